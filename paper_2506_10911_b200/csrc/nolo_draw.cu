@@ -6,6 +6,7 @@
 // counter = (i, boundary, slot, domain) and key = (seed, step); the permutation lists the
 // indices in ascending (key, index) order.  Integer arithmetic only, so the tables are
 // reproducible bit for bit on any machine.
+#include "nolo_draw.cuh"
 #include "nolo_internal.h"
 #include "nolo_philox.cuh"
 
@@ -13,32 +14,23 @@ namespace nolo {
 
 namespace {
 
-constexpr int kDrawThreads = 256;
-
-// One CTA per permutation.  Keys live in shared memory; element i's position is the number of
-// elements that sort before it (rank by counting: N <= 4096, so N^2 compares are cheap and need
-// no sort network).
-__global__ void __launch_bounds__(kDrawThreads)
+// One CTA per permutation, one thread per element up to N = 1024 and four above.  Bound by latency:
+// the ten dependent rounds of a key (about 0.4 us), then five barriers.
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS)
 draw_perm_kernel(uint64_t seed, uint64_t step, uint64_t domain, int N, int first_boundary, int slots_drawn,
                  int slots_total, int32_t* __restrict__ table) {
-    extern __shared__ uint64_t keys[];
+    extern __shared__ uint64_t raw[];
     const int b = first_boundary + blockIdx.x / slots_drawn;
     const int s = blockIdx.x % slots_drawn;
-    for (int i = threadIdx.x; i < N; i += blockDim.x)
-        keys[i] = draw_key((uint64_t)i, (uint64_t)b, (uint64_t)s, domain, seed, step);
-    __syncthreads();
     const int k_lo = (slots_drawn == slots_total) ? s : 0;
     const int k_hi = (slots_drawn == slots_total) ? s + 1 : slots_total;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
-        const uint64_t ki = keys[i];
-        int rank = 0;
-        for (int j = 0; j < N; ++j) {
-            const uint64_t kj = keys[j];
-            rank += (kj < ki) || (kj == ki && j < i);
-        }
-        for (int k = k_lo; k < k_hi; ++k)
-            table[((int64_t)b * slots_total + k) * N + rank] = i;
-    }
+    rank_by_buckets<THREADS>(
+        reinterpret_cast<unsigned char*>(raw), N,
+        [&](int i) { return draw_key((uint64_t)i, (uint64_t)b, (uint64_t)s, domain, seed, step); },
+        [&](int i, int rank) {
+            for (int k = k_lo; k < k_hi; ++k) table[((int64_t)b * slots_total + k) * N + rank] = i;
+        });
 }
 
 }  // namespace
@@ -48,9 +40,15 @@ cudaError_t launch_draw_range(uint64_t seed, uint64_t step, int domain, int N, i
                               cudaStream_t stream) {
     const int blocks = boundaries * slots_drawn;
     if (blocks <= 0 || N <= 0) return cudaSuccess;
-    draw_perm_kernel<<<blocks, kDrawThreads, (size_t)N * sizeof(uint64_t), stream>>>(
-        seed, step, (uint64_t)domain, N, first_boundary, slots_drawn, slots_total, table);
-    return cudaGetLastError();
+    auto launch = [&](auto kernel, int threads) {
+        kernel<<<blocks, threads, draw_scratch_bytes(N, threads), stream>>>(
+            seed, step, (uint64_t)domain, N, first_boundary, slots_drawn, slots_total, table);
+        return cudaGetLastError();
+    };
+    if (N <= 32) return launch(draw_perm_kernel<32>, 32);
+    if (N <= 128) return launch(draw_perm_kernel<128>, 128);
+    if (N <= 512) return launch(draw_perm_kernel<512>, 512);
+    return launch(draw_perm_kernel<1024>, 1024);
 }
 
 cudaError_t launch_draw(uint64_t seed, uint64_t step, int domain, int N, int boundaries,

@@ -69,6 +69,18 @@ def test_subgroup_tables_bit_exact(nolo, W, n):
     nolo.nolo_destroy(h)
 
 
+@pytest.mark.parametrize("W", [31, 32, 33, 127, 128, 129, 511, 512, 513, 1023, 1024, 1025, 2049, 4095, 4096])
+def test_permutation_draw_at_cta_size_boundaries(nolo, W):
+    """The draw uses CTAs of 32, 128, 512 and 1024 threads with up to four elements per thread."""
+    phi, theta, delta = (x.cuda() for x in synth.make_state(W, 8, 0))
+    h = nolo.nolo_create(W, 1, 8, 1, *F)
+    nolo.nolo_bind_state(h, phi, theta, delta)
+    for seed, step in [(3, 1), (2**64 - 1, 7)]:
+        nolo.nolo_outer_step(h, seed, step)
+        assert np.array_equal(nolo.nolo_get_groups(h), O.draw_groups(seed, step, W, 1))
+    nolo.nolo_destroy(h)
+
+
 # -------------------------------------------------------------- outer step
 
 def test_config1_full(nolo):
