@@ -44,6 +44,7 @@ struct KArgs {
     int64_t stride;
     int64_t P;
     int n;
+    int tail;                 // two-pass kernel, 1 when P % 4 != 0: the first CTA of every subgroup takes those columns
     float alpha, beta_over_n, gamma, inv_n, n_f;
     double inv_n_d;
 };
@@ -198,6 +199,68 @@ __device__ void scalar_tail(const KArgs& a, int g) {
     }
 }
 
+// Columns P - (P % 4) .. P-1 of one subgroup, element by element with float64 sums (rows are only
+// guaranteed to be padded to a multiple of 8, and padding must not be written).  Done by a CTA of its
+// own, the first of the subgroup: four neighbouring threads per member, so a pass over the members is
+// one or a few loads in flight per thread.  One thread walking the members column by column is a
+// serial chain of loads; one CTA is not: 3 extra columns cost 7.7 us before and nothing measurable now
+// at n = 20 (73.5 -> 67.4 us for W = 60, P = 2^18 + 3), 197 us at n = 256, 1.42 ms at n = 1024 (2531 ->
+// 1056 us for P = 2^18 + 3).
+template <typename ThetaT, int THREADS>
+__device__ __forceinline__ void ragged_tail(const KArgs& a, int g) {
+    constexpr int VEC = 4, WARPS = THREADS / 32, ROWS = THREADS / VEC;
+    __shared__ double2 part[WARPS][VEC];
+    const int n = a.n;
+    const int32_t* members = a.perm + (int64_t)g * n;
+    const int64_t c = (a.P & ~int64_t(VEC - 1)) + threadIdx.x % VEC;
+    const int first = threadIdx.x / VEC;
+    const bool mine = c < a.P;
+    double sD = 0.0, sP = 0.0;
+    if (mine) {
+#pragma unroll 4
+        for (int j = first; j < n; j += ROWS) {
+            const int64_t at = (int64_t)__ldg(members + j) * a.stride + c;
+            const float p = a.phi[at];
+            sD += (double)(p - load_theta1(static_cast<const ThetaT*>(a.theta), at));
+            sP += (double)p;
+        }
+    }
+#pragma unroll
+    for (int o = VEC; o < 32; o <<= 1) {
+        sD += __shfl_xor_sync(0xffffffffu, sD, o);
+        sP += __shfl_xor_sync(0xffffffffu, sP, o);
+    }
+    if ((threadIdx.x & 31) < VEC) part[threadIdx.x >> 5][threadIdx.x % VEC] = make_double2(sD, sP);
+    __syncthreads();
+    if (!mine) return;
+    sD = sP = 0.0;
+#pragma unroll
+    for (int w = 0; w < WARPS; ++w) { sD += part[w][threadIdx.x % VEC].x; sP += part[w][threadIdx.x % VEC].y; }
+    const double mP = a.mean_phi ? a.mean_phi[(int64_t)g * a.mean_stride + c] : sP * a.inv_n_d;
+    for (int j0 = first; j0 < n; j0 += 4 * ROWS) {        // four rows in flight
+        float p[4], d[4];
+        int64_t at[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (j0 + i * ROWS < n) {
+                at[i] = (int64_t)__ldg(members + j0 + i * ROWS) * a.stride + c;
+                p[i] = a.phi[at[i]];
+                d[i] = a.delta[at[i]];
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (j0 + i * ROWS < n) {
+                float dn;
+                const float pn = update1(p[i], (float)((double)p[i] - mP), d[i], (float)sD, a, &dn);
+                a.phi[at[i]] = pn;
+                a.delta[at[i]] = dn;
+                store_theta1(static_cast<ThetaT*>(a.theta), at[i], pn);
+            }
+        }
+    }
+}
+
 // ---- n <= 8: register-resident, subgroup size N known at compile time --------------------
 //
 // Each thread handles ITEMS quads (4 consecutive parameters) of the tile, 256 quads apart, for all
@@ -316,8 +379,12 @@ outer_step_twopass_kernel(const KArgs a) {
     const int part = ROWQ >= 32 ? slot : (threadIdx.x >> 5);
     const int g = blockIdx.y;
     const int n = a.n;
+    if (a.tail && blockIdx.x == 0) {
+        ragged_tail<ThetaT, THREADS>(a, g);
+        return;
+    }
     const int32_t* members = a.perm + (int64_t)g * n;
-    const int64_t q = (int64_t)blockIdx.x * ROWQ + ql;
+    const int64_t q = (int64_t)(blockIdx.x - a.tail) * ROWQ + ql;
     const bool ok = q < (a.P >> 2);
 
     float4 sD = f4_zero();
@@ -413,7 +480,6 @@ outer_step_twopass_kernel(const KArgs a) {
             }
         }
     }
-    if ((a.P & 3) && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) scalar_tail<ThetaT>(a, g);
 }
 
 // ---- subgroup means of phi alone (first half of the split-phase step) ------------------------
@@ -444,7 +510,19 @@ group_mean_kernel(const float* __restrict__ phi, const int32_t* __restrict__ per
                   int64_t P, double* __restrict__ mean, int64_t mean_stride, double inv_n) {
     const int g = blockIdx.y;
     const int32_t* members = perm + (int64_t)g * n;
-    const int64_t q0 = (int64_t)blockIdx.x * (kThreads * ITEMS) + threadIdx.x;
+    const int tail = (P & 3) != 0;
+    if (tail && blockIdx.x == 0) {            // the partial quad, one warp per column
+        const int64_t c = (P & ~int64_t(3)) + (threadIdx.x >> 5);
+        if (c >= P) return;
+        double t = 0.0;
+#pragma unroll 4
+        for (int j = threadIdx.x & 31; j < n; j += 32) t += (double)phi[(int64_t)__ldg(members + j) * stride + c];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if ((threadIdx.x & 31) == 0) mean[(int64_t)g * mean_stride + c] = t * inv_n;
+        return;
+    }
+    const int64_t q0 = (int64_t)(blockIdx.x - tail) * (kThreads * ITEMS) + threadIdx.x;
     const int64_t quads = P >> 2;
     PairSum s[ITEMS];
 #pragma unroll
@@ -480,13 +558,6 @@ group_mean_kernel(const float* __restrict__ phi, const int32_t* __restrict__ per
                               ((double)s[it].hi.z + (double)s[it].lo.z) * inv_n, ((double)s[it].hi.w + (double)s[it].lo.w) * inv_n);
         }
     }
-    if ((P & 3) && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
-        for (int64_t c = P & ~int64_t(3); c < P; ++c) {
-            double t = 0.0;
-            for (int j = 0; j < n; ++j) t += (double)phi[(int64_t)members[j] * stride + c];
-            mean[(int64_t)g * mean_stride + c] = t * inv_n;
-        }
-    }
 }
 
 // ---- launches ---------------------------------------------------------------------------
@@ -513,8 +584,9 @@ cudaError_t launch_reg(const KArgs& k, int groups, cudaStream_t stream) {
 
 template <typename ThetaT, int THREADS, int ROWQ, int U, int MINB>
 cudaError_t launch_twopass(const KArgs& k, int groups, cudaStream_t stream) {
-    dim3 grid;
-    if (!tile_grid(k, ROWQ, groups, &grid)) return cudaErrorInvalidConfiguration;
+    const int64_t tiles = ((k.P >> 2) + ROWQ - 1) / ROWQ + k.tail;
+    if (tiles > 0x7fffffffll) return cudaErrorInvalidConfiguration;
+    const dim3 grid((unsigned)tiles, (unsigned)groups);
     outer_step_twopass_kernel<ThetaT, THREADS, ROWQ, U, MINB><<<grid, THREADS, 0, stream>>>(k);
     return cudaGetLastError();
 }
@@ -559,9 +631,8 @@ cudaError_t launch_group_mean(const float* phi, const int32_t* perm, int W, int 
                               double* mean, int64_t mean_stride, cudaStream_t stream) {
     if (P <= 0 || W <= 0) return cudaSuccess;
     const int items = n <= 4 ? 2 : 1;
-    const int64_t quads = (P + 3) >> 2;
     const int64_t per_cta = (int64_t)kThreads * items;
-    const int64_t tiles = (quads + per_cta - 1) / per_cta;
+    const int64_t tiles = ((P >> 2) + per_cta - 1) / per_cta + ((P & 3) != 0);
     const int groups = W / n;
     if (tiles > 0x7fffffffll || groups > 65535) return cudaErrorInvalidConfiguration;
     dim3 grid((unsigned)tiles, (unsigned)groups);
@@ -580,6 +651,7 @@ cudaError_t launch_outer(const OuterArgs& a, cudaStream_t stream) {
     k.phi = a.phi; k.theta = a.theta; k.delta = a.delta; k.perm = a.perm;
     k.mean_phi = a.mean_phi; k.mean_stride = a.mean_stride;
     k.stride = a.stride; k.P = a.P; k.n = a.n;
+    k.tail = (a.P & 3) != 0;
     k.alpha = a.alpha; k.gamma = a.gamma;
     k.beta_over_n = a.beta / (float)a.n;
     k.inv_n = 1.0f / (float)a.n;

@@ -118,6 +118,13 @@ def test_small_and_odd_P(nolo, P, bf16):
     run_both(nolo, 6, 3, P, 1, 2, dt)
 
 
+@pytest.mark.parametrize("n", [2, 8, 12, 31, 32, 33, 64, 65, 128, 129, 300, 1024])
+@pytest.mark.parametrize("P", [1, 6, 1021])
+def test_ragged_columns(nolo, n, P):
+    """P % 4 columns are done by a CTA of their own with 32, 64 or 128 members in flight."""
+    run_both(nolo, 2 * n, n, P, 6, 9, torch.bfloat16 if P == 6 else torch.float32)
+
+
 @pytest.mark.parametrize("hp", [(0.0, 0.0, 1.0), (0.3, 0.7, 0.0), (0.9, 1.0, 1.5), (0.5, 0.7, 0.0)])
 def test_hyperparameter_corners(nolo, hp):
     hp = tuple(float(np.float32(x)) for x in hp)
