@@ -65,10 +65,7 @@ WORKLOADS = [
 # of the same kernel (dram__bytes_read.sum + dram__bytes_write.sum over the worker-parameters of
 # the captured launch); traffic grows in proportion to the columns processed.  None = not captured
 # since the kernel last changed.
-PROFILED_DRAM_BYTES_PER_PARAM = {
-    "outer_step_reg_kernel<2,bf16,1>": 2.627498e9 / (16 * 8388608),     # 19.58
-    "outer_step_reg_kernel<4,float,1>": 1.553978e9 / (8 * 8388608),      # 23.16
-}
+PROFILED_DRAM_BYTES_PER_PARAM = {}
 
 
 def bytes_per_param(theta: str) -> int:
@@ -79,8 +76,7 @@ def bytes_per_param(theta: str) -> int:
 def kernel_name(n: int, theta: str) -> str:
     t = "bf16" if theta == "bf16" else "float"
     if n <= 8:
-        items = 4 if n == 1 else (2 if (n == 2 and theta != "bf16") else 1)
-        return f"outer_step_reg_kernel<{n},{t},{items}>"
+        return f"outer_step_reg_kernel<{n},{t}>"
     shape = ("128 threads,128 quads,4 rows" if n <= 12 else "128 threads,64 quads,8 rows" if n <= 24 else
              "256 threads,64 quads,4 rows" if n <= 64 else "256 threads,64 quads,8 rows" if n <= 96 else
              "256 threads,32 quads,4 rows" if n <= 128 else "256 threads,32 quads,8 rows" if n <= 224 else

@@ -1,7 +1,7 @@
 // Fused NoLoCo outer step (Section 3.2, Eq. 1-3) for W workers resident in one GPU's memory.
 //
 // Work decomposition: one CTA owns one subgroup x one tile of parameters.  Every member's
-// phi / theta / delta element is fetched from HBM exactly once (128-bit coalesced, streaming
+// phi / theta / delta element is fetched from HBM exactly once (128- or 256-bit coalesced, streaming
 // cache policy) and every output element stored exactly once; the pseudo-gradients, their sum
 // and the subgroup mean of phi exist only on chip.  The path is bandwidth bound (about 15 flops
 // per 20-24 bytes), so there is no tensor-core work here.
@@ -12,7 +12,7 @@
 //   theta_i' = phi_i'   (start of the next inner phase)
 //
 // Two kernels cover the subgroup sizes:
-//   n <= 8        register-resident: one thread holds its quad of every member;
+//   n <= 8        register-resident: one thread holds its oct of every member;
 //   n > 8         two passes over the members, the second read of phi served by L1/L2.
 //
 // Arithmetic.  Delta_j is formed per member and summed in float32 in short fixed-order partial
@@ -32,7 +32,7 @@ namespace nolo {
 
 namespace {
 
-constexpr int kThreads = 256;   // CTA size of the register-resident kernel and of the helpers
+constexpr int kThreads = 256;   // CTA size of the subgroup-mean kernel
 
 struct KArgs {
     float* phi;
@@ -44,7 +44,7 @@ struct KArgs {
     int64_t stride;
     int64_t P;
     int n;
-    int tail;                 // two-pass kernel, 1 when P % 4 != 0: the first CTA of every subgroup takes those columns
+    int tail;                 // 1 when P is no multiple of a thread's columns: the first CTA of every subgroup takes the rest
     float alpha, beta_over_n, gamma, inv_n, n_f;
     double inv_n_d;
 };
@@ -54,9 +54,6 @@ __device__ __forceinline__ void f4_add(float4& s, const float4 v) {
 }
 __device__ __forceinline__ float4 f4_sub(const float4 a, const float4 b) {
     return make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w);
-}
-__device__ __forceinline__ float4 f4_scale(const float4 a, const float s) {
-    return make_float4(a.x * s, a.y * s, a.z * s, a.w * s);
 }
 __device__ __forceinline__ float4 f4_zero() { return make_float4(0.f, 0.f, 0.f, 0.f); }
 
@@ -146,6 +143,76 @@ __device__ __forceinline__ void store_theta1(__nv_bfloat16* row, int64_t c, floa
     row[c] = __float2bfloat16_rn(v);
 }
 
+// ---- 8 consecutive parameters -------------------------------------------------------------
+//
+// WIDE: one 256-bit access (rows are 32-byte aligned); else two 128-bit ones.
+struct Oct { float v[8]; };
+
+template <bool WIDE>
+__device__ __forceinline__ Oct load8(const float* p) {
+    Oct o;
+    if constexpr (WIDE) {
+        asm volatile("ld.global.cs.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                     : "=f"(o.v[0]), "=f"(o.v[1]), "=f"(o.v[2]), "=f"(o.v[3]), "=f"(o.v[4]), "=f"(o.v[5]), "=f"(o.v[6]),
+                       "=f"(o.v[7])
+                     : "l"(p));
+    } else {
+        const float4 x = __ldcs(reinterpret_cast<const float4*>(p)), y = __ldcs(reinterpret_cast<const float4*>(p) + 1);
+        o.v[0] = x.x; o.v[1] = x.y; o.v[2] = x.z; o.v[3] = x.w;
+        o.v[4] = y.x; o.v[5] = y.y; o.v[6] = y.z; o.v[7] = y.w;
+    }
+    return o;
+}
+template <bool WIDE>
+__device__ __forceinline__ void store8(float* p, const Oct& o) {
+    if constexpr (WIDE) {
+        asm volatile("st.global.cs.v8.f32 [%8], {%0, %1, %2, %3, %4, %5, %6, %7};" ::"f"(o.v[0]), "f"(o.v[1]), "f"(o.v[2]),
+                     "f"(o.v[3]), "f"(o.v[4]), "f"(o.v[5]), "f"(o.v[6]), "f"(o.v[7]), "l"(p)
+                     : "memory");
+    } else {
+        __stcs(reinterpret_cast<float4*>(p), make_float4(o.v[0], o.v[1], o.v[2], o.v[3]));
+        __stcs(reinterpret_cast<float4*>(p) + 1, make_float4(o.v[4], o.v[5], o.v[6], o.v[7]));
+    }
+}
+template <typename ThetaT> struct ThetaOct { using type = Oct; };
+template <> struct ThetaOct<__nv_bfloat16> { using type = uint4; };
+template <bool WIDE>
+__device__ __forceinline__ Oct load_theta8(const float* p) { return load8<WIDE>(p); }
+template <bool WIDE>
+__device__ __forceinline__ uint4 load_theta8(const __nv_bfloat16* p) { return __ldcs(reinterpret_cast<const uint4*>(p)); }
+__device__ __forceinline__ float widened(const Oct& o, int e) { return o.v[e]; }
+__device__ __forceinline__ float widened(const uint4& o, int e) {
+    const uint32_t w = e < 2 ? o.x : e < 4 ? o.y : e < 6 ? o.z : o.w;
+    return __uint_as_float(e & 1 ? w & 0xffff0000u : w << 16);
+}
+template <bool WIDE>
+__device__ __forceinline__ void store_theta8(float* p, const Oct& o) { store8<WIDE>(p, o); }
+template <bool WIDE>
+__device__ __forceinline__ void store_theta8(__nv_bfloat16* p, const Oct& o) {
+    uint32_t w[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const __nv_bfloat162 b = __floats2bfloat162_rn(o.v[2 * i], o.v[2 * i + 1]);   // round to nearest even
+        w[i] = *reinterpret_cast<const uint32_t*>(&b);
+    }
+    __stcs(reinterpret_cast<uint4*>(p), make_uint4(w[0], w[1], w[2], w[3]));
+}
+template <bool WIDE>
+__device__ __forceinline__ void load_means8(double (&m)[8], const double* p) {
+    if constexpr (WIDE) {
+#pragma unroll
+        for (int i = 0; i < 8; i += 4)
+            asm volatile("ld.global.nc.v4.f64 {%0, %1, %2, %3}, [%4];"
+                         : "=d"(m[i]), "=d"(m[i + 1]), "=d"(m[i + 2]), "=d"(m[i + 3]) : "l"(p + i));
+    } else {
+#pragma unroll
+        for (int i = 0; i < 8; i += 2) {
+            const double2 x = __ldg(reinterpret_cast<const double2*>(p + i));
+            m[i] = x.x; m[i + 1] = x.y;
+        }
+    }
+}
+
 // Eq. 2 and Eq. 3 for one parameter; dev = phi_i - mean phi.
 __device__ __forceinline__ float update1(float phi, float dev, float delta, float sum_Delta,
                                          const KArgs& a, float* delta_out) {
@@ -173,42 +240,16 @@ __device__ __forceinline__ void update_store(const KArgs& a, int64_t row_off, in
     store_theta4(static_cast<ThetaT*>(a.theta) + row_off, q, p);
 }
 
-// Columns P - (P % 4) .. P-1 of one subgroup, element by element in float64 (rows are only
-// guaranteed to be padded to a multiple of 8, and padding must not be written).
-template <typename ThetaT>
-__device__ void scalar_tail(const KArgs& a, int g) {
-    const int n = a.n;
-    for (int64_t c = a.P & ~int64_t(3); c < a.P; ++c) {
-        double sD = 0.0, sP = 0.0;
-        for (int j = 0; j < n; ++j) {
-            const int64_t row = (int64_t)a.perm[g * n + j] * a.stride;
-            const float p = a.phi[row + c];
-            sD += (double)(p - load_theta1(static_cast<const ThetaT*>(a.theta) + row, c));
-            sP += (double)p;
-        }
-        const double mP = a.mean_phi ? a.mean_phi[(int64_t)g * a.mean_stride + c] : sP * a.inv_n_d;
-        for (int j = 0; j < n; ++j) {
-            const int64_t row = (int64_t)a.perm[g * n + j] * a.stride;
-            float d;
-            const float p0 = a.phi[row + c];
-            const float p = update1(p0, (float)((double)p0 - mP), a.delta[row + c], (float)sD, a, &d);
-            a.phi[row + c] = p;
-            a.delta[row + c] = d;
-            store_theta1(static_cast<ThetaT*>(a.theta) + row, c, p);
-        }
-    }
-}
-
-// Columns P - (P % 4) .. P-1 of one subgroup, element by element with float64 sums (rows are only
-// guaranteed to be padded to a multiple of 8, and padding must not be written).  Done by a CTA of its
-// own, the first of the subgroup: four neighbouring threads per member, so a pass over the members is
-// one or a few loads in flight per thread.  One thread walking the members column by column is a
-// serial chain of loads; one CTA is not: 3 extra columns cost 7.7 us before and nothing measurable now
-// at n = 20 (73.5 -> 67.4 us for W = 60, P = 2^18 + 3), 197 us at n = 256, 1.42 ms at n = 1024 (2531 ->
-// 1056 us for P = 2^18 + 3).
-template <typename ThetaT, int THREADS>
+// Columns P - (P % VEC) .. P-1 of one subgroup (a thread has VEC columns elsewhere), element by element
+// with float64 sums (rows are only guaranteed to be padded to a multiple of 8, and padding must not be
+// written).  Done by a CTA of its own, the first of the subgroup: VEC neighbouring threads per member, so
+// a pass over the members is one or a few loads in flight per thread.  One thread walking the members
+// column by column is a serial chain of loads; one CTA is not: 3 extra columns cost 7.7 us before and
+// nothing measurable now at n = 20 (73.5 -> 67.4 us for W = 60, P = 2^18 + 3), 197 us at n = 256, 1.42 ms
+// at n = 1024 (2531 -> 1056 us for P = 2^18 + 3).
+template <typename ThetaT, int THREADS, int VEC>
 __device__ __forceinline__ void ragged_tail(const KArgs& a, int g) {
-    constexpr int VEC = 4, WARPS = THREADS / 32, ROWS = THREADS / VEC;
+    constexpr int WARPS = THREADS / 32, ROWS = THREADS / VEC;
     __shared__ double2 part[WARPS][VEC];
     const int n = a.n;
     const int32_t* members = a.perm + (int64_t)g * n;
@@ -263,71 +304,72 @@ __device__ __forceinline__ void ragged_tail(const KArgs& a, int g) {
 
 // ---- n <= 8: register-resident, subgroup size N known at compile time --------------------
 //
-// Each thread handles ITEMS quads (4 consecutive parameters) of the tile, 256 quads apart, for all
-// N members: phi_j stays in registers between the reduction and the update, so nothing is read
-// twice.  All loads of a thread are issued before the first use to keep many bytes in flight.
-// ITEMS = 4 for n = 1, 2 for pairs with float32 theta, 1 otherwise (chosen by measurement).
-template <int N, typename ThetaT, int ITEMS, bool PREPARED>
-__global__ void __launch_bounds__(kThreads, 1)
+// Each thread handles one oct (8 consecutive parameters) for all N members: phi_j stays in registers
+// between the reduction and the update, so nothing is read twice.  All loads of a thread are issued
+// before the first use to keep many bytes in flight.
+//
+// Bound by DRAM.  256-bit accesses make a row piece of one warp 1 KB long and halve the requests; against
+// quads in 128-bit accesses (256 threads) the rate rises with what is in flight per thread.  GB/s at W = 16,
+// P = 2^25, float32 / bfloat16 theta, quads -> octs: n = 1 6864 / 6800 -> 6905 / 6870, n = 2 6822 / 6824 -> 6923 /
+// 6850, n = 4 6770 / 6737 -> 6862 / 6800, n = 6 6521 / 6670 -> 6831 / 6695, n = 7 6673 / 6378 -> 6834 / 6740, n = 8
+// 6711 / 5568 -> 6828 / 6739; with prepared means n = 2 5988 / 6830 -> 6985 / 6976, n = 4 6655 -> 6890 (float32).
+// (The quad kernel with n = 7 and 8 left one CTA of 256 threads per SM.)
+template <int N, typename ThetaT, int THREADS, bool PREPARED, bool WIDE>
+__global__ void __launch_bounds__(THREADS, 1)
 outer_step_reg_kernel(const KArgs a) {
     const int g = blockIdx.y;
-    const int64_t full_quads = a.P >> 2;
-    const int64_t q0 = (int64_t)blockIdx.x * (kThreads * ITEMS) + threadIdx.x;
+    if (a.tail && blockIdx.x == 0) {
+        ragged_tail<ThetaT, THREADS, 8>(a, g);
+        return;
+    }
+    const int64_t c = ((int64_t)(blockIdx.x - a.tail) * THREADS + threadIdx.x) * 8;
+    if (c + 8 > a.P) return;
 
-    int row[N];
+    int64_t at[N];
 #pragma unroll
-    for (int j = 0; j < N; ++j) row[j] = __ldg(a.perm + g * N + j);
-    auto phi_row = [&](int j) { return a.phi + (int64_t)row[j] * a.stride; };
-    auto delta_row = [&](int j) { return a.delta + (int64_t)row[j] * a.stride; };
-    auto theta_row = [&](int j) { return static_cast<ThetaT*>(a.theta) + (int64_t)row[j] * a.stride; };
-
-    float4 phi[ITEMS][N], dlt[ITEMS][N];
-    typename ThetaRaw<ThetaT>::type the[ITEMS][N];
-    bool ok[ITEMS];
+    for (int j = 0; j < N; ++j) at[j] = (int64_t)__ldg(a.perm + g * N + j) * a.stride + c;
+    Oct phi[N], dlt[N];
+    typename ThetaOct<ThetaT>::type the[N];
 #pragma unroll
-    for (int it = 0; it < ITEMS; ++it) {
-        const int64_t q = q0 + (int64_t)it * kThreads;
-        ok[it] = q < full_quads;
-        if (ok[it]) {
-#pragma unroll
-            for (int j = 0; j < N; ++j) {
-                phi[it][j] = __ldcs(reinterpret_cast<const float4*>(phi_row(j)) + q);
-                the[it][j] = load_theta_raw(theta_row(j), q);
-            }
-#pragma unroll
-            for (int j = 0; j < N; ++j)
-                dlt[it][j] = __ldcs(reinterpret_cast<const float4*>(delta_row(j)) + q);
-        }
+    for (int j = 0; j < N; ++j) {
+        phi[j] = load8<WIDE>(a.phi + at[j]);
+        the[j] = load_theta8<WIDE>(static_cast<const ThetaT*>(a.theta) + at[j]);
     }
 #pragma unroll
-    for (int it = 0; it < ITEMS; ++it) {
-        if (!ok[it]) continue;
-        const int64_t q = q0 + (int64_t)it * kThreads;
+    for (int j = 0; j < N; ++j) dlt[j] = load8<WIDE>(a.delta + at[j]);
+    double mean[PREPARED ? 8 : 1];
+    if constexpr (PREPARED) load_means8<WIDE>(mean, a.mean_phi + (int64_t)g * a.mean_stride + c);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
         // Sums in the fixed member order (deterministic).  The mean of phi is formed in two
         // passes over the registers: a plain float32 mean, then the mean of the residuals
         // phi_j - mean, so that hi + lo keeps the precision of the spread of the replicas.
-        float4 sD = f4_zero(), s0 = f4_zero();
+        float sD = 0.f, s0 = 0.f, hi, lo;
 #pragma unroll
         for (int j = 0; j < N; ++j) {
-            f4_add(sD, f4_sub(phi[it][j], widen(the[it][j])));          // Eq. 1
-            f4_add(s0, phi[it][j]);
+            sD += phi[j].v[e] - widened(the[j], e);                      // Eq. 1
+            s0 += phi[j].v[e];
         }
-        PairSum mean;
-        if (PREPARED) {
-            mean = load_prepared_mean(a, g, q);
+        if constexpr (PREPARED) {
+            hi = (float)mean[e];
+            lo = (float)(mean[e] - (double)hi);
         } else {
-            mean.hi = f4_scale(s0, a.inv_n);
-            float4 sR = f4_zero();
+            hi = s0 * a.inv_n;
+            float sR = 0.f;
 #pragma unroll
-            for (int j = 0; j < N; ++j) f4_add(sR, f4_sub(phi[it][j], mean.hi));
-            mean.lo = f4_scale(sR, a.inv_n);
+            for (int j = 0; j < N; ++j) sR += phi[j].v[e] - hi;
+            lo = sR * a.inv_n;
         }
 #pragma unroll
         for (int j = 0; j < N; ++j)
-            update_store<ThetaT>(a, (int64_t)row[j] * a.stride, q, phi[it][j], mean.deviation(phi[it][j]),
-                                 dlt[it][j], sD);
+            phi[j].v[e] = update1(phi[j].v[e], (phi[j].v[e] - hi) - lo, dlt[j].v[e], sD, a, &dlt[j].v[e]);
     }
-    if ((a.P & 3) && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) scalar_tail<ThetaT>(a, g);
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+        store8<WIDE>(a.phi + at[j], phi[j]);
+        store8<WIDE>(a.delta + at[j], dlt[j]);
+        store_theta8<WIDE>(static_cast<ThetaT*>(a.theta) + at[j], phi[j]);
+    }
 }
 
 // ---- n > 8: two passes over the members, the second read of phi served by L1 / L2 ----------
@@ -380,7 +422,7 @@ outer_step_twopass_kernel(const KArgs a) {
     const int g = blockIdx.y;
     const int n = a.n;
     if (a.tail && blockIdx.x == 0) {
-        ragged_tail<ThetaT, THREADS>(a, g);
+        ragged_tail<ThetaT, THREADS, 4>(a, g);
         return;
     }
     const int32_t* members = a.perm + (int64_t)g * n;
@@ -562,31 +604,55 @@ group_mean_kernel(const float* __restrict__ phi, const int32_t* __restrict__ per
 
 // ---- launches ---------------------------------------------------------------------------
 
-// Tiles of `quads_per_cta` quads; a trailing partial quad still needs a CTA for the scalar tail.
-bool tile_grid(const KArgs& k, int64_t quads_per_cta, int groups, dim3* grid) {
-    const int64_t quads = (k.P + 3) >> 2;
-    const int64_t tiles = (quads + quads_per_cta - 1) / quads_per_cta;
+// Tiles of `cols_per_cta` columns (whole vectors of `vec` columns per thread), and one more CTA for
+// the columns that are left over.
+bool tile_grid(KArgs& k, int vec, int64_t cols_per_cta, int groups, dim3* grid) {
+    k.tail = k.P % vec != 0;
+    const int64_t tiles = (k.P - k.P % vec + cols_per_cta - 1) / cols_per_cta + k.tail;
     if (tiles > 0x7fffffffll) return false;
     *grid = dim3((unsigned)tiles, (unsigned)groups);
     return true;
 }
 
-template <int N, typename ThetaT, int ITEMS>
-cudaError_t launch_reg(const KArgs& k, int groups, cudaStream_t stream) {
+bool aligned32(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 31u) == 0; }
+
+template <int N, typename ThetaT, int THREADS, bool WIDE>
+cudaError_t launch_reg_shape(KArgs& k, int groups, cudaStream_t stream) {
     dim3 grid;
-    if (!tile_grid(k, (int64_t)kThreads * ITEMS, groups, &grid)) return cudaErrorInvalidConfiguration;
+    if (!tile_grid(k, 8, (int64_t)THREADS * 8, groups, &grid)) return cudaErrorInvalidConfiguration;
     if (k.mean_phi)
-        outer_step_reg_kernel<N, ThetaT, ITEMS, true><<<grid, kThreads, 0, stream>>>(k);
+        outer_step_reg_kernel<N, ThetaT, THREADS, true, WIDE><<<grid, THREADS, 0, stream>>>(k);
     else
-        outer_step_reg_kernel<N, ThetaT, ITEMS, false><<<grid, kThreads, 0, stream>>>(k);
+        outer_step_reg_kernel<N, ThetaT, THREADS, false, WIDE><<<grid, THREADS, 0, stream>>>(k);
     return cudaGetLastError();
 }
 
+// Larger CTAs stream longer pieces of a row and are the faster by up to 0.7 % where there are many octs
+// (n = 2 float32, 256 against 64 threads: 6912 / 6880 GB/s at 8.4 GB of phi, equal at 2^19 octs); below that
+// the ends of the grid weigh more (16.8 / 16.4 us at W = 4, P = 2^20).  The sizes are those that hold
+// their rate under the power cap as well, where the SM clock drops by a tenth: pairs with bfloat16 theta at
+// P = 123e6, W = 16, 320 threads 5757 us, 256 5777, 384 5765, 512 5748 at full clock but 5800 capped (the quad
+// kernel 5775).  With more than 4 members a thread needs the registers that 64-thread CTAs leave it.
+constexpr int64_t kRegManyOcts = 1 << 19;
+template <int N, typename ThetaT>
+constexpr int kRegThreads = N == 4 ? 192 : (N == 2 && sizeof(ThetaT) == 2) ? 320 : 256;
+
+template <int N, typename ThetaT>
+cudaError_t launch_reg(KArgs& k, int groups, cudaStream_t stream) {
+    // the strides are multiples of 32 bytes (of 16 for bfloat16 theta, which is read 16 bytes at a time)
+    const bool wide = aligned32(k.phi) && aligned32(k.delta) && (sizeof(ThetaT) == 2 || aligned32(k.theta)) &&
+                      aligned32(k.mean_phi);
+    if (!wide) return launch_reg_shape<N, ThetaT, 64, false>(k, groups, stream);
+    if constexpr (N <= 4) {
+        if (k.P / 8 * groups >= kRegManyOcts) return launch_reg_shape<N, ThetaT, kRegThreads<N, ThetaT>, true>(k, groups, stream);
+    }
+    return launch_reg_shape<N, ThetaT, 64, true>(k, groups, stream);
+}
+
 template <typename ThetaT, int THREADS, int ROWQ, int U, int MINB>
-cudaError_t launch_twopass(const KArgs& k, int groups, cudaStream_t stream) {
-    const int64_t tiles = ((k.P >> 2) + ROWQ - 1) / ROWQ + k.tail;
-    if (tiles > 0x7fffffffll) return cudaErrorInvalidConfiguration;
-    const dim3 grid((unsigned)tiles, (unsigned)groups);
+cudaError_t launch_twopass(KArgs& k, int groups, cudaStream_t stream) {
+    dim3 grid;
+    if (!tile_grid(k, 4, (int64_t)ROWQ * 4, groups, &grid)) return cudaErrorInvalidConfiguration;
     outer_step_twopass_kernel<ThetaT, THREADS, ROWQ, U, MINB><<<grid, THREADS, 0, stream>>>(k);
     return cudaGetLastError();
 }
@@ -602,17 +668,16 @@ constexpr int kTwoPassMaxN32Quads = 224;  // 256 x 32 x 8, 2 CTAs
 constexpr int kTwoPassMaxN8Warps = 640;   // 256 x 16 x 8, 2 CTAs; above: 512 x 16 x 8, 1 CTA
 
 template <typename ThetaT>
-cudaError_t dispatch(const KArgs& k, int groups, cudaStream_t stream) {
+cudaError_t dispatch(KArgs& k, int groups, cudaStream_t stream) {
     switch (k.n) {
-        case 1:  return launch_reg<1, ThetaT, 4>(k, groups, stream);
-        // pairs: 2 quads per thread with fp32 theta, 1 with bf16 theta measured best (+0.7 %)
-        case 2:  return launch_reg<2, ThetaT, (sizeof(ThetaT) == 4) ? 2 : 1>(k, groups, stream);
-        case 3:  return launch_reg<3, ThetaT, 1>(k, groups, stream);
-        case 4:  return launch_reg<4, ThetaT, 1>(k, groups, stream);
-        case 5:  return launch_reg<5, ThetaT, 1>(k, groups, stream);
-        case 6:  return launch_reg<6, ThetaT, 1>(k, groups, stream);
-        case 7:  return launch_reg<7, ThetaT, 1>(k, groups, stream);
-        case 8:  return launch_reg<8, ThetaT, 1>(k, groups, stream);
+        case 1:  return launch_reg<1, ThetaT>(k, groups, stream);
+        case 2:  return launch_reg<2, ThetaT>(k, groups, stream);
+        case 3:  return launch_reg<3, ThetaT>(k, groups, stream);
+        case 4:  return launch_reg<4, ThetaT>(k, groups, stream);
+        case 5:  return launch_reg<5, ThetaT>(k, groups, stream);
+        case 6:  return launch_reg<6, ThetaT>(k, groups, stream);
+        case 7:  return launch_reg<7, ThetaT>(k, groups, stream);
+        case 8:  return launch_reg<8, ThetaT>(k, groups, stream);
         default: break;
     }
     if (k.n <= kTwoPassMaxN1Slot) return launch_twopass<ThetaT, 128, 128, 4, 6>(k, groups, stream);
@@ -651,7 +716,6 @@ cudaError_t launch_outer(const OuterArgs& a, cudaStream_t stream) {
     k.phi = a.phi; k.theta = a.theta; k.delta = a.delta; k.perm = a.perm;
     k.mean_phi = a.mean_phi; k.mean_stride = a.mean_stride;
     k.stride = a.stride; k.P = a.P; k.n = a.n;
-    k.tail = (a.P & 3) != 0;
     k.alpha = a.alpha; k.gamma = a.gamma;
     k.beta_over_n = a.beta / (float)a.n;
     k.inv_n = 1.0f / (float)a.n;

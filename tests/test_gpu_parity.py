@@ -125,6 +125,53 @@ def test_ragged_columns(nolo, n, P):
     run_both(nolo, 2 * n, n, P, 6, 9, torch.bfloat16 if P == 6 else torch.float32)
 
 
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 5, 8])
+@pytest.mark.parametrize("bf16", [False, True])
+def test_rows_only_16_byte_aligned(nolo, n, bf16):
+    """Subgroups of up to 8 use 256-bit accesses where rows are 32-byte aligned, 128-bit ones elsewhere:
+    the same bits from either."""
+    W, P, stride = 2 * n, 2048 + 5, 2064
+    state = [x.cuda() for x in synth.make_state(W, P, 2, torch.bfloat16 if bf16 else torch.float32, stride=stride)]
+    results = []
+    for shift_bytes in (0, 16):
+        views = []
+        for x in state:
+            big = torch.zeros(W * stride + 16, dtype=x.dtype, device="cuda")
+            off = shift_bytes // x.element_size()
+            v = big[off:off + W * stride].view(W, stride)
+            v.copy_(x)
+            views.append(v)
+        h = nolo.nolo_create(W, n, P, 1, *F)
+        nolo.nolo_bind_state(h, *views)
+        nolo.nolo_outer_step(h, 3, 2)
+        torch.cuda.synchronize()
+        nolo.nolo_destroy(h)
+        results.append(views)
+    for a, b in zip(*results):
+        assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 4])
+@pytest.mark.parametrize("bf16", [False, True])
+def test_cta_sizes_agree(nolo, n, bf16):
+    """Large states of small subgroups run in CTAs of 192 to 320 threads, others in 64: the same columns give
+    the same bits through either.  The first 9000 columns go through a handle of their own."""
+    W = 16 * n
+    P = (1 << 19) * 8 // 16 + 4099
+    phi = torch.empty((W, P // 8 * 8 + 8), device="cuda").uniform_(-0.05, 0.05)
+    theta = (phi + 1e-3 * torch.randn_like(phi)).to(torch.bfloat16 if bf16 else torch.float32)
+    delta = 1e-4 * torch.randn_like(phi)
+    small = [x[:, :9008].clone() for x in (phi, theta, delta)]
+    for state, cols in (((phi, theta, delta), P), (small, 9000)):
+        h = nolo.nolo_create(W, n, cols, 1, *F)
+        nolo.nolo_bind_state(h, *state)
+        nolo.nolo_outer_step(h, 5, 6)
+        torch.cuda.synchronize()
+        nolo.nolo_destroy(h)
+    for a, b in zip((phi, theta, delta), small):
+        assert torch.equal(a[:, :9000], b[:, :9000])
+
+
 @pytest.mark.parametrize("hp", [(0.0, 0.0, 1.0), (0.3, 0.7, 0.0), (0.9, 1.0, 1.5), (0.5, 0.7, 0.0)])
 def test_hyperparameter_corners(nolo, hp):
     hp = tuple(float(np.float32(x)) for x in hp)
