@@ -365,7 +365,10 @@ int nolo_copy_probe(const void* src, void* dst, int64_t bytes, int iters, void* 
  * Device-time instrumentation.  With enable != 0 every later launch of the
  * fused outer-step kernel, the routing copy kernel, the divergence kernels and the
  * subgroup-mean kernel of nolo_outer_prepare is bracketed by CUDA
- * events on the bound stream (up to 4096 launches per kernel between reads).
+ * events on the bound stream (up to 4096 launches per kernel between reads).  So
+ * that these times are those of the data kernels alone, permutations are then
+ * drawn by kernels of their own at every size (small calls draw them inside the
+ * data kernel otherwise).
  * nolo_timing_read synchronises the stream, returns the summed device time in
  * milliseconds and the number of bracketed launches of `kernel`
  * (NOLO_KERNEL_OUTER / _ROUTE / _DIVERGENCE / _PREPARE) since the last read, and resets them.

@@ -128,7 +128,18 @@ struct Bracket {
     }
 };
 
-int enqueue_outer(nolo_handle* h, int64_t col0, int64_t cols, bool prepared = false) {
+int enqueue_group_draw(nolo_handle* h, uint64_t seed, uint64_t step) {
+    NOLO_CUDA(h, nolo::launch_draw(seed, step, nolo::kDomainGroups, h->W, 1, 1, 1, h->d_perm, h->stream));
+    ++h->launches;
+    return NOLO_OK;
+}
+
+// The outer step over columns [col0, col0 + cols).  draw: (seed, step) of a partition that is still to be
+// drawn; NULL when the table is there.
+struct Draw {
+    uint64_t seed, step;
+};
+int enqueue_outer(nolo_handle* h, int64_t col0, int64_t cols, const Draw* draw, bool prepared = false) {
     nolo::OuterArgs a;
     if (prepared) {
         a.mean_phi = h->mean_phi + col0;
@@ -144,18 +155,21 @@ int enqueue_outer(nolo_handle* h, int64_t col0, int64_t cols, bool prepared = fa
     a.n = h->n;
     a.theta_bf16 = h->theta_dtype == NOLO_BF16;
     a.alpha = h->alpha; a.beta = h->beta; a.gamma = h->gamma;
+    if (draw) {
+        a.seed = draw->seed;
+        a.step = draw->step;
+        a.draw = !h->timing && nolo::outer_draws(a);   // timed kernels do the same work at every size
+        if (!a.draw) {
+            const int rc = enqueue_group_draw(h, draw->seed, draw->step);
+            if (rc != NOLO_OK) return rc;
+        }
+    }
     Bracket br(h, NOLO_KERNEL_OUTER);
     NOLO_CUDA(h, nolo::launch_outer(a, h->stream));
     br.done();
     ++h->launches;
-    h->prepared_valid = false;   // phi has changed: means prepared from the old phi are stale
-    return NOLO_OK;
-}
-
-int enqueue_group_draw(nolo_handle* h, uint64_t seed, uint64_t step) {
-    NOLO_CUDA(h, nolo::launch_draw(seed, step, nolo::kDomainGroups, h->W, 1, 1, 1, h->d_perm, h->stream));
-    ++h->launches;
     h->groups_valid = true;
+    h->prepared_valid = false;   // phi has changed: means prepared from the old phi are stale
     return NOLO_OK;
 }
 
@@ -249,9 +263,8 @@ int nolo_bind_state(nolo_handle* h, void* phi, void* theta, void* delta, int the
 int nolo_outer_step(nolo_handle* h, uint64_t seed, uint64_t step) {
     if (!h) return NOLO_EINVAL;
     if (!h->state_bound) return fail(h, NOLO_ESTATE, "nolo_bind_state has not been called");
-    int rc = enqueue_group_draw(h, seed, step);
-    if (rc != NOLO_OK) return rc;
-    return enqueue_outer(h, 0, h->P);
+    const Draw draw = {seed, step};
+    return enqueue_outer(h, 0, h->P, &draw);
 }
 
 int nolo_bind_prepared(nolo_handle* h, void* mean_phi, int64_t mean_stride) {
@@ -299,9 +312,8 @@ int nolo_outer_step_prepared(nolo_handle* h, uint64_t seed, uint64_t step) {
         return fail(h, NOLO_ESTATE, "means were prepared for (seed %llu, step %llu), not for (seed %llu, step %llu)",
                     (unsigned long long)h->prepared_seed, (unsigned long long)h->prepared_step,
                     (unsigned long long)seed, (unsigned long long)step);
-    int rc = enqueue_group_draw(h, seed, step);
-    if (rc != NOLO_OK) return rc;
-    return enqueue_outer(h, 0, h->P, true);
+    const Draw draw = {seed, step};
+    return enqueue_outer(h, 0, h->P, &draw, true);
 }
 
 int nolo_outer_step_host(nolo_handle* h, uint64_t seed, uint64_t step, void* phi_host,
@@ -335,7 +347,7 @@ int nolo_outer_step_host(nolo_handle* h, uint64_t seed, uint64_t step, void* phi
         NOLO_CUDA(h, cudaMemcpy2DAsync(h->delta + c0, dp4, de_h, hp4, (size_t)cols * 4, h->W, cudaMemcpyHostToDevice, h->s_in));
         NOLO_CUDA(h, cudaEventRecord(h->ev_in, h->s_in));
         NOLO_CUDA(h, cudaStreamWaitEvent(h->stream, h->ev_in, 0));
-        rc = enqueue_outer(h, c0, cols);
+        rc = enqueue_outer(h, c0, cols, nullptr);
         if (rc != NOLO_OK) return rc;
         NOLO_CUDA(h, cudaEventRecord(h->ev_kernel, h->stream));
         NOLO_CUDA(h, cudaStreamWaitEvent(h->s_out, h->ev_kernel, 0));

@@ -8,6 +8,7 @@
 // reproducible bit for bit on any machine.
 #include "nolo_draw.cuh"
 #include "nolo_internal.h"
+#include "nolo_launch.cuh"
 #include "nolo_philox.cuh"
 
 namespace nolo {
@@ -15,7 +16,8 @@ namespace nolo {
 namespace {
 
 // One CTA per permutation, one thread per element up to N = 1024 and four above.  Bound by latency:
-// the ten dependent rounds of a key (about 0.4 us), then five barriers.
+// the ten dependent rounds of a key (about 0.4 us), then five barriers.  All of that needs nothing from
+// earlier kernels and is done while they still run; only the table is written after them.
 template <int THREADS>
 __global__ void __launch_bounds__(THREADS)
 draw_perm_kernel(uint64_t seed, uint64_t step, uint64_t domain, int N, int first_boundary, int slots_drawn,
@@ -25,12 +27,18 @@ draw_perm_kernel(uint64_t seed, uint64_t step, uint64_t domain, int N, int first
     const int s = blockIdx.x % slots_drawn;
     const int k_lo = (slots_drawn == slots_total) ? s : 0;
     const int k_hi = (slots_drawn == slots_total) ? s + 1 : slots_total;
+    let_successor_start();          // it waits for this kernel, and this kernel for all before it
+    int rank[kDrawPerThread];
     rank_by_buckets<THREADS>(
         reinterpret_cast<unsigned char*>(raw), N,
-        [&](int i) { return draw_key((uint64_t)i, (uint64_t)b, (uint64_t)s, domain, seed, step); },
-        [&](int i, int rank) {
-            for (int k = k_lo; k < k_hi; ++k) table[((int64_t)b * slots_total + k) * N + rank] = i;
-        });
+        [&](int i) { return draw_key((uint64_t)i, (uint64_t)b, (uint64_t)s, domain, seed, step); }, rank);
+    wait_for_predecessors();
+#pragma unroll
+    for (int m = 0; m < kDrawPerThread; ++m) {
+        const int i = threadIdx.x + m * THREADS;
+        if (i < N)
+            for (int k = k_lo; k < k_hi; ++k) table[((int64_t)b * slots_total + k) * N + rank[m]] = i;
+    }
 }
 
 }  // namespace
@@ -41,9 +49,8 @@ cudaError_t launch_draw_range(uint64_t seed, uint64_t step, int domain, int N, i
     const int blocks = boundaries * slots_drawn;
     if (blocks <= 0 || N <= 0) return cudaSuccess;
     auto launch = [&](auto kernel, int threads) {
-        kernel<<<blocks, threads, draw_scratch_bytes(N, threads), stream>>>(
-            seed, step, (uint64_t)domain, N, first_boundary, slots_drawn, slots_total, table);
-        return cudaGetLastError();
+        return launch_overlapped(kernel, dim3((unsigned)blocks), threads, draw_scratch_bytes(N, threads), stream, seed, step,
+                                 (uint64_t)domain, N, first_boundary, slots_drawn, slots_total, table);
     };
     if (N <= 32) return launch(draw_perm_kernel<32>, 32);
     if (N <= 128) return launch(draw_perm_kernel<128>, 128);

@@ -23,11 +23,31 @@ cudaError_t launch_draw_range(uint64_t seed, uint64_t step, int domain, int N, i
                               int boundaries, int slots_drawn, int slots_total, int32_t* table,
                               cudaStream_t stream);
 
+// Launch of a kernel that calls wait_for_predecessors() (nolo_launch.cuh): its CTAs may be set up
+// while the kernel before it in the stream is still running (programmatic dependent launch).
+template <typename... Params, typename... Args>
+cudaError_t launch_overlapped(void (*kernel)(Params...), dim3 grid, unsigned threads, size_t smem, cudaStream_t stream,
+                              Args... args) {
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 struct OuterArgs {
     float* phi;          // [W][stride]
     void* theta;         // [W][stride] float or bf16
     float* delta;        // [W][stride]
-    const int32_t* perm; // [W]; subgroup g = perm[g*n .. g*n+n-1]
+    int32_t* perm;       // [W]; subgroup g = perm[g*n .. g*n+n-1]
+    bool draw = false;   // the kernel draws perm itself from (seed, step) and writes it: see outer_draws
+    uint64_t seed = 0, step = 0;
     int64_t stride;      // elements between rows
     int64_t P;           // columns to process, starting at the pointers given
     int W, n;
@@ -38,6 +58,10 @@ struct OuterArgs {
     const double* mean_phi = nullptr;
     int64_t mean_stride = 0;
 };
+
+// Whether launch_outer can draw the partition itself (a.draw) at these sizes; otherwise perm has to be
+// drawn by launch_draw first.
+bool outer_draws(const OuterArgs& a);
 
 // Fused Eq. 1-3 + theta reset over columns [0, P) of the rows (pointers may be pre-offset by
 // a multiple of 8 columns).  One launch.

@@ -24,7 +24,9 @@
 // addition is recovered exactly and kept in lo).  Float64 accumulators would do the same, but
 // the float32 <-> float64 conversions they need run at 16 per clock per SM on B200 and cost
 // the wide-subgroup kernels 20-35 % of their bandwidth when measured.
+#include "nolo_draw.cuh"
 #include "nolo_internal.h"
+#include "nolo_launch.cuh"
 
 #include <cuda_bf16.h>
 
@@ -38,7 +40,9 @@ struct KArgs {
     float* phi;
     void* theta;
     float* delta;
-    const int32_t* perm;
+    int32_t* perm;
+    uint64_t seed, step;      // kernels that draw the partition themselves (DRAW)
+    int W;
     const double* mean_phi;   // subgroup means of phi prepared in advance, [groups][mean_stride]; or NULL
     int64_t mean_stride;
     int64_t stride;
@@ -240,6 +244,38 @@ __device__ __forceinline__ void update_store(const KArgs& a, int64_t row_off, in
     store_theta4(static_cast<ThetaT*>(a.theta) + row_off, q, p);
 }
 
+// ---- the members of a subgroup --------------------------------------------------------------
+//
+// DRAW = false: read from the table.  DRAW = true (at most 32 workers): the first warp of every CTA draws
+// the partition, before it waits for the kernels ahead of it, and keeps its subgroup's members in
+// shared memory; the first CTA writes the table as well.  Both wait for the kernels ahead of this one.
+template <bool DRAW> struct Members;
+template <> struct Members<false> {
+    const int32_t* list;
+    __device__ __forceinline__ void init(const KArgs& a, int g, int*) {
+        list = a.perm + (int64_t)g * a.n;
+        wait_for_predecessors();
+        let_successor_start();
+    }
+    __device__ __forceinline__ int operator[](int j) const { return __ldg(list + j); }
+};
+template <> struct Members<true> {
+    const int* list;                     // shared memory
+    __device__ __forceinline__ void init(const KArgs& a, int g, int* shared) {
+        list = shared;
+        int rank = 0;
+        if (threadIdx.x < 32) {
+            rank = rank_by_warp(a.W, 0, 0, kDomainGroups, a.seed, a.step);
+            if ((int)threadIdx.x < a.W && rank / a.n == g) shared[rank - g * a.n] = threadIdx.x;
+        }
+        wait_for_predecessors();
+        let_successor_start();
+        if (blockIdx.x == 0 && g == 0 && (int)threadIdx.x < a.W) a.perm[rank] = threadIdx.x;
+        __syncthreads();
+    }
+    __device__ __forceinline__ int operator[](int j) const { return list[j]; }
+};
+
 // Columns P - (P % VEC) .. P-1 of one subgroup (a thread has VEC columns elsewhere), element by element
 // with float64 sums (rows are only guaranteed to be padded to a multiple of 8, and padding must not be
 // written).  Done by a CTA of its own, the first of the subgroup: VEC neighbouring threads per member, so
@@ -247,12 +283,11 @@ __device__ __forceinline__ void update_store(const KArgs& a, int64_t row_off, in
 // column by column is a serial chain of loads; one CTA is not: 3 extra columns cost 7.7 us before and
 // nothing measurable now at n = 20 (73.5 -> 67.4 us for W = 60, P = 2^18 + 3), 197 us at n = 256, 1.42 ms
 // at n = 1024 (2531 -> 1056 us for P = 2^18 + 3).
-template <typename ThetaT, int THREADS, int VEC>
-__device__ __forceinline__ void ragged_tail(const KArgs& a, int g) {
+template <typename ThetaT, int THREADS, int VEC, typename M>
+__device__ __forceinline__ void ragged_tail(const KArgs& a, int g, const M& members) {
     constexpr int WARPS = THREADS / 32, ROWS = THREADS / VEC;
     __shared__ double2 part[WARPS][VEC];
     const int n = a.n;
-    const int32_t* members = a.perm + (int64_t)g * n;
     const int64_t c = (a.P & ~int64_t(VEC - 1)) + threadIdx.x % VEC;
     const int first = threadIdx.x / VEC;
     const bool mine = c < a.P;
@@ -260,7 +295,7 @@ __device__ __forceinline__ void ragged_tail(const KArgs& a, int g) {
     if (mine) {
 #pragma unroll 4
         for (int j = first; j < n; j += ROWS) {
-            const int64_t at = (int64_t)__ldg(members + j) * a.stride + c;
+            const int64_t at = (int64_t)members[j] * a.stride + c;
             const float p = a.phi[at];
             sD += (double)(p - load_theta1(static_cast<const ThetaT*>(a.theta), at));
             sP += (double)p;
@@ -284,7 +319,7 @@ __device__ __forceinline__ void ragged_tail(const KArgs& a, int g) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             if (j0 + i * ROWS < n) {
-                at[i] = (int64_t)__ldg(members + j0 + i * ROWS) * a.stride + c;
+                at[i] = (int64_t)members[j0 + i * ROWS] * a.stride + c;
                 p[i] = a.phi[at[i]];
                 d[i] = a.delta[at[i]];
             }
@@ -314,12 +349,15 @@ __device__ __forceinline__ void ragged_tail(const KArgs& a, int g) {
 // 6850, n = 4 6770 / 6737 -> 6862 / 6800, n = 6 6521 / 6670 -> 6831 / 6695, n = 7 6673 / 6378 -> 6834 / 6740, n = 8
 // 6711 / 5568 -> 6828 / 6739; with prepared means n = 2 5988 / 6830 -> 6985 / 6976, n = 4 6655 -> 6890 (float32).
 // (The quad kernel with n = 7 and 8 left one CTA of 256 threads per SM.)
-template <int N, typename ThetaT, int THREADS, bool PREPARED, bool WIDE>
+template <int N, typename ThetaT, int THREADS, bool PREPARED, bool WIDE, bool DRAW>
 __global__ void __launch_bounds__(THREADS, 1)
 outer_step_reg_kernel(const KArgs a) {
     const int g = blockIdx.y;
+    __shared__ int drawn[DRAW ? N : 1];
+    Members<DRAW> members;
+    members.init(a, g, drawn);
     if (a.tail && blockIdx.x == 0) {
-        ragged_tail<ThetaT, THREADS, 8>(a, g);
+        ragged_tail<ThetaT, THREADS, 8>(a, g, members);
         return;
     }
     const int64_t c = ((int64_t)(blockIdx.x - a.tail) * THREADS + threadIdx.x) * 8;
@@ -327,7 +365,7 @@ outer_step_reg_kernel(const KArgs a) {
 
     int64_t at[N];
 #pragma unroll
-    for (int j = 0; j < N; ++j) at[j] = (int64_t)__ldg(a.perm + g * N + j) * a.stride + c;
+    for (int j = 0; j < N; ++j) at[j] = (int64_t)members[j] * a.stride + c;
     Oct phi[N], dlt[N];
     typename ThetaOct<ThetaT>::type the[N];
 #pragma unroll
@@ -403,7 +441,7 @@ outer_step_reg_kernel(const KArgs a) {
 // (0.5-0.7: all CTAs in the same phase at once).  With the re-read of phi left out altogether
 // the 512-byte-piece loops reach only 0.92 / 0.91 / 0.89 of a plain copy at n = 128 / 256 / 1024:
 // what is lost is lost to streaming n x 3 rows in narrow pieces, not to the second read.
-template <typename ThetaT, int THREADS, int ROWQ, int U, int MINB>
+template <typename ThetaT, int THREADS, int ROWQ, int U, int MINB, bool DRAW>
 __global__ void __launch_bounds__(THREADS, MINB)
 outer_step_twopass_kernel(const KArgs a) {
     static_assert(THREADS % 32 == 0 && THREADS % ROWQ == 0, "slots tile the CTA");
@@ -421,11 +459,13 @@ outer_step_twopass_kernel(const KArgs a) {
     const int part = ROWQ >= 32 ? slot : (threadIdx.x >> 5);
     const int g = blockIdx.y;
     const int n = a.n;
+    __shared__ int drawn[DRAW ? 32 : 1];
+    Members<DRAW> members;
+    members.init(a, g, drawn);
     if (a.tail && blockIdx.x == 0) {
-        ragged_tail<ThetaT, THREADS, 4>(a, g);
+        ragged_tail<ThetaT, THREADS, 4>(a, g, members);
         return;
     }
-    const int32_t* members = a.perm + (int64_t)g * n;
     const int64_t q = (int64_t)(blockIdx.x - a.tail) * ROWQ + ql;
     const bool ok = q < (a.P >> 2);
 
@@ -440,7 +480,7 @@ outer_step_twopass_kernel(const KArgs a) {
             for (int i = 0; i < U; ++i) {
                 const int jj = j + i * SLOTS;
                 if (jj < n) {
-                    const int64_t off = (int64_t)__ldg(members + jj) * a.stride;
+                    const int64_t off = (int64_t)members[jj] * a.stride;
                     p[i] = reinterpret_cast<const float4*>(a.phi + off)[q];     // default policy: stays cached for pass 2
                     t[i] = load_theta_raw(static_cast<const ThetaT*>(a.theta) + off, q);
                 }
@@ -462,7 +502,7 @@ outer_step_twopass_kernel(const KArgs a) {
         for (int i = 0; i < U; ++i) {
             const int jj = j + i * SLOTS;
             if (jj < n) {
-                off2[i] = (int64_t)__ldg(members + jj) * a.stride;
+                off2[i] = (int64_t)members[jj] * a.stride;
                 p2[i] = __ldcs(reinterpret_cast<const float4*>(a.phi + off2[i]) + q);
                 d2[i] = __ldcs(reinterpret_cast<const float4*>(a.delta + off2[i]) + q);
             }
@@ -550,6 +590,8 @@ template <int ITEMS, bool WIDE>
 __global__ void __launch_bounds__(kThreads)
 group_mean_kernel(const float* __restrict__ phi, const int32_t* __restrict__ perm, int n, int64_t stride,
                   int64_t P, double* __restrict__ mean, int64_t mean_stride, double inv_n) {
+    wait_for_predecessors();
+    let_successor_start();
     const int g = blockIdx.y;
     const int32_t* members = perm + (int64_t)g * n;
     const int tail = (P & 3) != 0;
@@ -616,15 +658,13 @@ bool tile_grid(KArgs& k, int vec, int64_t cols_per_cta, int groups, dim3* grid) 
 
 bool aligned32(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 31u) == 0; }
 
-template <int N, typename ThetaT, int THREADS, bool WIDE>
+template <int N, typename ThetaT, int THREADS, bool WIDE, bool DRAW>
 cudaError_t launch_reg_shape(KArgs& k, int groups, cudaStream_t stream) {
     dim3 grid;
     if (!tile_grid(k, 8, (int64_t)THREADS * 8, groups, &grid)) return cudaErrorInvalidConfiguration;
-    if (k.mean_phi)
-        outer_step_reg_kernel<N, ThetaT, THREADS, true, WIDE><<<grid, THREADS, 0, stream>>>(k);
-    else
-        outer_step_reg_kernel<N, ThetaT, THREADS, false, WIDE><<<grid, THREADS, 0, stream>>>(k);
-    return cudaGetLastError();
+    return launch_overlapped(k.mean_phi ? outer_step_reg_kernel<N, ThetaT, THREADS, true, WIDE, DRAW>
+                                        : outer_step_reg_kernel<N, ThetaT, THREADS, false, WIDE, DRAW>,
+                             grid, THREADS, 0, stream, k);
 }
 
 // Larger CTAs stream longer pieces of a row and are the faster by up to 0.7 % where there are many octs
@@ -638,23 +678,31 @@ template <int N, typename ThetaT>
 constexpr int kRegThreads = N == 4 ? 192 : (N == 2 && sizeof(ThetaT) == 2) ? 320 : 256;
 
 template <int N, typename ThetaT>
-cudaError_t launch_reg(KArgs& k, int groups, cudaStream_t stream) {
+cudaError_t launch_reg(KArgs& k, bool draw, int groups, cudaStream_t stream) {
     // the strides are multiples of 32 bytes (of 16 for bfloat16 theta, which is read 16 bytes at a time)
     const bool wide = aligned32(k.phi) && aligned32(k.delta) && (sizeof(ThetaT) == 2 || aligned32(k.theta)) &&
                       aligned32(k.mean_phi);
-    if (!wide) return launch_reg_shape<N, ThetaT, 64, false>(k, groups, stream);
+    if (draw) return wide ? launch_reg_shape<N, ThetaT, 64, true, true>(k, groups, stream)
+                          : launch_reg_shape<N, ThetaT, 64, false, true>(k, groups, stream);
+    if (!wide) return launch_reg_shape<N, ThetaT, 64, false, false>(k, groups, stream);
     if constexpr (N <= 4) {
-        if (k.P / 8 * groups >= kRegManyOcts) return launch_reg_shape<N, ThetaT, kRegThreads<N, ThetaT>, true>(k, groups, stream);
+        if (k.P / 8 * groups >= kRegManyOcts)
+            return launch_reg_shape<N, ThetaT, kRegThreads<N, ThetaT>, true, false>(k, groups, stream);
     }
-    return launch_reg_shape<N, ThetaT, 64, true>(k, groups, stream);
+    return launch_reg_shape<N, ThetaT, 64, true, false>(k, groups, stream);
 }
 
 template <typename ThetaT, int THREADS, int ROWQ, int U, int MINB>
-cudaError_t launch_twopass(KArgs& k, int groups, cudaStream_t stream) {
+cudaError_t launch_twopass(KArgs& k, bool draw, int groups, cudaStream_t stream) {
     dim3 grid;
     if (!tile_grid(k, 4, (int64_t)ROWQ * 4, groups, &grid)) return cudaErrorInvalidConfiguration;
-    outer_step_twopass_kernel<ThetaT, THREADS, ROWQ, U, MINB><<<grid, THREADS, 0, stream>>>(k);
-    return cudaGetLastError();
+    if constexpr (ROWQ >= 64 && U * THREADS / ROWQ <= 16) {       // the shapes of up to 32 members
+        if (draw)
+            return launch_overlapped(outer_step_twopass_kernel<ThetaT, THREADS, ROWQ, U, MINB, true>, grid, THREADS, 0,
+                                     stream, k);
+    }
+    if (draw) return cudaErrorInvalidValue;
+    return launch_overlapped(outer_step_twopass_kernel<ThetaT, THREADS, ROWQ, U, MINB, false>, grid, THREADS, 0, stream, k);
 }
 
 // Subgroup sizes up to which each two-pass shape is used (by measurement, see the kernel's comment):
@@ -668,26 +716,26 @@ constexpr int kTwoPassMaxN32Quads = 224;  // 256 x 32 x 8, 2 CTAs
 constexpr int kTwoPassMaxN8Warps = 640;   // 256 x 16 x 8, 2 CTAs; above: 512 x 16 x 8, 1 CTA
 
 template <typename ThetaT>
-cudaError_t dispatch(KArgs& k, int groups, cudaStream_t stream) {
+cudaError_t dispatch(KArgs& k, bool draw, int groups, cudaStream_t stream) {
     switch (k.n) {
-        case 1:  return launch_reg<1, ThetaT>(k, groups, stream);
-        case 2:  return launch_reg<2, ThetaT>(k, groups, stream);
-        case 3:  return launch_reg<3, ThetaT>(k, groups, stream);
-        case 4:  return launch_reg<4, ThetaT>(k, groups, stream);
-        case 5:  return launch_reg<5, ThetaT>(k, groups, stream);
-        case 6:  return launch_reg<6, ThetaT>(k, groups, stream);
-        case 7:  return launch_reg<7, ThetaT>(k, groups, stream);
-        case 8:  return launch_reg<8, ThetaT>(k, groups, stream);
+        case 1:  return launch_reg<1, ThetaT>(k, draw, groups, stream);
+        case 2:  return launch_reg<2, ThetaT>(k, draw, groups, stream);
+        case 3:  return launch_reg<3, ThetaT>(k, draw, groups, stream);
+        case 4:  return launch_reg<4, ThetaT>(k, draw, groups, stream);
+        case 5:  return launch_reg<5, ThetaT>(k, draw, groups, stream);
+        case 6:  return launch_reg<6, ThetaT>(k, draw, groups, stream);
+        case 7:  return launch_reg<7, ThetaT>(k, draw, groups, stream);
+        case 8:  return launch_reg<8, ThetaT>(k, draw, groups, stream);
         default: break;
     }
-    if (k.n <= kTwoPassMaxN1Slot) return launch_twopass<ThetaT, 128, 128, 4, 6>(k, groups, stream);
-    if (k.n <= kTwoPassMaxN2Slots) return launch_twopass<ThetaT, 128, 64, 8, 4>(k, groups, stream);
-    if (k.n <= kTwoPassMaxN64Quads4) return launch_twopass<ThetaT, 256, 64, 4, 3>(k, groups, stream);
-    if (k.n <= kTwoPassMaxN64Quads8) return launch_twopass<ThetaT, 256, 64, 8, 2>(k, groups, stream);
-    if (k.n <= kTwoPassMaxN4Rows) return launch_twopass<ThetaT, 256, 32, 4, 3>(k, groups, stream);
-    if (k.n <= kTwoPassMaxN32Quads) return launch_twopass<ThetaT, 256, 32, 8, 2>(k, groups, stream);
-    if (k.n <= kTwoPassMaxN8Warps) return launch_twopass<ThetaT, 256, 16, 8, 2>(k, groups, stream);
-    return launch_twopass<ThetaT, 512, 16, 8, 1>(k, groups, stream);
+    if (k.n <= kTwoPassMaxN1Slot) return launch_twopass<ThetaT, 128, 128, 4, 6>(k, draw, groups, stream);
+    if (k.n <= kTwoPassMaxN2Slots) return launch_twopass<ThetaT, 128, 64, 8, 4>(k, draw, groups, stream);
+    if (k.n <= kTwoPassMaxN64Quads4) return launch_twopass<ThetaT, 256, 64, 4, 3>(k, draw, groups, stream);
+    if (k.n <= kTwoPassMaxN64Quads8) return launch_twopass<ThetaT, 256, 64, 8, 2>(k, draw, groups, stream);
+    if (k.n <= kTwoPassMaxN4Rows) return launch_twopass<ThetaT, 256, 32, 4, 3>(k, draw, groups, stream);
+    if (k.n <= kTwoPassMaxN32Quads) return launch_twopass<ThetaT, 256, 32, 8, 2>(k, draw, groups, stream);
+    if (k.n <= kTwoPassMaxN8Warps) return launch_twopass<ThetaT, 256, 16, 8, 2>(k, draw, groups, stream);
+    return launch_twopass<ThetaT, 512, 16, 8, 1>(k, draw, groups, stream);
 }
 
 }  // namespace
@@ -704,16 +752,26 @@ cudaError_t launch_group_mean(const float* phi, const int32_t* perm, int W, int 
     const double inv_n = 1.0 / (double)n;
     // rows of the means are 32-byte aligned when the base is (the stride is a multiple of 64 bytes)
     const bool wide = (reinterpret_cast<uintptr_t>(mean) & 31u) == 0;
-    auto launch = [&](auto kernel) { kernel<<<grid, kThreads, 0, stream>>>(phi, perm, n, stride, P, mean, mean_stride, inv_n); };
-    if (items == 2) launch(wide ? group_mean_kernel<2, true> : group_mean_kernel<2, false>);
-    else launch(wide ? group_mean_kernel<1, true> : group_mean_kernel<1, false>);
-    return cudaGetLastError();
+    auto launch = [&](auto kernel) {
+        return launch_overlapped(kernel, grid, kThreads, 0, stream, phi, perm, n, stride, P, mean, mean_stride, inv_n);
+    };
+    if (items == 2) return launch(wide ? group_mean_kernel<2, true> : group_mean_kernel<2, false>);
+    return launch(wide ? group_mean_kernel<1, true> : group_mean_kernel<1, false>);
 }
+
+// Drawing in the kernel saves the launch of the draw (2 us of host time, 1 to 2 us on the device) and costs
+// every CTA the draw's 0.3 us, which shows once there are several waves of them.  Measured, draw kernel /
+// drawn in the step, us per step: 2^17 worker-parameters 5.3 / 3.1-4.0, 2^22 14.0-22.8 / 13.3-20.9, 2^24 62.2 /
+// 61.3 (n = 2), 68.7 / 67.6 (n = 20) but 54.7 / 55.4 (n = 8, bfloat16 theta), 2^26 204 / 207 and 247.9 / 249.4.
+constexpr int64_t kDrawMaxParams = 1 << 23;   // worker-parameters
+
+bool outer_draws(const OuterArgs& a) { return a.W <= 32 && a.P * a.W <= kDrawMaxParams; }
 
 cudaError_t launch_outer(const OuterArgs& a, cudaStream_t stream) {
     if (a.P <= 0 || a.W <= 0) return cudaSuccess;
     KArgs k;
     k.phi = a.phi; k.theta = a.theta; k.delta = a.delta; k.perm = a.perm;
+    k.seed = a.seed; k.step = a.step; k.W = a.W;
     k.mean_phi = a.mean_phi; k.mean_stride = a.mean_stride;
     k.stride = a.stride; k.P = a.P; k.n = a.n;
     k.alpha = a.alpha; k.gamma = a.gamma;
@@ -723,7 +781,7 @@ cudaError_t launch_outer(const OuterArgs& a, cudaStream_t stream) {
     k.inv_n_d = 1.0 / (double)a.n;
     const int groups = a.W / a.n;
     if (groups > 65535) return cudaErrorInvalidConfiguration;
-    return a.theta_bf16 ? dispatch<__nv_bfloat16>(k, groups, stream) : dispatch<float>(k, groups, stream);
+    return a.theta_bf16 ? dispatch<__nv_bfloat16>(k, a.draw, groups, stream) : dispatch<float>(k, a.draw, groups, stream);
 }
 
 }  // namespace nolo

@@ -95,9 +95,6 @@ extern "C" int nolo_outer_step_static(int W, int n, int64_t P, float alpha, floa
     if (rc != NOLO_OK) return rc;
 
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    // The draw overwrites entries 0..W-1, all that the step reads: nothing has to start at zero.
-    cudaError_t e = nolo::launch_draw(seed, step, nolo::kDomainGroups, W, 1, 1, 1, perm, s);
-    if (e != cudaSuccess) return report(err, err_len, NOLO_ECUDA, "subgroup draw launch: %s", cudaGetErrorString(e));
     nolo::OuterArgs a;
     a.phi = static_cast<float*>(phi);
     a.theta = theta;
@@ -109,7 +106,14 @@ extern "C" int nolo_outer_step_static(int W, int n, int64_t P, float alpha, floa
     a.n = n;
     a.theta_bf16 = theta_dtype == NOLO_BF16;
     a.alpha = alpha; a.beta = beta; a.gamma = gamma;
-    e = nolo::launch_outer(a, s);
+    a.seed = seed; a.step = step;
+    a.draw = nolo::outer_draws(a);
+    if (!a.draw) {
+        // The draw overwrites entries 0..W-1, all that the step reads: nothing has to start at zero.
+        const cudaError_t e = nolo::launch_draw(seed, step, nolo::kDomainGroups, W, 1, 1, 1, perm, s);
+        if (e != cudaSuccess) return report(err, err_len, NOLO_ECUDA, "subgroup draw launch: %s", cudaGetErrorString(e));
+    }
+    const cudaError_t e = nolo::launch_outer(a, s);
     if (e != cudaSuccess) return report(err, err_len, NOLO_ECUDA, "outer step launch: %s", cudaGetErrorString(e));
     return NOLO_OK;
 }

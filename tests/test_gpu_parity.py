@@ -172,6 +172,32 @@ def test_cta_sizes_agree(nolo, n, bf16):
         assert torch.equal(a[:, :9000], b[:, :9000])
 
 
+@pytest.mark.parametrize("W,n", [(1, 1), (32, 8), (20, 20), (32, 32), (33, 11)])
+def test_drawn_in_the_step_or_ahead_of_it(nolo, W, n):
+    """Up to 32 workers and 2^23 worker-parameters the step draws its partition itself, else a kernel
+    ahead of it does: the same table and the same bits either way, for steps that follow each other
+    closely as well as for steps that are waited for."""
+    P = (1 << 23) // W // 8 * 8 + 8
+    state = [x.cuda() for x in synth.make_state(W, 5000, 3, stride=5008)]
+    big = [torch.zeros((W, P), device="cuda") for _ in state]
+    for b, x in zip(big, state):
+        b[:, :5000] = x[:, :5000]
+    again = [x.clone() for x in state]
+    for views, cols, wait, timed in ((state, 5000, False, False), (again, 5000, False, True), (big, P, True, False)):
+        h = nolo.nolo_create(W, n, cols, 1, *F)
+        nolo.nolo_bind_state(h, *views)
+        nolo.nolo_timing_enable(h, timed)               # timed steps have a draw kernel at every size
+        for step in range(12):
+            nolo.nolo_outer_step(h, 5, step)
+            if wait:
+                assert np.array_equal(nolo.nolo_get_groups(h), O.draw_groups(5, step, W, n))
+        assert np.array_equal(nolo.nolo_get_groups(h), O.draw_groups(5, 11, W, n))
+        assert nolo.nolo_launch_count(h) == (12 if W <= 32 and views is state else 24)
+        nolo.nolo_destroy(h)
+    for b, x, y in zip(big, state, again):
+        assert torch.equal(b[:, :5000], x[:, :5000]) and torch.equal(x[:, :5000], y[:, :5000])
+
+
 @pytest.mark.parametrize("hp", [(0.0, 0.0, 1.0), (0.3, 0.7, 0.0), (0.9, 1.0, 1.5), (0.5, 0.7, 0.0)])
 def test_hyperparameter_corners(nolo, hp):
     hp = tuple(float(np.float32(x)) for x in hp)
