@@ -646,10 +646,10 @@ def run_ours(args):
     }
     if M:
         rb = 2 * acts.numel() * acts.element_size()
-        line["route"] = stats_record("routing, forward, all boundaries", "route_copy16_kernel", route_stats, route_cnt,
+        line["route"] = stats_record("routing, forward, all boundaries", "route_copy_kernel", route_stats, route_cnt,
                                      rb, peak, copy_gbs)
         if back_stats is not None:
-            line["route_backward"] = stats_record("routing, backward, all boundaries", "route_copy16_kernel",
+            line["route_backward"] = stats_record("routing, backward, all boundaries", "route_copy_kernel",
                                                   back_stats, back_cnt, rb, peak, copy_gbs)
     nolo.nolo_destroy(h)
     del phi, theta, delta, acts, acts_out

@@ -173,22 +173,27 @@ int enqueue_outer(nolo_handle* h, int64_t col0, int64_t cols, const Draw* draw, 
     return NOLO_OK;
 }
 
-int enqueue_route(nolo_handle* h, uint64_t seed, uint64_t step, const void* in, void* out, int backward) {
-    const int B = h->stages - 1;
-    if (B == 0) return NOLO_OK;
-    const int drawn = h->per_microbatch ? h->K : 1;
-    NOLO_CUDA(h, nolo::launch_draw(seed, step, nolo::kDomainRoute, h->W, B, drawn, h->K, h->d_route, h->stream));
-    ++h->launches;
-    h->route_valid = true;
+// Boundaries [b0, b0 + count); in and out begin with boundary b0.
+int enqueue_route(nolo_handle* h, uint64_t seed, uint64_t step, int b0, int count, const void* in, void* out, int backward) {
+    if (count == 0) return NOLO_OK;
     nolo::RouteArgs a;
-    a.in = in; a.out = out; a.table = h->d_route;
-    a.B = B; a.R = h->W; a.K = h->K; a.E = h->E;
+    a.in = in; a.out = out; a.table = h->d_route + (size_t)b0 * h->K * h->W;
+    a.B = count; a.R = h->W; a.K = h->K; a.E = h->E;
     a.elem_size = elem_size(h->act_dtype);
     a.backward = backward;
+    a.seed = seed; a.step = step; a.first_boundary = b0; a.per_microbatch = h->per_microbatch;
+    a.draw = !h->timing && nolo::route_draws(a);       // timed kernels do the same work at every size
+    if (!a.draw) {
+        const int drawn = h->per_microbatch ? h->K : 1;
+        NOLO_CUDA(h, nolo::launch_draw_range(seed, step, nolo::kDomainRoute, h->W, b0, count, drawn, h->K, h->d_route,
+                                             h->stream));
+        ++h->launches;
+    }
     Bracket br(h, NOLO_KERNEL_ROUTE);
     NOLO_CUDA(h, nolo::launch_route(a, h->stream));
     br.done();
     ++h->launches;
+    h->route_valid = true;
     return NOLO_OK;
 }
 
@@ -394,7 +399,7 @@ int nolo_route(nolo_handle* h, uint64_t seed, uint64_t step, const void* acts) {
     if (!aligned16(acts)) return fail(h, NOLO_EALIGN, "acts must be 16-byte aligned");
     if (overlap(acts, route_bytes(h), h->acts_out, route_bytes(h)))
         return fail(h, NOLO_EINVAL, "acts overlaps acts_out");
-    return enqueue_route(h, seed, step, acts, h->acts_out, 0);
+    return enqueue_route(h, seed, step, 0, h->stages - 1, acts, h->acts_out, 0);
 }
 
 int nolo_route_boundary(nolo_handle* h, uint64_t seed, uint64_t step, int boundary, const void* acts_b,
@@ -407,22 +412,7 @@ int nolo_route_boundary(nolo_handle* h, uint64_t seed, uint64_t step, int bounda
     if (!aligned16(acts_b) || !aligned16(out_b)) return fail(h, NOLO_EALIGN, "pointers must be 16-byte aligned");
     const size_t bytes = route_bytes(h) / (size_t)(h->stages - 1);
     if (overlap(acts_b, bytes, out_b, bytes)) return fail(h, NOLO_EINVAL, "acts_b overlaps out_b");
-    const int drawn = h->per_microbatch ? h->K : 1;
-    NOLO_CUDA(h, nolo::launch_draw_range(seed, step, nolo::kDomainRoute, h->W, boundary, 1, drawn, h->K,
-                                         h->d_route, h->stream));
-    ++h->launches;
-    h->route_valid = true;
-    nolo::RouteArgs a;
-    a.in = acts_b; a.out = out_b;
-    a.table = h->d_route + (size_t)boundary * h->K * h->W;
-    a.B = 1; a.R = h->W; a.K = h->K; a.E = h->E;
-    a.elem_size = elem_size(h->act_dtype);
-    a.backward = 0;
-    Bracket br(h, NOLO_KERNEL_ROUTE);
-    NOLO_CUDA(h, nolo::launch_route(a, h->stream));
-    br.done();
-    ++h->launches;
-    return NOLO_OK;
+    return enqueue_route(h, seed, step, boundary, 1, acts_b, out_b, 0);
 }
 
 int nolo_route_backward(nolo_handle* h, uint64_t seed, uint64_t step, const void* grads, void* grads_out) {
@@ -433,7 +423,7 @@ int nolo_route_backward(nolo_handle* h, uint64_t seed, uint64_t step, const void
     if (!aligned16(grads) || !aligned16(grads_out)) return fail(h, NOLO_EALIGN, "pointers must be 16-byte aligned");
     if (overlap(grads, route_bytes(h), grads_out, route_bytes(h)))
         return fail(h, NOLO_EINVAL, "grads overlaps grads_out");
-    return enqueue_route(h, seed, step, grads, grads_out, 1);
+    return enqueue_route(h, seed, step, 0, h->stages - 1, grads, grads_out, 1);
 }
 
 int nolo_route_host(nolo_handle* h, uint64_t seed, uint64_t step, const void* acts_host,
@@ -446,7 +436,7 @@ int nolo_route_host(nolo_handle* h, uint64_t seed, uint64_t step, const void* ac
     const size_t bytes = route_bytes(h);
     if (overlap(acts_dev, bytes, h->acts_out, bytes)) return fail(h, NOLO_EINVAL, "acts_dev overlaps acts_out");
     NOLO_CUDA(h, cudaMemcpyAsync(acts_dev, acts_host, bytes, cudaMemcpyHostToDevice, h->stream));
-    int rc = enqueue_route(h, seed, step, acts_dev, h->acts_out, 0);
+    int rc = enqueue_route(h, seed, step, 0, h->stages - 1, acts_dev, h->acts_out, 0);
     if (rc != NOLO_OK) return rc;
     NOLO_CUDA(h, cudaMemcpyAsync(out_host, h->acts_out, bytes, cudaMemcpyDeviceToHost, h->stream));
     NOLO_CUDA(h, cudaStreamSynchronize(h->stream));

@@ -75,12 +75,19 @@ cudaError_t launch_group_mean(const float* phi, const int32_t* perm, int W, int 
 struct RouteArgs {
     const void* in;        // [B][R][K][E]
     void* out;             // [B][R][K][E]
-    const int32_t* table;  // [B][K][R]
+    int32_t* table;        // [B][K][R]
     int B, R, K;
     int64_t E;
     int elem_size;         // bytes
     int backward;          // 0: out[b][r][k] = in[b][table[b][k][r]][k]; 1: the inverse
+    bool draw = false;     // the kernel draws the table itself and writes it: see route_draws
+    uint64_t seed = 0, step = 0;
+    int first_boundary = 0, per_microbatch = 0;
 };
+
+// Whether launch_route can draw the table itself (a.draw) at these sizes; otherwise it has to be drawn by
+// launch_draw first.
+bool route_draws(const RouteArgs& a);
 
 cudaError_t launch_route(const RouteArgs& a, cudaStream_t stream);
 

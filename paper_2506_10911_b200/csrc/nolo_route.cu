@@ -1,77 +1,163 @@
 // Random pipeline routing (Section 3.1, Algorithm 1) as a permutation gather of micro-batch
 // activations between the replicas of consecutive stages.  A pure copy: every byte is read once
-// and written once, 128 bits per access, streaming cache policy.
+// and written once, 128 or 256 bits per access, streaming cache policy.
 //
 //   forward :  out[b][r][k][:] = in[b][table[b][k][r]][k][:]
 //   backward:  out[b][table[b][k][r]][k][:] = in[b][r][k][:]     (same path, reversed)
+//
+// Bound by DRAM for all but the smallest calls, which are bound by latency: kernels are launched while
+// their predecessor runs, and up to 32 replicas draw their permutation inside the copy.
+#include "nolo_draw.cuh"
 #include "nolo_internal.h"
+#include "nolo_launch.cuh"
 
 namespace nolo {
 
 namespace {
 
-constexpr int kThreads = 256;
-constexpr int kVecPerThread = 4;                      // 128-bit loads in flight per thread (routing: 4 measured 15 % above 2)
-constexpr int kTileVecs = kThreads * kVecPerThread;   // vectors per tile
-
-struct Blocks {
-    int64_t src, dst;   // block indices into [B][R][K]
+struct CopyArgs {
+    const unsigned char* in;
+    unsigned char* out;
+    int32_t* table;           // [B][K][R]
+    int B, R, K;
+    int64_t bytes;            // of one block
+    int backward;
+    // kernels that draw the table themselves (DRAW)
+    uint64_t seed, step;
+    int first_boundary, per_microbatch;
 };
 
-__device__ __forceinline__ Blocks resolve(int64_t blk, const int32_t* __restrict__ table, int R, int K,
-                                          int backward) {
-    const int k = (int)(blk % K);
-    const int r = (int)((blk / K) % R);
-    const int64_t b = blk / ((int64_t)K * R);
-    const int peer = __ldg(table + (b * K + k) * R + r);
-    const int64_t other = (b * R + peer) * K + k;
-    Blocks o;
-    o.src = backward ? blk : other;
-    o.dst = backward ? other : blk;
-    return o;
-}
-
-// Blocks of `vecs` 16-byte vectors each; tiles of kTileVecs vectors; one tile per CTA.
-__global__ void __launch_bounds__(kThreads)
-route_copy16_kernel(const uint4* __restrict__ in, uint4* __restrict__ out,
-                    const int32_t* __restrict__ table, int R, int K, int64_t vecs,
-                    int64_t tiles_per_block, int64_t total_tiles, int backward) {
-    for (int64_t tile = blockIdx.x; tile < total_tiles; tile += gridDim.x) {
-        const int64_t blk = tile / tiles_per_block;
-        const int64_t v0 = (tile - blk * tiles_per_block) * kTileVecs + threadIdx.x;
-        const Blocks w = resolve(blk, table, R, K, backward);
-        const uint4* s = in + w.src * vecs;
-        uint4* d = out + w.dst * vecs;
-        uint4 v[kVecPerThread];
-#pragma unroll
-        for (int i = 0; i < kVecPerThread; ++i) {
-            const int64_t x = v0 + (int64_t)i * kThreads;
-            if (x < vecs) v[i] = __ldcs(s + x);
+// The replica of the other side for slot k of replica r at boundary b.  DRAW: drawn by the first warp
+// before the kernels ahead are waited for; one CTA per permutation writes the table.
+template <bool DRAW>
+__device__ __forceinline__ int peer_of(const CopyArgs& a, int b, int r, int k) {
+    int32_t* row = a.table + ((int64_t)b * a.K + k) * a.R;
+    if constexpr (!DRAW) {
+        return __ldg(row + r);
+    } else {
+        __shared__ int peer;
+        int rank = 0;
+        if (threadIdx.x < 32) {
+            rank = rank_by_warp(a.R, a.first_boundary + b, a.per_microbatch ? k : 0, kDomainRoute, a.seed, a.step);
+            if (rank == r) peer = threadIdx.x;
         }
-#pragma unroll
-        for (int i = 0; i < kVecPerThread; ++i) {
-            const int64_t x = v0 + (int64_t)i * kThreads;
-            if (x < vecs) __stcs(d + x, v[i]);
-        }
+        wait_for_predecessors();
+        if (r == 0 && blockIdx.x == 0 && (int)threadIdx.x < a.R) row[rank] = threadIdx.x;
+        __syncthreads();
+        const int p = peer;
+        __syncthreads();      // before the next draw of this CTA
+        return p;
     }
 }
 
-// Fallback for blocks whose byte size is not a multiple of 16: element-wise copy.
-template <typename T>
-__global__ void __launch_bounds__(kThreads)
-route_copy_elem_kernel(const T* __restrict__ in, T* __restrict__ out, const int32_t* __restrict__ table,
-                       int R, int K, int64_t E, int64_t tiles_per_block, int64_t total_tiles,
-                       int backward) {
-    for (int64_t tile = blockIdx.x; tile < total_tiles; tile += gridDim.x) {
-        const int64_t blk = tile / tiles_per_block;
-        const int64_t e0 = (tile - blk * tiles_per_block) * kTileVecs + threadIdx.x;
-        const Blocks w = resolve(blk, table, R, K, backward);
-        const T* s = in + w.src * E;
-        T* d = out + w.dst * E;
+// A 256-bit vector, moved by one access.
+struct __align__(32) Wide { uint4 a, b; };
+__device__ __forceinline__ Wide load_stream(const Wide* p) {
+    Wide v;
+    asm volatile("ld.global.cs.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(v.a.x), "=r"(v.a.y), "=r"(v.a.z), "=r"(v.a.w), "=r"(v.b.x), "=r"(v.b.y), "=r"(v.b.z), "=r"(v.b.w)
+                 : "l"(p));
+    return v;
+}
+__device__ __forceinline__ void store_stream(Wide* p, const Wide& v) {
+    asm volatile("st.global.cs.v8.b32 [%8], {%0, %1, %2, %3, %4, %5, %6, %7};" ::"r"(v.a.x), "r"(v.a.y), "r"(v.a.z), "r"(v.a.w),
+                 "r"(v.b.x), "r"(v.b.y), "r"(v.b.z), "r"(v.b.w), "l"(p)
+                 : "memory");
+}
+__device__ __forceinline__ uint4 load_stream(const uint4* p) { return __ldcs(p); }
+__device__ __forceinline__ void store_stream(uint4* p, const uint4& v) { __stcs(p, v); }
+
+// A tile of THREADS x N vectors V of one block, block and vectors aligned to V.
+template <typename V, int THREADS, int N>
+__device__ __forceinline__ void copy_tile(const unsigned char* src, unsigned char* dst, int64_t bytes) {
+    const int64_t vecs = bytes / sizeof(V), v0 = (int64_t)blockIdx.x * (THREADS * N) + threadIdx.x;
+    V v[N];
 #pragma unroll
-        for (int i = 0; i < kVecPerThread; ++i) {
-            const int64_t x = e0 + (int64_t)i * kThreads;
-            if (x < E) d[x] = s[x];
+    for (int i = 0; i < N; ++i) {
+        const int64_t x = v0 + (int64_t)i * THREADS;
+        if (x < vecs) v[i] = load_stream(reinterpret_cast<const V*>(src) + x);
+    }
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        const int64_t x = v0 + (int64_t)i * THREADS;
+        if (x < vecs) store_stream(reinterpret_cast<V*>(dst) + x, v[i]);
+    }
+}
+
+constexpr int kLine = 128;
+
+// Bytes s .. s+15 of two neighbouring 16-byte vectors.
+__device__ __forceinline__ uint4 shifted(const uint4& x, const uint4& y, int s) {
+    const uint32_t w[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
+    const int words = s >> 2, bits = (s & 3) * 8;
+    uint32_t v[5];
+#pragma unroll
+    for (int i = 0; i < 5; ++i)
+        v[i] = words == 0 ? w[i] : words == 1 ? w[i + 1] : words == 2 ? w[i + 2] : w[i + 3];
+    return make_uint4(__funnelshift_r(v[0], v[1], bits), __funnelshift_r(v[1], v[2], bits), __funnelshift_r(v[2], v[3], bits),
+                      __funnelshift_r(v[3], v[4], bits));
+}
+
+// The same for blocks of elements T that begin anywhere (at a multiple of sizeof(T)), the source at
+// another offset from a 16-byte boundary than the destination: 16-byte vectors of the destination, from its
+// first 128-byte line on, so that no two warps share one, are each put together from the two aligned source
+// vectors they straddle.  A warp has N x 32 consecutive vectors, so that the second one comes from the next lane
+// by shuffle (holding both in registers measured 10-20 % slower: fewer bytes in flight); the bytes before
+// the first and after the last vector go one T at a time.  No access leaves the buffers: a vector that
+// would need a source vector reaching beyond in_end is left to the elements.
+template <typename T, int THREADS, int N>
+__device__ __forceinline__ void copy_tile_shifted(const unsigned char* src, unsigned char* dst, int64_t bytes,
+                                                  const unsigned char* in_end) {
+    static_assert(THREADS * sizeof(T) >= kLine + 32, "one element per thread at the ends");
+    int64_t head = (kLine - (reinterpret_cast<uintptr_t>(dst) & (kLine - 1))) & (kLine - 1);
+    if (head > bytes) head = bytes;
+    const int shift = (int)(reinterpret_cast<uintptr_t>(src + head) & 15);
+    const uint4* from = reinterpret_cast<const uint4*>(src + head - shift);
+    const int second = shift != 0;
+    const int64_t inside = (in_end - reinterpret_cast<const unsigned char*>(from)) / 16 - second;
+    int64_t vecs = (bytes - head) / 16;
+    if (vecs > inside) vecs = inside > 0 ? inside : 0;        // one less, at the end of the whole input
+    const int lane = threadIdx.x & 31;
+    const int64_t v0 = ((int64_t)blockIdx.x * (THREADS / 32) + (threadIdx.x >> 5)) * (32 * N) + lane;
+    uint4 v[N + 1];
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+        if (v0 + 32 * i < vecs + second) v[i] = __ldcs(from + v0 + 32 * i);
+    if (lane == 0 && v0 + 32 * N < vecs + second) v[N] = __ldg(from + v0 + 32 * N);
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        const uint4 give = lane == 0 ? v[i + 1] : v[i];
+        uint4 next;
+        next.x = __shfl_sync(0xffffffffu, give.x, (lane + 1) & 31);
+        next.y = __shfl_sync(0xffffffffu, give.y, (lane + 1) & 31);
+        next.z = __shfl_sync(0xffffffffu, give.z, (lane + 1) & 31);
+        next.w = __shfl_sync(0xffffffffu, give.w, (lane + 1) & 31);
+        if (v0 + 32 * i < vecs) __stcs(reinterpret_cast<uint4*>(dst + head) + v0 + 32 * i, shifted(v[i], next, shift));
+    }
+    if (blockIdx.x == 0 && threadIdx.x < (kLine + 32) / sizeof(T)) {
+        const int e = threadIdx.x * sizeof(T);
+        const int64_t at = e < kLine ? e : head + 16 * vecs + (e - kLine);
+        if (e < kLine ? at < head : at < bytes) *reinterpret_cast<T*>(dst + at) = *reinterpret_cast<const T*>(src + at);
+    }
+}
+
+// One tile of one block per CTA.  V: Wide or uint4 for blocks that are a multiple of it, else the element.
+template <typename V, int THREADS, int N, bool DRAW>
+__global__ void __launch_bounds__(THREADS)
+route_copy_kernel(const CopyArgs a) {
+    if constexpr (!DRAW) wait_for_predecessors();
+    let_successor_start();
+    for (int b = blockIdx.z; b < a.B; b += gridDim.z) {
+        for (int rk = blockIdx.y; rk < a.R * a.K; rk += gridDim.y) {
+            const int r = rk / a.K, k = rk - r * a.K;
+            const int peer = peer_of<DRAW>(a, b, r, k);
+            const int64_t here = ((int64_t)b * a.R + r) * a.K + k, there = ((int64_t)b * a.R + peer) * a.K + k;
+            const unsigned char* src = a.in + (a.backward ? here : there) * a.bytes;
+            unsigned char* dst = a.out + (a.backward ? there : here) * a.bytes;
+            if constexpr (sizeof(V) >= 16)
+                copy_tile<V, THREADS, N>(src, dst, a.bytes);
+            else
+                copy_tile_shifted<V, THREADS, N>(src, dst, a.bytes, a.in + (int64_t)a.B * a.R * a.K * a.bytes);
         }
     }
 }
@@ -80,30 +166,24 @@ route_copy_elem_kernel(const T* __restrict__ in, T* __restrict__ out, const int3
 // routing copy: the yardstick the other kernels are compared with.  Two vectors per thread is the
 // fastest plain copy found on B200 (6.97 TB/s against 6.90 with four and 6.87 with eight; 256-bit
 // loads and stores gave the same 6.9-7.0).
+constexpr int kProbeThreads = 256;
 constexpr int kProbeVecPerThread = 2;
-constexpr int kProbeTileVecs = kThreads * kProbeVecPerThread;
+constexpr int kProbeTileVecs = kProbeThreads * kProbeVecPerThread;
 
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kProbeThreads)
 copy_probe_kernel(const uint4* __restrict__ in, uint4* __restrict__ out, int64_t vecs) {
     const int64_t v0 = (int64_t)blockIdx.x * kProbeTileVecs + threadIdx.x;
     uint4 v[kProbeVecPerThread];
 #pragma unroll
     for (int i = 0; i < kProbeVecPerThread; ++i) {
-        const int64_t x = v0 + (int64_t)i * kThreads;
+        const int64_t x = v0 + (int64_t)i * kProbeThreads;
         if (x < vecs) v[i] = __ldcs(in + x);
     }
 #pragma unroll
     for (int i = 0; i < kProbeVecPerThread; ++i) {
-        const int64_t x = v0 + (int64_t)i * kThreads;
+        const int64_t x = v0 + (int64_t)i * kProbeThreads;
         if (x < vecs) __stcs(out + x, v[i]);
     }
-}
-
-// One CTA per tile (a one-shot grid streams through memory in address order, which measured
-// about 10 % faster on B200 than a resident grid striding over the tiles); the kernels still loop
-// so that a tile count beyond the grid limit stays correct.
-int tile_grid(int64_t total_tiles) {
-    return (int)(total_tiles < 0x7fffffffll ? total_tiles : 0x7fffffffll);
 }
 
 }  // namespace
@@ -113,36 +193,54 @@ cudaError_t launch_copy_probe(const void* in, void* out, int64_t bytes, cudaStre
     const int64_t tiles = (vecs + kProbeTileVecs - 1) / kProbeTileVecs;
     if (tiles <= 0) return cudaSuccess;
     if (tiles > 0x7fffffffll) return cudaErrorInvalidConfiguration;
-    copy_probe_kernel<<<(unsigned)tiles, kThreads, 0, stream>>>(static_cast<const uint4*>(in),
+    copy_probe_kernel<<<(unsigned)tiles, kProbeThreads, 0, stream>>>(static_cast<const uint4*>(in),
                                                                 static_cast<uint4*>(out), vecs);
     return cudaGetLastError();
 }
 
+// Drawing in the copy saves the launch of the draw and costs every CTA the draw's 0.3 us.  Measured, draw
+// kernel / drawn in the copy, us for a forward and a backward call: 2 MB 12.0 / 7.4, 25 MB 20.7 / 18.7 (22.5 / 22.5 for
+// blocks at odd offsets), 76 MB 50.7 / 49.1 but 51.2 / 55.0 at odd offsets, 100 MB 64.4 / 67.5.
+constexpr int64_t kDrawMaxBytes = 32ll << 20;
+
+bool route_draws(const RouteArgs& a) {
+    return a.R <= 32 && (int64_t)a.B * a.R * a.K * a.E * a.elem_size <= kDrawMaxBytes;
+}
+
+template <typename V, int THREADS, int N>
+cudaError_t launch_shape(const CopyArgs& c, bool draw, cudaStream_t stream) {
+    constexpr int64_t tile = (int64_t)THREADS * N * (sizeof(V) < 16 ? 16 : sizeof(V));
+    const int64_t tiles = (c.bytes + tile - 1) / tile, rk = (int64_t)c.R * c.K;
+    if (tiles > 0x7fffffffll) return cudaErrorInvalidConfiguration;
+    const dim3 grid((unsigned)tiles, (unsigned)(rk < 65535 ? rk : 65535), (unsigned)(c.B < 65535 ? c.B : 65535));
+    return launch_overlapped(draw ? route_copy_kernel<V, THREADS, N, true> : route_copy_kernel<V, THREADS, N, false>, grid,
+                             THREADS, 0, stream, c);
+}
+
+// One CTA per tile: a one-shot grid streams through memory in address order, which measured about 10 %
+// faster on B200 than a resident grid striding over the tiles (the kernel loops only where a grid
+// dimension ends).  CTA shapes, us for a forward and a backward call of 96 blocks of 64 MB: 256 threads x 4
+// vectors of 16 bytes 3724, 256 x 2 3685, 512 x 2 3646; of 32 bytes 256 x 2 3698, 256 x 1 3689, 384 x 1 3676, 512 x 1
+// 3657; on a device under its power cap (SM clock down by a tenth) the shapes of 512 and more threads took 3750, so the
+// choice is the largest that keeps its rate there.  Over blocks of 1 MB all are within 2 %; copies that draw
+// want few CTAs.  Blocks at any offset (96 of 4 MB, bfloat16, GB/s): 128 x 8 6780, 128 x 4 6490, 256 x 4 6030, 256 x 1
+// 2910 (what a CTA does before its loads is a chain of several hundred cycles, so it has to have many in
+// flight); one 2-byte element per access, as before, 2180.
 cudaError_t launch_route(const RouteArgs& a, cudaStream_t stream) {
-    const int64_t blocks = (int64_t)a.B * a.R * a.K;
-    if (blocks <= 0 || a.E <= 0) return cudaSuccess;
-    const int64_t bytes = a.E * a.elem_size;
-    if (bytes % 16 == 0) {
-        const int64_t vecs = bytes / 16;
-        const int64_t tpb = (vecs + kTileVecs - 1) / kTileVecs;
-        const int64_t total = tpb * blocks;
-        route_copy16_kernel<<<tile_grid(total), kThreads, 0, stream>>>(
-            static_cast<const uint4*>(a.in), static_cast<uint4*>(a.out), a.table, a.R, a.K, vecs, tpb,
-            total, a.backward);
-    } else {
-        const int64_t tpb = (a.E + kTileVecs - 1) / kTileVecs;
-        const int64_t total = tpb * blocks;
-        const int grid = tile_grid(total);
-        if (a.elem_size == 4)
-            route_copy_elem_kernel<uint32_t><<<grid, kThreads, 0, stream>>>(
-                static_cast<const uint32_t*>(a.in), static_cast<uint32_t*>(a.out), a.table, a.R, a.K,
-                a.E, tpb, total, a.backward);
-        else
-            route_copy_elem_kernel<uint16_t><<<grid, kThreads, 0, stream>>>(
-                static_cast<const uint16_t*>(a.in), static_cast<uint16_t*>(a.out), a.table, a.R, a.K,
-                a.E, tpb, total, a.backward);
-    }
-    return cudaGetLastError();
+    CopyArgs c;
+    c.in = static_cast<const unsigned char*>(a.in);
+    c.out = static_cast<unsigned char*>(a.out);
+    c.table = a.table;
+    c.B = a.B; c.R = a.R; c.K = a.K;
+    c.bytes = a.E * a.elem_size;
+    c.backward = a.backward;
+    c.seed = a.seed; c.step = a.step;
+    c.first_boundary = a.first_boundary; c.per_microbatch = a.per_microbatch;
+    if (a.B <= 0 || a.R <= 0 || a.K <= 0 || c.bytes <= 0) return cudaSuccess;
+    const bool wide = c.bytes % 32 == 0 && ((reinterpret_cast<uintptr_t>(a.in) | reinterpret_cast<uintptr_t>(a.out)) & 31) == 0;
+    if (wide) return a.draw ? launch_shape<Wide, 256, 2>(c, true, stream) : launch_shape<Wide, 384, 1>(c, false, stream);
+    if (c.bytes % 16 == 0) return a.draw ? launch_shape<uint4, 256, 4>(c, true, stream) : launch_shape<uint4, 256, 2>(c, false, stream);
+    return a.elem_size == 4 ? launch_shape<uint32_t, 128, 8>(c, a.draw, stream) : launch_shape<uint16_t, 128, 8>(c, a.draw, stream);
 }
 
 }  // namespace nolo

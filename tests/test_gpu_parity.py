@@ -436,6 +436,33 @@ def test_route_bit_exact(nolo, S, R, K, E, dt, pm):
     nolo.nolo_destroy(h)
 
 
+@pytest.mark.parametrize("R,K", [(1, 1), (4, 3), (32, 2), (33, 2)])
+@pytest.mark.parametrize("dt", [torch.float32, torch.bfloat16])
+def test_route_blocks_at_any_offset(nolo, R, K, dt):
+    """Blocks that are no multiple of 16 bytes: every combination of source and destination offset from
+    a 16-byte boundary, blocks shorter than a vector, whole tiles and one element more or less; up to 32
+    replicas draw inside the copy.  Nothing outside the output is written."""
+    S = 3
+    tile = 16384 // (4 if dt == torch.float32 else 2)
+    for E in (1, 3, 5, 7, 8, 9, 15, 17, 33, tile - 1, tile, tile + 1, tile + 9, 2 * tile + 3):
+        acts = synth.make_acts(S - 1, R, K, E, E, dt).cuda()
+        big = torch.full((acts.numel() + 64,), -5.0, dtype=dt, device="cuda")
+        out = big[32:32 + acts.numel()].view_as(acts)
+        back = torch.zeros_like(acts)
+        h = nolo.nolo_create(R, 1, 8, S, *F)
+        for pm in (False, True):
+            nolo.nolo_bind_route(h, R * K, E, out, per_microbatch=pm)
+            nolo.nolo_route(h, 9, E, acts)
+            table = O.draw_route(9, E, S, R, K, pm)
+            assert np.array_equal(nolo.nolo_get_route(h), table)
+            assert np.array_equal(to_np(out), O.route_forward(to_np(acts), table)), E
+            nolo.nolo_route_backward(h, 9, E, out, back)
+            torch.cuda.synchronize()
+            assert torch.equal(back, acts), E
+        assert bool((big[:32] == -5.0).all()) and bool((big[-32:] == -5.0).all())
+        nolo.nolo_destroy(h)
+
+
 @pytest.mark.parametrize("pm", [False, True])
 def test_route_one_boundary_at_a_time(nolo, pm):
     S, R, K, E = 4, 8, 2, 3000
