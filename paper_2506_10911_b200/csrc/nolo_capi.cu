@@ -616,9 +616,10 @@ int nolo_sim_straggler(int W, int n, int H, int T, double mu, double sigma, int6
     if ((double)W * (double)H * (double)T * (double)trials > (double)NOLO_SIM_MAX_SAMPLES) return NOLO_EINVAL;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     double* d = nullptr;
-    cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&d), sizeof(double) * (2 * (size_t)trials + 4));
+    const size_t results = sizeof(double) * (2 * (size_t)trials + 4);
+    cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&d), results + nolo::straggler_scratch(W, T, trials));
     if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? NOLO_ENOMEM : NOLO_ECUDA;
-    e = nolo::launch_straggler(W, n, H, T, mu, sigma, trials, seed, d + 4, d, s);
+    e = nolo::launch_straggler(W, n, H, T, mu, sigma, trials, seed, d + 4, d, reinterpret_cast<char*>(d) + results, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(host_stats, d, 4 * sizeof(double), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess && host_trials)
         e = cudaMemcpyAsync(host_trials, d + 4, sizeof(double) * 2 * (size_t)trials, cudaMemcpyDeviceToHost, s);

@@ -7,148 +7,270 @@
 //  * straggler effect: inner-step times LogNormal(mu, sigma^2); DiLoCo waits at a global barrier
 //    after every H inner steps, NoLoCo only for the members of its random subgroup of n.
 //
-// Random numbers: every Philox-4x64-10 block yields four times.  Words -> u = ((x >> 11) + 0.5) 2^-53;
-// Box-Muller on the word pairs (0,1) and (2,3), r = sqrt(-2 ln u_a), gives the normals
-// [r01 cos, r01 sin, r23 cos, r23 sin] of the angle 2 pi u_b; t = exp(mu + sigma z).  Sample j of a
-// stream is position j % 4 of block j / 4.  float64 throughout.
+// The random times and their stream are those of nolo_lognormal.cuh: four per Philox block, sample j of a
+// stream in position j % 4 of block j / 4.  float64 throughout.
+#include "nolo.h"
+#include "nolo_draw.cuh"
 #include "nolo_internal.h"
+#include "nolo_lognormal.cuh"
 #include "nolo_philox.cuh"
+
+#include <cmath>
 
 namespace nolo {
 
 namespace {
 
-constexpr int kTreeThreads = 128;   // small CTAs: the upper tree levels leave few threads busy
+constexpr int kSimThreads = 256;
 constexpr uint64_t kDomainTree = 3;
 constexpr uint64_t kDomainStraggler = 4;
 
-__device__ __forceinline__ double uniform_open(uint64_t x) {
-    return ((double)(x >> 11) + 0.5) * 0x1.0p-53;
+// ---- tree all-reduce ---------------------------------------------------------------------------
+//
+// A group of threads per trial: `group` = W/2 of them (one Philox block of each direction each) up to 256;
+// a CTA holds kSimThreads / group trials at a time and strides over the trials.  The times of all edges
+// of one direction are made first, by all threads at once, into shared memory, indexed like a binary
+// heap (root 1, children of p are 2p and 2p+1, leaves W .. 2W-1; block q holds those above the nodes 4q ..
+// 4q+3); then the levels are swept.  Bound by issue slots (the log-normal times); the sweeps are chains of
+// a dozen short steps that other trials of the SM fill.  A sweep of the levels that draws its times on
+// the way, one CTA per trial, leaves most threads idle near the root and computes every block twice.  Whole
+// call, before -> now: 20 000 trials of 1024 workers 2.0 -> 1.27 ms, 100 000 of 256 6.2 -> 1.6, 400 000 of 16
+// 7.2 -> 1.2 (0.6 ms of each is the allocation of the result).
+
+// Barrier of one trial's threads.  Groups are a power of two: parts of a warp, or whole CTAs' worth of warps.
+__device__ __forceinline__ void sync_group(int group) {
+    if (group <= 32) __syncwarp();
+    else __syncthreads();      // a group of more than a warp is the whole CTA
 }
 
-// The two log-normal times of one word pair: cosine first, sine second.
-__device__ __forceinline__ void lognormal2(uint64_t wa, uint64_t wb, double mu, double sigma, double& t_cos,
-                                           double& t_sin) {
-    double s, c;
-    const double r = sqrt(-2.0 * log(uniform_open(wa)));
-    sincospi(2.0 * uniform_open(wb), &s, &c);
-    t_cos = exp(mu + sigma * (r * c));
-    t_sin = exp(mu + sigma * (r * s));
-}
-
-// The four log-normal times of one block.
-__device__ __forceinline__ void lognormal4(const Philox4& b, double mu, double sigma, double (&t)[4]) {
-    lognormal2(b.w0, b.w1, mu, sigma, t[0], t[1]);
-    lognormal2(b.w2, b.w3, mu, sigma, t[2], t[3]);
-}
-
-// Maximum over the CTA, returned to every thread.  Contains two barriers.
-__device__ __forceinline__ double block_max(double v, double* scratch /*[32]*/) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, off));
-    __syncthreads();                      // scratch may still be read from a previous call
-    if ((threadIdx.x & 31) == 0) scratch[threadIdx.x >> 5] = v;
+template <bool TAME>
+__global__ void __launch_bounds__(kSimThreads)
+tree_allreduce_kernel(int W, int group, int64_t trials, LogNormal q, uint64_t seed, double* __restrict__ out) {
+    extern __shared__ double nodes[];                 // [trials of the CTA][2W]
+    __shared__ LogNormalTables tables;
+    __shared__ double part[kSimThreads / 32];
+    fill_tables(tables);
     __syncthreads();
-    const int warps = (blockDim.x + 31) >> 5;
-    double m = scratch[0];
-    for (int w = 1; w < warps; ++w) m = fmax(m, scratch[w]);
-    return m;
-}
-
-// One CTA per trial.  node[] holds ready times on the way up and arrival times on the way down,
-// indexed like a binary heap: root 1, children of p are 2p and 2p+1, leaves W .. 2W-1.
-__global__ void tree_allreduce_kernel(int W, double mu, double sigma, uint64_t seed,
-                                      double* __restrict__ out) {
-    extern __shared__ double node[];      // [2W]
-    __shared__ double scratch[32];
-    const uint64_t trial = blockIdx.x;
-    for (int i = threadIdx.x; i < 2 * W; i += blockDim.x) node[i] = 0.0;
-    __syncthreads();
-    // A block serves the four nodes 4q .. 4q+3; two siblings 2p, 2p+1 share one of its word pairs.  One
-    // thread per sibling pair: the levels near the root have few nodes, so the work of a block is
-    // split over two threads (each recomputes the block's integer rounds) rather than halving the
-    // number of busy threads.
-    for (int first = W >> 1; first >= 1; first >>= 1) {          // parents of one level: first .. 2*first-1
-        for (int p = first + threadIdx.x; p < 2 * first; p += blockDim.x) {
-            const Philox4 b = philox4x64_10(p >> 1, trial, 0, kDomainTree, seed, 0);   // children 2p, 2p+1 are in block p/2
-            double ta, tb;
-            if (p & 1) lognormal2(b.w2, b.w3, mu, sigma, ta, tb);
-            else lognormal2(b.w0, b.w1, mu, sigma, ta, tb);
-            node[p] = fmax(node[2 * p] + ta, node[2 * p + 1] + tb);
-        }
-        __syncthreads();
-    }
-    for (int first = 2; first < 2 * W; first <<= 1) {            // children of one level, top down, in sibling pairs
-        for (int c = first + 2 * threadIdx.x; c < 2 * first; c += 2 * blockDim.x) {
-            const Philox4 b = philox4x64_10(c >> 2, trial, 1, kDomainTree, seed, 0);
-            double ta, tb;
-            if (c & 2) lognormal2(b.w2, b.w3, mu, sigma, ta, tb);
-            else lognormal2(b.w0, b.w1, mu, sigma, ta, tb);
-            const double parent = node[c >> 1];
-            node[c] = parent + ta;
-            node[c + 1] = parent + tb;
-        }
-        __syncthreads();
-    }
-    double m = 0.0;
-    for (int leaf = W + threadIdx.x; leaf < 2 * W; leaf += blockDim.x) m = fmax(m, node[leaf]);
-    m = block_max(m, scratch);
-    if (threadIdx.x == 0) out[trial] = m;
-}
-
-// One CTA per trial; thread w (striding) owns worker w.
-__global__ void straggler_kernel(int W, int n, int H, int T, double mu, double sigma, uint64_t seed,
-                                 double* __restrict__ out /*[trials][2]*/) {
-    extern __shared__ unsigned char raw[];
-    uint64_t* keys = reinterpret_cast<uint64_t*>(raw);            // [W]
-    double* done = reinterpret_cast<double*>(keys + W);           // [W] clock + work of this step
-    double* clock = done + W;                                     // [W]
-    int* perm = reinterpret_cast<int*>(clock + W);                // [W]
-    __shared__ double scratch[32];
-    const uint64_t trial = blockIdx.x;
-    for (int w = threadIdx.x; w < W; w += blockDim.x) clock[w] = 0.0;
-    double barrier_clock = 0.0;
-    __syncthreads();
-    for (int t = 0; t < T; ++t) {
-        double longest = 0.0;
-        for (int w = threadIdx.x; w < W; w += blockDim.x) {
-            double work = 0.0;
-            for (int k0 = 0; k0 < H; k0 += 4) {                   // inner steps k0 .. k0+3 share a block
-                double step[4];
-                lognormal4(philox4x64_10(k0 >> 2, w, t, kDomainStraggler, seed, trial), mu, sigma, step);
-#pragma unroll
-                for (int l = 0; l < 4; ++l)
-                    if (k0 + l < H) work += step[l];
+    const int per_cta = blockDim.x / group, mine = threadIdx.x / group, lane = threadIdx.x % group;
+    double* node = nodes + (size_t)mine * 2 * W;
+    const int blocks = W / 2 > 1 ? W / 2 : 1;         // of four times each, the first two of block 0 above no node
+    for (int64_t first_trial = (int64_t)blockIdx.x * per_cta; first_trial < trials; first_trial += (int64_t)gridDim.x * per_cta) {
+        const int64_t trial = first_trial + mine;
+        const bool live = trial < trials;             // the threads of other trials only keep the barriers company
+        auto draw = [&](int phase) {
+            if (!live) return;
+            for (int b = lane; b < blocks; b += group) {
+                double t[4];
+                lognormal4<TAME>(tables, philox4x64_10(b, trial, phase, kDomainTree, seed, 0), q, t);
+                double2* to = reinterpret_cast<double2*>(node + 4 * b);
+                to[0] = make_double2(t[0], t[1]);
+                if (4 * b + 2 < 2 * W) to[1] = make_double2(t[2], t[3]);
             }
-            longest = fmax(longest, work);
-            done[w] = clock[w] + work;
-            keys[w] = draw_key(w, trial, 0, kDomainGroups, seed, t);
-        }
-        barrier_clock += block_max(longest, scratch);             // its barriers also publish done[] and keys[]
-        for (int w = threadIdx.x; w < W; w += blockDim.x) {
-            const uint64_t kw = keys[w];
-            int rank = 0;
-            for (int j = 0; j < W; ++j) {
-                const uint64_t kj = keys[j];
-                rank += (kj < kw) || (kj == kw && j < w);
+        };
+        // up: node[c] = time at which c's message has reached its parent
+        draw(0);
+        sync_group(group);
+        for (int first = W >> 1; first >= 2; first >>= 1) {          // parents of one level: first .. 2*first-1
+            for (int i = lane; i < first; i += group) {
+                const double2 c = reinterpret_cast<const double2*>(node)[first + i];
+                node[first + i] += fmax(c.x, c.y);
             }
-            perm[rank] = w;
+            sync_group(group);
         }
-        __syncthreads();
-        for (int i = threadIdx.x; i < W; i += blockDim.x) {      // position i of the permutation
-            const int g0 = (i / n) * n;
-            double m = done[perm[g0]];
-            for (int j = 1; j < n; ++j) m = fmax(m, done[perm[g0 + j]]);
-            clock[perm[i]] = m;
+        const double root = fmax(node[2], node[3]);
+        sync_group(group);
+        // down: node[c] = time at which the result has reached c
+        draw(1);
+        sync_group(group);
+        for (int i = lane; i < 2; i += group) node[2 + i] += root;
+        sync_group(group);
+        for (int first = 4; first < 2 * W; first <<= 1) {
+            for (int i = lane; i < first / 2; i += group) {           // sibling pairs
+                double2* c = reinterpret_cast<double2*>(node) + first / 2 + i;
+                const double parent = node[first / 2 + i];
+                *c = make_double2(parent + c->x, parent + c->y);
+            }
+            sync_group(group);
         }
-        __syncthreads();
+        double m = 0.0;
+        for (int leaf = W + lane; leaf < 2 * W; leaf += group) m = fmax(m, node[leaf]);
+        for (int o = (group < 32 ? group : 32) / 2; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+        if (group > 32) {
+            if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = m;
+            __syncthreads();
+            for (int w = 0; w < group / 32; ++w) m = fmax(m, part[w]);
+        }
+        if (live && lane == 0) out[trial] = m;
+        sync_group(group);                            // node[] and part[] are used again
     }
+}
+
+// ---- straggler simulation --------------------------------------------------------------------------
+//
+// Only the clocks depend on the iteration before: the work of every worker in every iteration and the
+// partitions do not.  So a slab of iterations is done by three kernels: the work sums (all of the random
+// times; bound by issue slots, any number of trials fills the chip), the partitions with the longest
+// work of each iteration (one CTA or warp each), and the clocks (one CTA per trial, a few exchanges
+// through shared memory per iteration).  One CTA per trial for everything used as many SMs as there were
+// trials, ranked the keys by O(W^2) comparisons in each iteration, and waited for itself.  Whole call, before ->
+// now, (W, n, H, T, trials): (1024, 2, 100, 250, 148) 39.0 -> 25.8 ms, (1024, 512, 100, 500, 8) 91.7 -> 4.3,
+// (100, 100, 100, 500, 50) 16.9 -> 2.6, (4, 2, 100, 500, 592) 15.7 -> 1.75, (64, 2, 50, 100, 8) 2.3 -> 0.69.
+struct Slab {
+    int W, n, H;
+    int iterations;            // of this slab, from t0 on
+    int64_t t0, trial0, trials;
+    LogNormal q;
+    uint64_t seed;
+    double* work;              // [trials][iterations][W]
+    uint16_t* order;           // [trials][iterations][W]: the worker in each position of the partition
+    double* longest;           // [trials][iterations]
+    double* clock;             // [trials][W], from slab to slab
+    double* out;               // [trials][2]: barrier and subgroup time so far
+};
+
+// lanes (a power of two, at most 32) threads share the blocks of one item (trial, iteration, worker).
+template <bool TAME>
+__global__ void __launch_bounds__(kSimThreads, 4)
+straggler_work_kernel(const Slab s, int lanes, int64_t items) {
+    __shared__ LogNormalTables tables;
+    fill_tables(tables);
+    __syncthreads();
+    const int64_t thread = (int64_t)blockIdx.x * kSimThreads + threadIdx.x;
+    const int64_t item = thread / lanes;
+    const int lane = (int)(thread % lanes);
+    double work = 0.0;
+    if (item < items) {
+        const int64_t row = item / s.W;
+        const int w = (int)(item - row * s.W);
+        const int64_t trial = row / s.iterations, t = row - trial * s.iterations;
+        for (int k = lane; 4 * k < s.H; k += lanes) {                // inner steps 4k .. 4k+3 share a block
+            double step[4];
+            lognormal4<TAME>(tables, philox4x64_10(k, w, s.t0 + t, kDomainStraggler, s.seed, s.trial0 + trial), s.q, step);
+            if (4 * k + 4 <= s.H) {
+                work += (step[0] + step[1]) + (step[2] + step[3]);
+            } else {
+                for (int l = 0; l < s.H - 4 * k; ++l) work += step[l];
+            }
+        }
+    }
+    for (int o = lanes / 2; o > 0; o >>= 1) work += __shfl_xor_sync(0xffffffffu, work, o);
+    if (item < items && lane == 0) s.work[item] = work;
+}
+
+// One row (trial, iteration) per CTA of THREADS; with 32 threads and W <= 32, one per warp of a larger CTA.
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS)
+straggler_order_kernel(const Slab s) {
+    extern __shared__ uint64_t raw[];
+    __shared__ double part[THREADS / 32];
+    const int64_t row = blockIdx.x;
+    const int64_t trial = row / s.iterations, t = row - trial * s.iterations;
+    int rank[kDrawPerThread];
+    rank_by_buckets<THREADS>(
+        reinterpret_cast<unsigned char*>(raw), s.W,
+        [&](int i) { return draw_key(i, s.trial0 + trial, 0, kDomainGroups, s.seed, s.t0 + t); }, rank);
     double m = 0.0;
-    for (int w = threadIdx.x; w < W; w += blockDim.x) m = fmax(m, clock[w]);
-    m = block_max(m, scratch);
+#pragma unroll
+    for (int k = 0; k < kDrawPerThread; ++k) {
+        const int w = threadIdx.x + k * THREADS;
+        if (w < s.W) {
+            s.order[row * s.W + rank[k]] = (uint16_t)w;
+            m = fmax(m, s.work[row * s.W + w]);
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = m;
+    __syncthreads();
     if (threadIdx.x == 0) {
-        out[2 * trial] = barrier_clock;
-        out[2 * trial + 1] = m;
+        for (int w = 1; w < THREADS / 32; ++w) m = fmax(m, part[w]);
+        s.longest[row] = m;
+    }
+}
+
+__global__ void __launch_bounds__(kSimThreads)
+straggler_order_warp_kernel(const Slab s, int64_t rows) {
+    const int64_t row = ((int64_t)blockIdx.x * kSimThreads + threadIdx.x) >> 5;
+    if (row >= rows) return;
+    const int lane = threadIdx.x & 31;
+    const int64_t trial = row / s.iterations, t = row - trial * s.iterations;
+    const int rank = rank_by_warp(s.W, s.trial0 + trial, 0, kDomainGroups, s.seed, s.t0 + t);
+    double m = 0.0;
+    if (lane < s.W) {
+        s.order[row * s.W + rank] = (uint16_t)lane;
+        m = s.work[row * s.W + lane];
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (lane == 0) s.longest[row] = m;
+}
+
+// The clocks of one trial per CTA.  `lanes` (a power of two, at most 32 and n) threads share a subgroup.
+__global__ void __launch_bounds__(1024)
+straggler_clock_kernel(const Slab s, int lanes) {
+    extern __shared__ uint64_t raw[];
+    double* clock = reinterpret_cast<double*>(raw);           // [W] when each worker is done with its work
+    uint16_t* order = reinterpret_cast<uint16_t*>(clock + s.W);   // [W]
+    const int64_t trial = blockIdx.x;
+    const int lane = threadIdx.x % lanes, groups = s.W / s.n;
+    for (int w = threadIdx.x; w < s.W; w += blockDim.x) clock[w] = s.t0 ? s.clock[trial * s.W + w] : 0.0;
+    double barrier = s.t0 ? s.out[2 * trial] : 0.0;
+    // the work and the partition of an iteration are read one iteration ahead
+    constexpr int kMost = NOLO_MAX_WORKERS / 1024;
+    double work[kMost], longest;
+    uint16_t position[kMost];
+    auto read = [&](int i) {
+        const int64_t row = trial * s.iterations + i;
+#pragma unroll
+        for (int k = 0; k < kMost; ++k) {
+            const int w = threadIdx.x + k * blockDim.x;
+            if (w < s.W) {
+                work[k] = s.work[row * s.W + w];
+                position[k] = s.order[row * s.W + w];
+            }
+        }
+        longest = s.longest[row];
+    };
+    read(0);
+    __syncthreads();
+    for (int i = 0; i < s.iterations; ++i) {
+#pragma unroll
+        for (int k = 0; k < kMost; ++k) {
+            const int w = threadIdx.x + k * blockDim.x;
+            if (w < s.W) {
+                clock[w] += work[k];
+                order[w] = position[k];
+            }
+        }
+        barrier += longest;
+        if (i + 1 < s.iterations) read(i + 1);
+        __syncthreads();
+        for (int g0 = 0; g0 < groups; g0 += blockDim.x / lanes) {     // every lane of a subgroup takes the same turns
+            const int g = g0 + threadIdx.x / lanes;
+            const uint16_t* member = order + (g < groups ? g : 0) * s.n;
+            double m = 0.0;
+            if (g < groups)
+                for (int j = lane; j < s.n; j += lanes) m = fmax(m, clock[member[j]]);
+            for (int o = lanes / 2; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+            if (g < groups)
+                for (int j = lane; j < s.n; j += lanes) clock[member[j]] = m;
+        }
+        __syncthreads();
+    }
+    double m = 0.0;
+    for (int w = threadIdx.x; w < s.W; w += blockDim.x) {
+        m = fmax(m, clock[w]);
+        s.clock[trial * s.W + w] = clock[w];
+    }
+    __shared__ double part[32];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < (int)blockDim.x / 32; ++w) m = fmax(m, part[w]);
+        s.out[2 * trial] = barrier;
+        s.out[2 * trial + 1] = m;
     }
 }
 
@@ -187,36 +309,92 @@ column_stats_kernel(const double* __restrict__ x, int64_t rows, int cols, double
     }
 }
 
-int round_up_threads(int want) {
-    const int t = (want + 31) / 32 * 32;
-    return t < 32 ? 32 : (t > 1024 ? 1024 : t);
+// Iterations and trials whose work sums are held at a time.
+constexpr int64_t kSlabItems = 1 << 21;
+
+int64_t slab_trials(int W, int64_t trials) {
+    const int64_t most = kSlabItems / W;
+    return trials < most ? trials : most;
+}
+
+int64_t slab_iterations(int W, int T, int64_t trials) {
+    const int64_t most = kSlabItems / (W * slab_trials(W, trials));
+    return T < most ? T : most;
 }
 
 }  // namespace
 
 cudaError_t launch_tree_allreduce(int W, double mu, double sigma, int64_t trials, uint64_t seed,
                                   double* per_trial, double* stats, cudaStream_t stream) {
-    const size_t smem = sizeof(double) * 2 * (size_t)W;
-    cudaError_t e = cudaFuncSetAttribute(tree_allreduce_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    const int blocks = W / 2 > 1 ? W / 2 : 1;
+    const int group = blocks < kSimThreads ? blocks : kSimThreads;
+    const int threads = group <= 32 ? kSimThreads : group;
+    const int per_cta = threads / group;
+    const size_t smem = sizeof(double) * 2 * (size_t)W * per_cta;
+    auto kernel = LogNormal::tame(mu, sigma) ? tree_allreduce_kernel<true> : tree_allreduce_kernel<false>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    tree_allreduce_kernel<<<(unsigned)trials, round_up_threads(W / 2 < kTreeThreads ? W / 2 : kTreeThreads), smem, stream>>>(W, mu, sigma, seed,
-                                                                                        per_trial);
+    int device = 0, sms = 0, resident = 0;
+    e = cudaGetDevice(&device);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, kernel, threads, smem);
+    if (e != cudaSuccess) return e;
+    const int64_t ctas = (trials + per_cta - 1) / per_cta, most = (int64_t)sms * (resident > 0 ? resident : 1);
+    kernel<<<(unsigned)(ctas < most ? ctas : most), threads, smem, stream>>>(W, group, trials, LogNormal::make(mu, sigma), seed,
+                                                                            per_trial);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     column_stats_kernel<<<1, 1024, 0, stream>>>(per_trial, trials, 1, stats);
     return cudaGetLastError();
 }
 
-cudaError_t launch_straggler(int W, int n, int H, int T, double mu, double sigma, int64_t trials,
-                             uint64_t seed, double* per_trial, double* stats, cudaStream_t stream) {
-    const size_t smem = (size_t)W * (8 + 8 + 8 + 4);
-    cudaError_t e = cudaFuncSetAttribute(straggler_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    straggler_kernel<<<(unsigned)trials, round_up_threads(W), smem, stream>>>(W, n, H, T, mu, sigma, seed,
-                                                                              per_trial);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+size_t straggler_scratch(int W, int T, int64_t trials) {
+    const size_t rows = (size_t)slab_trials(W, trials) * slab_iterations(W, T, trials);
+    return rows * W * (sizeof(double) + sizeof(uint16_t)) + rows * sizeof(double) +
+           (size_t)slab_trials(W, trials) * W * sizeof(double) + 64;
+}
+
+cudaError_t launch_straggler(int W, int n, int H, int T, double mu, double sigma, int64_t trials, uint64_t seed,
+                             double* per_trial, double* stats, void* scratch, cudaStream_t stream) {
+    const int64_t group = slab_trials(W, trials), iterations = slab_iterations(W, T, trials);
+    Slab s;
+    s.W = W; s.n = n; s.H = H;
+    s.q = LogNormal::make(mu, sigma);
+    s.seed = seed;
+    s.work = static_cast<double*>(scratch);
+    s.clock = s.work + group * iterations * W;
+    s.longest = s.clock + group * W;
+    s.order = reinterpret_cast<uint16_t*>(s.longest + group * iterations);
+    auto work_kernel = LogNormal::tame(mu, sigma) ? straggler_work_kernel<true> : straggler_work_kernel<false>;
+    const int threads = W >= 1024 ? 1024 : (W + 31) / 32 * 32;
+    int lanes = 1;
+    while (2 * lanes <= n && lanes < 32) lanes *= 2;
+    for (int64_t trial0 = 0; trial0 < trials; trial0 += group) {
+        s.trial0 = trial0;
+        s.trials = trials - trial0 < group ? trials - trial0 : group;
+        s.out = per_trial + 2 * trial0;
+        for (int64_t t0 = 0; t0 < T; t0 += iterations) {
+            s.t0 = t0;
+            s.iterations = (int)(T - t0 < iterations ? T - t0 : iterations);
+            const int64_t rows = s.trials * s.iterations, items = rows * W;
+            // Threads per item: enough to fill the chip about twice, at most one per block of the item.
+            int split = 1;
+            while (items * split < (1 << 18) && split < 32 && 4 * split < H) split *= 2;
+            const int64_t work_ctas = (items * split + kSimThreads - 1) / kSimThreads;
+            work_kernel<<<(unsigned)work_ctas, kSimThreads, 0, stream>>>(s, split, items);
+            auto order = [&](auto kernel, int order_threads) {
+                kernel<<<(unsigned)rows, order_threads, draw_scratch_bytes(W, order_threads), stream>>>(s);
+            };
+            if (W <= 32)
+                straggler_order_warp_kernel<<<(unsigned)((rows * 32 + kSimThreads - 1) / kSimThreads), kSimThreads, 0, stream>>>(s, rows);
+            else if (W <= 512) order(straggler_order_kernel<128>, 128);
+            else if (W <= 2048) order(straggler_order_kernel<512>, 512);
+            else order(straggler_order_kernel<1024>, 1024);
+            straggler_clock_kernel<<<(unsigned)s.trials, threads, (size_t)W * 10, stream>>>(s, lanes);
+            const cudaError_t e = cudaGetLastError();
+            if (e != cudaSuccess) return e;
+        }
+    }
     column_stats_kernel<<<1, 1024, 0, stream>>>(per_trial, trials, 2, stats);
     return cudaGetLastError();
 }

@@ -21,7 +21,7 @@ def nolo():
 
 @pytest.mark.parametrize("W,mu,sigma,trials,seed", [
     (2, 0.5, 0.8, 50, 3), (4, 0.0, 1.0, 40, 2), (64, 1.0, math.sqrt(0.5), 12, 9), (1024, -0.3, 0.25, 3, 1),
-    (4096, 0.0, 0.5, 1, 5),
+    (4096, 0.0, 0.5, 1, 5), (8, 0.0, 1.0, 300, 4), (32, 0.2, 0.7, 70, 4), (128, 0.2, 0.7, 5, 4), (512, 0.1, 1.0, 2, 4),
 ])
 def test_tree_allreduce_trials_match_oracle(nolo, W, mu, sigma, trials, seed):
     mean, se, per = nolo.nolo_sim_tree_allreduce(W, mu, sigma, trials, seed, return_trials=True)
@@ -60,6 +60,37 @@ def test_straggler_trials_match_oracle(nolo, W, n, H, T, trials, seed):
     assert stats[0] == pytest.approx(want[:, 0].mean(), rel=RTOL)
     assert stats[1] == pytest.approx(want[:, 1].mean(), rel=RTOL)
     assert (per[:, 1] <= per[:, 0] * (1 + 1e-15)).all()
+
+
+@pytest.mark.parametrize("W,n,H,T,trials", [
+    (2, 1, 1, 1, 3), (31, 31, 5, 3, 2), (32, 16, 4, 3, 2), (33, 11, 9, 3, 2), (96, 48, 33, 2, 2), (512, 128, 3, 2, 1),
+    (513, 27, 3, 2, 1), (1025, 205, 3, 2, 1), (4096, 4096, 2, 2, 1), (4096, 1, 130, 1, 1),
+])
+def test_straggler_kernel_boundaries(nolo, W, n, H, T, trials):
+    """Sizes where the kernels change: warps or CTAs of 128, 512 or 1024 threads per partition, subgroups
+    shared by up to 32 threads, items shared by up to 32 threads, inner steps that fill no block."""
+    *_, per = nolo.nolo_sim_straggler(W, n, H, T, 0.5, 0.9, trials, 12, return_trials=True)
+    np.testing.assert_allclose(per, L.sim_straggler(W, n, H, T, 0.5, 0.9, trials, 12), rtol=RTOL)
+
+
+def test_straggler_in_slabs_agrees_with_itself(nolo):
+    """2^21 work sums are held at a time.  The first trials of a call that needs several slabs of
+    iterations (and of trials) have the times that a call of those trials alone gives."""
+    for W, T, trials in ((2048, 30, 40), (4096, 3, 600)):
+        *_, per = nolo.nolo_sim_straggler(W, 2, 2, T, 0.0, 0.5, trials, 3, return_trials=True)
+        *_, few = nolo.nolo_sim_straggler(W, 2, 2, T, 0.0, 0.5, 2, 3, return_trials=True)
+        np.testing.assert_allclose(per[:2], few, rtol=1e-14)
+        assert (per[:, 1] <= per[:, 0] * (1 + 1e-15)).all() and (per > 0).all()
+
+
+@pytest.mark.parametrize("mu,sigma", [(0.0, 80.0), (690.0, 0.5), (705.0, 1.0), (-740.0, 0.1), (0.0, 0.0), (0.0, 400.0)])
+def test_times_at_the_ends_of_the_range(nolo, mu, sigma):
+    """Times that leave the normal numbers are taken by the general form of exp; either form agrees with
+    the oracle (relative to e^|exponent|'s own rounding: 2^-53 of an exponent of 700 is 8e-14)."""
+    with np.errstate(over="ignore"):
+        want = L.sim_tree_allreduce(16, mu, sigma, 40, 8)
+    *_, per = nolo.nolo_sim_tree_allreduce(16, mu, sigma, 40, 8, return_trials=True)
+    np.testing.assert_allclose(per, want, rtol=1e-11, atol=1e-320)
 
 
 def test_straggler_reproduces_the_papers_figure_at_full_size(nolo):
