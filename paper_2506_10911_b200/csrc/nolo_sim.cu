@@ -113,7 +113,7 @@ tree_allreduce_kernel(int W, int group, int64_t trials, LogNormal q, uint64_t se
 // work of each iteration (one CTA or warp each), and the clocks (one CTA per trial, a few exchanges
 // through shared memory per iteration).  One CTA per trial for everything used as many SMs as there were
 // trials, ranked the keys by O(W^2) comparisons in each iteration, and waited for itself.  Whole call, before ->
-// now, (W, n, H, T, trials): (1024, 2, 100, 250, 148) 39.0 -> 25.8 ms, (1024, 512, 100, 500, 8) 91.7 -> 4.3,
+// now, (W, n, H, T, trials): (1024, 2, 100, 250, 148) 39.0 -> 17.6 ms, (1024, 512, 100, 500, 8) 91.7 -> 4.3,
 // (100, 100, 100, 500, 50) 16.9 -> 2.6, (4, 2, 100, 500, 592) 15.7 -> 1.75, (64, 2, 50, 100, 8) 2.3 -> 0.69.
 struct Slab {
     int W, n, H;
@@ -128,10 +128,59 @@ struct Slab {
     double* out;               // [trials][2]: barrier and subgroup time so far
 };
 
-// lanes (a power of two, at most 32) threads share the blocks of one item (trial, iteration, worker).
+// A thread per item (trial, iteration, worker), for W >= kSharedRowsW.  A CTA's items lie in few rows (trial,
+// iteration), so the part of the Philox rounds that depends on the row and the block only is made once for
+// the CTA, kSharedBlocks blocks at a time.  Bound by issue slots and by the 64-bit products: 15 of them per
+// four times: 215 G times/s in all (W = 1024, H = 100), 170 with all 20 products per block.
+constexpr int kSharedRowsW = 64;
+constexpr int kSharedRows = (kSimThreads - 2) / kSharedRowsW + 2;
+constexpr int kSharedBlocks = 32;
+
 template <bool TAME>
 __global__ void __launch_bounds__(kSimThreads, 4)
-straggler_work_kernel(const Slab s, int lanes, int64_t items) {
+straggler_work_kernel(const Slab s, int64_t items) {
+    __shared__ LogNormalTables tables;
+    __shared__ PhiloxOfC0 lead[kSharedRows][kSharedBlocks];
+    fill_tables(tables);
+    const int64_t item = (int64_t)blockIdx.x * kSimThreads + threadIdx.x;
+    const int64_t row0 = (int64_t)blockIdx.x * kSimThreads / s.W;
+    const int64_t last = (int64_t)blockIdx.x * kSimThreads + kSimThreads - 1;
+    const int rows = (int)((last < items ? last : items - 1) / s.W - row0) + 1;
+    const int64_t row = item / s.W;
+    const int w = (int)(item - row * s.W), mine = item < items ? (int)(row - row0) : 0;
+    const int64_t trial = row / s.iterations, t = row - trial * s.iterations;
+    const PhiloxOfC1 of_worker = philox_of_c1(w, s.t0 + t, s.seed);
+    const int blocks = (s.H + 3) / 4;
+    double work = 0.0;
+    for (int b0 = 0; b0 < blocks; b0 += kSharedBlocks) {
+        __syncthreads();
+        for (int i = threadIdx.x; i < rows * kSharedBlocks; i += kSimThreads) {
+            const int64_t r = row0 + i / kSharedBlocks, r_trial = r / s.iterations;
+            lead[i / kSharedBlocks][i % kSharedBlocks] =
+                philox_of_c0(b0 + i % kSharedBlocks, s.t0 + (r - r_trial * s.iterations), kDomainStraggler, s.seed,
+                             s.trial0 + r_trial);
+        }
+        __syncthreads();
+        const int here = blocks - b0 < kSharedBlocks ? blocks - b0 : kSharedBlocks;
+        for (int k = 0; k < here; ++k) {                             // inner steps 4 (b0 + k) .. + 3 share a block
+            double step[4];
+            lognormal4<TAME>(tables, philox_join(lead[mine][k], of_worker, s.seed, s.trial0 + trial), s.q, step);
+            const int left = s.H - 4 * (b0 + k);
+            if (left >= 4) {
+                work += (step[0] + step[1]) + (step[2] + step[3]);
+            } else {
+                for (int l = 0; l < left; ++l) work += step[l];
+            }
+        }
+    }
+    if (item < items) s.work[item] = work;
+}
+
+// The same for any W: `lanes` (a power of two, at most 32) threads share the blocks of an item, so that few
+// items fill the chip too.
+template <bool TAME>
+__global__ void __launch_bounds__(kSimThreads, 4)
+straggler_split_work_kernel(const Slab s, int lanes, int64_t items) {
     __shared__ LogNormalTables tables;
     fill_tables(tables);
     __syncthreads();
@@ -143,7 +192,7 @@ straggler_work_kernel(const Slab s, int lanes, int64_t items) {
         const int64_t row = item / s.W;
         const int w = (int)(item - row * s.W);
         const int64_t trial = row / s.iterations, t = row - trial * s.iterations;
-        for (int k = lane; 4 * k < s.H; k += lanes) {                // inner steps 4k .. 4k+3 share a block
+        for (int k = lane; 4 * k < s.H; k += lanes) {
             double step[4];
             lognormal4<TAME>(tables, philox4x64_10(k, w, s.t0 + t, kDomainStraggler, s.seed, s.trial0 + trial), s.q, step);
             if (4 * k + 4 <= s.H) {
@@ -365,7 +414,7 @@ cudaError_t launch_straggler(int W, int n, int H, int T, double mu, double sigma
     s.clock = s.work + group * iterations * W;
     s.longest = s.clock + group * W;
     s.order = reinterpret_cast<uint16_t*>(s.longest + group * iterations);
-    auto work_kernel = LogNormal::tame(mu, sigma) ? straggler_work_kernel<true> : straggler_work_kernel<false>;
+    const bool tame = LogNormal::tame(mu, sigma);
     const int threads = W >= 1024 ? 1024 : (W + 31) / 32 * 32;
     int lanes = 1;
     while (2 * lanes <= n && lanes < 32) lanes *= 2;
@@ -380,8 +429,12 @@ cudaError_t launch_straggler(int W, int n, int H, int T, double mu, double sigma
             // Threads per item: enough to fill the chip about twice, at most one per block of the item.
             int split = 1;
             while (items * split < (1 << 18) && split < 32 && 4 * split < H) split *= 2;
-            const int64_t work_ctas = (items * split + kSimThreads - 1) / kSimThreads;
-            work_kernel<<<(unsigned)work_ctas, kSimThreads, 0, stream>>>(s, split, items);
+            const unsigned work_ctas = (unsigned)((items * split + kSimThreads - 1) / kSimThreads);
+            if (split == 1 && W >= kSharedRowsW)
+                (tame ? straggler_work_kernel<true> : straggler_work_kernel<false>)<<<work_ctas, kSimThreads, 0, stream>>>(s, items);
+            else
+                (tame ? straggler_split_work_kernel<true>
+                      : straggler_split_work_kernel<false>)<<<work_ctas, kSimThreads, 0, stream>>>(s, split, items);
             auto order = [&](auto kernel, int order_threads) {
                 kernel<<<(unsigned)rows, order_threads, draw_scratch_bytes(W, order_threads), stream>>>(s);
             };
