@@ -310,7 +310,8 @@ int nolo_divergence(nolo_handle* h, double* host_out);
  *   stream  cudaStream_t for the kernels
  *   host_stats   host, 2 doubles: mean completion time, its standard error
  *   host_trials  host, [trials] completion times, or NULL
- * float64 arithmetic.  Synchronous; allocates and frees its own scratch.
+ * float64 arithmetic.  Synchronous; allocates its own scratch, of which the
+ * library keeps up to 64 MB for later calls until a handle is destroyed.
  * Errors: NOLO_EINVAL, NOLO_ENOMEM, NOLO_ECUDA.
  */
 int nolo_sim_tree_allreduce(int W, double mu, double sigma, int64_t trials, uint64_t seed,
@@ -338,7 +339,7 @@ double nolo_expected_pair_exchange(double mu, double sigma);
  *   host_stats   host, 4 doubles: mean time with the global barrier, mean time
  *           with subgroup waits, then the standard errors of the two means
  *   host_trials  host, [trials][2] (barrier, subgroup) per trial, or NULL
- * Synchronous; allocates and frees its own scratch.  trials 1..2^20, and the
+ * Synchronous; scratch as above (at most about 40 MB).  trials 1..2^20, and the
  * total number of samples W*H*T*trials at most NOLO_SIM_MAX_SAMPLES (2^40, about
  * 20 s of GPU time): a larger request is refused with NOLO_EINVAL rather than
  * left to occupy the device.

@@ -34,8 +34,8 @@ constexpr uint64_t kDomainStraggler = 4;
 // 4q+3); then the levels are swept.  Bound by issue slots (the log-normal times); the sweeps are chains of
 // a dozen short steps that other trials of the SM fill.  A sweep of the levels that draws its times on
 // the way, one CTA per trial, leaves most threads idle near the root and computes every block twice.  Whole
-// call, before -> now: 20 000 trials of 1024 workers 2.0 -> 1.27 ms, 100 000 of 256 6.2 -> 1.6, 400 000 of 16
-// 7.2 -> 1.2 (0.6 ms of each is the allocation of the result).
+// call, before -> now: 20 000 trials of 1024 workers 2.0 -> 0.56 ms, 100 000 of 256 3.4 -> 0.87, 400 000 of 16
+// 4.0 -> 0.54 (0.65 ms of each was the allocation of the result).
 
 // Barrier of one trial's threads.  Groups are a power of two: parts of a warp, or whole CTAs' worth of warps.
 __device__ __forceinline__ void sync_group(int group) {
@@ -113,8 +113,8 @@ tree_allreduce_kernel(int W, int group, int64_t trials, LogNormal q, uint64_t se
 // work of each iteration (one CTA or warp each), and the clocks (one CTA per trial, a few exchanges
 // through shared memory per iteration).  One CTA per trial for everything used as many SMs as there were
 // trials, ranked the keys by O(W^2) comparisons in each iteration, and waited for itself.  Whole call, before ->
-// now, (W, n, H, T, trials): (1024, 2, 100, 250, 148) 39.0 -> 17.6 ms, (1024, 512, 100, 500, 8) 91.7 -> 4.3,
-// (100, 100, 100, 500, 50) 16.9 -> 2.6, (4, 2, 100, 500, 592) 15.7 -> 1.75, (64, 2, 50, 100, 8) 2.3 -> 0.69.
+// now, (W, n, H, T, trials): (1024, 2, 100, 250, 148) 39.0 -> 16.8 ms, (1024, 512, 100, 500, 8) 91.7 -> 3.1,
+// (100, 100, 100, 500, 50) 16.9 -> 1.6, (4, 2, 100, 500, 592) 15.7 -> 1.04, (64, 2, 50, 100, 8) 2.3 -> 0.13.
 struct Slab {
     int W, n, H;
     int iterations;            // of this slab, from t0 on

@@ -103,6 +103,32 @@ def test_straggler_reproduces_the_papers_figure_at_full_size(nolo):
     assert b == pytest.approx(500 * math.e, rel=1e-12) and s == pytest.approx(b, rel=1e-15)
 
 
+def test_simulations_from_several_threads_and_streams(nolo):
+    """Each call has scratch of its own: calls that overlap give what they give alone, also when handles
+    are destroyed in between (which gives kept scratch back)."""
+    import threading
+    import torch
+    want = {s: (nolo.nolo_sim_tree_allreduce(64, 0.0, 1.0, 5000, s, return_trials=True)[2],
+                nolo.nolo_sim_straggler(64, 2, 10, 20, 0.0, 0.5, 40, s, return_trials=True)[4]) for s in range(6)}
+    bad = []
+
+    def work(s):
+        stream = torch.cuda.Stream()
+        for _ in range(10):
+            a = nolo.nolo_sim_tree_allreduce(64, 0.0, 1.0, 5000, s, stream, return_trials=True)[2]
+            b = nolo.nolo_sim_straggler(64, 2, 10, 20, 0.0, 0.5, 40, s, stream, return_trials=True)[4]
+            nolo.nolo_destroy(nolo.nolo_create(2, 1, 8, 1, 0.5, 0.7, 0.5))
+            if not (np.array_equal(a, want[s][0]) and np.array_equal(b, want[s][1])):
+                bad.append(s)
+
+    threads = [threading.Thread(target=work, args=(s,)) for s in range(6)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad
+
+
 def test_simulation_argument_checks(nolo):
     for bad in [(6, 0.0, 1.0, 10), (1, 0.0, 1.0, 10), (8, 0.0, -1.0, 10), (8, 0.0, 1.0, 0), (8, float("nan"), 1.0, 1)]:
         with pytest.raises(nolo.NoloError) as e:
