@@ -370,7 +370,7 @@ def time_outer_cases(nolo, dev, W, P, theta, variants, peak, copy_gbs, warmup=3,
             for _ in range(steps):
                 nolo.nolo_divergence(h)
             st, cnt = nolo.nolo_timing_stats(h, nolo.NOLO_KERNEL_DIVERGENCE)
-            recs.append(stats_record(f"{name}: divergence", "divergence_partial_kernel + divergence_final_kernel",
+            recs.append(stats_record(f"{name}: divergence", "divergence_kernel + divergence_finish_kernel",
                                      st, cnt, 4 * W * P, peak, copy_gbs, W=W, P=P,
                                      note="read-only pass; the read-only ceiling is above the copy figure"))
             # split-phase step: subgroup means of phi prepared ahead, then the step that uses them

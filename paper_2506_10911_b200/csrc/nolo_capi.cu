@@ -57,8 +57,8 @@ struct nolo_handle {
     bool route_valid = false;
 
     // divergence metric scratch (allocated on first use)
-    void* d_div_partials = nullptr;
-    double* d_div_out = nullptr;
+    void* d_div = nullptr;       // partial sums, then the counter of arrived CTAs
+    double* div_out = nullptr;   // page-locked host memory that the kernel writes
 
     // host-streaming helpers (created on first use)
     cudaStream_t s_in = nullptr, s_out = nullptr;
@@ -547,21 +547,29 @@ int nolo_divergence(nolo_handle* h, double* host_out) {
     if (!h) return NOLO_EINVAL;
     if (!host_out) return fail(h, NOLO_EINVAL, "host_out must not be NULL");
     if (!h->state_bound) return fail(h, NOLO_ESTATE, "nolo_bind_state has not been called");
-    if (!h->d_div_partials) {
-        cudaError_t e = cudaMalloc(&h->d_div_partials, (size_t)nolo::divergence_partials(h->P) * 16);
-        if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&h->d_div_out), 2 * sizeof(double));
+    const size_t partials = (size_t)nolo::divergence_partials(h->W, h->P) * 16;
+    if (!h->d_div) {
+        void* d = nullptr;
+        cudaError_t e = cudaMalloc(&d, partials + 16);
+        if (e == cudaSuccess) e = cudaMemsetAsync(static_cast<char*>(d) + partials, 0, 16, h->stream);
+        if (e == cudaSuccess && !h->div_out)
+            e = cudaHostAlloc(reinterpret_cast<void**>(&h->div_out), 2 * sizeof(double), cudaHostAllocMapped);
         if (e != cudaSuccess) {
-            if (h->d_div_partials) { cudaFree(h->d_div_partials); h->d_div_partials = nullptr; }
+            if (d) cudaFree(d);
             return fail(h, e == cudaErrorMemoryAllocation ? NOLO_ENOMEM : NOLO_ECUDA,
                         "divergence scratch allocation: %s", cudaGetErrorString(e));
         }
+        h->d_div = d;
     }
     Bracket br(h, NOLO_KERNEL_DIVERGENCE);
-    NOLO_CUDA(h, nolo::launch_divergence(h->phi, h->W, h->stride, h->P, h->d_div_partials, h->d_div_out, h->stream));
+    NOLO_CUDA(h, nolo::launch_divergence(h->phi, h->W, h->stride, h->P, h->d_div,
+                                         reinterpret_cast<unsigned*>(static_cast<char*>(h->d_div) + partials), h->div_out,
+                                         h->stream));
     br.done();
-    h->launches += 2;
-    NOLO_CUDA(h, cudaMemcpyAsync(host_out, h->d_div_out, 2 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+    ++h->launches;
     NOLO_CUDA(h, cudaStreamSynchronize(h->stream));
+    host_out[0] = h->div_out[0];
+    host_out[1] = h->div_out[1];
     return NOLO_OK;
 }
 
@@ -642,8 +650,8 @@ int nolo_destroy(nolo_handle* h) {
     }
     if (h->d_perm) cudaFree(h->d_perm);
     if (h->d_route) cudaFree(h->d_route);
-    if (h->d_div_partials) cudaFree(h->d_div_partials);
-    if (h->d_div_out) cudaFree(h->d_div_out);
+    if (h->d_div) cudaFree(h->d_div);
+    if (h->div_out) cudaFreeHost(h->div_out);
     delete h;
     g_scratch.give_back();
     return NOLO_OK;

@@ -96,9 +96,10 @@ cudaError_t launch_copy_probe(const void* in, void* out, int64_t bytes, cudaStre
 
 // Replica divergence of phi (Fig. 3b): out2[0] = mean over parameters of the across-worker
 // population standard deviation, out2[1] = sqrt(mean over parameters of the across-worker variance).
-// `partials` is device scratch of divergence_partials(P) * 16 bytes; out2 is device memory.
-int64_t divergence_partials(int64_t P);
-cudaError_t launch_divergence(const float* phi, int W, int64_t stride, int64_t P, void* partials,
+// `partials` is device scratch of divergence_partials(W, P) * 16 bytes, `arrived` a device counter that is zero
+// before and after; out2 is device or mapped host memory.  One launch.
+int64_t divergence_partials(int W, int64_t P);
+cudaError_t launch_divergence(const float* phi, int W, int64_t stride, int64_t P, void* partials, unsigned* arrived,
                               double* out2, cudaStream_t stream);
 
 // Latency simulations (Section 4.3).  per_trial: device [trials] resp. [trials][2];

@@ -4,136 +4,228 @@
 // For every parameter p the population variance of phi[0..W-1][p] across the workers is computed
 // with Welford's update in float32 (stable when the replicas are close, as they are), and the
 // per-parameter standard deviation and variance are summed over all parameters in float64: first
-// inside each CTA, then over the CTAs by a second kernel, both in a fixed order, so the result is
-// reproducible.  A read-only pass: 4 bytes per worker-parameter.
+// inside each CTA, then over the CTAs by the last of them to finish, both in a fixed order, so the result
+// is reproducible.  A read-only pass: 4 bytes per worker-parameter.
 #include "nolo_internal.h"
+#include "nolo_launch.cuh"
 
 namespace nolo {
 
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kItems = 4;     // quads per thread
-constexpr int kUnroll = 4;    // worker rows in flight per thread
-
-struct Welford4 {
-    float4 mean, m2;
-    __device__ __forceinline__ void init() {
-        mean = make_float4(0.f, 0.f, 0.f, 0.f);
-        m2 = mean;
+// One column's mean and sum of squared deviations over some workers.
+struct Moments {
+    float mean, m2;
+    __device__ __forceinline__ void push(float x, float inv_k) {
+        const float d = x - mean;
+        mean += d * inv_k;
+        m2 += d * (x - mean);
     }
-    __device__ __forceinline__ void push(float4 x, float inv_k) {
-        float d;
-        d = x.x - mean.x; mean.x += d * inv_k; m2.x += d * (x.x - mean.x);
-        d = x.y - mean.y; mean.y += d * inv_k; m2.y += d * (x.y - mean.y);
-        d = x.z - mean.z; mean.z += d * inv_k; m2.z += d * (x.z - mean.z);
-        d = x.w - mean.w; mean.w += d * inv_k; m2.w += d * (x.w - mean.w);
+    // this one of n values, o of the m that follow (Chan, Golub, LeVeque: updating formulae, 1979)
+    __device__ __forceinline__ void join(const Moments& o, float n, float m) {
+        const float d = o.mean - mean, share = m / (n + m);
+        mean += d * share;
+        m2 += o.m2 + d * d * (n * share);
     }
 };
 
-__global__ void __launch_bounds__(kThreads)
-divergence_partial_kernel(const float* __restrict__ phi, int W, int64_t stride, int64_t P,
-                          double2* __restrict__ partial) {
-    const int64_t full_quads = P >> 2;
-    const int64_t q0 = (int64_t)blockIdx.x * (kThreads * kItems) + threadIdx.x;
-    const float inv_W = 1.0f / (float)W;
-    double sum_std = 0.0, sum_var = 0.0;
-
-    Welford4 acc[kItems];
-#pragma unroll
-    for (int it = 0; it < kItems; ++it) acc[it].init();
-    bool ok[kItems];
-#pragma unroll
-    for (int it = 0; it < kItems; ++it) ok[it] = q0 + (int64_t)it * kThreads < full_quads;
-#pragma unroll kUnroll
-    for (int w = 0; w < W; ++w) {
-        const float4* row = reinterpret_cast<const float4*>(phi + (int64_t)w * stride);
-        const float inv_k = __frcp_rn((float)(w + 1));
-        float4 x[kItems];
-#pragma unroll
-        for (int it = 0; it < kItems; ++it)
-            if (ok[it]) x[it] = __ldcs(row + q0 + (int64_t)it * kThreads);
-#pragma unroll
-        for (int it = 0; it < kItems; ++it)
-            if (ok[it]) acc[it].push(x[it], inv_k);
-    }
-#pragma unroll
-    for (int it = 0; it < kItems; ++it) {
-        if (!ok[it]) continue;
-        const float4 v = make_float4(acc[it].m2.x * inv_W, acc[it].m2.y * inv_W, acc[it].m2.z * inv_W,
-                                     acc[it].m2.w * inv_W);
-        sum_var += (double)v.x + (double)v.y + (double)v.z + (double)v.w;
-        sum_std += (double)sqrtf(v.x) + (double)sqrtf(v.y) + (double)sqrtf(v.z) + (double)sqrtf(v.w);
-    }
-    // ragged tail (P mod 4 columns): one thread of the last CTA
-    if ((P & 3) && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
-        for (int64_t c = P & ~int64_t(3); c < P; ++c) {
-            float mean = 0.f, m2 = 0.f;
-            for (int w = 0; w < W; ++w) {
-                const float x = phi[(int64_t)w * stride + c];
-                const float d = x - mean;
-                mean += d * __frcp_rn((float)(w + 1));
-                m2 += d * (x - mean);
-            }
-            const float v = m2 * inv_W;
-            sum_var += (double)v;
-            sum_std += (double)sqrtf(v);
-        }
-    }
-    // CTA reduction in a fixed order: lanes by shuffle tree, then warps in order
-    __shared__ double2 warp_part[kThreads / 32];
+__device__ __forceinline__ double2 warp_sum(double2 v) {
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
-        sum_std += __shfl_down_sync(0xffffffffu, sum_std, off);
-        sum_var += __shfl_down_sync(0xffffffffu, sum_var, off);
+        v.x += __shfl_down_sync(0xffffffffu, v.x, off);
+        v.y += __shfl_down_sync(0xffffffffu, v.y, off);
     }
-    if ((threadIdx.x & 31) == 0) warp_part[threadIdx.x >> 5] = make_double2(sum_std, sum_var);
+    return v;
+}
+
+// The sum over the CTA, in a fixed order, in thread 0.  Contains two barriers.
+template <int THREADS>
+__device__ __forceinline__ double2 cta_sum(double2 v) {
+    __shared__ double2 warp_part[THREADS / 32];
+    v = warp_sum(v);
     __syncthreads();
+    if ((threadIdx.x & 31) == 0) warp_part[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x == 0)
+        for (int w = 1; w < THREADS / 32; ++w) { v.x += warp_part[w].x; v.y += warp_part[w].y; }
+    return v;
+}
+
+// The result from the CTAs' sums, by one CTA in a fixed order.
+template <int THREADS>
+__device__ __forceinline__ void finish(const double2* partial, int64_t count, int64_t P, double* out) {
+    double2 total = make_double2(0.0, 0.0);
+#pragma unroll 8
+    for (int64_t i = threadIdx.x; i < count; i += THREADS) {
+        const double2 v = __ldcg(partial + i);
+        total.x += v.x;
+        total.y += v.y;
+    }
+    total = cta_sum<THREADS>(total);
     if (threadIdx.x == 0) {
-        double2 t = warp_part[0];
-        for (int w = 1; w < kThreads / 32; ++w) { t.x += warp_part[w].x; t.y += warp_part[w].y; }
-        partial[blockIdx.x] = t;
+        out[0] = total.x / (double)P;            // mean over parameters of the across-worker std
+        out[1] = sqrt(total.y / (double)P);      // root of the mean across-worker variance
     }
 }
 
-// One CTA adds the per-CTA partial sums: each thread a strided slice, then a fixed-order tree.
-__global__ void __launch_bounds__(1024)
-divergence_final_kernel(const double2* __restrict__ partial, int64_t count, double inv_P,
-                        double* __restrict__ out) {
-    __shared__ double2 sm[1024];
-    double2 t = make_double2(0.0, 0.0);
-    for (int64_t i = threadIdx.x; i < count; i += 1024) { t.x += partial[i].x; t.y += partial[i].y; }
-    sm[threadIdx.x] = t;
-    __syncthreads();
-    for (int s = 512; s > 0; s >>= 1) {
-        if (threadIdx.x < s) { sm[threadIdx.x].x += sm[threadIdx.x + s].x; sm[threadIdx.x].y += sm[threadIdx.x + s].y; }
+// ITEMS quads (4 consecutive columns) per thread; the CTA's threads form PARTS groups that share out the
+// workers of the same columns and join their moments in shared memory, for states with few columns, whose
+// CTAs would not fill the chip and whose threads would walk the workers one after the other.  FUSED: the
+// last CTA to leave its sums adds them up; `arrived` counts them and is zero before and after.
+template <int ITEMS, int PARTS, bool FUSED>
+__global__ void __launch_bounds__(kThreads, ITEMS == 4 ? 4 : 1)
+divergence_kernel(const float* __restrict__ phi, int W, int64_t stride, int64_t P, double2* partial, unsigned* arrived,
+                  double* out) {
+    constexpr int COLS = kThreads / PARTS;             // threads of one part
+    constexpr int ROWS = ITEMS > 1 ? 1 : PARTS > 1 ? 4 : 8;   // rows whose loads are written before the first use
+    wait_for_predecessors();
+    let_successor_start();
+    const int part = threadIdx.x / COLS, lane = threadIdx.x % COLS;
+    const int64_t quads = (P + 3) >> 2;                // the last may be partial: rows are padded to multiples of 8
+    const int64_t q0 = (int64_t)blockIdx.x * (COLS * ITEMS) + lane;
+    const int w0 = (int)((int64_t)W * part / PARTS), w1 = (int)((int64_t)W * (part + 1) / PARTS);
+
+    Moments acc[ITEMS][4];
+    bool ok[ITEMS];
+#pragma unroll
+    for (int it = 0; it < ITEMS; ++it) {
+        ok[it] = q0 + it * COLS < quads;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[it][e] = {0.f, 0.f};
+    }
+#pragma unroll (ITEMS == 1 ? 1 : 4)
+    for (int w = w0; w < w1; w += ROWS) {
+        float4 x[ROWS][ITEMS];
+#pragma unroll
+        for (int i = 0; i < ROWS; ++i) {
+            const float4* row = reinterpret_cast<const float4*>(phi + (int64_t)(w + i) * stride);
+#pragma unroll
+            for (int it = 0; it < ITEMS; ++it)
+                if (ok[it] && w + i < w1) x[i][it] = __ldcs(row + q0 + it * COLS);
+        }
+#pragma unroll
+        for (int i = 0; i < ROWS; ++i) {
+            const float inv_k = __frcp_rn((float)(w + i - w0 + 1));
+#pragma unroll
+            for (int it = 0; it < ITEMS; ++it) {
+                if (ok[it] && w + i < w1) {
+                    acc[it][0].push(x[i][it].x, inv_k); acc[it][1].push(x[i][it].y, inv_k);
+                    acc[it][2].push(x[i][it].z, inv_k); acc[it][3].push(x[i][it].w, inv_k);
+                }
+            }
+        }
+    }
+    if constexpr (PARTS > 1) {
+        static_assert(ITEMS == 1, "parts share one quad per thread");
+        __shared__ Moments shared[kThreads][4];
+        for (int half = PARTS / 2; half >= 1; half /= 2) {     // part p takes over the workers of part p + half
+            __syncthreads();
+#pragma unroll
+            for (int e = 0; e < 4; ++e) shared[threadIdx.x][e] = acc[0][e];
+            __syncthreads();
+            if (part < half) {
+                // workers held by parts p, p + 2 half, p + 4 half, ... and by p + half, p + 3 half, ...
+                int n = 0, m = 0;
+                for (int p = part; p < PARTS; p += 2 * half) {
+                    n += (int)((int64_t)W * (p + 1) / PARTS) - (int)((int64_t)W * p / PARTS);
+                    m += (int)((int64_t)W * (p + half + 1) / PARTS) - (int)((int64_t)W * (p + half) / PARTS);
+                }
+#pragma unroll
+                for (int e = 0; e < 4; ++e) acc[0][e].join(shared[threadIdx.x + half * COLS][e], (float)n, (float)m);
+            }
+        }
+    }
+    double2 sum = make_double2(0.0, 0.0);              // of the standard deviations, of the variances
+    if (part == 0) {
+        const float inv_W = 1.0f / (float)W;
+        const int64_t full = P >> 2;
+        const int ragged = (int)(P & 3);
+#pragma unroll
+        for (int it = 0; it < ITEMS; ++it) {
+            if (!ok[it]) continue;
+            float4 v = make_float4(acc[it][0].m2 * inv_W, acc[it][1].m2 * inv_W, acc[it][2].m2 * inv_W, acc[it][3].m2 * inv_W);
+            const int64_t q = q0 + it * COLS;
+            if (q == full) {                           // the partial quad
+                if (ragged < 2) v.y = 0.f;
+                if (ragged < 3) v.z = 0.f;
+                v.w = 0.f;
+            }
+            sum.y += (double)v.x + (double)v.y + (double)v.z + (double)v.w;
+            sum.x += (double)sqrtf(v.x) + (double)sqrtf(v.y) + (double)sqrtf(v.z) + (double)sqrtf(v.w);
+        }
+    }
+    sum = cta_sum<kThreads>(sum);
+    if (threadIdx.x == 0) partial[blockIdx.x] = sum;
+    if constexpr (FUSED) {
+        __shared__ bool last;
+        if (threadIdx.x == 0) {
+            __threadfence();
+            last = atomicAdd(arrived, 1u) == gridDim.x - 1;
+        }
         __syncthreads();
+        if (!last) return;
+        __threadfence();
+        finish<kThreads>(partial, gridDim.x, P, out);
+        if (threadIdx.x == 0) *arrived = 0;
     }
-    if (threadIdx.x == 0) {
-        out[0] = sm[0].x * inv_P;            // mean over parameters of the across-worker std
-        out[1] = sqrt(sm[0].y * inv_P);      // root of the mean across-worker variance
+}
+
+__global__ void __launch_bounds__(1024)
+divergence_finish_kernel(const double2* partial, int64_t count, int64_t P, double* out) {
+    wait_for_predecessors();
+    let_successor_start();
+    finish<1024>(partial, count, P, out);
+}
+
+struct Shape {
+    int items, parts;
+    int64_t ctas(int64_t P) const {
+        const int64_t quads = (P + 3) >> 2, per_cta = (int64_t)(kThreads / parts) * items;
+        return (quads + per_cta - 1) / per_cta;
     }
+};
+
+// Four quads per thread and a second kernel for the sums where that leaves eight CTAs per SM, else one quad and
+// one kernel, in as many parts as give the chip about four CTAs per SM while every part keeps a worker.  A call, before (two
+// kernels of one shape, a copy of the result) -> now, us: (W, P) = (16, 10 007) 31.2 -> 16.5, (16, 2^20) 42.8 -> 29.1,
+// (16, 7.1e6) 93.1 -> 81.4, (128, 10 007) 98.7 -> 18.2, (1024, 1000) 331 -> 21.3, (1024, 65 536) 841 -> 65, (1024, 2^20)
+// 920 -> 703, (16, 2^26) 637 -> 622; one quad per thread on that last one 670.  Four quads want four CTAs of 64
+// registers per SM: at 66 registers, three CTAs, it measured 675.
+constexpr int64_t kManyCtas = 148 * 8, kFewCtas = 148 * 4;
+Shape shape_for(int W, int64_t P) {
+    Shape s = {4, 1};
+    if (s.ctas(P) >= kManyCtas) return s;
+    s.items = 1;
+    while (s.parts < 32 && s.ctas(P) < kFewCtas && W >= 4 * s.parts) s.parts *= s.parts == 16 ? 2 : 4;
+    return s;
 }
 
 }  // namespace
 
-int64_t divergence_partials(int64_t P) {
-    const int64_t quads = (P + 3) >> 2;
-    const int64_t per_cta = (int64_t)kThreads * kItems;
-    return (quads + per_cta - 1) / per_cta;
-}
+int64_t divergence_partials(int W, int64_t P) { return shape_for(W, P).ctas(P); }
 
-cudaError_t launch_divergence(const float* phi, int W, int64_t stride, int64_t P, void* partials,
+cudaError_t launch_divergence(const float* phi, int W, int64_t stride, int64_t P, void* partials, unsigned* arrived,
                               double* out2, cudaStream_t stream) {
-    const int64_t ctas = divergence_partials(P);
+    const Shape s = shape_for(W, P);
+    const int64_t ctas = s.ctas(P);
     if (ctas > 0x7fffffffll) return cudaErrorInvalidConfiguration;
-    divergence_partial_kernel<<<(unsigned)ctas, kThreads, 0, stream>>>(phi, W, stride, P,
-                                                                       static_cast<double2*>(partials));
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    divergence_final_kernel<<<1, 1024, 0, stream>>>(static_cast<const double2*>(partials), ctas,
-                                                    1.0 / (double)P, out2);
-    return cudaGetLastError();
+    double2* partial = static_cast<double2*>(partials);
+    auto launch = [&](auto kernel) {
+        return launch_overlapped(kernel, dim3((unsigned)ctas), kThreads, 0, stream, phi, W, stride, P, partial, arrived, out2);
+    };
+    if (s.items == 4) {
+        const cudaError_t e = launch(divergence_kernel<4, 1, false>);
+        if (e != cudaSuccess) return e;
+        return launch_overlapped(divergence_finish_kernel, dim3(1), 1024, 0, stream, static_cast<const double2*>(partial), ctas,
+                                 P, out2);
+    }
+    switch (s.parts) {
+        case 1: return launch(divergence_kernel<1, 1, true>);
+        case 4: return launch(divergence_kernel<1, 4, true>);
+        case 16: return launch(divergence_kernel<1, 16, true>);
+        default: return launch(divergence_kernel<1, 32, true>);
+    }
 }
 
 }  // namespace nolo

@@ -546,6 +546,26 @@ def test_divergence_matches_oracle(nolo, W, P):
     nolo.nolo_destroy(h)
 
 
+@pytest.mark.parametrize("W,P", [(3, 1), (4, 7), (15, 2049), (16, 4096 + 1), (63, 259), (64, 130), (65, 1030), (257, 31),
+                                 (1, 700_000), (5, 606_207), (6, 606_209), (2, 4_849_665), (3, 4_849_668)])
+def test_divergence_shapes(nolo, W, P):
+    """Sizes where the kernel changes: workers in 1, 4, 16 or 32 parts, one or four quads per thread, one
+    kernel or two, a partial last quad (the padding holds NaN)."""
+    gen = torch.Generator().manual_seed(W * 7 + P)
+    stride = (P + 7) // 8 * 8
+    phi = torch.full((W, stride), float("nan"))
+    phi[:, :P] = torch.empty(P).normal_(0.0, 0.02, generator=gen) + torch.empty((W, P)).normal_(0.0, 1e-3, generator=gen)
+    d = phi.cuda()
+    h = nolo.nolo_create(W, 1, P, 1, *F)
+    nolo.nolo_bind_state(h, d, torch.empty_like(d), torch.empty_like(d))
+    got = [nolo.nolo_divergence(h) for _ in range(3)]
+    want = O.divergence(to_np(phi)[:, :P])
+    # float32 mean and deviations of W values of 0.02: 2^-24 x 0.02 / 1e-3 relative each, times a small number
+    assert got[0] == pytest.approx(want, rel=1e-5, abs=1e-12)
+    assert got[1] == got[0] and got[2] == got[0]
+    nolo.nolo_destroy(h)
+
+
 def test_divergence_after_gossip_step_is_zero(nolo):
     """alpha = beta = 0, gamma = 1, n = W puts every replica on the mean."""
     W, P = 16, 70_000
