@@ -174,8 +174,21 @@ int enqueue_outer(nolo_handle* h, int64_t col0, int64_t cols, const Draw* draw, 
     return NOLO_OK;
 }
 
-// Boundaries [b0, b0 + count); in and out begin with boundary b0.
-int enqueue_route(nolo_handle* h, uint64_t seed, uint64_t step, int b0, int count, const void* in, void* out, int backward) {
+int enqueue_route_draw(nolo_handle* h, uint64_t seed, uint64_t step, int b0, int count) {
+    const int drawn = h->per_microbatch ? h->K : 1;
+    NOLO_CUDA(h, nolo::launch_draw_range(seed, step, nolo::kDomainRoute, h->W, b0, count, drawn, h->K, h->d_route,
+                                         h->stream));
+    ++h->launches;
+    return NOLO_OK;
+}
+
+// Boundaries [b0, b0 + count); in and out begin with boundary b0.  part: the elements of every block to copy
+// with the table that is there; NULL for whole blocks and a new table.
+struct Part {
+    int64_t first, count;
+};
+int enqueue_route(nolo_handle* h, uint64_t seed, uint64_t step, int b0, int count, const void* in, void* out, int backward,
+                  const Part* part = nullptr) {
     if (count == 0) return NOLO_OK;
     nolo::RouteArgs a;
     a.in = in; a.out = out; a.table = h->d_route + (size_t)b0 * h->K * h->W;
@@ -183,12 +196,15 @@ int enqueue_route(nolo_handle* h, uint64_t seed, uint64_t step, int b0, int coun
     a.elem_size = elem_size(h->act_dtype);
     a.backward = backward;
     a.seed = seed; a.step = step; a.first_boundary = b0; a.per_microbatch = h->per_microbatch;
-    a.draw = !h->timing && nolo::route_draws(a);       // timed kernels do the same work at every size
-    if (!a.draw) {
-        const int drawn = h->per_microbatch ? h->K : 1;
-        NOLO_CUDA(h, nolo::launch_draw_range(seed, step, nolo::kDomainRoute, h->W, b0, count, drawn, h->K, h->d_route,
-                                             h->stream));
-        ++h->launches;
+    if (part) {
+        a.first_element = part->first;
+        a.elements = part->count;
+    } else {
+        a.draw = !h->timing && nolo::route_draws(a);   // timed kernels do the same work at every size
+        if (!a.draw) {
+            const int rc = enqueue_route_draw(h, seed, step, b0, count);
+            if (rc != NOLO_OK) return rc;
+        }
     }
     Bracket br(h, NOLO_KERNEL_ROUTE);
     NOLO_CUDA(h, nolo::launch_route(a, h->stream));
@@ -196,6 +212,21 @@ int enqueue_route(nolo_handle* h, uint64_t seed, uint64_t step, int b0, int coun
     ++h->launches;
     h->route_valid = true;
     return NOLO_OK;
+}
+
+// Items (columns, elements) per chunk of a transfer through the device of `items` in all, of `bytes` each.  The copy in, the kernel and the copy out of consecutive chunks overlap, so the first
+// copy in and the last copy out are what is not hidden; but a chunk costs about 30 us of host time and the copies
+// of small ones run below the link's rate.  Outer step and routing, ms, in one or two chunks before (335 MB) ->
+// 1/8 of the transfer, 4 to 64 MB, now (1/32 | 1/16): 8 x 7.3 M columns (586 MB each way) 18.56 -> 14.30 (14.26 | 14.18),
+// 8 x 1 M 3.36 -> 2.45 (2.82 | 2.74), 32 x 0.1 M 1.52 -> 1.29 (1.51 | 1.50), 32 x 3 M 90.3 -> 60.6 (60.3 | 62.5); with
+// chunks of 2 MB and less 15.8, 3.5, 1.7.
+int64_t host_chunk(int64_t items, int64_t bytes) {
+    constexpr int64_t kMultiple = 4096;          // rows of at least 8 KB
+    int64_t target = items * bytes / 8;
+    const int64_t least = int64_t(4) << 20, most = int64_t(64) << 20;
+    target = target < least ? least : target > most ? most : target;
+    const int64_t chunk = target / bytes / kMultiple * kMultiple;
+    return chunk < kMultiple ? kMultiple : chunk;
 }
 
 size_t route_bytes(const nolo_handle* h) {
@@ -414,9 +445,7 @@ int nolo_outer_step_host(nolo_handle* h, uint64_t seed, uint64_t step, void* phi
     if (rc != NOLO_OK) return rc;
 
     const int ts = elem_size(h->theta_dtype);
-    // Column chunks of about 128 MB per fp32 tensor, a multiple of 8 columns.
-    int64_t chunk = ((int64_t(32) << 20) / h->W) & ~int64_t(7);
-    if (chunk < 8) chunk = 8;
+    const int64_t chunk = host_chunk(h->P, (int64_t)h->W * (8 + ts));
     // Earlier work on the bound stream may still use the device buffers.
     NOLO_CUDA(h, cudaEventRecord(h->ev_fence, h->stream));
     NOLO_CUDA(h, cudaStreamWaitEvent(h->s_in, h->ev_fence, 0));
@@ -516,10 +545,38 @@ int nolo_route_host(nolo_handle* h, uint64_t seed, uint64_t step, const void* ac
     if (!aligned16(acts_dev)) return fail(h, NOLO_EALIGN, "acts_dev must be 16-byte aligned");
     const size_t bytes = route_bytes(h);
     if (overlap(acts_dev, bytes, h->acts_out, bytes)) return fail(h, NOLO_EINVAL, "acts_dev overlaps acts_out");
-    NOLO_CUDA(h, cudaMemcpyAsync(acts_dev, acts_host, bytes, cudaMemcpyHostToDevice, h->stream));
-    int rc = enqueue_route(h, seed, step, 0, h->stages - 1, acts_dev, h->acts_out, 0);
+    const int64_t es = elem_size(h->act_dtype), blocks = (int64_t)(h->stages - 1) * h->W * h->K;
+    const int64_t chunk = host_chunk(h->E, blocks * es);
+    if (chunk >= h->E) {
+        NOLO_CUDA(h, cudaMemcpyAsync(acts_dev, acts_host, bytes, cudaMemcpyHostToDevice, h->stream));
+        int rc = enqueue_route(h, seed, step, 0, h->stages - 1, acts_dev, h->acts_out, 0);
+        if (rc != NOLO_OK) return rc;
+        NOLO_CUDA(h, cudaMemcpyAsync(out_host, h->acts_out, bytes, cudaMemcpyDeviceToHost, h->stream));
+        NOLO_CUDA(h, cudaStreamSynchronize(h->stream));
+        return NOLO_OK;
+    }
+    int rc = ensure_host_streams(h);
+    if (rc == NOLO_OK) rc = enqueue_route_draw(h, seed, step, 0, h->stages - 1);
     if (rc != NOLO_OK) return rc;
-    NOLO_CUDA(h, cudaMemcpyAsync(out_host, h->acts_out, bytes, cudaMemcpyDeviceToHost, h->stream));
+    // Earlier work on the bound stream may still use the device buffers.
+    NOLO_CUDA(h, cudaEventRecord(h->ev_fence, h->stream));
+    NOLO_CUDA(h, cudaStreamWaitEvent(h->s_in, h->ev_fence, 0));
+    const size_t pitch = (size_t)(h->E * es);
+    for (int64_t e0 = 0; e0 < h->E; e0 += chunk) {
+        const Part part = {e0, h->E - e0 < chunk ? h->E - e0 : chunk};
+        const size_t width = (size_t)(part.count * es), skip = (size_t)(e0 * es);
+        NOLO_CUDA(h, cudaMemcpy2DAsync(static_cast<char*>(acts_dev) + skip, pitch, static_cast<const char*>(acts_host) + skip,
+                                       pitch, width, (size_t)blocks, cudaMemcpyHostToDevice, h->s_in));
+        NOLO_CUDA(h, cudaEventRecord(h->ev_in, h->s_in));
+        NOLO_CUDA(h, cudaStreamWaitEvent(h->stream, h->ev_in, 0));
+        rc = enqueue_route(h, seed, step, 0, h->stages - 1, acts_dev, h->acts_out, 0, &part);
+        if (rc != NOLO_OK) return rc;
+        NOLO_CUDA(h, cudaEventRecord(h->ev_kernel, h->stream));
+        NOLO_CUDA(h, cudaStreamWaitEvent(h->s_out, h->ev_kernel, 0));
+        NOLO_CUDA(h, cudaMemcpy2DAsync(static_cast<char*>(out_host) + skip, pitch, static_cast<const char*>(h->acts_out) + skip,
+                                       pitch, width, (size_t)blocks, cudaMemcpyDeviceToHost, h->s_out));
+    }
+    NOLO_CUDA(h, cudaStreamSynchronize(h->s_out));
     NOLO_CUDA(h, cudaStreamSynchronize(h->stream));
     return NOLO_OK;
 }

@@ -83,6 +83,7 @@ struct RouteArgs {
     bool draw = false;     // the kernel draws the table itself and writes it: see route_draws
     uint64_t seed = 0, step = 0;
     int first_boundary = 0, per_microbatch = 0;
+    int64_t first_element = 0, elements = 0;   // the part of every block to copy; 0 elements = all of it
 };
 
 // Whether launch_route can draw the table itself (a.draw) at these sizes; otherwise it has to be drawn by

@@ -20,7 +20,9 @@ struct CopyArgs {
     unsigned char* out;
     int32_t* table;           // [B][K][R]
     int B, R, K;
-    int64_t bytes;            // of one block
+    int64_t bytes;            // of one block, or of the part of it that is copied
+    int64_t stride;           // bytes between blocks
+    const unsigned char* in_end;
     int backward;
     // kernels that draw the table themselves (DRAW)
     uint64_t seed, step;
@@ -152,12 +154,12 @@ route_copy_kernel(const CopyArgs a) {
             const int r = rk / a.K, k = rk - r * a.K;
             const int peer = peer_of<DRAW>(a, b, r, k);
             const int64_t here = ((int64_t)b * a.R + r) * a.K + k, there = ((int64_t)b * a.R + peer) * a.K + k;
-            const unsigned char* src = a.in + (a.backward ? here : there) * a.bytes;
-            unsigned char* dst = a.out + (a.backward ? there : here) * a.bytes;
+            const unsigned char* src = a.in + (a.backward ? here : there) * a.stride;
+            unsigned char* dst = a.out + (a.backward ? there : here) * a.stride;
             if constexpr (sizeof(V) >= 16)
                 copy_tile<V, THREADS, N>(src, dst, a.bytes);
             else
-                copy_tile_shifted<V, THREADS, N>(src, dst, a.bytes, a.in + (int64_t)a.B * a.R * a.K * a.bytes);
+                copy_tile_shifted<V, THREADS, N>(src, dst, a.bytes, a.in_end);
         }
     }
 }
@@ -228,18 +230,22 @@ cudaError_t launch_shape(const CopyArgs& c, bool draw, cudaStream_t stream) {
 // flight); one 2-byte element per access, as before, 2180.
 cudaError_t launch_route(const RouteArgs& a, cudaStream_t stream) {
     CopyArgs c;
-    c.in = static_cast<const unsigned char*>(a.in);
-    c.out = static_cast<unsigned char*>(a.out);
+    const int64_t skip = a.first_element * a.elem_size;
+    c.in = static_cast<const unsigned char*>(a.in) + skip;
+    c.out = static_cast<unsigned char*>(a.out) + skip;
     c.table = a.table;
     c.B = a.B; c.R = a.R; c.K = a.K;
-    c.bytes = a.E * a.elem_size;
+    c.bytes = (a.elements > 0 ? a.elements : a.E) * a.elem_size;
+    c.stride = a.E * a.elem_size;
+    c.in_end = static_cast<const unsigned char*>(a.in) + (int64_t)a.B * a.R * a.K * c.stride;
     c.backward = a.backward;
     c.seed = a.seed; c.step = a.step;
     c.first_boundary = a.first_boundary; c.per_microbatch = a.per_microbatch;
     if (a.B <= 0 || a.R <= 0 || a.K <= 0 || c.bytes <= 0) return cudaSuccess;
-    const bool wide = c.bytes % 32 == 0 && ((reinterpret_cast<uintptr_t>(a.in) | reinterpret_cast<uintptr_t>(a.out)) & 31) == 0;
+    const int64_t aligned = c.bytes | c.stride | (int64_t)reinterpret_cast<uintptr_t>(c.in) | (int64_t)reinterpret_cast<uintptr_t>(c.out);
+    const bool wide = aligned % 32 == 0;
     if (wide) return a.draw ? launch_shape<Wide, 256, 2>(c, true, stream) : launch_shape<Wide, 384, 1>(c, false, stream);
-    if (c.bytes % 16 == 0) return a.draw ? launch_shape<uint4, 256, 4>(c, true, stream) : launch_shape<uint4, 256, 2>(c, false, stream);
+    if (aligned % 16 == 0) return a.draw ? launch_shape<uint4, 256, 4>(c, true, stream) : launch_shape<uint4, 256, 2>(c, false, stream);
     return a.elem_size == 4 ? launch_shape<uint32_t, 128, 8>(c, a.draw, stream) : launch_shape<uint16_t, 128, 8>(c, a.draw, stream);
 }
 

@@ -514,6 +514,32 @@ def test_route_single_stage_is_a_noop(nolo):
     nolo.nolo_destroy(h)
 
 
+@pytest.mark.parametrize("W,P,E,dt", [(8, 100_003, 70_001, torch.bfloat16), (32, 40_000, 8192 * 3, torch.float32)])
+def test_host_paths_in_several_chunks(nolo, W, P, E, dt):
+    """Transfers above 4 MB go in chunks of 4096 columns (elements) and more, copies and kernel overlapped; the last
+    chunk is shorter.  Twice over, so that a chunk of the second call meets buffers of the first."""
+    S, K = 3, 2
+    dev = [x.cuda() for x in synth.make_state(W, P, 3, dt)]
+    host = [x.cpu().pin_memory() for x in dev]
+    stage = [torch.zeros_like(x) for x in dev]
+    acts = synth.make_acts(S - 1, W, K, E, 5, dt)
+    out, d_out, src = torch.zeros_like(acts).pin_memory(), torch.zeros_like(acts).cuda(), acts.pin_memory()
+    hd, hh = nolo.nolo_create(W, 2, P, S, *F), nolo.nolo_create(W, 2, P, S, *F)
+    nolo.nolo_bind_state(hd, *dev)
+    nolo.nolo_bind_state(hh, *stage)
+    nolo.nolo_bind_route(hh, W * K, E, d_out)
+    for step in range(2):
+        nolo.nolo_outer_step(hd, 1, step)
+        nolo.nolo_outer_step_host(hh, 1, step, *host)
+        nolo.nolo_route_host(hh, 1, step, src, out, torch.empty_like(d_out))
+        for a, b, c in zip(dev, host, stage):
+            assert torch.equal(a[:, :P].cpu(), b[:, :P]) and torch.equal(a[:, :P], c[:, :P])
+        want = O.route_forward(to_np(acts), O.draw_route(1, step, S, W, K))
+        assert np.array_equal(to_np(out), want) and np.array_equal(to_np(d_out), want)
+    nolo.nolo_destroy(hd)
+    nolo.nolo_destroy(hh)
+
+
 def test_route_host_path(nolo):
     S, R, K, E = 3, 4, 2, 4096
     acts = synth.make_acts(S - 1, R, K, E, 8, torch.bfloat16)
