@@ -743,10 +743,11 @@ int nolo_sim_tree_allreduce(int W, double mu, double sigma, int64_t trials, uint
         return NOLO_EINVAL;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     Scratch scratch;
-    cudaError_t e = scratch.take(sizeof(double) * ((size_t)trials + 4));
+    const size_t results = sizeof(double) * (((size_t)trials + 5) & ~size_t(1));
+    cudaError_t e = scratch.take(results + nolo::tree_scratch());
     if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? NOLO_ENOMEM : NOLO_ECUDA;
     double* d = static_cast<double*>(scratch.p);
-    e = nolo::launch_tree_allreduce(W, mu, sigma, trials, seed, d + 4, d, s);
+    e = nolo::launch_tree_allreduce(W, mu, sigma, trials, seed, d + 4, d, static_cast<char*>(scratch.p) + results, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(host_stats, d, 2 * sizeof(double), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess && host_trials)
         e = cudaMemcpyAsync(host_trials, d + 4, sizeof(double) * (size_t)trials, cudaMemcpyDeviceToHost, s);

@@ -44,7 +44,7 @@ template <int THREADS, typename Key>
 __device__ __forceinline__ void rank_by_buckets(unsigned char* raw, int N, Key key, int (&rank)[kDrawPerThread]) {
     static_assert(THREADS >= 32 && (THREADS & (THREADS - 1)) == 0, "whole warps, a power of two");
     constexpr int kMost = kDrawPerThread;
-    constexpr int kShift = 64 - (THREADS == 32 ? 5 : THREADS == 128 ? 7 : THREADS == 512 ? 9 : 10);
+    constexpr int kShift = 64 - (THREADS == 32 ? 5 : THREADS == 128 ? 7 : THREADS == 256 ? 8 : THREADS == 512 ? 9 : 10);
     static_assert((1ull << (64 - kShift)) == THREADS, "one bucket per thread");
     __shared__ uint32_t warp_total[THREADS / 32];
     uint64_t* keys = reinterpret_cast<uint64_t*>(raw);            // [N]

@@ -12,6 +12,7 @@
 #include "nolo.h"
 #include "nolo_draw.cuh"
 #include "nolo_internal.h"
+#include "nolo_launch.cuh"
 #include "nolo_lognormal.cuh"
 #include "nolo_philox.cuh"
 
@@ -28,80 +29,149 @@ constexpr uint64_t kDomainStraggler = 4;
 // ---- tree all-reduce ---------------------------------------------------------------------------
 //
 // A group of threads per trial: `group` = W/2 of them (one Philox block of each direction each) up to 256;
-// a CTA holds kSimThreads / group trials at a time and strides over the trials.  The times of all edges
-// of one direction are made first, by all threads at once, into shared memory, indexed like a binary
-// heap (root 1, children of p are 2p and 2p+1, leaves W .. 2W-1; block q holds those above the nodes 4q ..
-// 4q+3); then the levels are swept.  Bound by issue slots (the log-normal times); the sweeps are chains of
-// a dozen short steps that other trials of the SM fill.  A sweep of the levels that draws its times on
-// the way, one CTA per trial, leaves most threads idle near the root and computes every block twice.  Whole
-// call, before -> now: 20 000 trials of 1024 workers 2.0 -> 0.56 ms, 100 000 of 256 3.4 -> 0.87, 400 000 of 16
-// 4.0 -> 0.54 (0.65 ms of each was the allocation of the result).
+// a CTA holds several trials at a time and strides over the trials.  The times of all edges of one
+// direction are made first, by all threads at once, into shared memory, indexed like a binary heap (root 1,
+// children of p are 2p and 2p+1, leaves W .. 2W-1; block q holds those above the nodes 4q .. 4q+3); then the
+// levels are swept, the upper ones by one warp.  (Subtrees per warp need fewer barriers still, but more
+// instructions on part-filled warps, and measured slower.)  What Philox makes of a block's number is the same
+// for all trials, what it makes of a trial's for all blocks: both are kept (LEAD).  Bound by issue slots
+// (the log-normal times).  Whole call, (W, trials): one CTA per trial that drew the times level by level,
+// two threads for a block -> all times first, a barrier per level -> now, ms: (1024, 20 000) 2.0 -> 0.54 -> 0.52,
+// (256, 100 000) 3.3 -> 0.79 -> 0.74, (16, 400 000) 3.8 -> 0.30 -> 0.22 (0.65 of the first was an allocation).
 
-// Barrier of one trial's threads.  Groups are a power of two: parts of a warp, or whole CTAs' worth of warps.
+constexpr int kTreeThreads = 512;
+// Trials of a CTA whose part of Philox is made at a time: a multiple of those that it has at once.
+__host__ __device__ constexpr int trials_ahead(int per_cta) { return per_cta > 32 ? per_cta : 32; }
+constexpr int kLeadMaxW = 1024;      // 32 KB of shared memory; above, one trial per CTA and no LEAD
+
+// Barrier of the threads of one trial.  Trials of more than a warp share the CTA's barrier: all trials of a CTA
+// take the same steps.  (Named barriers, one per trial, cost CTAs per SM: all 16 of a CTA are set aside.)
 __device__ __forceinline__ void sync_group(int group) {
     if (group <= 32) __syncwarp();
-    else __syncthreads();      // a group of more than a warp is the whole CTA
+    else __syncthreads();
 }
 
-template <bool TAME>
-__global__ void __launch_bounds__(kSimThreads)
+template <bool TAME, bool LEAD>
+__global__ void __launch_bounds__(LEAD ? kTreeThreads : 256, LEAD ? 3 : 5)
 tree_allreduce_kernel(int W, int group, int64_t trials, LogNormal q, uint64_t seed, double* __restrict__ out) {
-    extern __shared__ double nodes[];                 // [trials of the CTA][2W]
+    extern __shared__ double2 dynamic[];
     __shared__ LogNormalTables tables;
-    __shared__ double part[kSimThreads / 32];
-    fill_tables(tables);
-    __syncthreads();
-    const int per_cta = blockDim.x / group, mine = threadIdx.x / group, lane = threadIdx.x % group;
-    double* node = nodes + (size_t)mine * 2 * W;
+    __shared__ double part[kTreeThreads / 32];
     const int blocks = W / 2 > 1 ? W / 2 : 1;         // of four times each, the first two of block 0 above no node
-    for (int64_t first_trial = (int64_t)blockIdx.x * per_cta; first_trial < trials; first_trial += (int64_t)gridDim.x * per_cta) {
+    const int per_cta = blockDim.x / group, mine = threadIdx.x / group, lane = threadIdx.x % group;
+    const int keep = trials_ahead(per_cta);
+    // [direction][block] a, b and c, d; [trial][direction]; then the nodes of each trial of the CTA
+    ulonglong2* lead_ab = reinterpret_cast<ulonglong2*>(dynamic);
+    ulonglong2* lead_cd = lead_ab + (LEAD ? 2 * blocks : 0);
+    PhiloxOfC1* of_trials = reinterpret_cast<PhiloxOfC1*>(lead_cd + (LEAD ? 2 * blocks : 0));
+    fill_tables(tables);
+    if constexpr (LEAD) {
+        for (int i = threadIdx.x; i < 2 * blocks; i += blockDim.x) {
+            const PhiloxOfC0 l = philox_of_c0(i % blocks, i / blocks, kDomainTree, seed, 0);
+            lead_ab[i] = make_ulonglong2(l.a, l.b);
+            lead_cd[i] = make_ulonglong2(l.c, l.d);
+        }
+    }
+    __syncthreads();
+    double* node = reinterpret_cast<double*>(of_trials + (LEAD ? 2 * keep : 0)) + (size_t)mine * 2 * W;
+    const int wide = group > 32 ? 32 : group;         // threads of the warp, or of the part of one, that a trial has
+    int turn = 0;                                     // of the CTA; its trials' part of Philox is made `keep` at a time
+    for (int64_t first_trial = (int64_t)blockIdx.x * per_cta; first_trial < trials;
+         first_trial += (int64_t)gridDim.x * per_cta, ++turn) {
         const int64_t trial = first_trial + mine;
+        const int ahead = turn * per_cta & (keep - 1);
+        if constexpr (LEAD) {
+            if (ahead == 0) {
+                __syncthreads();
+                for (int i = threadIdx.x; i < 2 * keep; i += blockDim.x) {
+                    const int later = i / 2 / per_cta, which = i / 2 % per_cta;
+                    of_trials[i] = philox_of_c1(first_trial + (int64_t)later * gridDim.x * per_cta + which, i & 1, seed);
+                }
+                __syncthreads();
+            }
+        }
         const bool live = trial < trials;             // the threads of other trials only keep the barriers company
-        auto draw = [&](int phase) {
+        auto draw = [&](int direction) {
             if (!live) return;
+            PhiloxOfC1 of_trial;
+            if constexpr (LEAD) of_trial = of_trials[2 * (ahead + mine) + direction];
             for (int b = lane; b < blocks; b += group) {
+                Philox4 x;
+                if constexpr (LEAD) {
+                    const ulonglong2 ab = lead_ab[direction * blocks + b], cd = lead_cd[direction * blocks + b];
+                    x = philox_join({ab.x, ab.y, cd.x, cd.y}, of_trial, seed, 0);
+                } else {
+                    x = philox4x64_10(b, trial, direction, kDomainTree, seed, 0);
+                }
                 double t[4];
-                lognormal4<TAME>(tables, philox4x64_10(b, trial, phase, kDomainTree, seed, 0), q, t);
+                lognormal4<TAME>(tables, x, q, t);
                 double2* to = reinterpret_cast<double2*>(node + 4 * b);
                 to[0] = make_double2(t[0], t[1]);
                 if (4 * b + 2 < 2 * W) to[1] = make_double2(t[2], t[3]);
             }
         };
-        // up: node[c] = time at which c's message has reached its parent
-        draw(0);
-        sync_group(group);
-        for (int first = W >> 1; first >= 2; first >>= 1) {          // parents of one level: first .. 2*first-1
-            for (int i = lane; i < first; i += group) {
+        // up: node[c] = time at which c's message has reached its parent.  The parents of one level are first ..
+        // 2 * first - 1.
+        auto up = [&](int first, int threads) {
+            for (int i = lane; i < first; i += threads) {
                 const double2 c = reinterpret_cast<const double2*>(node)[first + i];
                 node[first + i] += fmax(c.x, c.y);
             }
+        };
+        draw(0);
+        sync_group(group);
+        int first = W >> 1;
+        for (; first > 32; first >>= 1) {
+            up(first, group);
             sync_group(group);
         }
+        if (lane < wide) {
+            for (; first >= 2; first >>= 1) {
+                up(first, wide);
+                __syncwarp();
+            }
+        }
+        sync_group(group);
         const double root = fmax(node[2], node[3]);
         sync_group(group);
-        // down: node[c] = time at which the result has reached c
-        draw(1);
-        sync_group(group);
-        for (int i = lane; i < 2; i += group) node[2 + i] += root;
-        sync_group(group);
-        for (int first = 4; first < 2 * W; first <<= 1) {
-            for (int i = lane; i < first / 2; i += group) {           // sibling pairs
-                double2* c = reinterpret_cast<double2*>(node) + first / 2 + i;
-                const double parent = node[first / 2 + i];
+        // down: node[c] = time at which the result has reached c.  Children in sibling pairs, those of the
+        // parents pairs .. 2 * pairs - 1.
+        auto down = [&](int pairs, int threads) {
+            for (int i = lane; i < pairs; i += threads) {
+                double2* c = reinterpret_cast<double2*>(node) + pairs + i;
+                const double parent = node[pairs + i];
                 *c = make_double2(parent + c->x, parent + c->y);
             }
+        };
+        draw(1);
+        sync_group(group);
+        if (lane < wide) {
+            if (lane == 0) {
+                node[2] += root;
+                node[3] += root;
+            }
+            __syncwarp();
+            for (int pairs = 2; pairs < W && pairs <= 32; pairs <<= 1) {
+                down(pairs, wide);
+                __syncwarp();
+            }
+        }
+        sync_group(group);
+        for (int pairs = 64; pairs < W; pairs <<= 1) {
+            down(pairs, group);
             sync_group(group);
         }
         double m = 0.0;
         for (int leaf = W + lane; leaf < 2 * W; leaf += group) m = fmax(m, node[leaf]);
-        for (int o = (group < 32 ? group : 32) / 2; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+        for (int o = wide / 2; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
         if (group > 32) {
             if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = m;
-            __syncthreads();
-            for (int w = 0; w < group / 32; ++w) m = fmax(m, part[w]);
+            sync_group(group);
+            if (lane == 0)
+                for (int w = 1; w < group / 32; ++w) m = fmax(m, part[(threadIdx.x >> 5) + w]);
         }
         if (live && lane == 0) out[trial] = m;
-        sync_group(group);                            // node[] and part[] are used again
+        sync_group(group);                      // node[] and part[] are used again
     }
 }
 
@@ -212,12 +282,14 @@ __global__ void __launch_bounds__(THREADS)
 straggler_order_kernel(const Slab s) {
     extern __shared__ uint64_t raw[];
     __shared__ double part[THREADS / 32];
+    let_successor_start();          // it waits for this kernel, and this kernel for all before it
     const int64_t row = blockIdx.x;
     const int64_t trial = row / s.iterations, t = row - trial * s.iterations;
     int rank[kDrawPerThread];
     rank_by_buckets<THREADS>(
         reinterpret_cast<unsigned char*>(raw), s.W,
         [&](int i) { return draw_key(i, s.trial0 + trial, 0, kDomainGroups, s.seed, s.t0 + t); }, rank);
+    wait_for_predecessors();
     double m = 0.0;
 #pragma unroll
     for (int k = 0; k < kDrawPerThread; ++k) {
@@ -240,6 +312,8 @@ straggler_order_kernel(const Slab s) {
 __global__ void __launch_bounds__(kSimThreads)
 straggler_order_warp_kernel(const Slab s, int64_t rows) {
     const int64_t row = ((int64_t)blockIdx.x * kSimThreads + threadIdx.x) >> 5;
+    wait_for_predecessors();
+    let_successor_start();
     if (row >= rows) return;
     const int lane = threadIdx.x & 31;
     const int64_t trial = row / s.iterations, t = row - trial * s.iterations;
@@ -254,7 +328,10 @@ straggler_order_warp_kernel(const Slab s, int64_t rows) {
     if (lane == 0) s.longest[row] = m;
 }
 
-// The clocks of one trial per CTA.  `lanes` (a power of two, at most 32 and n) threads share a subgroup.
+// The clocks of one trial per CTA.  `lanes` (a power of two, at most 32 and n) threads share a subgroup.  The
+// work and the partition of an iteration are read AHEAD iterations ahead: an iteration is two short exchanges
+// through shared memory, a read from L2 several times that.
+template <int MOST, int AHEAD>
 __global__ void __launch_bounds__(1024)
 straggler_clock_kernel(const Slab s, int lanes) {
     extern __shared__ uint64_t raw[];
@@ -262,49 +339,54 @@ straggler_clock_kernel(const Slab s, int lanes) {
     uint16_t* order = reinterpret_cast<uint16_t*>(clock + s.W);   // [W]
     const int64_t trial = blockIdx.x;
     const int lane = threadIdx.x % lanes, groups = s.W / s.n;
+    let_successor_start();
     for (int w = threadIdx.x; w < s.W; w += blockDim.x) clock[w] = s.t0 ? s.clock[trial * s.W + w] : 0.0;
     double barrier = s.t0 ? s.out[2 * trial] : 0.0;
-    // the work and the partition of an iteration are read one iteration ahead
-    constexpr int kMost = NOLO_MAX_WORKERS / 1024;
-    double work[kMost], longest;
-    uint16_t position[kMost];
-    auto read = [&](int i) {
+    double work[AHEAD][MOST], longest[AHEAD];
+    uint16_t position[AHEAD][MOST];
+    auto read = [&](int slot, int i) {
+        if (i >= s.iterations) return;
         const int64_t row = trial * s.iterations + i;
 #pragma unroll
-        for (int k = 0; k < kMost; ++k) {
+        for (int k = 0; k < MOST; ++k) {
             const int w = threadIdx.x + k * blockDim.x;
             if (w < s.W) {
-                work[k] = s.work[row * s.W + w];
-                position[k] = s.order[row * s.W + w];
+                work[slot][k] = s.work[row * s.W + w];
+                position[slot][k] = s.order[row * s.W + w];
             }
         }
-        longest = s.longest[row];
+        longest[slot] = s.longest[row];
     };
-    read(0);
-    __syncthreads();
-    for (int i = 0; i < s.iterations; ++i) {
 #pragma unroll
-        for (int k = 0; k < kMost; ++k) {
-            const int w = threadIdx.x + k * blockDim.x;
-            if (w < s.W) {
-                clock[w] += work[k];
-                order[w] = position[k];
+    for (int u = 0; u < AHEAD; ++u) read(u, u);
+    __syncthreads();
+    for (int i0 = 0; i0 < s.iterations; i0 += AHEAD) {
+#pragma unroll
+        for (int u = 0; u < AHEAD; ++u) {
+            if (i0 + u >= s.iterations) break;
+#pragma unroll
+            for (int k = 0; k < MOST; ++k) {
+                const int w = threadIdx.x + k * blockDim.x;
+                if (w < s.W) {
+                    clock[w] += work[u][k];
+                    order[w] = position[u][k];
+                }
             }
+            barrier += longest[u];
+            read(u, i0 + u + AHEAD);
+            __syncthreads();
+            for (int g0 = 0; g0 < groups; g0 += blockDim.x / lanes) {     // every lane of a subgroup takes the same turns
+                const int g = g0 + threadIdx.x / lanes;
+                const uint16_t* member = order + (g < groups ? g : 0) * s.n;
+                double m = 0.0;
+                if (g < groups)
+                    for (int j = lane; j < s.n; j += lanes) m = fmax(m, clock[member[j]]);
+                for (int o = lanes / 2; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+                if (g < groups)
+                    for (int j = lane; j < s.n; j += lanes) clock[member[j]] = m;
+            }
+            __syncthreads();
         }
-        barrier += longest;
-        if (i + 1 < s.iterations) read(i + 1);
-        __syncthreads();
-        for (int g0 = 0; g0 < groups; g0 += blockDim.x / lanes) {     // every lane of a subgroup takes the same turns
-            const int g = g0 + threadIdx.x / lanes;
-            const uint16_t* member = order + (g < groups ? g : 0) * s.n;
-            double m = 0.0;
-            if (g < groups)
-                for (int j = lane; j < s.n; j += lanes) m = fmax(m, clock[member[j]]);
-            for (int o = lanes / 2; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-            if (g < groups)
-                for (int j = lane; j < s.n; j += lanes) clock[member[j]] = m;
-        }
-        __syncthreads();
     }
     double m = 0.0;
     for (int w = threadIdx.x; w < s.W; w += blockDim.x) {
@@ -323,39 +405,81 @@ straggler_clock_kernel(const Slab s, int lanes) {
     }
 }
 
-// Column means of a [rows][cols] array by one CTA, in a fixed order, to out[c]; the standard error
-// of each mean, sqrt(sample variance / rows), to out[cols + c].
-__global__ void __launch_bounds__(1024)
-column_stats_kernel(const double* __restrict__ x, int64_t rows, int cols, double* __restrict__ out) {
-    __shared__ double sm[1024];
-    for (int c = 0; c < cols; ++c) {
-        double s = 0.0;
-        for (int64_t i = threadIdx.x; i < rows; i += 1024) s += x[i * cols + c];
-        sm[threadIdx.x] = s;
-        __syncthreads();
-        for (int k = 512; k > 0; k >>= 1) {
-            if (threadIdx.x < k) sm[threadIdx.x] += sm[threadIdx.x + k];
-            __syncthreads();
+// ---- means and standard errors ------------------------------------------------------------------------
+
+constexpr int kStatsThreads = 512, kStatsCtas = 64;
+
+__device__ __forceinline__ double cta_sum(double v) {          // in a fixed order, to every thread
+    __shared__ double part[kStatsThreads / 32];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    __syncthreads();                                            // part[] may still be read from the call before
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = v;
+    __syncthreads();
+    v = part[0];
+#pragma unroll
+    for (int w = 1; w < kStatsThreads / 32; ++w) v += part[w];
+    return v;
+}
+
+// Sum, and sum of squared deviations from the mean, of each column of rows [r0, r1) of x[][COLS], one slice of
+// the rows per CTA; the slices are put together by the next kernel.  stats[cta][column] = {sum, deviations}.
+template <int COLS>
+__global__ void __launch_bounds__(kStatsThreads)
+column_moments_kernel(const double* __restrict__ x, int64_t rows, double2* __restrict__ moments) {
+    wait_for_predecessors();
+    let_successor_start();
+    const int64_t r0 = rows * blockIdx.x / gridDim.x, r1 = rows * (blockIdx.x + 1) / gridDim.x;
+    double sum[COLS] = {}, dev[COLS] = {};
+#pragma unroll 4
+    for (int64_t i = r0 + threadIdx.x; i < r1; i += kStatsThreads)
+        for (int c = 0; c < COLS; ++c) sum[c] += x[i * COLS + c];
+#pragma unroll
+    for (int c = 0; c < COLS; ++c) sum[c] = cta_sum(sum[c]);
+#pragma unroll 4
+    for (int64_t i = r0 + threadIdx.x; i < r1; i += kStatsThreads) {
+        for (int c = 0; c < COLS; ++c) {
+            const double d = x[i * COLS + c] - sum[c] / (double)(r1 - r0);
+            dev[c] += d * d;
         }
-        const double mean = sm[0] / (double)rows;
-        __syncthreads();
-        double q = 0.0;
-        for (int64_t i = threadIdx.x; i < rows; i += 1024) {
-            const double d = x[i * cols + c] - mean;
-            q += d * d;
-        }
-        sm[threadIdx.x] = q;
-        __syncthreads();
-        for (int k = 512; k > 0; k >>= 1) {
-            if (threadIdx.x < k) sm[threadIdx.x] += sm[threadIdx.x + k];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) {
-            out[c] = mean;
-            out[cols + c] = rows > 1 ? sqrt(sm[0] / (double)(rows - 1) / (double)rows) : 0.0;
-        }
-        __syncthreads();
     }
+#pragma unroll
+    for (int c = 0; c < COLS; ++c) {
+        dev[c] = cta_sum(dev[c]);
+        if (threadIdx.x == 0) moments[blockIdx.x * COLS + c] = make_double2(sum[c], dev[c]);
+    }
+}
+
+// Column means to out[c]; the standard error of each mean, sqrt(sample variance / rows), to out[COLS + c].
+template <int COLS>
+__global__ void __launch_bounds__(32)
+column_stats_kernel(const double2* __restrict__ moments, int slices, int64_t rows, double* __restrict__ out) {
+    wait_for_predecessors();
+    let_successor_start();
+    const int c = threadIdx.x;
+    if (c >= COLS) return;
+    double total = 0.0;
+    for (int k = 0; k < slices; ++k) total += moments[k * COLS + c].x;
+    const double mean = total / (double)rows;
+    double dev = 0.0;
+    for (int k = 0; k < slices; ++k) {
+        const double n = (double)(rows * (k + 1) / slices - rows * k / slices), d = moments[k * COLS + c].x / n - mean;
+        dev += moments[k * COLS + c].y + n * d * d;
+    }
+    out[c] = mean;
+    out[COLS + c] = rows > 1 ? sqrt(dev / (double)(rows - 1) / (double)rows) : 0.0;
+}
+
+template <int COLS>
+cudaError_t launch_stats(const double* x, int64_t rows, double* out, void* scratch, cudaStream_t stream) {
+    const int64_t wanted = rows / 4096;
+    const int slices = (int)(wanted < 1 ? 1 : wanted > kStatsCtas ? kStatsCtas : wanted);
+    double2* moments = static_cast<double2*>(scratch);
+    const cudaError_t e = launch_overlapped(column_moments_kernel<COLS>, dim3((unsigned)slices), kStatsThreads, 0, stream, x,
+                                            rows, moments);
+    if (e != cudaSuccess) return e;
+    return launch_overlapped(column_stats_kernel<COLS>, dim3(1), 32, 0, stream, static_cast<const double2*>(moments), slices, rows,
+                             out);
 }
 
 // Iterations and trials whose work sums are held at a time.
@@ -373,14 +497,19 @@ int64_t slab_iterations(int W, int T, int64_t trials) {
 
 }  // namespace
 
+size_t tree_scratch() { return sizeof(double2) * kStatsCtas; }
+
 cudaError_t launch_tree_allreduce(int W, double mu, double sigma, int64_t trials, uint64_t seed,
-                                  double* per_trial, double* stats, cudaStream_t stream) {
+                                  double* per_trial, double* stats, void* scratch, cudaStream_t stream) {
     const int blocks = W / 2 > 1 ? W / 2 : 1;
-    const int group = blocks < kSimThreads ? blocks : kSimThreads;
-    const int threads = group <= 32 ? kSimThreads : group;
+    const int group = blocks < 256 ? blocks : 256;
+    const bool lead = W <= kLeadMaxW, tame = LogNormal::tame(mu, sigma);
+    const int threads = group <= 128 ? 256 : lead ? 512 : 256;
     const int per_cta = threads / group;
-    const size_t smem = sizeof(double) * 2 * (size_t)W * per_cta;
-    auto kernel = LogNormal::tame(mu, sigma) ? tree_allreduce_kernel<true> : tree_allreduce_kernel<false>;
+    const size_t smem = sizeof(double) * 2 * (size_t)W * per_cta + 
+                        (lead ? sizeof(PhiloxOfC0) * 2 * (size_t)blocks + sizeof(PhiloxOfC1) * 2 * trials_ahead(per_cta) : 0);
+    auto kernel = tame ? (lead ? tree_allreduce_kernel<true, true> : tree_allreduce_kernel<true, false>)
+                       : (lead ? tree_allreduce_kernel<false, true> : tree_allreduce_kernel<false, false>);
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int device = 0, sms = 0, resident = 0;
@@ -393,14 +522,13 @@ cudaError_t launch_tree_allreduce(int W, double mu, double sigma, int64_t trials
                                                                             per_trial);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    column_stats_kernel<<<1, 1024, 0, stream>>>(per_trial, trials, 1, stats);
-    return cudaGetLastError();
+    return launch_stats<1>(per_trial, trials, stats, scratch, stream);
 }
 
 size_t straggler_scratch(int W, int T, int64_t trials) {
     const size_t rows = (size_t)slab_trials(W, trials) * slab_iterations(W, T, trials);
     return rows * W * (sizeof(double) + sizeof(uint16_t)) + rows * sizeof(double) +
-           (size_t)slab_trials(W, trials) * W * sizeof(double) + 64;
+           (size_t)slab_trials(W, trials) * W * sizeof(double) + sizeof(double2) * 2 * kStatsCtas;
 }
 
 cudaError_t launch_straggler(int W, int n, int H, int T, double mu, double sigma, int64_t trials, uint64_t seed,
@@ -435,21 +563,28 @@ cudaError_t launch_straggler(int W, int n, int H, int T, double mu, double sigma
             else
                 (tame ? straggler_split_work_kernel<true>
                       : straggler_split_work_kernel<false>)<<<work_ctas, kSimThreads, 0, stream>>>(s, split, items);
+            cudaError_t e = cudaGetLastError();
+            if (e != cudaSuccess) return e;
             auto order = [&](auto kernel, int order_threads) {
-                kernel<<<(unsigned)rows, order_threads, draw_scratch_bytes(W, order_threads), stream>>>(s);
+                return launch_overlapped(kernel, dim3((unsigned)rows), order_threads, draw_scratch_bytes(W, order_threads), stream, s);
             };
-            if (W <= 32)
-                straggler_order_warp_kernel<<<(unsigned)((rows * 32 + kSimThreads - 1) / kSimThreads), kSimThreads, 0, stream>>>(s, rows);
-            else if (W <= 512) order(straggler_order_kernel<128>, 128);
-            else if (W <= 2048) order(straggler_order_kernel<512>, 512);
-            else order(straggler_order_kernel<1024>, 1024);
-            straggler_clock_kernel<<<(unsigned)s.trials, threads, (size_t)W * 10, stream>>>(s, lanes);
-            const cudaError_t e = cudaGetLastError();
+            e = W <= 32 ? launch_overlapped(straggler_order_warp_kernel, dim3((unsigned)((rows * 32 + kSimThreads - 1) / kSimThreads)),
+                                            kSimThreads, 0, stream, s, rows)
+              : W <= 512  ? order(straggler_order_kernel<128>, 128)
+              : W <= 1024 ? order(straggler_order_kernel<256>, 256)
+              : W <= 2048 ? order(straggler_order_kernel<512>, 512)
+                          : order(straggler_order_kernel<1024>, 1024);
+            if (e != cudaSuccess) return e;
+            // Not ahead of the order kernel's end: CTAs that come in as it leaves crowd on the first free SMs, and these
+            // run for long (1.03 -> 1.16 ms in all for (4, 2, 100, 500, 592)).
+            auto clock = [&](auto kernel) { kernel<<<(unsigned)s.trials, threads, (size_t)W * 10, stream>>>(s, lanes); };
+            if (W <= 1024) clock(straggler_clock_kernel<1, 4>);
+            else clock(straggler_clock_kernel<NOLO_MAX_WORKERS / 1024, 1>);
+            e = cudaGetLastError();
             if (e != cudaSuccess) return e;
         }
     }
-    column_stats_kernel<<<1, 1024, 0, stream>>>(per_trial, trials, 2, stats);
-    return cudaGetLastError();
+    return launch_stats<2>(per_trial, trials, stats, scratch, stream);      // the slabs are done with it
 }
 
 }  // namespace nolo

@@ -73,6 +73,18 @@ def test_straggler_kernel_boundaries(nolo, W, n, H, T, trials):
     np.testing.assert_allclose(per, L.sim_straggler(W, n, H, T, 0.5, 0.9, trials, 12), rtol=RTOL)
 
 
+@pytest.mark.parametrize("trials", [1, 2, 4095, 8191, 8192, 8193, 12_289, 300_001])
+def test_means_and_standard_errors_of_many_trials(nolo, trials):
+    """The rows are summed in slices of 4096 and more, 64 at most; float64 sums of up to 3e5 terms of one sign."""
+    mean, se, per = nolo.nolo_sim_tree_allreduce(2, 0.1, 0.6, trials, 5, return_trials=True)
+    assert mean == pytest.approx(per.mean(), rel=1e-13)
+    assert se == (pytest.approx(per.std(ddof=1) / math.sqrt(trials), rel=1e-11) if trials > 1 else 0.0)
+    b, s, eb, es, per = nolo.nolo_sim_straggler(2, 1, 1, 1, 0.1, 0.6, trials, 5, return_trials=True)
+    assert (b, s) == pytest.approx(tuple(per.mean(0)), rel=1e-13)
+    if trials > 1:
+        assert (eb, es) == pytest.approx(tuple(per.std(0, ddof=1) / math.sqrt(trials)), rel=1e-11)
+
+
 def test_straggler_in_slabs_agrees_with_itself(nolo):
     """2^21 work sums are held at a time.  The first trials of a call that needs several slabs of
     iterations (and of trials) have the times that a call of those trials alone gives."""
