@@ -29,9 +29,20 @@ struct CopyArgs {
     int first_boundary, per_microbatch;
 };
 
+// Asks for the whole 16-byte vectors of this CTA's tile of an input block.
+template <int TILE>
+__device__ __forceinline__ void prefetch_tile(const CopyArgs& a, int64_t block) {
+    const int64_t first = (int64_t)blockIdx.x * TILE, left = a.bytes - first;
+    const uintptr_t from = reinterpret_cast<uintptr_t>(a.in + block * a.stride + first);
+    const uintptr_t lo = (from + 15) & ~uintptr_t(15), hi = (from + (left < TILE ? left : TILE)) & ~uintptr_t(15);
+    prefetch_to_l2(reinterpret_cast<const void*>(lo), (int64_t)(hi - lo));
+}
+
 // The replica of the other side for slot k of replica r at boundary b.  DRAW: drawn by the first warp
-// before the kernels ahead are waited for; one CTA per permutation writes the table.
-template <bool DRAW>
+// before the kernels ahead are waited for; one CTA per permutation writes the table.  The lane that finds the
+// replica has the tile brought to L2 while the kernels ahead end: us for a forward and a backward call, without
+// / with, 17 MB 13.4 / 11.5, 33 MB 25.0 / 21.2 (alone 36.0 / 33.8).
+template <bool DRAW, int TILE>
 __device__ __forceinline__ int peer_of(const CopyArgs& a, int b, int r, int k) {
     int32_t* row = a.table + ((int64_t)b * a.K + k) * a.R;
     if constexpr (!DRAW) {
@@ -41,7 +52,10 @@ __device__ __forceinline__ int peer_of(const CopyArgs& a, int b, int r, int k) {
         int rank = 0;
         if (threadIdx.x < 32) {
             rank = rank_by_warp(a.R, a.first_boundary + b, a.per_microbatch ? k : 0, kDomainRoute, a.seed, a.step);
-            if (rank == r) peer = threadIdx.x;
+            if (rank == r) {
+                peer = threadIdx.x;
+                prefetch_tile<TILE>(a, ((int64_t)b * a.R + (a.backward ? r : (int)threadIdx.x)) * a.K + k);
+            }
         }
         wait_for_predecessors();
         if (r == 0 && blockIdx.x == 0 && (int)threadIdx.x < a.R) row[rank] = threadIdx.x;
@@ -149,10 +163,11 @@ __global__ void __launch_bounds__(THREADS)
 route_copy_kernel(const CopyArgs a) {
     if constexpr (!DRAW) wait_for_predecessors();
     let_successor_start();
+    constexpr int TILE = THREADS * N * (sizeof(V) < 16 ? 16 : (int)sizeof(V));
     for (int b = blockIdx.z; b < a.B; b += gridDim.z) {
         for (int rk = blockIdx.y; rk < a.R * a.K; rk += gridDim.y) {
             const int r = rk / a.K, k = rk - r * a.K;
-            const int peer = peer_of<DRAW>(a, b, r, k);
+            const int peer = peer_of<DRAW, TILE>(a, b, r, k);
             const int64_t here = ((int64_t)b * a.R + r) * a.K + k, there = ((int64_t)b * a.R + peer) * a.K + k;
             const unsigned char* src = a.in + (a.backward ? here : there) * a.stride;
             unsigned char* dst = a.out + (a.backward ? there : here) * a.stride;
@@ -200,13 +215,16 @@ cudaError_t launch_copy_probe(const void* in, void* out, int64_t bytes, cudaStre
     return cudaGetLastError();
 }
 
-// Drawing in the copy saves the launch of the draw and costs every CTA the draw's 0.3 us.  Measured, draw
-// kernel / drawn in the copy, us for a forward and a backward call: 2 MB 12.0 / 7.4, 25 MB 20.7 / 18.7 (22.5 / 22.5 for
-// blocks at odd offsets), 76 MB 50.7 / 49.1 but 51.2 / 55.0 at odd offsets, 100 MB 64.4 / 67.5.
-constexpr int64_t kDrawMaxBytes = 32ll << 20;
+// Drawing in the copy saves the launch of the draw, lets the copy ask for its data ahead of its wait, and costs every
+// CTA the draw's 0.3 us.  Measured, draw kernel / drawn in the copy, us for a forward and a backward call: 2 MB
+// 12.0 / 7.4, 50 MB 35.1 / 30.3, 100 MB 64.1 / 58.8, 134 MB 83.0 / 77.8, 400 MB 236 / 233 (alone 248 / 251); blocks that
+// are no multiple of 32 bytes 96 MB 61.0 / 61.0, 400 MB 237 / 255; at odd offsets 14 MB 17.4 / 15.7, 77 MB 51.8 / 49.0,
+// 115 MB 74.2 / 73.4-75.5 (alone 86 / 88).
+constexpr int64_t kDrawMaxBytes = 64ll << 20, kDrawMaxBytesWide = 128ll << 20;   // the latter for multiples of 32 bytes
 
 bool route_draws(const RouteArgs& a) {
-    return a.R <= 32 && (int64_t)a.B * a.R * a.K * a.E * a.elem_size <= kDrawMaxBytes;
+    const int64_t block = a.E * a.elem_size;
+    return a.R <= 32 && (int64_t)a.B * a.R * a.K * block <= (block % 32 == 0 ? kDrawMaxBytesWide : kDrawMaxBytes);
 }
 
 template <typename V, int THREADS, int N>

@@ -174,10 +174,10 @@ def test_cta_sizes_agree(nolo, n, bf16):
 
 @pytest.mark.parametrize("W,n", [(1, 1), (32, 8), (20, 20), (32, 32), (33, 11)])
 def test_drawn_in_the_step_or_ahead_of_it(nolo, W, n):
-    """Up to 32 workers and 2^23 worker-parameters the step draws its partition itself, else a kernel
+    """Up to 32 workers and 2^25 (n <= 4) or 2^24 worker-parameters the step draws its partition itself, else a kernel
     ahead of it does: the same table and the same bits either way, for steps that follow each other
     closely as well as for steps that are waited for."""
-    P = (1 << 23) // W // 8 * 8 + 8
+    P = (1 << (25 if n <= 4 else 24)) // W // 8 * 8 + 8
     state = [x.cuda() for x in synth.make_state(W, 5000, 3, stride=5008)]
     big = [torch.zeros((W, P), device="cuda") for _ in state]
     for b, x in zip(big, state):
@@ -196,6 +196,32 @@ def test_drawn_in_the_step_or_ahead_of_it(nolo, W, n):
         nolo.nolo_destroy(h)
     for b, x, y in zip(big, state, again):
         assert torch.equal(b[:, :5000], x[:, :5000]) and torch.equal(x[:, :5000], y[:, :5000])
+
+
+@pytest.mark.parametrize("W,n,params", [(2, 2, (1 << 25) - 6), (8, 1, 1 << 23), (16, 4, (1 << 23) + 16 * 77), (12, 3, (1 << 22) + 36),
+                                        (8, 8, (1 << 24) - 8 * 3), (10, 5, (1 << 22) - 10)])
+@pytest.mark.parametrize("bf16", [False, True])
+def test_steps_that_ask_for_data_early(nolo, W, n, params, bf16):
+    """A step that draws its partition may ask for its tiles while the step before still writes them:
+    steps that follow each other closely give the bits of steps whose partition is drawn ahead, and whose
+    kernel asks for nothing before its wait.  Sizes on both sides of each CTA size and of 2^22
+    worker-parameters; ragged ends."""
+    P = params // W
+    torch.manual_seed(3)
+    phi = torch.empty((W, P // 8 * 8 + 8), device="cuda").uniform_(-0.05, 0.05)
+    state = (phi, (phi + 1e-3 * torch.randn_like(phi)).to(torch.bfloat16 if bf16 else torch.float32), 1e-4 * torch.randn_like(phi))
+    other = [x.clone() for x in state]
+    for views, timed in ((state, False), (other, True)):
+        h = nolo.nolo_create(W, n, P, 1, *F)
+        nolo.nolo_bind_state(h, *views)
+        nolo.nolo_timing_enable(h, timed)
+        for step in range(4):
+            nolo.nolo_outer_step(h, 5, step)
+        torch.cuda.synchronize()
+        assert nolo.nolo_launch_count(h) == (8 if timed else 4)
+        nolo.nolo_destroy(h)
+    for x, y in zip(state, other):
+        assert torch.equal(x, y)
 
 
 @pytest.mark.parametrize("hp", [(0.0, 0.0, 1.0), (0.3, 0.7, 0.0), (0.9, 1.0, 1.5), (0.5, 0.7, 0.0)])
