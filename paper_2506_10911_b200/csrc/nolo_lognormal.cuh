@@ -3,12 +3,12 @@
 // Words -> u = ((x >> 11) + 0.5) 2^-53; Box-Muller on the word pairs (0,1) and (2,3), r = sqrt(-2 ln u_a),
 // gives the normals [r01 cos, r01 sin, r23 cos, r23 sin] of the angle 2 pi u_b; t = exp(mu + sigma z).
 //
-// Bound by issue slots.  The logarithm, sine and cosine and exponential are table-driven in the manner of
+// Bound by the pipes of the float64 operations and of Philox's products.  The logarithm, sine and cosine and exponential are table-driven in the manner of
 // P. T. P. Tang (ACM TOMS 15, 1989, "Table-driven implementation of the exponential function in IEEE
 // floating-point arithmetic", and TOMS 16, 1990, for the logarithm): a table in shared memory takes the
 // leading bits, a Taylor polynomial the rest.  The arguments are confined (u in (0, 1], angles as
 // integers, exponents checked once on the host), so no special case is left in the loop, the angle is
-// reduced in integers and the factors 2, pi, sigma and 256 / ln 2 are folded into constants.  About 27
+// reduced in integers and the factors 2, pi, sigma and 256 / ln 2 are folded into constants.  About 23
 // float64 operations per time; each step is good to one or two units in the last place.
 #pragma once
 
@@ -176,35 +176,43 @@ __device__ const double kSinTable[64] = {
 
 constexpr int kSinCosEntries = 256;
 
+// exp(mu + sigma z) = 2^((mu' + sigma' z) / 256)
+struct LogNormal {
+    double mu, sigma;            // as given
+    double mu_scaled;
+    double square;               // sigma'^2, a factor of everything that makes up sigma'^2 (-2 ln u)
+    double log_poly[7];          // of r^1 .. r^7, times it
+
+    __host__ static LogNormal make(double mu, double sigma) {
+        constexpr double k256_over_ln2 = 0x1.71547652b82fep+8;
+        // (a sigma of 0 as one that changes no time but leaves the square root a positive argument)
+        const double scaled = (sigma > 1e-100 ? sigma : 1e-100) * k256_over_ln2, square = scaled * scaled;
+        return {mu, sigma, mu * k256_over_ln2, square,
+                {-2.0 * square, square, -2.0 / 3.0 * square, 0.5 * square, -2.0 / 5.0 * square, 1.0 / 3.0 * square,
+                 -2.0 / 7.0 * square}};
+    }
+    // |z| < 8.7, so exp stays within the normal numbers and the table-driven form applies.
+    __host__ static bool tame(double mu, double sigma) { return fabs(mu) + 8.7 * sigma < 700.0; }
+};
+
 struct LogNormalTables {
-    double2 log[128];                      // c_i, 2 ln c_i
+    double2 log[128];                      // c_i, 2 ln c_i sigma'^2
     double2 sin_cos[kSinCosEntries];       // of 2 pi (j + 1/2) / 256
     double exp2[256];
+    double exponent[56];                   // 2 ln 2 (54 - j) sigma'^2
 };
 
 // Filled by the whole CTA; a barrier has to follow.
-__device__ __forceinline__ void fill_tables(LogNormalTables& t) {
+__device__ __forceinline__ void fill_tables(LogNormalTables& t, const LogNormal& q) {
     for (int i = threadIdx.x; i < 256; i += blockDim.x) {
         t.exp2[i] = kExpTable[i];
-        if (i < 128) t.log[i] = kLogTable[i];
+        if (i < 128) t.log[i] = make_double2(kLogTable[i].x, kLogTable[i].y * q.square);
+        if (i < 56) t.exponent[i] = (54 - i) * 0x1.62e42fefa39efp+0 * q.square;
         const double a = kSinTable[i & 63], b = kSinTable[63 - (i & 63)];
         const double s = i & 64 ? b : a, c = i & 64 ? -a : b;              // second quadrant: cos, -sin
         t.sin_cos[i] = i & 128 ? make_double2(-s, -c) : make_double2(s, c);
     }
 }
-
-// exp(mu + sigma z) = 2^((mu' + sigma' z) / 256)
-struct LogNormal {
-    double mu, sigma;            // as given
-    double mu_scaled, sigma_scaled;
-
-    __host__ static LogNormal make(double mu, double sigma) {
-        constexpr double k256_over_ln2 = 0x1.71547652b82fep+8;
-        return {mu, sigma, mu * k256_over_ln2, sigma * k256_over_ln2};
-    }
-    // |z| < 8.7, so exp stays within the normal numbers and the table-driven form applies.
-    __host__ static bool tame(double mu, double sigma) { return fabs(mu) + 8.7 * sigma < 700.0; }
-};
 
 // 2^(y / 256): y = k + f, |f| <= 1/2, k by adding 1.5 * 2^52.
 __device__ __forceinline__ double exp2_256(const LogNormalTables& t, double y) {
@@ -233,38 +241,36 @@ __device__ __forceinline__ void lognormal2(const LogNormalTables& t, uint64_t wa
         t_sin = exp(q.mu + q.sigma * (r * s));
         return;
     }
-    // -2 ln u, u = v 2^-53 = m 2^e with m in [0.6875, 1.375), m c_i = 1 + r, |r| <= 2^-7.  Near u = 1 both e and
-    // ln c_i vanish and nothing cancels; the 2^-120 kept in their place makes the result positive at u = 1.
+    // sigma'^2 (-2 ln u), u = v 2^-53 = m 2^e with m in [0.6875, 1.375), m c_i = 1 + r, |r| <= 2^-7.  Near u = 1 both e
+    // and ln c_i vanish and nothing cancels; the 2^-120 kept in their place makes the result positive at u = 1.
     const double v = (double)(wa >> 11) + 0.5;
     const int above = __double2hiint(v) - 0x3FE60000;
-    const int e = above >> 20;
+    const int e = above >> 20;                                            // -1 .. 53
     const double m = __hiloint2double(__double2hiint(v) - (e << 20), __double2loint(v));
     const double2 cl = t.log[(above >> 13) & 127];
     const double r = fma(m, cl.x, -1.0);
-    double p = fma(r, -2.0 / 7.0, 1.0 / 3.0);
-    p = fma(p, r, -2.0 / 5.0);
-    p = fma(p, r, 0.5);
-    p = fma(p, r, -2.0 / 3.0);
-    p = fma(p, r, 1.0);
-    const double exponent = __hiloint2double(0x43300000, (e - 53) ^ 0x80000000) - (0x1.0p52 + 0x1.0p31);
-    const double head = fma(exponent, -0x1.62e42fefa39efp+0, cl.y);      // -2 ln2
-    const double x = fma(p, r * r, fma(r, -2.0, head));
-    // sigma' sqrt(x): y = x^-1/2 (1 + O(2^-20)), one step of third order
+    double p = fma(r, q.log_poly[6], q.log_poly[5]);
+    p = fma(p, r, q.log_poly[4]);
+    p = fma(p, r, q.log_poly[3]);
+    p = fma(p, r, q.log_poly[2]);
+    p = fma(p, r, q.log_poly[1]);
+    const double x = fma(p, r * r, fma(r, q.log_poly[0], t.exponent[e + 1] + cl.y));
+    // sqrt(x): y = x^-1/2 (1 + O(2^-20)), one step of third order
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
     const double h = x * y, d = fma(-h, y, 1.0);
-    const double radius = fma(h * d, fma(d, 0.375, 0.5), h) * q.sigma_scaled;
-    // angle: the table entry of the leading 8 bits, turned by the rest (|a| <= pi / 256)
+    const double radius = fma(h * d, fma(d, 0.375, 0.5), h);
+    // angle: the table entry of the leading 8 bits, turned by the rest, a = pi 2^-53 i (|a| <= pi / 256)
     const uint32_t hi = (uint32_t)(wb >> 32), lo = (uint32_t)wb;
-    const double a = (__hiloint2double(0x43300000 | ((hi >> 10) & 0x3FFF), __funnelshift_r(lo, hi, 10) | 1) -
-                      (0x1.0p52 + 0x1.0p45)) *
-                     0x1.921fb54442d18p-52;   // pi 2^-53
+    const double i = __hiloint2double(0x43300000 | ((hi >> 10) & 0x3FFF), __funnelshift_r(lo, hi, 10) | 1) -
+                     (0x1.0p52 + 0x1.0p45);
+    constexpr double k = 0x1.921fb54442d18p-52;   // pi 2^-53
     const double2 sc = t.sin_cos[hi >> 24];
-    const double a2 = a * a;
-    const double sa = fma(a * a2, fma(a2, 1.0 / 120.0, -1.0 / 6.0), a);
-    const double ca = a2 * fma(a2, fma(a2, -1.0 / 720.0, 1.0 / 24.0), -0.5);       // cos a - 1
-    const double s = sc.x + fma(sc.y, sa, sc.x * ca);
-    const double c = sc.y + fma(-sc.x, sa, sc.y * ca);
+    const double i2 = i * i;
+    const double sa = fma(i2, fma(i2, k * k * k * k * k / 120.0, -k * k * k / 6.0), k) * i;
+    const double ca = fma(i2, fma(i2, -k * k * k * k * k * k / 720.0, k * k * k * k / 24.0), -0.5 * k * k) * i2;   // cos a - 1
+    const double s = fma(sc.y, sa, fma(sc.x, ca, sc.x));
+    const double c = fma(-sc.x, sa, fma(sc.y, ca, sc.y));
     t_cos = exp2_256(t, fma(radius, c, q.mu_scaled));
     t_sin = exp2_256(t, fma(radius, s, q.mu_scaled));
 }

@@ -64,7 +64,7 @@ tree_allreduce_kernel(int W, int group, int64_t trials, LogNormal q, uint64_t se
     ulonglong2* lead_ab = reinterpret_cast<ulonglong2*>(dynamic);
     ulonglong2* lead_cd = lead_ab + (LEAD ? 2 * blocks : 0);
     PhiloxOfC1* of_trials = reinterpret_cast<PhiloxOfC1*>(lead_cd + (LEAD ? 2 * blocks : 0));
-    fill_tables(tables);
+    fill_tables(tables, q);
     if constexpr (LEAD) {
         for (int i = threadIdx.x; i < 2 * blocks; i += blockDim.x) {
             const PhiloxOfC0 l = philox_of_c0(i % blocks, i / blocks, kDomainTree, seed, 0);
@@ -183,13 +183,12 @@ tree_allreduce_kernel(int W, int group, int64_t trials, LogNormal q, uint64_t se
 // work of each iteration (one CTA or warp each), and the clocks (one CTA per trial, a few exchanges
 // through shared memory per iteration).  One CTA per trial for everything used as many SMs as there were
 // trials, ranked the keys by O(W^2) comparisons in each iteration, and waited for itself.  Whole call, before ->
-// now, (W, n, H, T, trials): (1024, 2, 100, 250, 148) 39.0 -> 16.8 ms, (1024, 512, 100, 500, 8) 91.7 -> 3.1,
-// (100, 100, 100, 500, 50) 16.9 -> 1.6, (4, 2, 100, 500, 592) 15.7 -> 1.04, (64, 2, 50, 100, 8) 2.3 -> 0.13.
+// now, (W, n, H, T, trials): (1024, 2, 100, 250, 148) 39.0 -> 16.1 ms, (1024, 512, 100, 500, 8) 91.7 -> 3.1,
+// (100, 100, 100, 500, 50) 16.9 -> 1.54, (4, 2, 100, 500, 592) 15.7 -> 0.94, (64, 2, 50, 100, 8) 2.3 -> 0.13.
 struct Slab {
     int W, n, H;
     int iterations;            // of this slab, from t0 on
     int64_t t0, trial0, trials;
-    LogNormal q;
     uint64_t seed;
     double* work;              // [trials][iterations][W]
     uint16_t* order;           // [trials][iterations][W]: the worker in each position of the partition
@@ -200,18 +199,20 @@ struct Slab {
 
 // A thread per item (trial, iteration, worker), for W >= kSharedRowsW.  A CTA's items lie in few rows (trial,
 // iteration), so the part of the Philox rounds that depends on the row and the block only is made once for
-// the CTA, kSharedBlocks blocks at a time.  Bound by issue slots and by the 64-bit products: 15 of them per
-// four times: 215 G times/s in all (W = 1024, H = 100), 170 with all 20 products per block.
+// the CTA, kSharedBlocks blocks at a time.  Bound by the 64-bit products, 15 per four times, and the float64
+// operations, whose pipes are busy 60 and 35 % of the time and measure as one: 2 to 5 CTAs per SM, two blocks in
+// flight per thread or the next block's Philox ahead of this one's times all gave 16.5 to 17.6 ms where this shape
+// gave 16.7, four float64 operations fewer per pair 16.1.  235 G times/s in all (W = 1024, H = 100).
 constexpr int kSharedRowsW = 64;
 constexpr int kSharedRows = (kSimThreads - 2) / kSharedRowsW + 2;
 constexpr int kSharedBlocks = 32;
 
 template <bool TAME>
 __global__ void __launch_bounds__(kSimThreads, 4)
-straggler_work_kernel(const Slab s, int64_t items) {
+straggler_work_kernel(const Slab s, const LogNormal q, int64_t items) {
     __shared__ LogNormalTables tables;
     __shared__ PhiloxOfC0 lead[kSharedRows][kSharedBlocks];
-    fill_tables(tables);
+    fill_tables(tables, q);
     const int64_t item = (int64_t)blockIdx.x * kSimThreads + threadIdx.x;
     const int64_t row0 = (int64_t)blockIdx.x * kSimThreads / s.W;
     const int64_t last = (int64_t)blockIdx.x * kSimThreads + kSimThreads - 1;
@@ -234,12 +235,14 @@ straggler_work_kernel(const Slab s, int64_t items) {
         const int here = blocks - b0 < kSharedBlocks ? blocks - b0 : kSharedBlocks;
         for (int k = 0; k < here; ++k) {                             // inner steps 4 (b0 + k) .. + 3 share a block
             double step[4];
-            lognormal4<TAME>(tables, philox_join(lead[mine][k], of_worker, s.seed, s.trial0 + trial), s.q, step);
+            lognormal4<TAME>(tables, philox_join(lead[mine][k], of_worker, s.seed, s.trial0 + trial), q, step);
             const int left = s.H - 4 * (b0 + k);
             if (left >= 4) {
                 work += (step[0] + step[1]) + (step[2] + step[3]);
             } else {
-                for (int l = 0; l < left; ++l) work += step[l];
+#pragma unroll
+                for (int l = 0; l < 3; ++l)
+                    if (l < left) work += step[l];
             }
         }
     }
@@ -250,9 +253,9 @@ straggler_work_kernel(const Slab s, int64_t items) {
 // items fill the chip too.
 template <bool TAME>
 __global__ void __launch_bounds__(kSimThreads, 4)
-straggler_split_work_kernel(const Slab s, int lanes, int64_t items) {
+straggler_split_work_kernel(const Slab s, const LogNormal q, int lanes, int64_t items) {
     __shared__ LogNormalTables tables;
-    fill_tables(tables);
+    fill_tables(tables, q);
     __syncthreads();
     const int64_t thread = (int64_t)blockIdx.x * kSimThreads + threadIdx.x;
     const int64_t item = thread / lanes;
@@ -264,11 +267,13 @@ straggler_split_work_kernel(const Slab s, int lanes, int64_t items) {
         const int64_t trial = row / s.iterations, t = row - trial * s.iterations;
         for (int k = lane; 4 * k < s.H; k += lanes) {
             double step[4];
-            lognormal4<TAME>(tables, philox4x64_10(k, w, s.t0 + t, kDomainStraggler, s.seed, s.trial0 + trial), s.q, step);
+            lognormal4<TAME>(tables, philox4x64_10(k, w, s.t0 + t, kDomainStraggler, s.seed, s.trial0 + trial), q, step);
             if (4 * k + 4 <= s.H) {
                 work += (step[0] + step[1]) + (step[2] + step[3]);
             } else {
-                for (int l = 0; l < s.H - 4 * k; ++l) work += step[l];
+#pragma unroll
+                for (int l = 0; l < 3; ++l)
+                    if (l < s.H - 4 * k) work += step[l];
             }
         }
     }
@@ -536,7 +541,7 @@ cudaError_t launch_straggler(int W, int n, int H, int T, double mu, double sigma
     const int64_t group = slab_trials(W, trials), iterations = slab_iterations(W, T, trials);
     Slab s;
     s.W = W; s.n = n; s.H = H;
-    s.q = LogNormal::make(mu, sigma);
+    const LogNormal q = LogNormal::make(mu, sigma);
     s.seed = seed;
     s.work = static_cast<double*>(scratch);
     s.clock = s.work + group * iterations * W;
@@ -559,10 +564,10 @@ cudaError_t launch_straggler(int W, int n, int H, int T, double mu, double sigma
             while (items * split < (1 << 18) && split < 32 && 4 * split < H) split *= 2;
             const unsigned work_ctas = (unsigned)((items * split + kSimThreads - 1) / kSimThreads);
             if (split == 1 && W >= kSharedRowsW)
-                (tame ? straggler_work_kernel<true> : straggler_work_kernel<false>)<<<work_ctas, kSimThreads, 0, stream>>>(s, items);
+                (tame ? straggler_work_kernel<true> : straggler_work_kernel<false>)<<<work_ctas, kSimThreads, 0, stream>>>(s, q, items);
             else
                 (tame ? straggler_split_work_kernel<true>
-                      : straggler_split_work_kernel<false>)<<<work_ctas, kSimThreads, 0, stream>>>(s, split, items);
+                      : straggler_split_work_kernel<false>)<<<work_ctas, kSimThreads, 0, stream>>>(s, q, split, items);
             cudaError_t e = cudaGetLastError();
             if (e != cudaSuccess) return e;
             auto order = [&](auto kernel, int order_threads) {
