@@ -65,7 +65,7 @@ WORKLOADS = [
 # of the same kernel (dram__bytes_read.sum + dram__bytes_write.sum over the worker-parameters of
 # the captured launch); traffic grows in proportion to the columns processed.  None = not captured
 # since the kernel last changed.
-PROFILED_DRAM_BYTES_PER_PARAM = {}
+PROFILED_DRAM_BYTES_PER_PARAM = {"outer_step_reg_kernel<2,bf16>": 19.59, "outer_step_reg_kernel<4,float>": 23.15}
 
 
 def bytes_per_param(theta: str) -> int:
@@ -425,7 +425,7 @@ def extra_configs(nolo, dev, peak, copy_gbs, args):
 # square root and sine/cosine pair plus one exponential in float64 per sample; the tree kernel
 # computes every block twice (one thread per sibling pair) and walks the tree.  The bound is
 # SMs x 4 schedulers x 32 lanes x SM clock / that count.
-SIM_THREAD_INSTR_PER_SAMPLE = {"straggler_kernel": 278.0, "tree_allreduce_kernel": 420.0}
+SIM_THREAD_INSTR_PER_SAMPLE = {"straggler_work_kernel": 278.0, "tree_allreduce_kernel": 420.0}
 
 
 def sim_records(nolo):
@@ -441,7 +441,7 @@ def sim_records(nolo):
     sms = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
     slots = sms * 4 * 32 * sm_hz                                  # thread-instructions per second
     out = []
-    cases = [("simulation: straggler barrier (Fig. 5b), W=1024 n=2 H=100 T=250, 592 trials", "straggler_kernel",
+    cases = [("simulation: straggler barrier (Fig. 5b), W=1024 n=2 H=100 T=250, 592 trials", "straggler_work_kernel",
               lambda: nolo.nolo_sim_straggler(1024, 2, 100, 250, 1.0, math.sqrt(0.5), 592, 0), 592 * 1024 * 100 * 250),
              ("simulation: tree all-reduce vs pair exchange (Fig. 5a), W=1024 sigma=1, 100000 trials",
               "tree_allreduce_kernel", lambda: nolo.nolo_sim_tree_allreduce(1024, 0.0, 1.0, 100_000, 0),
@@ -460,7 +460,7 @@ def sim_records(nolo):
                "roofline": {"bound": "alu", "achieved": rate / 1e9, "peak": peak / 1e9, "unit": "G samples/s",
                             "frac": rate / peak, "peak_kind": "issue slots: SMs x 4 schedulers x 32 lanes x SM clock / "
                                                               f"{SIM_THREAD_INSTR_PER_SAMPLE[kernel]:.0f} profiled thread-instructions per sample"}}
-        if kernel == "straggler_kernel":
+        if kernel == "straggler_work_kernel":
             rec["barrier_over_subgroup"] = res[0] / res[1]
         else:
             rec["tree_over_pair"] = res[0] / nolo.nolo_expected_pair_exchange(0.0, 1.0)

@@ -3,13 +3,13 @@
 // Words -> u = ((x >> 11) + 0.5) 2^-53; Box-Muller on the word pairs (0,1) and (2,3), r = sqrt(-2 ln u_a),
 // gives the normals [r01 cos, r01 sin, r23 cos, r23 sin] of the angle 2 pi u_b; t = exp(mu + sigma z).
 //
-// Bound by the pipes of the float64 operations and of Philox's products.  The logarithm, sine and cosine and exponential are table-driven in the manner of
-// P. T. P. Tang (ACM TOMS 15, 1989, "Table-driven implementation of the exponential function in IEEE
-// floating-point arithmetic", and TOMS 16, 1990, for the logarithm): a table in shared memory takes the
-// leading bits, a Taylor polynomial the rest.  The arguments are confined (u in (0, 1], angles as
-// integers, exponents checked once on the host), so no special case is left in the loop, the angle is
-// reduced in integers and the factors 2, pi, sigma and 256 / ln 2 are folded into constants.  About 23
-// float64 operations per time; each step is good to one or two units in the last place.
+// Bound by the pipes of the float64 operations and of Philox's products.  The logarithm, sine and cosine and
+// exponential are table-driven in the manner of P. T. P. Tang (ACM TOMS 15, 1989, "Table-driven implementation of
+// the exponential function in IEEE floating-point arithmetic", and TOMS 16, 1990, for the logarithm): a table in
+// shared memory takes the leading bits, a Taylor polynomial the rest.  The arguments are confined (u in (0, 1],
+// angles as integers, exponents checked once on the host), so no special case is left in the loop, the angle
+// is reduced in integers and the factors 2, pi, sigma and 256 / ln 2 are folded into constants.  About 24 float64
+// operations per time; each step is good to one or two units in the last place.
 #pragma once
 
 #include <stdint.h>
