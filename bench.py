@@ -420,12 +420,11 @@ def extra_configs(nolo, dev, peak, copy_gbs, args):
 
 
 # Issue-slot bound of the simulation kernels.  Thread-instructions per log-normal sample, from a
-# profiler capture of each kernel (warp instructions x 32 / samples): the straggler kernel spends a
-# quarter of a Philox block (ten rounds of two 64 x 64 -> 128-bit products) and half a logarithm,
-# square root and sine/cosine pair plus one exponential in float64 per sample; the tree kernel
-# computes every block twice (one thread per sibling pair) and walks the tree.  The bound is
-# SMs x 4 schedulers x 32 lanes x SM clock / that count.
-SIM_THREAD_INSTR_PER_SAMPLE = {"straggler_work_kernel": 278.0, "tree_allreduce_kernel": 420.0}
+# profiler capture of each kernel (warp instructions x 32 / samples): a quarter of a Philox block (15 of
+# its 20 64 x 64 -> 128-bit products, the rest is shared) and half a table-driven logarithm, square root
+# and sine/cosine pair plus one exponential in float64 per sample; the tree kernel also walks the tree.
+# The bound is SMs x 4 schedulers x 32 lanes x SM clock / that count.
+SIM_THREAD_INSTR_PER_SAMPLE = {"straggler_work_kernel": 95.1, "tree_allreduce_kernel": 130.8}
 
 
 def sim_records(nolo):
