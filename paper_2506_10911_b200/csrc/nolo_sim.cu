@@ -32,12 +32,14 @@ constexpr uint64_t kDomainStraggler = 4;
 // a CTA holds several trials at a time and strides over the trials.  The times of all edges of one
 // direction are made first, by all threads at once, into shared memory, indexed like a binary heap (root 1,
 // children of p are 2p and 2p+1, leaves W .. 2W-1; block q holds those above the nodes 4q .. 4q+3); then the
-// levels are swept, the upper ones by one warp.  (Subtrees per warp need fewer barriers still, but more
+// levels are swept, the upper ones (nodes below 128) by one warp, which alone makes and reads those nodes'
+// times: between the last wide level up and the first wide level down no barrier is needed, and the other warps
+// make the times of the way down meanwhile.  (Subtrees per warp need fewer barriers still, but more
 // instructions on part-filled warps, and measured slower.)  What Philox makes of a block's number is the same
-// for all trials, what it makes of a trial's for all blocks: both are kept (LEAD).  Bound by issue slots
-// (the log-normal times).  Whole call, (W, trials): one CTA per trial that drew the times level by level,
-// two threads for a block -> all times first, a barrier per level -> now, ms: (1024, 20 000) 2.0 -> 0.54 -> 0.52,
-// (256, 100 000) 3.3 -> 0.79 -> 0.74, (16, 400 000) 3.8 -> 0.30 -> 0.22 (0.65 of the first was an allocation).
+// for all trials, what it makes of a trial's for all blocks: both are kept (LEAD).  Bound by the
+// log-normal times and the barriers (root to wide level without any: 0.505 -> 0.492 at W = 1024).  Whole call, (W, trials): one CTA per trial that drew the times level by level,
+// two threads for a block -> all times first, a barrier per level -> now, ms: (1024, 20 000) 2.0 -> 0.54 -> 0.49,
+// (256, 100 000) 3.3 -> 0.79 -> 0.73, (16, 400 000) 3.8 -> 0.30 -> 0.22 (0.65 of the first was an allocation).
 
 constexpr int kTreeThreads = 512;
 // Trials of a CTA whose part of Philox is made at a time: a multiple of those that it has at once.
@@ -131,9 +133,8 @@ tree_allreduce_kernel(int W, int group, int64_t trials, LogNormal q, uint64_t se
                 __syncwarp();
             }
         }
-        sync_group(group);
-        const double root = fmax(node[2], node[3]);
-        sync_group(group);
+        const double root = lane < wide ? fmax(node[2], node[3]) : 0.0;
+        __syncwarp();
         // down: node[c] = time at which the result has reached c.  Children in sibling pairs, those of the
         // parents pairs .. 2 * pairs - 1.
         auto down = [&](int pairs, int threads) {
@@ -144,7 +145,7 @@ tree_allreduce_kernel(int W, int group, int64_t trials, LogNormal q, uint64_t se
             }
         };
         draw(1);
-        sync_group(group);
+        __syncwarp();
         if (lane < wide) {
             if (lane == 0) {
                 node[2] += root;
