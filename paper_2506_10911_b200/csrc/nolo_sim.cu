@@ -36,10 +36,11 @@ constexpr uint64_t kDomainStraggler = 4;
 // times: between the last wide level up and the first wide level down no barrier is needed, and the other warps
 // make the times of the way down meanwhile.  (Subtrees per warp need fewer barriers still, but more
 // instructions on part-filled warps, and measured slower.)  What Philox makes of a block's number is the same
-// for all trials, what it makes of a trial's for all blocks: both are kept (LEAD).  Bound by the
-// log-normal times and the barriers (root to wide level without any: 0.505 -> 0.492 at W = 1024).  Whole call, (W, trials): one CTA per trial that drew the times level by level,
-// two threads for a block -> all times first, a barrier per level -> now, ms: (1024, 20 000) 2.0 -> 0.54 -> 0.49,
-// (256, 100 000) 3.3 -> 0.79 -> 0.73, (16, 400 000) 3.8 -> 0.30 -> 0.22 (0.65 of the first was an allocation).
+// for all trials, what it makes of a trial's for all blocks: both are kept (LEAD).  Bound by the log-normal times
+// and the barriers (0.505 -> 0.492 ms without those around the root, W = 1024).  Whole call, (W, trials): one CTA
+// per trial that drew the times level by level, two threads for a block -> all times first, a barrier per level ->
+// now, ms: (1024, 20 000) 2.0 -> 0.54 -> 0.49, (256, 100 000) 3.3 -> 0.79 -> 0.73, (16, 400 000) 3.8 -> 0.30 -> 0.21
+// (0.65 of the first was an allocation).
 
 constexpr int kTreeThreads = 512;
 // Trials of a CTA whose part of Philox is made at a time: a multiple of those that it has at once.
