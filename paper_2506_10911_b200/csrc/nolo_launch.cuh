@@ -1,11 +1,27 @@
 // Device side of kernels that are launched while their predecessor in the stream still runs.
 #pragma once
 
+#include <stdint.h>
+
 namespace nolo {
 
 // Returns when everything before this kernel in the stream is complete and visible.  Nothing that an
 // earlier kernel writes may be read, and nothing that it reads or writes may be written, before this.
 __device__ __forceinline__ void wait_for_predecessors() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Reads, after the wait, of what an earlier kernel wrote.  Not __ldg (ld.global.nc) and not through const __restrict__
+// pointers: both promise that nothing writes the memory as long as the kernel runs, and the kernel is running
+// while its predecessor still writes.  volatile keeps them behind the wait.
+__device__ __forceinline__ int32_t load_written(const int32_t* p) {
+    int32_t v;
+    asm volatile("ld.global.b32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ double2 load_written(const double2* p) {
+    double2 v;
+    asm volatile("ld.global.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
+    return v;
+}
 
 // Lets the next kernel of the stream be set up once every CTA of this one has got here or has ended.
 // The next kernel's own wait is for the whole of this one; every kernel here waits for its predecessors

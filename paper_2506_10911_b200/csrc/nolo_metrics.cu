@@ -75,7 +75,7 @@ __device__ __forceinline__ void finish(const double2* partial, int64_t count, in
 // last CTA to leave its sums adds them up; `arrived` counts them and is zero before and after.
 template <int ITEMS, int PARTS, bool FUSED>
 __global__ void __launch_bounds__(kThreads, ITEMS == 4 ? 4 : 1)
-divergence_kernel(const float* __restrict__ phi, int W, int64_t stride, int64_t P, double2* partial, unsigned* arrived,
+divergence_kernel(const float* phi, int W, int64_t stride, int64_t P, double2* partial, unsigned* arrived,
                   double* out) {
     constexpr int COLS = kThreads / PARTS;             // threads of one part
     constexpr int ROWS = ITEMS > 1 ? 1 : PARTS > 1 ? 4 : 8;   // rows whose loads are written before the first use

@@ -98,7 +98,7 @@ struct PairSum {
 // The mean of subgroup g for quad q prepared in advance (float64 in memory), split into hi + lo.
 __device__ __forceinline__ PairSum load_prepared_mean(const KArgs& a, int g, int64_t q) {
     const double2* m = reinterpret_cast<const double2*>(a.mean_phi + (int64_t)g * a.mean_stride) + 2 * q;
-    const double2 u = __ldg(m), v = __ldg(m + 1);
+    const double2 u = load_written(m), v = load_written(m + 1);
     PairSum p;
     p.hi = make_float4((float)u.x, (float)u.y, (float)v.x, (float)v.y);
     p.lo = make_float4((float)(u.x - (double)p.hi.x), (float)(u.y - (double)p.hi.y),
@@ -207,12 +207,12 @@ __device__ __forceinline__ void load_means8(double (&m)[8], const double* p) {
     if constexpr (WIDE) {
 #pragma unroll
         for (int i = 0; i < 8; i += 4)
-            asm volatile("ld.global.nc.v4.f64 {%0, %1, %2, %3}, [%4];"
+            asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];"
                          : "=d"(m[i]), "=d"(m[i + 1]), "=d"(m[i + 2]), "=d"(m[i + 3]) : "l"(p + i));
     } else {
 #pragma unroll
         for (int i = 0; i < 8; i += 2) {
-            const double2 x = __ldg(reinterpret_cast<const double2*>(p + i));
+            const double2 x = load_written(reinterpret_cast<const double2*>(p + i));
             m[i] = x.x; m[i + 1] = x.y;
         }
     }
@@ -265,7 +265,7 @@ template <> struct Members<false> {
         wait_for_predecessors();
         let_successor_start();
     }
-    __device__ __forceinline__ int operator[](int j) const { return __ldg(list + j); }
+    __device__ __forceinline__ int operator[](int j) const { return load_written(list + j); }
 };
 template <> struct Members<true> {
     const int* list;                     // shared memory
@@ -619,7 +619,7 @@ __device__ __forceinline__ void store_mean4(double* out, double a, double b, dou
 // quad, so each thread takes two quads up to n = 4.
 template <int ITEMS, bool WIDE>
 __global__ void __launch_bounds__(kThreads)
-group_mean_kernel(const float* __restrict__ phi, const int32_t* __restrict__ perm, int n, int64_t stride,
+group_mean_kernel(const float* phi, const int32_t* perm, int n, int64_t stride,
                   int64_t P, double* __restrict__ mean, int64_t mean_stride, double inv_n) {
     wait_for_predecessors();
     let_successor_start();
@@ -631,7 +631,7 @@ group_mean_kernel(const float* __restrict__ phi, const int32_t* __restrict__ per
         if (c >= P) return;
         double t = 0.0;
 #pragma unroll 4
-        for (int j = threadIdx.x & 31; j < n; j += 32) t += (double)phi[(int64_t)__ldg(members + j) * stride + c];
+        for (int j = threadIdx.x & 31; j < n; j += 32) t += (double)phi[(int64_t)load_written(members + j) * stride + c];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
         if ((threadIdx.x & 31) == 0) mean[(int64_t)g * mean_stride + c] = t * inv_n;
@@ -647,7 +647,7 @@ group_mean_kernel(const float* __restrict__ phi, const int32_t* __restrict__ per
 #pragma unroll
         for (int i = 0; i < kMeanUnroll; ++i) {
             if (j + i < n) {
-                const float4* row = reinterpret_cast<const float4*>(phi + (int64_t)__ldg(members + j + i) * stride);
+                const float4* row = reinterpret_cast<const float4*>(phi + (int64_t)load_written(members + j + i) * stride);
 #pragma unroll
                 for (int it = 0; it < ITEMS; ++it) {
                     const int64_t q = q0 + (int64_t)it * kThreads;

@@ -46,7 +46,7 @@ template <bool DRAW, int TILE>
 __device__ __forceinline__ int peer_of(const CopyArgs& a, int b, int r, int k) {
     int32_t* row = a.table + ((int64_t)b * a.K + k) * a.R;
     if constexpr (!DRAW) {
-        return __ldg(row + r);
+        return load_written(row + r);
     } else {
         __shared__ int peer;
         int rank = 0;
@@ -139,7 +139,7 @@ __device__ __forceinline__ void copy_tile_shifted(const unsigned char* src, unsi
 #pragma unroll
     for (int i = 0; i < N; ++i)
         if (v0 + 32 * i < vecs + second) v[i] = __ldcs(from + v0 + 32 * i);
-    if (lane == 0 && v0 + 32 * N < vecs + second) v[N] = __ldg(from + v0 + 32 * N);
+    if (lane == 0 && v0 + 32 * N < vecs + second) v[N] = __ldcs(from + v0 + 32 * N);
 #pragma unroll
     for (int i = 0; i < N; ++i) {
         const uint4 give = lane == 0 ? v[i + 1] : v[i];
@@ -188,7 +188,7 @@ constexpr int kProbeVecPerThread = 2;
 constexpr int kProbeTileVecs = kProbeThreads * kProbeVecPerThread;
 
 __global__ void __launch_bounds__(kProbeThreads)
-copy_probe_kernel(const uint4* __restrict__ in, uint4* __restrict__ out, int64_t vecs) {
+copy_probe_kernel(const uint4* in, uint4* out, int64_t vecs) {
     const int64_t v0 = (int64_t)blockIdx.x * kProbeTileVecs + threadIdx.x;
     uint4 v[kProbeVecPerThread];
 #pragma unroll

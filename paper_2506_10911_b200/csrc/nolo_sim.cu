@@ -433,7 +433,7 @@ __device__ __forceinline__ double cta_sum(double v) {          // in a fixed ord
 // the rows per CTA; the slices are put together by the next kernel.  stats[cta][column] = {sum, deviations}.
 template <int COLS>
 __global__ void __launch_bounds__(kStatsThreads)
-column_moments_kernel(const double* __restrict__ x, int64_t rows, double2* __restrict__ moments) {
+column_moments_kernel(const double* x, int64_t rows, double2* __restrict__ moments) {
     wait_for_predecessors();
     let_successor_start();
     const int64_t r0 = rows * blockIdx.x / gridDim.x, r1 = rows * (blockIdx.x + 1) / gridDim.x;
@@ -460,7 +460,7 @@ column_moments_kernel(const double* __restrict__ x, int64_t rows, double2* __res
 // Column means to out[c]; the standard error of each mean, sqrt(sample variance / rows), to out[COLS + c].
 template <int COLS>
 __global__ void __launch_bounds__(32)
-column_stats_kernel(const double2* __restrict__ moments, int slices, int64_t rows, double* __restrict__ out) {
+column_stats_kernel(const double2* moments, int slices, int64_t rows, double* __restrict__ out) {
     wait_for_predecessors();
     let_successor_start();
     const int c = threadIdx.x;
