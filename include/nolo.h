@@ -17,6 +17,12 @@
  *   - Calls that enqueue GPU work are asynchronous on the bound stream unless
  *     stated otherwise.  One handle serves one stream at a time and is not
  *     thread-safe.
+ *   - In a stream the calls behave as ordinary kernels and copies do.  A caller's
+ *     kernel that is launched by programmatic stream serialization may start
+ *     before nolo_route*() and nolo_outer_prepare() have written their output,
+ *     and has to execute griddepcontrol.wait before it reads that, as behind any
+ *     kernel that allows it; it does not start before an outer step has written
+ *     the state, nor before anything ahead of the call is done.
  *   - Streams are passed as void* holding a cudaStream_t (NULL = default
  *     stream), so that this header needs no CUDA header.
  *

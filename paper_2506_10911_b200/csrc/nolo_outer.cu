@@ -263,7 +263,6 @@ template <> struct Members<false> {
     __device__ __forceinline__ void init(const KArgs& a, int g, int*) {
         list = a.perm + (int64_t)g * a.n;
         wait_for_predecessors();
-        let_successor_start();
     }
     __device__ __forceinline__ int operator[](int j) const { return load_written(list + j); }
 };
@@ -283,7 +282,6 @@ template <> struct Members<true> {
             if ((int)(blockIdx.y * gridDim.x + blockIdx.x) < EARLY) prefetch<ThetaT, THREADS, COLS>(a);
         }
         wait_for_predecessors();
-        let_successor_start();
         if (blockIdx.x == 0 && g == 0 && (int)threadIdx.x < a.W) a.perm[rank] = threadIdx.x;
         if (!ahead) __syncthreads();
     }

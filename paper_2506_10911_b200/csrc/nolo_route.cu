@@ -58,6 +58,7 @@ __device__ __forceinline__ int peer_of(const CopyArgs& a, int b, int r, int k) {
             }
         }
         wait_for_predecessors();
+        let_successor_start();      // not before: it may count on all that went before this kernel
         if (r == 0 && blockIdx.x == 0 && (int)threadIdx.x < a.R) row[rank] = threadIdx.x;
         __syncthreads();
         const int p = peer;
@@ -161,8 +162,10 @@ __device__ __forceinline__ void copy_tile_shifted(const unsigned char* src, unsi
 template <typename V, int THREADS, int N, bool DRAW>
 __global__ void __launch_bounds__(THREADS)
 route_copy_kernel(const CopyArgs a) {
-    if constexpr (!DRAW) wait_for_predecessors();
-    let_successor_start();
+    if constexpr (!DRAW) {
+        wait_for_predecessors();
+        let_successor_start();
+    }
     constexpr int TILE = THREADS * N * (sizeof(V) < 16 ? 16 : (int)sizeof(V));
     for (int b = blockIdx.z; b < a.B; b += gridDim.z) {
         for (int rk = blockIdx.y; rk < a.R * a.K; rk += gridDim.y) {

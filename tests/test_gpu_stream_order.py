@@ -75,3 +75,65 @@ def test_routes_are_those_of_their_step(nolo, E, pm):
                                 O.draw_route(9, 100 + step, S, R, K, pm))
     assert np.array_equal(to_np(a), want)
     nolo.nolo_destroy(h)
+
+
+FOREIGN = r"""
+#include <cuda_runtime.h>
+// Reads samples of x ahead of its wait, as kernels do with weights.
+__global__ void early_reader(const volatile float* x, long long stride, float* seen) {
+    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    seen[i] = x[i * stride];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+extern "C" int launch_early_reader(const float* x, long long stride, float* seen, int blocks, void* stream) {
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(32);
+    cfg.stream = static_cast<cudaStream_t>(stream);
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, early_reader, (const volatile float*)x, stride, seen);
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def early_reader(tmp_path_factory):
+    import ctypes
+    import subprocess
+    from paper_2506_10911_b200 import build
+    d = tmp_path_factory.mktemp("foreign")
+    (d / "foreign.cu").write_text(FOREIGN)
+    subprocess.run([build.find_nvcc(), *build.NVCC_FLAGS, "-o", str(d / "foreign.so"), str(d / "foreign.cu")], check=True)
+    fn = ctypes.CDLL(str(d / "foreign.so")).launch_early_reader
+    fn.argtypes = [ctypes.c_void_p, ctypes.c_longlong, ctypes.c_void_p, ctypes.c_int, ctypes.c_void_p]
+    return fn
+
+
+@pytest.mark.parametrize("W,n", [(8, 2), (64, 8), (20, 20), (128, 128)])
+@pytest.mark.parametrize("routed", [False, True])
+def test_a_callers_kernel_sees_the_new_weights_ahead_of_its_wait(nolo, early_reader, W, n, routed):
+    """Also with a routing call between the step and the caller's kernel."""
+    P, blocks = (1 << 25) // W // 8 * 8, 64
+    phi = torch.empty((W, P), device="cuda").uniform_(-0.05, 0.05)
+    theta = torch.full_like(phi, 7.0)                       # fast weights far from anything a step leaves
+    h = nolo.nolo_create(W, n, P, 2, *F)
+    nolo.nolo_bind_state(h, phi, theta, torch.zeros_like(phi))
+    acts = torch.zeros((1, W, 1, 1 << 12), device="cuda")
+    out = torch.zeros_like(acts)
+    nolo.nolo_bind_route(h, W, 1 << 12, out)
+    stride = W * P // (blocks * 32)
+    stream = torch.cuda.current_stream().cuda_stream
+    for step in range(4):
+        theta.fill_(7.0)
+        seen = torch.empty(blocks * 32, device="cuda")
+        nolo.nolo_outer_step(h, 1, step)
+        if routed:
+            nolo.nolo_route(h, 1, step, acts)
+        assert early_reader(theta.data_ptr(), stride, seen.data_ptr(), blocks, stream) == 0
+        assert torch.equal(seen, theta.view(-1)[::stride][:blocks * 32])
+        assert not bool((seen == 7.0).any())
+    nolo.nolo_destroy(h)
