@@ -43,7 +43,6 @@ struct KArgs {
     int32_t* perm;
     uint64_t seed, step;      // kernels that draw the partition themselves (DRAW)
     int W;
-    int prefetch;             // 1 when their first CTAs ask for phi and theta ahead of the wait
     const double* mean_phi;   // subgroup means of phi prepared in advance, [groups][mean_stride]; or NULL
     int64_t mean_stride;
     int64_t stride;
@@ -250,16 +249,12 @@ __device__ __forceinline__ void update_store(const KArgs& a, int64_t row_off, in
 // DRAW = false: read from the table.  DRAW = true (at most 32 workers): the first warp of every CTA draws
 // the partition, before it waits for the kernels ahead of it, and keeps its subgroup's members in
 // shared memory; the first CTA writes the table as well.  Both wait for the kernels ahead of this one.
-// EARLY: CTAs that may be resident while the kernel ahead ends.  They have phi and theta of their tile brought to
-// L2 meanwhile, which DRAM does while that kernel's last CTAs leave it idle.  us per step, without / with, steps
-// that follow each other (alone in brackets): W = 4, P = 2^20, n = 2 16.8 / 15.9 (28.0 / 28.0), n = 8
-// 33.3 / 32.5 (44.1 / 44.5); behind a routing copy 21.5 / 19.6.  With delta as well a CTA alone loses what it
-// gains.  Below 2^22 worker-parameters the state may well be in L2 (n = 8, 2^21: 7.4 / 7.7), and in the two-pass
-// kernel the requests for all rows cost as much as they give (n = 20, P = 800001 65.9 / 66.5).
+// (Having phi and theta of the first tiles brought to L2 ahead of the wait measured no gain since the kernel ahead is
+// mostly done by then: 61.0 us with, 60.5 without for steps that follow each other, W = 4, P = 2^22, n = 2; 63.6 / 63.9
+// behind a routing copy.)
 template <bool DRAW> struct Members;
 template <> struct Members<false> {
     const int32_t* list;
-    template <typename ThetaT, int THREADS, int COLS, int EARLY>
     __device__ __forceinline__ void init(const KArgs& a, int g, int*) {
         list = a.perm + (int64_t)g * a.n;
         wait_for_predecessors();
@@ -268,7 +263,6 @@ template <> struct Members<false> {
 };
 template <> struct Members<true> {
     const int* list;                     // shared memory
-    template <typename ThetaT, int THREADS, int COLS, int EARLY>
     __device__ __forceinline__ void init(const KArgs& a, int g, int* shared) {
         list = shared;
         int rank = 0;
@@ -276,29 +270,9 @@ template <> struct Members<true> {
             rank = rank_by_warp(a.W, 0, 0, kDomainGroups, a.seed, a.step);
             if ((int)threadIdx.x < a.W && rank / a.n == g) shared[rank - g * a.n] = threadIdx.x;
         }
-        const bool ahead = EARLY > 0 && a.prefetch;
-        if (ahead) {          // (a barrier on this side for every kernel costs small states up to 0.4 us)
-            __syncthreads();
-            if ((int)(blockIdx.y * gridDim.x + blockIdx.x) < EARLY) prefetch<ThetaT, THREADS, COLS>(a);
-        }
         wait_for_predecessors();
         if (blockIdx.x == 0 && g == 0 && (int)threadIdx.x < a.W) a.perm[rank] = threadIdx.x;
-        if (!ahead) __syncthreads();
-    }
-    // One line of the members' phi or theta per thread and turn.
-    template <typename ThetaT, int THREADS, int COLS>
-    __device__ __forceinline__ void prefetch(const KArgs& a) const {
-        constexpr int kPhi = 128 / sizeof(float), kTheta = 128 / sizeof(ThetaT);              // columns of a line
-        constexpr int kPhiLines = COLS / kPhi, kLines = kPhiLines + COLS / kTheta;
-        const int64_t c0 = (int64_t)((int)blockIdx.x - a.tail) * COLS;
-        if (c0 < 0) return;
-        for (int i = threadIdx.x; i < a.n * kLines; i += THREADS) {
-            const int j = i / kLines, l = i % kLines;
-            const int64_t c = c0 + (l < kPhiLines ? l * kPhi : (l - kPhiLines) * kTheta);
-            const int64_t at = (int64_t)list[j] * a.stride + c;
-            if (c < a.P)
-                prefetch_to_l2(l < kPhiLines ? (const void*)(a.phi + at) : (const void*)(static_cast<const ThetaT*>(a.theta) + at));
-        }
+        __syncthreads();
     }
     __device__ __forceinline__ int operator[](int j) const { return list[j]; }
 };
@@ -376,15 +350,13 @@ __device__ __forceinline__ void ragged_tail(const KArgs& a, int g, const M& memb
 // 6850, n = 4 6770 / 6737 -> 6862 / 6800, n = 6 6521 / 6670 -> 6831 / 6695, n = 7 6673 / 6378 -> 6834 / 6740, n = 8
 // 6711 / 5568 -> 6828 / 6739; with prepared means n = 2 5988 / 6830 -> 6985 / 6976, n = 4 6655 -> 6890 (float32).
 // (The quad kernel with n = 7 and 8 left one CTA of 256 threads per SM.)
-template <int N, int THREADS>
-constexpr int kRegResident = 148 * (65536 / (THREADS * (24 * N + 30)));     // CTAs, by the registers a thread takes
 template <int N, typename ThetaT, int THREADS, bool PREPARED, bool WIDE, bool DRAW>
 __global__ void __launch_bounds__(THREADS, 1)
 outer_step_reg_kernel(const KArgs a) {
     const int g = blockIdx.y;
     __shared__ int drawn[DRAW ? N : 1];
     Members<DRAW> members;
-    members.template init<ThetaT, THREADS, THREADS * 8, kRegResident<N, THREADS>>(a, g, drawn);
+    members.init(a, g, drawn);
     if (a.tail && blockIdx.x == 0) {
         ragged_tail<ThetaT, THREADS, 8>(a, g, members);
         return;
@@ -490,7 +462,7 @@ outer_step_twopass_kernel(const KArgs a) {
     const int n = a.n;
     __shared__ int drawn[DRAW ? 32 : 1];
     Members<DRAW> members;
-    members.template init<ThetaT, THREADS, ROWQ * 4, 0>(a, g, drawn);
+    members.init(a, g, drawn);
     if (a.tail && blockIdx.x == 0) {
         ragged_tail<ThetaT, THREADS, 4>(a, g, members);
         return;
@@ -795,7 +767,6 @@ cudaError_t launch_group_mean(const float* phi, const int32_t* perm, int W, int 
 // theta), 52.0 / 51.5 (n = 12), 66.5 / 65.9 (n = 20), 2^25 121.5 / 119.4 (n = 4); 2^26 236.1 / 234-237 and, alone,
 // 248 / 250 (n = 2), 240.5 / 241.0 and 252 / 256 (n = 8).
 constexpr int64_t kDrawMaxParams = 1 << 25, kDrawMaxParamsWide = 1 << 24;   // worker-parameters; n <= 4 and above
-constexpr int64_t kPrefetchParams = 1 << 22;
 
 bool outer_draws(const OuterArgs& a) {
     return a.W <= 32 && a.P * a.W <= (a.n <= 4 ? kDrawMaxParams : kDrawMaxParamsWide);
@@ -806,7 +777,6 @@ cudaError_t launch_outer(const OuterArgs& a, cudaStream_t stream) {
     KArgs k;
     k.phi = a.phi; k.theta = a.theta; k.delta = a.delta; k.perm = a.perm;
     k.seed = a.seed; k.step = a.step; k.W = a.W;
-    k.prefetch = a.P * a.W >= kPrefetchParams;
     k.mean_phi = a.mean_phi; k.mean_stride = a.mean_stride;
     k.stride = a.stride; k.P = a.P; k.n = a.n;
     k.alpha = a.alpha; k.gamma = a.gamma;
