@@ -10,6 +10,7 @@
 #include "nolo_draw.cuh"
 #include "nolo_internal.h"
 #include "nolo_launch.cuh"
+#include "nolo_shifted.h"
 
 namespace nolo {
 
@@ -101,8 +102,6 @@ __device__ __forceinline__ void copy_tile(const unsigned char* src, unsigned cha
     }
 }
 
-constexpr int kLine = 128;
-
 // Bytes s .. s+15 of two neighbouring 16-byte vectors.
 __device__ __forceinline__ uint4 shifted(const uint4& x, const uint4& y, int s) {
     const uint32_t w[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
@@ -116,31 +115,23 @@ __device__ __forceinline__ uint4 shifted(const uint4& x, const uint4& y, int s) 
 }
 
 // The same for blocks of elements T that begin anywhere (at a multiple of sizeof(T)), the source at
-// another offset from a 16-byte boundary than the destination: 16-byte vectors of the destination, from its
-// first 128-byte line on, so that no two warps share one, are each put together from the two aligned source
-// vectors they straddle.  A warp has N x 32 consecutive vectors, so that the second one comes from the next lane
-// by shuffle (holding both in registers measured 10-20 % slower: fewer bytes in flight); the bytes before
-// the first and after the last vector go one T at a time.  No access leaves the buffers: a vector that
-// would need a source vector reaching beyond in_end is left to the elements.
+// another offset from a 16-byte boundary than the destination: each 16-byte vector of the destination is put
+// together from the two aligned source vectors it straddles (see ShiftedSpan).  A warp has N x 32 consecutive vectors,
+// so that the second one comes from the next lane by shuffle (holding both in registers measured 10-20 % slower:
+// fewer bytes in flight).
 template <typename T, int THREADS, int N>
 __device__ __forceinline__ void copy_tile_shifted(const unsigned char* src, unsigned char* dst, int64_t bytes,
                                                   const unsigned char* in_end) {
     static_assert(THREADS * sizeof(T) >= kLine + 32, "one element per thread at the ends");
-    int64_t head = (kLine - (reinterpret_cast<uintptr_t>(dst) & (kLine - 1))) & (kLine - 1);
-    if (head > bytes) head = bytes;
-    const int shift = (int)(reinterpret_cast<uintptr_t>(src + head) & 15);
-    const uint4* from = reinterpret_cast<const uint4*>(src + head - shift);
-    const int second = shift != 0;
-    const int64_t inside = (in_end - reinterpret_cast<const unsigned char*>(from)) / 16 - second;
-    int64_t vecs = (bytes - head) / 16;
-    if (vecs > inside) vecs = inside > 0 ? inside : 0;        // one less, at the end of the whole input
+    const ShiftedSpan p = shifted_span(src, dst, bytes, in_end);
+    const uint4* from = reinterpret_cast<const uint4*>(p.from);
     const int lane = threadIdx.x & 31;
     const int64_t v0 = ((int64_t)blockIdx.x * (THREADS / 32) + (threadIdx.x >> 5)) * (32 * N) + lane;
     uint4 v[N + 1];
 #pragma unroll
     for (int i = 0; i < N; ++i)
-        if (v0 + 32 * i < vecs + second) v[i] = __ldcs(from + v0 + 32 * i);
-    if (lane == 0 && v0 + 32 * N < vecs + second) v[N] = __ldcs(from + v0 + 32 * N);
+        if (v0 + 32 * i < p.loads) v[i] = __ldcs(from + v0 + 32 * i);
+    if (lane == 0 && v0 + 32 * N < p.loads) v[N] = __ldcs(from + v0 + 32 * N);
 #pragma unroll
     for (int i = 0; i < N; ++i) {
         const uint4 give = lane == 0 ? v[i + 1] : v[i];
@@ -149,12 +140,12 @@ __device__ __forceinline__ void copy_tile_shifted(const unsigned char* src, unsi
         next.y = __shfl_sync(0xffffffffu, give.y, (lane + 1) & 31);
         next.z = __shfl_sync(0xffffffffu, give.z, (lane + 1) & 31);
         next.w = __shfl_sync(0xffffffffu, give.w, (lane + 1) & 31);
-        if (v0 + 32 * i < vecs) __stcs(reinterpret_cast<uint4*>(dst + head) + v0 + 32 * i, shifted(v[i], next, shift));
+        if (v0 + 32 * i < p.vecs) __stcs(reinterpret_cast<uint4*>(dst + p.head) + v0 + 32 * i, shifted(v[i], next, p.shift));
     }
     if (blockIdx.x == 0 && threadIdx.x < (kLine + 32) / sizeof(T)) {
         const int e = threadIdx.x * sizeof(T);
-        const int64_t at = e < kLine ? e : head + 16 * vecs + (e - kLine);
-        if (e < kLine ? at < head : at < bytes) *reinterpret_cast<T*>(dst + at) = *reinterpret_cast<const T*>(src + at);
+        const int64_t at = e < kLine ? e : p.head + 16 * p.vecs + (e - kLine);
+        if (e < kLine ? at < p.head : at < bytes) *reinterpret_cast<T*>(dst + at) = *reinterpret_cast<const T*>(src + at);
     }
 }
 

@@ -1,4 +1,7 @@
-"""Shared test helpers: tolerance checks and tensor <-> numpy conversion."""
+"""Shared test helpers: tolerance checks, tensor <-> numpy conversion, host code of the library compiled alone."""
+
+import os
+import subprocess
 
 import numpy as np
 import torch
@@ -84,3 +87,18 @@ def assert_outer_step_parity(got_phi, got_delta, got_theta, want, bf16: bool, wh
         assert_bf16_within_1ulp(got_theta, want[2], f"{what}theta(bf16)", carried=want[1])
     else:
         assert_close_f32(got_theta, want[2], f"{what}theta", carried=want[1])
+
+
+def run_host_code(tmp_path, source: str) -> str:
+    """Compile a C++ program that includes headers of the library's csrc with the host compiler, run it, return
+    its output; a failed check in it is a failed test."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    src, exe = tmp_path / "check.cpp", tmp_path / "check"
+    src.write_text(source)
+    res = subprocess.run(["g++", "-std=c++17", "-O1", "-fsanitize=undefined", "-fno-sanitize-recover=all", "-pthread",
+                          "-I", os.path.join(root, "paper_2506_10911_b200", "csrc"), "-o", str(exe), str(src)],
+                         capture_output=True, text=True)
+    assert res.returncode == 0, res.stderr
+    res = subprocess.run([str(exe)], capture_output=True, text=True, timeout=300)
+    assert res.returncode == 0, res.stdout + res.stderr
+    return res.stdout
