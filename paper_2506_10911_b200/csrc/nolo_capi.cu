@@ -547,7 +547,10 @@ int nolo_route_host(nolo_handle* h, uint64_t seed, uint64_t step, const void* ac
     if (overlap(acts_dev, bytes, h->acts_out, bytes)) return fail(h, NOLO_EINVAL, "acts_dev overlaps acts_out");
     const int64_t es = elem_size(h->act_dtype), blocks = (int64_t)(h->stages - 1) * h->W * h->K;
     const int64_t chunk = host_chunk(h->E, blocks * es);
-    if (chunk >= h->E) {
+    // Chunks of the result come back while later chunks of the input are read: not where they would land on them.
+    const bool in_place = acts_host == out_host;      // every chunk comes back to where it was read
+    const bool crossed = !in_place && overlap(acts_host, bytes, out_host, bytes);
+    if (chunk >= h->E || crossed) {
         NOLO_CUDA(h, cudaMemcpyAsync(acts_dev, acts_host, bytes, cudaMemcpyHostToDevice, h->stream));
         int rc = enqueue_route(h, seed, step, 0, h->stages - 1, acts_dev, h->acts_out, 0);
         if (rc != NOLO_OK) return rc;

@@ -566,6 +566,24 @@ def test_host_paths_in_several_chunks(nolo, W, P, E, dt):
     nolo.nolo_destroy(hh)
 
 
+@pytest.mark.parametrize("shift", [0, 1, 7, 8 * 600_000])
+def test_route_host_path_with_overlapping_host_buffers(nolo, shift):
+    """The whole input is read before a byte of the result lands on it: host buffers may overlap, at any offset."""
+    S, R, K, E = 2, 4, 2, 600_000                       # in several chunks where the buffers are apart
+    n = (S - 1) * R * K * E
+    for forwards in (True, False):
+        buf = torch.empty(n + shift).uniform_(-1, 1).pin_memory()
+        a, b = buf[:n], buf[shift:shift + n]
+        src, dst = (a, b) if forwards else (b, a)
+        want = O.route_forward(to_np(src).copy().reshape(S - 1, R, K, E), O.draw_route(4, 2, S, R, K))
+        d_in, d_out = torch.empty(n, device="cuda"), torch.empty((S - 1, R, K, E), device="cuda")
+        h = nolo.nolo_create(R, 1, 8, S, *F)
+        nolo.nolo_bind_route(h, R * K, E, d_out)
+        nolo.nolo_route_host(h, 4, 2, src, dst, d_in)
+        assert np.array_equal(to_np(dst).reshape(want.shape), want)
+        nolo.nolo_destroy(h)
+
+
 def test_route_host_path(nolo):
     S, R, K, E = 3, 4, 2, 4096
     acts = synth.make_acts(S - 1, R, K, E, 8, torch.bfloat16)
