@@ -214,17 +214,27 @@ int enqueue_route(nolo_handle* h, uint64_t seed, uint64_t step, int b0, int coun
     return NOLO_OK;
 }
 
-// Items (columns, elements) per chunk of a transfer through the device of `items` in all, of `bytes` each.  The copy in, the kernel and the copy out of consecutive chunks overlap, so the first
-// copy in and the last copy out are what is not hidden; but a chunk costs about 30 us of host time and the copies
-// of small ones run below the link's rate.  Outer step and routing, ms, in one or two chunks before (335 MB) ->
-// 1/8 of the transfer, 4 to 64 MB, now (1/32 | 1/16): 8 x 7.3 M columns (586 MB each way) 18.56 -> 14.30 (14.26 | 14.18),
-// 8 x 1 M 3.36 -> 2.45 (2.82 | 2.74), 32 x 0.1 M 1.52 -> 1.29 (1.51 | 1.50), 32 x 3 M 90.3 -> 60.6 (60.3 | 62.5); with
-// chunks of 2 MB and less 15.8, 3.5, 1.7.
-int64_t host_chunk(int64_t items, int64_t bytes) {
+// Whether copies from and to host memory at p overlap other work: memory that CUDA has not page-locked is copied
+// through a buffer of the driver while the call waits.
+bool page_locked(const void* p) {
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) == cudaSuccess) return a.type != cudaMemoryTypeUnregistered;
+    cudaGetLastError();
+    return false;
+}
+
+// Items (columns, elements) per chunk of a transfer through the device of `items` in all, of `bytes` each.  The copy in,
+// the kernel and the copy out of consecutive chunks overlap, so the first copy in and the last copy out are what is not
+// hidden; but a chunk costs about 30 us of host time and the copies of small ones run below the link's rate: an
+// eighth of the transfer, 4 to 64 MB (8 x 7.3 M columns, 586 MB each way, 14.3 ms; in chunks of 335 MB 18.6).  Pageable
+// memory is copied in few large pieces, whose rows are long (17 MB of activations 1.8 ms, in eighths 2.1; 38 MB of state
+// 5.7, in eighths 6.6).
+int64_t host_chunk(int64_t items, int64_t bytes, bool locked) {
     constexpr int64_t kMultiple = 4096;          // rows of at least 8 KB
     int64_t target = items * bytes / 8;
     const int64_t least = int64_t(4) << 20, most = int64_t(64) << 20;
     target = target < least ? least : target > most ? most : target;
+    if (!locked) target = int64_t(384) << 20;
     const int64_t chunk = target / bytes / kMultiple * kMultiple;
     return chunk < kMultiple ? kMultiple : chunk;
 }
@@ -445,7 +455,8 @@ int nolo_outer_step_host(nolo_handle* h, uint64_t seed, uint64_t step, void* phi
     if (rc != NOLO_OK) return rc;
 
     const int ts = elem_size(h->theta_dtype);
-    const int64_t chunk = host_chunk(h->P, (int64_t)h->W * (8 + ts));
+    const int64_t chunk = host_chunk(h->P, (int64_t)h->W * (8 + ts),
+                                     page_locked(phi_host) && page_locked(theta_host) && page_locked(delta_host));
     // Earlier work on the bound stream may still use the device buffers.
     NOLO_CUDA(h, cudaEventRecord(h->ev_fence, h->stream));
     NOLO_CUDA(h, cudaStreamWaitEvent(h->s_in, h->ev_fence, 0));
@@ -546,7 +557,7 @@ int nolo_route_host(nolo_handle* h, uint64_t seed, uint64_t step, const void* ac
     const size_t bytes = route_bytes(h);
     if (overlap(acts_dev, bytes, h->acts_out, bytes)) return fail(h, NOLO_EINVAL, "acts_dev overlaps acts_out");
     const int64_t es = elem_size(h->act_dtype), blocks = (int64_t)(h->stages - 1) * h->W * h->K;
-    const int64_t chunk = host_chunk(h->E, blocks * es);
+    const int64_t chunk = host_chunk(h->E, blocks * es, page_locked(acts_host) && page_locked(out_host));
     // Chunks of the result come back while later chunks of the input are read: not where they would land on them.
     const bool in_place = acts_host == out_host;      // every chunk comes back to where it was read
     const bool crossed = !in_place && overlap(acts_host, bytes, out_host, bytes);

@@ -744,3 +744,24 @@ def test_non_default_stream(nolo):
     want = O.outer_step(to_np(phi), to_np(theta), to_np(delta), perm, n, *F)
     assert_close_f32(to_np(dev[0]), want[0], "phi")
     nolo.nolo_destroy(h)
+
+
+def test_host_paths_of_pageable_memory(nolo):
+    """Pageable buffers are copied in pieces of 384 MB: two of the state here, the activations whole."""
+    W, P, S, K, E = 4, 9_000_003, 2, 2, 1_000_003
+    state = synth.make_state(W, P, 6)
+    dev, stage, host = [x.cuda() for x in state], [torch.zeros_like(x, device="cuda") for x in state], [x.clone() for x in state]
+    acts = synth.make_acts(S - 1, W, K, E, 6, torch.float32)
+    out, d_in, d_out = torch.zeros_like(acts), torch.empty_like(acts, device="cuda"), torch.empty_like(acts, device="cuda")
+    hd, hh = nolo.nolo_create(W, 2, P, S, *F), nolo.nolo_create(W, 2, P, S, *F)
+    nolo.nolo_bind_state(hd, *dev)
+    nolo.nolo_bind_state(hh, *stage)
+    nolo.nolo_bind_route(hh, W * K, E, d_out)
+    nolo.nolo_outer_step(hd, 2, 3)
+    nolo.nolo_outer_step_host(hh, 2, 3, *host)
+    nolo.nolo_route_host(hh, 2, 3, acts, out, d_in)
+    for a, b in zip(dev, host):
+        assert torch.equal(a[:, :P].cpu(), b[:, :P])
+    assert np.array_equal(to_np(out), O.route_forward(to_np(acts), O.draw_route(2, 3, S, W, K)))
+    nolo.nolo_destroy(hd)
+    nolo.nolo_destroy(hh)
