@@ -15,6 +15,7 @@
 #include "nolo_launch.cuh"
 #include "nolo_lognormal.cuh"
 #include "nolo_philox.cuh"
+#include "nolo_steps.h"
 
 #include <cmath>
 
@@ -223,7 +224,7 @@ straggler_work_kernel(const Slab s, const LogNormal q, int64_t items) {
     const int w = (int)(item - row * s.W), mine = item < items ? (int)(row - row0) : 0;
     const int64_t trial = row / s.iterations, t = row - trial * s.iterations;
     const PhiloxOfC1 of_worker = philox_of_c1(w, s.t0 + t, s.seed);
-    const int blocks = (s.H + 3) / 4;
+    const int blocks = step_blocks(s.H);
     double work = 0.0;
     for (int b0 = 0; b0 < blocks; b0 += kSharedBlocks) {
         __syncthreads();
@@ -238,13 +239,13 @@ straggler_work_kernel(const Slab s, const LogNormal q, int64_t items) {
         for (int k = 0; k < here; ++k) {                             // inner steps 4 (b0 + k) .. + 3 share a block
             double step[4];
             lognormal4<TAME>(tables, philox_join(lead[mine][k], of_worker, s.seed, s.trial0 + trial), q, step);
-            const int left = s.H - 4 * (b0 + k);
-            if (left >= 4) {
+            const int steps = steps_in_block(s.H, b0 + k);
+            if (steps == 4) {
                 work += (step[0] + step[1]) + (step[2] + step[3]);
             } else {
 #pragma unroll
                 for (int l = 0; l < 3; ++l)
-                    if (l < left) work += step[l];
+                    if (l < steps) work += step[l];
             }
         }
     }
@@ -267,15 +268,17 @@ straggler_split_work_kernel(const Slab s, const LogNormal q, int lanes, int64_t 
         const int64_t row = item / s.W;
         const int w = (int)(item - row * s.W);
         const int64_t trial = row / s.iterations, t = row - trial * s.iterations;
-        for (int k = lane; 4 * k < s.H; k += lanes) {
+        const int blocks = step_blocks(s.H);
+        for (int k = lane; k < blocks; k += lanes) {
             double step[4];
             lognormal4<TAME>(tables, philox4x64_10(k, w, s.t0 + t, kDomainStraggler, s.seed, s.trial0 + trial), q, step);
-            if (4 * k + 4 <= s.H) {
+            const int steps = steps_in_block(s.H, k);
+            if (steps == 4) {
                 work += (step[0] + step[1]) + (step[2] + step[3]);
             } else {
 #pragma unroll
                 for (int l = 0; l < 3; ++l)
-                    if (l < s.H - 4 * k) work += step[l];
+                    if (l < steps) work += step[l];
             }
         }
     }

@@ -35,3 +35,35 @@ int main() {
     return 0;
 }
 """)
+
+
+def test_inner_steps_of_any_int_count(tmp_path):
+    """Up to the largest int, by any number of lanes: each lane's loop ends, the blocks hold H steps in all, and no
+    signed sum overflows (the sanitizer is on)."""
+    run_host_code(tmp_path, r"""
+#include "nolo_steps.h"
+#include <climits>
+#include <cstdio>
+int main() {
+    for (int i = 0; i < 400; ++i) {
+        const int H = i < 200 ? 1 + i : INT_MAX - (i - 200);
+        const int blocks = nolo::step_blocks(H);
+        long long steps = 0;
+        for (int lanes = 1; lanes <= 32; lanes *= 2) {
+            steps = 0;
+            for (int lane = 0; lane < lanes; ++lane) {
+                // the last turns of this lane; all before them have whole blocks
+                int k = blocks > 4096 ? (blocks - 1024) / lanes * lanes + lane : lane;
+                steps += 4ll * (k / lanes);
+                for (; k < blocks; k += lanes) {
+                    const int n = nolo::steps_in_block(H, k);
+                    if (n < 1 || n > 4 || (n < 4 && k != blocks - 1)) return printf("H %d k %d: %d\n", H, k, n), 1;
+                    steps += n;
+                }
+            }
+            if (steps != H) return printf("H %d, %d lanes: %lld\n", H, lanes, steps), 1;
+        }
+    }
+    return 0;
+}
+""")
