@@ -2,12 +2,12 @@
 // which the kernels are enqueued.  All arithmetic of the method lives in the kernels.
 #include "nolo.h"
 #include "nolo_internal.h"
+#include "nolo_scratch.h"
 
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
-#include <mutex>
 #include <new>
 
 namespace {
@@ -244,83 +244,32 @@ size_t route_bytes(const nolo_handle* h) {
 }
 
 // Device scratch of the simulations, which have no handle to keep it in.  cudaMalloc and cudaFree cost 0.65 ms a
-// call on B200 (measured; more when the device is busy), several times what a small simulation takes, so a
-// few blocks are kept: at most kBlocks of at most kMostBytes in all, each used by one call at a time and put
-// back when the GPU is done with it.  They are given back when a handle is destroyed and when an
-// allocation here fails.
-class ScratchBlocks {
-public:
-    cudaError_t take(size_t bytes, void** out) {
-        int device = 0;
-        cudaError_t e = cudaGetDevice(&device);
-        if (e != cudaSuccess) return e;
-        {
-            std::lock_guard<std::mutex> lock(mutex_);
-            Block* best = nullptr;
-            for (Block& b : blocks_)
-                if (b.p && b.device == device && b.bytes >= bytes && (!best || b.bytes < best->bytes)) best = &b;
-            if (best) {
-                *out = best->p;
-                best->p = nullptr;
-                kept_ -= best->bytes;
-                return cudaSuccess;
-            }
-        }
-        e = cudaMalloc(out, bytes);
-        if (e == cudaErrorMemoryAllocation) {
-            cudaGetLastError();
-            give_back();
-            e = cudaMalloc(out, bytes);
-        }
+// call on B200 (measured; more when the device is busy), several times what a small simulation takes.  What is kept is
+// given back when a handle is destroyed and when an allocation here fails.
+struct DeviceMemory {
+    using Status = cudaError_t;
+    static constexpr Status kOk = cudaSuccess;
+    static Status device(int* d) { return cudaGetDevice(d); }
+    static Status allocate(void** p, size_t bytes) {
+        const Status e = cudaMalloc(p, bytes);
+        if (e != cudaSuccess) cudaGetLastError();
         return e;
     }
-    // p is no longer in use on the GPU; bytes as it was taken or less.
-    void put(void* p, size_t bytes) {
-        int device = 0;
-        if (cudaGetDevice(&device) == cudaSuccess) {
-            std::lock_guard<std::mutex> lock(mutex_);
-            for (Block& b : blocks_) {
-                if (b.p || kept_ + bytes > kMostBytes) continue;
-                b.p = p;
-                b.bytes = bytes;
-                b.device = device;
-                kept_ += bytes;
-                return;
-            }
-        }
-        cudaFree(p);
-    }
-    void give_back() {
-        void* p[kBlocks];
-        {
-            std::lock_guard<std::mutex> lock(mutex_);
-            for (int i = 0; i < kBlocks; ++i) { p[i] = blocks_[i].p; blocks_[i].p = nullptr; }
-            kept_ = 0;
-        }
-        for (void* q : p) if (q) cudaFree(q);
-    }
-
-private:
-    static constexpr int kBlocks = 4;
-    static constexpr size_t kMostBytes = size_t(64) << 20;
-    struct Block { void* p = nullptr; size_t bytes = 0; int device = 0; };
-    std::mutex mutex_;
-    Block blocks_[kBlocks];
-    size_t kept_ = 0;
+    static bool exhausted(Status e) { return e == cudaErrorMemoryAllocation; }
+    static void release(void* p) { cudaFree(p); }
 };
+using Scratches = nolo::ScratchBlocks<DeviceMemory>;
 
-ScratchBlocks g_scratch;
+Scratches g_scratch;
 
 // Scratch of one simulation call, kept for the next one if the call comes to its end.
 struct Scratch {
-    void* p = nullptr;
-    size_t bytes = 0;
+    Scratches::Block block;
     cudaError_t take(size_t want) {
-        bytes = want < (size_t(1) << 20) ? size_t(1) << 20 : want;      // small calls of all sizes share blocks
-        return g_scratch.take(bytes, &p);
+        return g_scratch.take(want < (size_t(1) << 20) ? size_t(1) << 20 : want, &block);   // small calls of all sizes share blocks
     }
-    ~Scratch() { if (p) cudaFree(p); }
-    void keep() { g_scratch.put(p, bytes); p = nullptr; }
+    ~Scratch() { if (block.p) cudaFree(block.p); }
+    void keep() { g_scratch.put(block); block.p = nullptr; }
 };
 
 int ensure_host_streams(nolo_handle* h) {
@@ -760,8 +709,8 @@ int nolo_sim_tree_allreduce(int W, double mu, double sigma, int64_t trials, uint
     const size_t results = sizeof(double) * (((size_t)trials + 5) & ~size_t(1));
     cudaError_t e = scratch.take(results + nolo::tree_scratch());
     if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? NOLO_ENOMEM : NOLO_ECUDA;
-    double* d = static_cast<double*>(scratch.p);
-    e = nolo::launch_tree_allreduce(W, mu, sigma, trials, seed, d + 4, d, static_cast<char*>(scratch.p) + results, s);
+    double* d = static_cast<double*>(scratch.block.p);
+    e = nolo::launch_tree_allreduce(W, mu, sigma, trials, seed, d + 4, d, static_cast<char*>(scratch.block.p) + results, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(host_stats, d, 2 * sizeof(double), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess && host_trials)
         e = cudaMemcpyAsync(host_trials, d + 4, sizeof(double) * (size_t)trials, cudaMemcpyDeviceToHost, s);
@@ -783,7 +732,7 @@ int nolo_sim_straggler(int W, int n, int H, int T, double mu, double sigma, int6
     const size_t results = sizeof(double) * (2 * (size_t)trials + 4);
     cudaError_t e = scratch.take(results + nolo::straggler_scratch(W, T, trials));
     if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? NOLO_ENOMEM : NOLO_ECUDA;
-    double* d = static_cast<double*>(scratch.p);
+    double* d = static_cast<double*>(scratch.block.p);
     e = nolo::launch_straggler(W, n, H, T, mu, sigma, trials, seed, d + 4, d, reinterpret_cast<char*>(d) + results, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(host_stats, d, 4 * sizeof(double), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess && host_trials)

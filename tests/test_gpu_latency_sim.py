@@ -150,3 +150,35 @@ def test_simulation_argument_checks(nolo):
         with pytest.raises(nolo.NoloError) as e:
             nolo.nolo_sim_straggler(*bad, 1.0, 0.5, 1, 0)
         assert e.value.status == nolo.NOLO_EINVAL
+
+
+def test_scratch_is_kept_and_bounded(nolo):
+    """What is kept stays below 64 MB however large and small calls follow each other, and the largest of growing
+    calls is kept (the driver hands memory out in pieces of 2 MB)."""
+    import torch
+
+    def call(mb):
+        nolo.nolo_sim_tree_allreduce(2, 0.0, 0.5, (mb << 17) - 1000, 1)
+
+    def give_back():
+        nolo.nolo_destroy(nolo.nolo_create(2, 1, 8, 1, 0.5, 0.7, 0.5))
+        torch.cuda.synchronize()
+
+    call(1)
+    give_back()
+    free = torch.cuda.mem_get_info()[0]
+    for small in (1, 2, 3):
+        call(40)
+        call(small)
+        assert free - torch.cuda.mem_get_info()[0] <= (64 + 8) << 20
+    give_back()
+    for mb in (1, 2, 4, 8, 16, 32, 48):
+        call(mb)
+        assert free - torch.cuda.mem_get_info()[0] <= (64 + 8) << 20
+    kept = torch.cuda.mem_get_info()[0]
+    assert free - kept >= 48 << 20
+    for mb in (48, 3, 48, 1, 2, 48):
+        call(mb)
+        assert torch.cuda.mem_get_info()[0] == kept
+    give_back()
+    assert free - torch.cuda.mem_get_info()[0] <= 4 << 20

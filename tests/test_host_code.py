@@ -67,3 +67,131 @@ int main() {
     return 0;
 }
 """)
+
+
+SCRATCH = r"""
+#include "nolo_scratch.h"
+#include <cstdio>
+#include <cstdlib>
+#include <map>
+#include <thread>
+#include <vector>
+#define CHECK(x) do { if (!(x)) { printf("line %d: %s\n", __LINE__, #x); exit(1); } } while (0)
+struct Fake {
+    using Status = int;
+    static constexpr int kOk = 0;
+    static inline std::mutex m;
+    static inline std::map<void*, size_t> held;
+    static inline size_t total = 0, room = ~size_t(0);
+    static inline int allocations = 0, fail_with = 0;
+    static inline thread_local int current = 0;
+    static int device(int* d) { *d = current; return 0; }
+    static int allocate(void** p, size_t bytes) {
+        std::lock_guard<std::mutex> lock(m);
+        if (fail_with) return fail_with;
+        if (total + bytes > room) return 2;
+        *p = malloc(1);
+        held[*p] = bytes; total += bytes; ++allocations;
+        return 0;
+    }
+    static bool exhausted(int e) { return e == 2; }
+    static void release(void* p) {
+        std::lock_guard<std::mutex> lock(m);
+        CHECK(held.count(p));
+        total -= held[p]; held.erase(p); free(p);
+    }
+};
+using Pool = nolo::ScratchBlocks<Fake>;
+const size_t MB = size_t(1) << 20;
+void call(Pool& pool, size_t bytes) {
+    Pool::Block b;
+    CHECK(pool.take(bytes, &b) == 0 && b.p && b.bytes >= bytes);
+    { std::lock_guard<std::mutex> lock(Fake::m); CHECK(Fake::held[b.p] == b.bytes); }
+    pool.put(b);
+}
+"""
+
+
+def test_scratch_keeps_its_bound_and_its_blocks(tmp_path):
+    run_host_code(tmp_path, SCRATCH + r"""
+int main() {
+    {   // a large block lent to small calls is a large block still
+        Pool pool;
+        for (int i = 0; i < 40; ++i) {
+            call(pool, 40 * MB);
+            call(pool, (1 + i % 3) * MB);
+            CHECK(Fake::total <= Pool::kMostBytes);
+        }
+        CHECK(Fake::allocations == 1);
+        // ... also to small calls that overlap
+        Pool::Block b[4];
+        for (int turn = 0; turn < 10; ++turn) {
+            for (Pool::Block& x : b) CHECK(pool.take(MB, &x) == 0);
+            for (Pool::Block& x : b) pool.put(x);
+            CHECK(Fake::total <= Pool::kMostBytes);
+        }
+        CHECK(Fake::allocations == 4);
+        pool.give_back();
+        CHECK(Fake::total == 0);
+    }
+    {   // growing sizes: the largest, repeated, is not allocated again
+        Pool pool;
+        for (size_t mb = 1; mb <= 32; mb *= 2) { call(pool, mb * MB); CHECK(Fake::total <= Pool::kMostBytes); }
+        call(pool, 33 * MB);
+        const int before = Fake::allocations;
+        for (int i = 0; i < 5; ++i) call(pool, 33 * MB);
+        CHECK(Fake::allocations == before && Fake::total <= Pool::kMostBytes);
+        call(pool, Pool::kMostBytes);
+        CHECK(Fake::total == Pool::kMostBytes);
+        call(pool, Pool::kMostBytes + 1);            // not kept
+        CHECK(Fake::total == Pool::kMostBytes);
+        pool.give_back();
+        CHECK(Fake::total == 0);
+    }
+    {   // another device finds room, and never the first one's blocks
+        Pool pool;
+        for (int mb = 10; mb <= 16; mb += 2) call(pool, mb * MB);
+        Fake::current = 1;
+        call(pool, MB);
+        const int before = Fake::allocations;
+        for (int i = 0; i < 5; ++i) call(pool, MB);
+        CHECK(Fake::allocations == before);
+        Fake::current = 0;
+        call(pool, 16 * MB);
+        CHECK(Fake::allocations == before);
+        pool.give_back();
+    }
+    {   // where memory is short what is kept goes first; other errors are passed on
+        Pool pool;
+        call(pool, 10 * MB);
+        call(pool, 20 * MB);
+        Fake::room = 40 * MB;
+        call(pool, 35 * MB);
+        CHECK(Fake::total == 35 * MB);
+        Pool::Block b;
+        CHECK(pool.take(41 * MB, &b) == 2 && !b.p);
+        Fake::room = ~size_t(0);
+        Fake::fail_with = 5;
+        CHECK(pool.take(MB, &b) == 5 && !b.p);
+        Fake::fail_with = 0;
+        pool.give_back();
+    }
+    {   // threads
+        Pool pool;
+        std::vector<std::thread> threads;
+        for (int t = 0; t < 8; ++t)
+            threads.emplace_back([&pool, t] {
+                Fake::current = t & 1;
+                for (int i = 0; i < 2000; ++i) {
+                    call(pool, (1 + (i * 7 + t) % 40) * MB);
+                    if (i % 100 == 0) pool.give_back();
+                }
+            });
+        for (std::thread& t : threads) t.join();
+        CHECK(Fake::total <= Pool::kMostBytes);
+        pool.give_back();
+        CHECK(Fake::total == 0);
+    }
+    return 0;
+}
+""")
