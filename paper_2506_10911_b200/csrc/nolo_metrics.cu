@@ -26,7 +26,7 @@ struct Moments {
     __device__ __forceinline__ void join(const Moments& o, float n, float m) {
         const float d = o.mean - mean, share = m / (n + m);
         mean += d * share;
-        m2 += o.m2 + d * d * (n * share);
+        m2 += o.m2 + d * (n * share * d);      // (d * d may overflow where this does not)
     }
 };
 

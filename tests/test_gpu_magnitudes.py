@@ -81,3 +81,16 @@ def test_larger_state_register_path(nolo):
     """Pairs and fours over enough columns to meet the rare near-cancellations of phi + delta'."""
     for n, dt in ((2, torch.bfloat16), (4, torch.float32), (8, torch.bfloat16)):
         step_and_compare(nolo, 16, n, 300_001, dt, (0.5, 0.7, 0.5), seed=5 + n)
+
+
+@pytest.mark.parametrize("W,far", [(4, 2.0e19), (16, 1.9e19), (64, 1.852e19)])
+def test_divergence_of_one_far_replica(nolo, W, far):
+    """One replica so far off that the square of its distance leaves float32, but the sum of the squared deviations
+    does not: finite, whichever worker it is and however the workers are shared out."""
+    phi = torch.zeros((W, 64))
+    phi[torch.arange(64) % W, torch.arange(64)] = far
+    d = phi.cuda()
+    h = nolo.nolo_create(W, 1, 64, 1, 0.5, 0.7, 0.5)
+    nolo.nolo_bind_state(h, d, torch.zeros_like(d), torch.zeros_like(d))
+    assert nolo.nolo_divergence(h) == pytest.approx(O.divergence(to_np(phi)), rel=1e-6)
+    nolo.nolo_destroy(h)
