@@ -291,7 +291,7 @@ int nolo_get_route(nolo_handle* h, int32_t* host_out);
  *   host_out[1] = sqrt((1/P) sum_p var_p)      root of the mean variance
  * (the paper does not say which of the two scalars it plots).  Read-only on
  * phi; float32 per parameter, float64 sums in a fixed order (reproducible).
- * Allocates 16 bytes per 4096 parameters (at most 40 KB more for small states) of
+ * Allocates 16 bytes per 4096 parameters (at most 60 KB more for small states) of
  * device scratch and 16 bytes of page-locked host memory on first use.
  * Synchronous: returns when the two doubles are in host memory.
  * Errors: NOLO_EINVAL, NOLO_ESTATE, NOLO_ENOMEM, NOLO_ECUDA.
@@ -346,7 +346,7 @@ double nolo_expected_pair_exchange(double mu, double sigma);
  *   host_stats   host, 4 doubles: mean time with the global barrier, mean time
  *           with subgroup waits, then the standard errors of the two means
  *   host_trials  host, [trials][2] (barrier, subgroup) per trial, or NULL
- * Synchronous; scratch as above (at most about 40 MB).  trials 1..2^20, and the
+ * Synchronous; scratch as above (at most about 63 MB).  trials 1..2^20, and the
  * total number of samples W*H*T*trials at most NOLO_SIM_MAX_SAMPLES (2^40, about
  * 20 s of GPU time): a larger request is refused with NOLO_EINVAL rather than
  * left to occupy the device.

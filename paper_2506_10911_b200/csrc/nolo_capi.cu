@@ -581,12 +581,13 @@ int nolo_divergence(nolo_handle* h, double* host_out) {
         }
         h->d_div = d;
     }
+    int launches = 0;
     Bracket br(h, NOLO_KERNEL_DIVERGENCE);
     NOLO_CUDA(h, nolo::launch_divergence(h->phi, h->W, h->stride, h->P, h->d_div,
                                          reinterpret_cast<unsigned*>(static_cast<char*>(h->d_div) + partials), h->div_out,
-                                         h->stream));
+                                         h->stream, &launches));
     br.done();
-    ++h->launches;
+    h->launches += launches;
     NOLO_CUDA(h, cudaStreamSynchronize(h->stream));
     host_out[0] = h->div_out[0];
     host_out[1] = h->div_out[1];

@@ -98,10 +98,10 @@ cudaError_t launch_copy_probe(const void* in, void* out, int64_t bytes, cudaStre
 // Replica divergence of phi (Fig. 3b): out2[0] = mean over parameters of the across-worker
 // population standard deviation, out2[1] = sqrt(mean over parameters of the across-worker variance).
 // `partials` is device scratch of divergence_partials(W, P) * 16 bytes, `arrived` a device counter that is zero
-// before and after; out2 is device or mapped host memory.  One launch.
+// before and after; out2 is device or mapped host memory.  *launches receives the number of kernels, one or two.
 int64_t divergence_partials(int W, int64_t P);
 cudaError_t launch_divergence(const float* phi, int W, int64_t stride, int64_t P, void* partials, unsigned* arrived,
-                              double* out2, cudaStream_t stream);
+                              double* out2, cudaStream_t stream, int* launches);
 
 // Latency simulations (Section 4.3).  per_trial: device [trials] resp. [trials][2];
 // stats: device, the column means followed by their standard errors.
@@ -109,7 +109,7 @@ cudaError_t launch_divergence(const float* phi, int W, int64_t stride, int64_t P
 size_t tree_scratch();
 cudaError_t launch_tree_allreduce(int W, double mu, double sigma, int64_t trials, uint64_t seed,
                                   double* per_trial, double* stats, void* scratch, cudaStream_t stream);
-// scratch: device, straggler_scratch() bytes (at most about 40 MB).
+// scratch: device, straggler_scratch() bytes (at most about 46 MB).
 size_t straggler_scratch(int W, int T, int64_t trials);
 cudaError_t launch_straggler(int W, int n, int H, int T, double mu, double sigma, int64_t trials,
                              uint64_t seed, double* per_trial, double* stats, void* scratch, cudaStream_t stream);

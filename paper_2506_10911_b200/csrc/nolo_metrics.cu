@@ -206,7 +206,7 @@ Shape shape_for(int W, int64_t P) {
 int64_t divergence_partials(int W, int64_t P) { return shape_for(W, P).ctas(P); }
 
 cudaError_t launch_divergence(const float* phi, int W, int64_t stride, int64_t P, void* partials, unsigned* arrived,
-                              double* out2, cudaStream_t stream) {
+                              double* out2, cudaStream_t stream, int* launches) {
     const Shape s = shape_for(W, P);
     const int64_t ctas = s.ctas(P);
     if (ctas > 0x7fffffffll) return cudaErrorInvalidConfiguration;
@@ -214,6 +214,7 @@ cudaError_t launch_divergence(const float* phi, int W, int64_t stride, int64_t P
     auto launch = [&](auto kernel) {
         return launch_overlapped(kernel, dim3((unsigned)ctas), kThreads, 0, stream, phi, W, stride, P, partial, arrived, out2);
     };
+    *launches = s.items == 4 ? 2 : 1;
     if (s.items == 4) {
         const cudaError_t e = launch(divergence_kernel<4, 1, false>);
         if (e != cudaSuccess) return e;

@@ -765,3 +765,14 @@ def test_host_paths_of_pageable_memory(nolo):
     assert np.array_equal(to_np(out), O.route_forward(to_np(acts), O.draw_route(2, 3, S, W, K)))
     nolo.nolo_destroy(hd)
     nolo.nolo_destroy(hh)
+
+
+@pytest.mark.parametrize("W,P,kernels", [(16, 10_000, 1), (2, 4_800_000, 1), (2, 4_849_665, 2), (64, 1 << 20, 1)])
+def test_divergence_counts_its_kernels(nolo, W, P, kernels):
+    phi = torch.zeros((W, (P + 7) // 8 * 8), device="cuda")
+    h = nolo.nolo_create(W, 1, P, 1, *F)
+    nolo.nolo_bind_state(h, phi, torch.zeros_like(phi), torch.zeros_like(phi))
+    for calls in (1, 2):
+        nolo.nolo_divergence(h)
+        assert nolo.nolo_launch_count(h) == calls * kernels
+    nolo.nolo_destroy(h)
