@@ -186,16 +186,18 @@ struct Shape {
     }
 };
 
-// Four quads per thread and a second kernel for the sums where that leaves eight CTAs per SM, else one quad and
-// one kernel, in as many parts as give the chip about four CTAs per SM while every part keeps a worker.  A call, before (two
-// kernels of one shape, a copy of the result) -> now, us: (W, P) = (16, 10 007) 31.2 -> 16.5, (16, 2^20) 42.8 -> 29.1,
-// (16, 7.1e6) 93.1 -> 81.4, (128, 10 007) 98.7 -> 18.2, (1024, 1000) 331 -> 21.3, (1024, 65 536) 841 -> 65, (1024, 2^20)
-// 920 -> 703, (16, 2^26) 637 -> 622; one quad per thread on that last one 670.  Four quads want four CTAs of 64
-// registers per SM: at 66 registers, three CTAs, it measured 675.
-constexpr int64_t kManyCtas = 148 * 8, kFewCtas = 148 * 4;
+// Four quads per thread and a second kernel for the sums where that leaves enough CTAs, else one quad and one
+// kernel, in as many parts as give the chip about four CTAs per SM while every part keeps a worker.  Enough are eight per
+// SM, so that the last, part-filled wave of four weighs little ((128, 3e6) 247 us with one quad, 301 with four, which
+// are 1.2 waves); with few workers a CTA is soon done and their number weighs more, the one counter that they all
+// add to included: three per SM ((1, 2^22) 45 us with one quad, 29 with four, (12, 3e6) 57 / 53, (16, 3e6) 58 / 62).
+// Few columns in parts: (1024, 1000) 331 us unparted, 21 now.  Four quads want four CTAs of 64 registers per SM: at 66
+// registers, three CTAs, (16, 2^26) measured 675 us instead of 622.
+constexpr int64_t kManyCtas = 148 * 8, kManyShortCtas = 148 * 3, kFewCtas = 148 * 4;
+constexpr int kShortMaxW = 12;
 Shape shape_for(int W, int64_t P) {
     Shape s = {4, 1};
-    if (s.ctas(P) >= kManyCtas) return s;
+    if (s.ctas(P) >= (W <= kShortMaxW ? kManyShortCtas : kManyCtas)) return s;
     s.items = 1;
     while (s.parts < 32 && s.ctas(P) < kFewCtas && W >= 4 * s.parts) s.parts *= s.parts == 16 ? 2 : 4;
     return s;

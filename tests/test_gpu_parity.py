@@ -767,12 +767,16 @@ def test_host_paths_of_pageable_memory(nolo):
     nolo.nolo_destroy(hh)
 
 
-@pytest.mark.parametrize("W,P,kernels", [(16, 10_000, 1), (2, 4_800_000, 1), (2, 4_849_665, 2), (64, 1 << 20, 1)])
+@pytest.mark.parametrize("W,P,kernels", [(16, 10_000, 1), (13, 4_845_568, 1), (13, 4_845_569, 2), (64, 1 << 20, 1),
+                                         (1, 1_814_528, 1), (1, 1_814_529, 2), (12, 1_814_528, 1), (12, 1_814_529, 2)])
 def test_divergence_counts_its_kernels(nolo, W, P, kernels):
+    """One kernel, or two from 1184 CTAs of 4096 columns on (444 for up to 12 workers), with the same result."""
     phi = torch.zeros((W, (P + 7) // 8 * 8), device="cuda")
+    phi[:, P - 3:P] = torch.arange(W, device="cuda").view(-1, 1)
     h = nolo.nolo_create(W, 1, P, 1, *F)
     nolo.nolo_bind_state(h, phi, torch.zeros_like(phi), torch.zeros_like(phi))
     for calls in (1, 2):
-        nolo.nolo_divergence(h)
+        var = (W * W - 1) / 12                       # of 0 .. W-1
+        assert nolo.nolo_divergence(h) == pytest.approx((3 / P * var**0.5, (3 / P * var)**0.5), rel=1e-6, abs=1e-12)
         assert nolo.nolo_launch_count(h) == calls * kernels
     nolo.nolo_destroy(h)
