@@ -6,7 +6,9 @@
 // Bound by the pipes of the float64 operations and of Philox's products.  The logarithm, sine and cosine and
 // exponential are table-driven in the manner of P. T. P. Tang (ACM TOMS 15, 1989, "Table-driven implementation of
 // the exponential function in IEEE floating-point arithmetic", and TOMS 16, 1990, for the logarithm): a table in
-// shared memory takes the leading bits, a Taylor polynomial the rest.  The arguments are confined (u in (0, 1],
+// shared memory takes the leading bits, a Taylor polynomial the rest.  The logarithm's intervals (128 of equal high
+// word, from 0.6875 on, with a reciprocal of 1 next to 1) are laid out as in the log of Arm's optimized-routines; the
+// tables' values are computed from their definitions.  The arguments are confined (u in (0, 1],
 // angles as integers, exponents checked once on the host), so no special case is left in the loop, the angle
 // is reduced in integers and the factors 2, pi, sigma and 256 / ln 2 are folded into constants.  About 24 float64
 // operations per time; each step is good to one or two units in the last place.
