@@ -18,12 +18,12 @@ per outer step).  With N GPUs, N independent replicas run (the path has no
 cross-GPU exchange); the job's time is the slowest rank's.  Launched without a
 process launcher, `--gpus N` starts the N rank processes itself.
 
-At N=1 the line also carries `configs`: one record per paper-shaped
-configuration, per kernel path for large subgroups, and for the routing,
-divergence and split-phase kernels, each timed with the library's own CUDA
-event brackets around the kernel.
-
-Prints one JSON line on rank 0.
+Prints one JSON line on rank 0, short enough to be read off the end of a log.
+What stands behind it goes to standard error, one JSON record per line: the
+spread of the timed launches, routing, the end-to-end slice and the CPU sample,
+and at N=1 one record per paper-shaped configuration, per kernel path for large
+subgroups, for the divergence and split-phase kernels (each timed with the
+library's own CUDA event brackets around the kernel) and for the simulations.
 """
 
 from __future__ import annotations
@@ -66,6 +66,19 @@ WORKLOADS = [
 # the captured launch); traffic grows in proportion to the columns processed.  None = not captured
 # since the kernel last changed.
 PROFILED_DRAM_BYTES_PER_PARAM = {"outer_step_reg_kernel<2,bf16>": 19.59, "outer_step_reg_kernel<4,float>": 23.15}
+
+
+def rounded(x):
+    """The same with floats of ten significant digits."""
+    if isinstance(x, dict):
+        return {k: rounded(v) for k, v in x.items()}
+    if isinstance(x, (list, tuple)):
+        return [rounded(v) for v in x]
+    return float(f"{x:.10g}") if isinstance(x, float) else x
+
+
+def print_record(**rec):
+    print(json.dumps(rounded(rec)), file=sys.stderr, flush=True)
 
 
 def bytes_per_param(theta: str) -> int:
@@ -111,10 +124,10 @@ def config_dict(wl, sh, n_gpus):
              f"{wl['stages']} stages") if wl["M"] else ", outer step (single stage: no routing)"
     th = "bf16 theta" if wl["theta"] == "bf16" else "fp32 theta"
     return {
-        "workload": f"{wl['name']}: W={wl['W']} n={wl['n']} {wl['text']} (P={sh['P']}), fp32 phi/delta, {th}{route}",
+        "workload": f"{wl['name']}: W={wl['W']} n={wl['n']} {wl['text']}, fp32 phi/delta, {th}{route}",
         "W": wl["W"], "n": wl["n"], "P": sh["P"], "stages": wl["stages"], "microbatches": wl["M"], "E": sh["E"],
         "alpha": ALPHA, "beta": BETA, "gamma": GAMMA, "replicas": n_gpus,
-        "l2": f"state ({sh['state_bytes'] / GB:.1f} GB per replica) is larger than L2; no flush needed",
+        "l2": f"no flush: state of {sh['state_bytes'] / GB:.1f} GB",
     }
 
 
@@ -270,9 +283,8 @@ def cpu_baseline(wl, sh, cols: int):
     W = wl["W"]
     what = "outer step + routing" if wl["M"] else "outer step"
     rec = {"value": W * cols / tc, "unit": UNIT, "cores": cores, "kind": "oracle",
-           "sample": f"1 step ({what}) on {cols} of {sh['P']} columns x {W} workers, numpy float64: "
-                     f"{tc:.1f} s with the columns spread over {cores} threads, {t1:.1f} s on one thread",
-           "single_thread": {"value": W * cols / t1, "unit": UNIT, "cores": 1}}
+           "sample": f"1 step ({what}), {cols} of {sh['P']} columns, numpy float64, {tc:.1f} s",
+           "single_thread": {"value": W * cols / t1, "unit": UNIT, "cores": 1, "seconds": t1}}
     try:
         c1 = c_oracle_step(wl, state, 0, 1)
         cc = min(c_oracle_step(wl, state, 0, cores) for _ in range(2))
@@ -625,47 +637,48 @@ def run_ours(args):
         "warmup": args.warmup, "ms_per_step": job_ms / args.steps, "higher_is_better": True, "scaling": "weak",
         "vs_baseline": None, "dtype": "f32", "data": "synthetic",
         "config": config_dict(wl, sh, world),
-        "hbm_gbs": achieved, "pct_of_8tbs_nominal": achieved / 8000.0,
         "clocks": clocks,
-        "e2e": e2e if e2e is not None else {"value": None, "unit": UNIT, "note": e2e_note or "skipped"},
+        "e2e": {k: e2e[k] for k in ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step")} if e2e is not None
+               else {"value": None, "unit": UNIT, "note": e2e_note or "skipped"},
         "gpu_launches": launches,
         "roofline": {"bound": "hbm", "kernel": kname, "achieved": achieved, "peak": peak,
-                     "unit": "GB/s", "frac": achieved / peak, "peak_kind": f"of {peak_kind}",
+                     "unit": "GB/s", "frac": achieved / peak,
                      "frac_of_same_run_copy": achieved / copy_gbs if copy_gbs else None,
-                     "frac_note": "peak is a plain torch copy measured earlier on this pool; our own one-shot "
-                                  "128-bit copy timed in this run is the tighter ceiling (frac_of_same_run_copy)",
                      "traffic": dram_bpp * W * P if dram_bpp else None,
-                     "traffic_note": "profiler dram bytes of a small case of this kernel scaled by columns"
-                                     if dram_bpp else "not captured since the kernel last changed",
-                     "bytes_per_launch": bpp * W * P,
-                     "ms_per_launch": per_launch_ms, "ms_per_launch_min": outer_stats["min"],
-                     "ms_per_launch_median": outer_stats["median"], "ms_per_launch_max": outer_stats["max"],
-                     "launches_timed": outer_cnt,
-                     "plain_copy_same_run_gbs": copy_gbs},
+                     "bytes_per_launch": bpp * W * P, "ms_per_launch": per_launch_ms, "launches_timed": outer_cnt},
     }
+    print_record(name="outer step, spread of the timed launches", ms=outer_stats, hbm_gbs=achieved,
+                 of_8tbs_nominal=achieved / 8000.0, plain_copy_same_run_gbs=copy_gbs,
+                 peak_kind=f"of {peak_kind}: a plain torch copy; our own one-shot 128-bit copy timed in this run is the "
+                           "tighter ceiling (frac_of_same_run_copy)",
+                 traffic="profiler dram bytes of a small case of this kernel scaled by columns" if dram_bpp
+                         else "not captured since the kernel last changed")
+    if e2e is not None:
+        print_record(name="end to end", **e2e)
     if M:
         rb = 2 * acts.numel() * acts.element_size()
-        line["route"] = stats_record("routing, forward, all boundaries", "route_copy_kernel", route_stats, route_cnt,
-                                     rb, peak, copy_gbs)
+        print_record(**stats_record("routing, forward, all boundaries", "route_copy_kernel", route_stats, route_cnt,
+                                    rb, peak, copy_gbs))
         if back_stats is not None:
-            line["route_backward"] = stats_record("routing, backward, all boundaries", "route_copy_kernel",
-                                                  back_stats, back_cnt, rb, peak, copy_gbs)
+            print_record(**stats_record("routing, backward, all boundaries", "route_copy_kernel", back_stats, back_cnt,
+                                        rb, peak, copy_gbs))
     nolo.nolo_destroy(h)
     del phi, theta, delta, acts, acts_out
     torch.cuda.empty_cache()
     if world == 1 and not args.no_configs:
         args.headline = wl["name"]
-        headline_rec = stats_record(f"{wl['name']} (the headline workload above): W={W} n={n} {wl['text']}", kname,
+        print_record(**stats_record(f"{wl['name']} (the headline workload): W={W} n={n} {wl['text']}", kname,
                                     outer_stats, outer_cnt, bpp * W * P, peak, copy_gbs, W=W, n=n, P=P,
                                     theta=wl["theta"], resident_gb=sh["state_bytes"] / GB,
-                                    params_per_s=W * P / (per_launch_ms * 1e-3))
-        line["configs"] = [headline_rec] + extra_configs(nolo, dev, peak, copy_gbs, args)
-        line["simulations"] = sim_records(nolo)
-    if args.no_cpu_baseline or world > 1:
-        line["cpu_baseline"] = None
-    else:
-        line["cpu_baseline"] = cpu_baseline(wl, sh, args.cpu_cols)
-    print(json.dumps(line), flush=True)
+                                    params_per_s=W * P / (per_launch_ms * 1e-3)))
+        for rec in extra_configs(nolo, dev, peak, copy_gbs, args) + sim_records(nolo):
+            print_record(**rec)
+    line["cpu_baseline"] = None
+    if not args.no_cpu_baseline and world == 1:
+        cpu = cpu_baseline(wl, sh, args.cpu_cols)
+        print_record(name="CPU baseline", **cpu)
+        line["cpu_baseline"] = {k: cpu[k] for k in ("value", "unit", "cores", "kind", "sample")}
+    print(json.dumps(rounded(line)), flush=True)
     return 0
 
 
