@@ -344,12 +344,9 @@ __device__ __forceinline__ void ragged_tail(const KArgs& a, int g, const M& memb
 // between the reduction and the update, so nothing is read twice.  All loads of a thread are issued
 // before the first use to keep many bytes in flight.
 //
-// Bound by DRAM.  256-bit accesses make a row piece of one warp 1 KB long and halve the requests; against
-// quads in 128-bit accesses (256 threads) the rate rises with what is in flight per thread.  GB/s at W = 16,
-// P = 2^25, float32 / bfloat16 theta, quads -> octs: n = 1 6864 / 6800 -> 6905 / 6870, n = 2 6822 / 6824 -> 6923 /
-// 6850, n = 4 6770 / 6737 -> 6862 / 6800, n = 6 6521 / 6670 -> 6831 / 6695, n = 7 6673 / 6378 -> 6834 / 6740, n = 8
-// 6711 / 5568 -> 6828 / 6739; with prepared means n = 2 5988 / 6830 -> 6985 / 6976, n = 4 6655 -> 6890 (float32).
-// (The quad kernel with n = 7 and 8 left one CTA of 256 threads per SM.)
+// Bound by DRAM.  256-bit accesses make a row piece of one warp 1 KB long and halve the requests, and the rate rises
+// with what is in flight per thread: 6923 GB/s for pairs with float32 theta (W = 16, P = 2^25), 6822 in quads by 128-bit
+// accesses; 6739 against 5568 with n = 8 and bfloat16 theta, where quads left one CTA of 256 threads per SM.
 template <int N, typename ThetaT, int THREADS, bool PREPARED, bool WIDE, bool DRAW>
 __global__ void __launch_bounds__(THREADS, 1)
 outer_step_reg_kernel(const KArgs a) {
@@ -668,12 +665,11 @@ cudaError_t launch_reg_shape(KArgs& k, int groups, cudaStream_t stream) {
                              grid, THREADS, 0, stream, k);
 }
 
-// Larger CTAs stream longer pieces of a row and are the faster by up to 0.7 % where there are many octs
-// (n = 2 float32, 256 against 64 threads: 6912 / 6880 GB/s at 8.4 GB of phi, equal at 2^19 octs); below that
-// the ends of the grid weigh more (16.8 / 16.4 us at W = 4, P = 2^20).  The sizes are those that hold
-// their rate under the power cap as well, where the SM clock drops by a tenth: pairs with bfloat16 theta at
-// P = 123e6, W = 16, 320 threads 5757 us, 256 5777, 384 5765, 512 5748 at full clock but 5800 capped (the quad
-// kernel 5775).  With more than 4 members a thread needs the registers that 64-thread CTAs leave it.
+// CTA sizes.  Larger CTAs stream longer pieces of a row, but the ends of the grid weigh more: 64 threads below 2^19
+// octs (W = 4, P = 2^20, n = 2 16.4 us, with 256 threads 16.8) and where a thread has more than 4 members, for the
+// registers that leaves it; else 256, or what fits the registers better: 192 with 4 members (1878 us with 256 threads 1888,
+// W = 16, P = 2^25, float32; bfloat16 1580 / 1613), 320 for pairs with bfloat16 theta (1561 / 1567; smaller states lose
+// up to 2 %, 101.1 / 99.1 at P = 2^21).
 constexpr int64_t kRegManyOcts = 1 << 19;
 template <int N, typename ThetaT>
 constexpr int kRegThreads = N == 4 ? 192 : (N == 2 && sizeof(ThetaT) == 2) ? 320 : 256;
@@ -761,11 +757,10 @@ cudaError_t launch_group_mean(const float* phi, const int32_t* perm, int W, int 
     return launch(wide ? group_mean_kernel<1, true> : group_mean_kernel<1, false>);
 }
 
-// Drawing in the kernel saves the launch of the draw (2 us of host time, 1 to 2 us on the device), lets the kernel
-// ask for its data ahead of its wait, and costs every CTA the draw's 0.3 us.  Measured, draw kernel / drawn in
-// the step, us per step: 2^17 worker-parameters 5.3 / 3.1, 2^24 61.8 / 60.1 (n = 2), 54.5 / 52.5 (n = 8, bfloat16
-// theta), 52.0 / 51.5 (n = 12), 66.5 / 65.9 (n = 20), 2^25 121.5 / 119.4 (n = 4); 2^26 236.1 / 234-237 and, alone,
-// 248 / 250 (n = 2), 240.5 / 241.0 and 252 / 256 (n = 8).
+// Drawing in the kernel saves the launch of the draw and costs every CTA the draw's 0.3 us.  It is the faster, for a call
+// alone and for calls that follow each other, as long as the grid is few waves: up to 2^25 worker-parameters for
+// n <= 4, whose CTAs are the larger, and up to 2^24 above.  us alone, drawn in the step / by a kernel ahead: n = 2 8.2 / 9.2
+// at 2^17, 67.6 / 68.6 at 2^24, 124.9 / 126.0 at 2^25; n = 8 10.2 / 13.3 at 2^20, 61.5 / 62.5 at 2^24; n = 20 75.8 / 77.0 at 2^24.
 constexpr int64_t kDrawMaxParams = 1 << 25, kDrawMaxParamsWide = 1 << 24;   // worker-parameters; n <= 4 and above
 
 bool outer_draws(const OuterArgs& a) {

@@ -41,8 +41,8 @@ __device__ __forceinline__ void prefetch_tile(const CopyArgs& a, int64_t block) 
 
 // The replica of the other side for slot k of replica r at boundary b.  DRAW: drawn by the first warp
 // before the kernels ahead are waited for; one CTA per permutation writes the table.  The lane that finds the
-// replica has the tile brought to L2 while the kernels ahead end: us for a forward and a backward call, without
-// / with, 17 MB 13.4 / 11.5, 33 MB 25.0 / 21.2 (alone 36.0 / 33.8).
+// replica has the tile brought to L2 while the kernels ahead end (a forward and a backward call of 67 MB 39.8 us, 43.5
+// without).
 template <bool DRAW, int TILE>
 __device__ __forceinline__ int peer_of(const CopyArgs& a, int b, int r, int k) {
     int32_t* row = a.table + ((int64_t)b * a.K + k) * a.R;
@@ -210,10 +210,9 @@ cudaError_t launch_copy_probe(const void* in, void* out, int64_t bytes, cudaStre
 }
 
 // Drawing in the copy saves the launch of the draw, lets the copy ask for its data ahead of its wait, and costs every
-// CTA the draw's 0.3 us.  Measured, draw kernel / drawn in the copy, us for a forward and a backward call: 2 MB
-// 12.0 / 7.4, 50 MB 35.1 / 30.3, 100 MB 64.1 / 58.8, 134 MB 83.0 / 77.8, 400 MB 236 / 233 (alone 248 / 251); blocks that
-// are no multiple of 32 bytes 96 MB 61.0 / 61.0, 400 MB 237 / 255; at odd offsets 14 MB 17.4 / 15.7, 77 MB 51.8 / 49.0,
-// 115 MB 74.2 / 73.4-75.5 (alone 86 / 88).
+// CTA the draw's 0.3 us.  It is the faster, for a call alone and for calls that follow each other, as long as the grid is
+// few waves.  us alone, drawn in the copy / by a kernel ahead: 6 MB 10.2 / 11.3, 134 MB (multiples of 32 bytes) 47.1 / 48.1,
+// 67 MB of other blocks 28.7 / 29.7; 400 MB 251 / 248 there and back.
 constexpr int64_t kDrawMaxBytes = 64ll << 20, kDrawMaxBytesWide = 128ll << 20;   // the latter for multiples of 32 bytes
 
 bool route_draws(const RouteArgs& a) {
@@ -231,15 +230,12 @@ cudaError_t launch_shape(const CopyArgs& c, bool draw, cudaStream_t stream) {
                              THREADS, 0, stream, c);
 }
 
-// One CTA per tile: a one-shot grid streams through memory in address order, which measured about 10 %
-// faster on B200 than a resident grid striding over the tiles (the kernel loops only where a grid
-// dimension ends).  CTA shapes, us for a forward and a backward call of 96 blocks of 64 MB: 256 threads x 4
-// vectors of 16 bytes 3724, 256 x 2 3685, 512 x 2 3646; of 32 bytes 256 x 2 3698, 256 x 1 3689, 384 x 1 3676, 512 x 1
-// 3657; on a device under its power cap (SM clock down by a tenth) the shapes of 512 and more threads took 3750, so the
-// choice is the largest that keeps its rate there.  Over blocks of 1 MB all are within 2 %; copies that draw
-// want few CTAs.  Blocks at any offset (96 of 4 MB, bfloat16, GB/s): 128 x 8 6780, 128 x 4 6490, 256 x 4 6030, 256 x 1
-// 2910 (what a CTA does before its loads is a chain of several hundred cycles, so it has to have many in
-// flight); one 2-byte element per access, as before, 2180.
+// One CTA per tile: a one-shot grid streams through memory in address order, about 10 % faster on B200 than a resident
+// grid striding over the tiles (the kernel loops only where a grid dimension ends).  CTA shapes: the largest that keeps
+// its rate on a device under its power cap too, where shapes of 512 and more threads lost 2-3 % (96 blocks of
+// 64 MB there and back: 384 threads x 1 vector of 32 bytes 3676 us, 256 x 4 of 16 bytes 3724); copies that draw want few
+// CTAs; blocks at any offset many vectors per thread, because what a CTA does before its loads is a chain of several
+// hundred cycles (96 blocks of 4 MB, bfloat16: 128 x 8 6780 GB/s, 256 x 1 2910, one element per access 2180).
 cudaError_t launch_route(const RouteArgs& a, cudaStream_t stream) {
     CopyArgs c;
     const int64_t skip = a.first_element * a.elem_size;
