@@ -65,7 +65,7 @@ WORKLOADS = [
 # of the same kernel (dram__bytes_read.sum + dram__bytes_write.sum over the worker-parameters of
 # the captured launch); traffic grows in proportion to the columns processed.  None = not captured
 # since the kernel last changed.
-PROFILED_DRAM_BYTES_PER_PARAM = {"outer_step_reg_kernel<2,bf16>": 19.59, "outer_step_reg_kernel<4,float>": 23.15}
+PROFILED_DRAM_BYTES_PER_PARAM = {"outer_step_reg_kernel<2,bf16>": 19.58, "outer_step_reg_kernel<4,float>": 23.14}
 
 
 def rounded(x):
@@ -436,7 +436,7 @@ def extra_configs(nolo, dev, peak, copy_gbs, args):
 # its 20 64 x 64 -> 128-bit products, the rest is shared) and half a table-driven logarithm, square root
 # and sine/cosine pair plus one exponential in float64 per sample; the tree kernel also walks the tree.
 # The bound is SMs x 4 schedulers x 32 lanes x SM clock / that count.
-SIM_THREAD_INSTR_PER_SAMPLE = {"straggler_work_kernel": 95.1, "tree_allreduce_kernel": 130.8}
+SIM_THREAD_INSTR_PER_SAMPLE = {"straggler_work_kernel": 95.1, "tree_allreduce_kernel": 129.7}
 
 
 def sim_records(nolo):
