@@ -137,3 +137,51 @@ def test_a_callers_kernel_sees_the_new_weights_ahead_of_its_wait(nolo, early_rea
         assert torch.equal(seen, theta.view(-1)[::stride][:blocks * 32])
         assert not bool((seen == 7.0).any())
     nolo.nolo_destroy(h)
+
+
+@pytest.mark.parametrize("W,P", [(8, 5000), (40, 70_003)])
+def test_captured_calls_replay_as_they_run(nolo, W, P):
+    """Both ways round, the step, the prepared step and the same from a second stream that joins in, captured into
+    a graph: tables drawn inside the kernels (8 workers) and ahead of them (40)."""
+    K, E, n = 2, 3001, 2
+    state = [x.cuda() for x in synth.make_state(W, P, 4)]
+    acts = synth.make_acts(1, W, K, E, 2, torch.bfloat16).cuda()
+    results = []
+    for captured in (False, True):
+        mine = [x.clone() for x in state]
+        out, back = torch.zeros_like(acts), torch.zeros_like(acts)
+        mean = torch.zeros((W // n, mine[0].shape[1]), dtype=torch.float64, device="cuda")
+        side, other = torch.cuda.Stream(), torch.cuda.Stream()
+        torch.cuda.synchronize()
+
+        def calls():
+            for step in range(3):
+                nolo.nolo_route(h, 3, step, acts)
+                nolo.nolo_route_backward(h, 3, step, out, back)
+                nolo.nolo_outer_step(h, 3, step)
+                other.wait_stream(side)
+                with torch.cuda.stream(other):
+                    mine[2].mul_(0.5)
+                side.wait_stream(other)
+                nolo.nolo_outer_prepare(h, 3, step + 100)
+                nolo.nolo_outer_step_prepared(h, 3, step + 100)
+
+        h = nolo.nolo_create(W, n, P, 2, *F)
+        nolo.nolo_bind_state(h, *mine, stream=side)
+        nolo.nolo_bind_prepared(h, mean)
+        nolo.nolo_bind_route(h, W * K, E, out)
+        with torch.cuda.stream(side):
+            if captured:
+                graph = torch.cuda.CUDAGraph()
+                graph.capture_begin()
+                calls()
+                graph.capture_end()
+                graph.replay()
+            else:
+                calls()
+        torch.cuda.synchronize()
+        assert torch.equal(back, acts)
+        results.append((*mine, out, mean))
+        nolo.nolo_destroy(h)
+    for x, y in zip(*results):
+        assert torch.equal(x, y)
