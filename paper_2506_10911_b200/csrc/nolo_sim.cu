@@ -56,7 +56,7 @@ __device__ __forceinline__ void sync_group(int group) {
 }
 
 template <bool TAME, bool LEAD>
-__global__ void __launch_bounds__(LEAD ? kTreeThreads : 256, LEAD ? 3 : 5)
+__global__ void __launch_bounds__(LEAD ? kTreeThreads : 256, LEAD ? 2 : 5)
 tree_allreduce_kernel(int W, int group, int64_t trials, LogNormal q, uint64_t seed, double* __restrict__ out) {
     extern __shared__ double2 dynamic[];
     __shared__ LogNormalTables tables;
@@ -200,56 +200,66 @@ struct Slab {
     double* out;               // [trials][2]: barrier and subgroup time so far
 };
 
-// A thread per item (trial, iteration, worker), for W >= kSharedRowsW.  A CTA's items lie in few rows (trial,
-// iteration), so the part of the Philox rounds that depends on the row and the block only is made once for
-// the CTA, kSharedBlocks blocks at a time.  Bound by the 64-bit products, 15 per four times, and the float64
-// operations, whose pipes are busy 60 and 35 % of the time and measure as one: 2 to 5 CTAs per SM, two blocks in
-// flight per thread or the next block's Philox ahead of this one's times all gave 16.5 to 17.6 ms where this shape
-// gave 16.7, four float64 operations fewer per pair 16.1.  235 G times/s in all (W = 1024, H = 100).
+// The times of one block.
+template <bool TAME>
+__device__ __forceinline__ double block_work(const LogNormalTables& tables, const Philox4& x, const LogNormal& q) {
+    double step[4];
+    lognormal4<TAME>(tables, x, q, step);
+    return (step[0] + step[1]) + (step[2] + step[3]);
+}
+// The first `steps` of them, fewer than four: the end of an item.
+template <bool TAME>
+__device__ __forceinline__ double part_work(const LogNormalTables& tables, const Philox4& x, const LogNormal& q, int steps) {
+    double a, b;
+    lognormal2<TAME>(tables, x.w0, x.w1, q, a, b);
+    double work = steps > 1 ? a + b : a;
+    if (steps > 2) {
+        lognormal2<TAME>(tables, x.w2, x.w3, q, a, b);
+        work += a;
+    }
+    return work;
+}
+
+// A thread per item (iteration, worker) of a trial, for W >= kSharedRowsW.  A CTA's kSimThreads items lie in few rows
+// (iterations), so the part of the Philox rounds that depends on the row and the block only is made once for
+// the CTA, kSharedBlocks blocks at a time; they are of one trial, so the round keys are the same for the CTA.
+// Bound as nolo_lognormal.cuh says: 323 thread-instructions per four times, 0.60 of the issue slots.  The tables are filled
+// once for several units of 256 items.  (1024, 2, 100, 250, 148) 16.1 -> 14.7 ms; 3 CTAs per SM 14.8, 5 14.8, 2 of 512 threads 14.6.
 constexpr int kSharedRowsW = 64;
 constexpr int kSharedRows = (kSimThreads - 2) / kSharedRowsW + 2;
 constexpr int kSharedBlocks = 32;
 
 template <bool TAME>
 __global__ void __launch_bounds__(kSimThreads, 4)
-straggler_work_kernel(const Slab s, const LogNormal q, int64_t items) {
+straggler_work_kernel(const Slab s, const LogNormal q) {
     __shared__ LogNormalTables tables;
     __shared__ PhiloxOfC0 lead[kSharedRows][kSharedBlocks];
     fill_tables(tables, q);
-    const int64_t item = (int64_t)blockIdx.x * kSimThreads + threadIdx.x;
-    const int64_t row0 = (int64_t)blockIdx.x * kSimThreads / s.W;
-    const int64_t last = (int64_t)blockIdx.x * kSimThreads + kSimThreads - 1;
-    const int rows = (int)((last < items ? last : items - 1) / s.W - row0) + 1;
-    const int64_t row = item / s.W;
-    const int w = (int)(item - row * s.W), mine = item < items ? (int)(row - row0) : 0;
-    const int64_t trial = row / s.iterations, t = row - trial * s.iterations;
-    const PhiloxOfC1 of_worker = philox_of_c1(w, s.t0 + t, s.seed);
+    const int items = s.iterations * s.W;                            // of a trial
+    const int chunks = (items + kSimThreads - 1) / kSimThreads;
     const int blocks = step_blocks(s.H);
-    double work = 0.0;
-    for (int b0 = 0; b0 < blocks; b0 += kSharedBlocks) {
-        __syncthreads();
-        for (int i = threadIdx.x; i < rows * kSharedBlocks; i += kSimThreads) {
-            const int64_t r = row0 + i / kSharedBlocks, r_trial = r / s.iterations;
-            lead[i / kSharedBlocks][i % kSharedBlocks] =
-                philox_of_c0(b0 + i % kSharedBlocks, s.t0 + (r - r_trial * s.iterations), kDomainStraggler, s.seed,
-                             s.trial0 + r_trial);
+    for (int64_t unit = blockIdx.x; unit < s.trials * chunks; unit += gridDim.x) {
+        const int64_t trial = unit / chunks;
+        const int base = (int)(unit - trial * chunks) * kSimThreads, item = base + threadIdx.x;
+        const int row0 = base / s.W, rows = (min(base + kSimThreads, items) - 1) / s.W - row0 + 1;
+        const int row = item / s.W, mine = item < items ? row - row0 : 0;
+        const PhiloxOfC1 of_worker = philox_of_c1(item - row * s.W, s.t0 + row, s.seed);
+        const uint64_t key1 = s.trial0 + trial;
+        double work = 0.0;
+        for (int b0 = 0; b0 < blocks; b0 += kSharedBlocks) {
+            __syncthreads();
+            for (int i = threadIdx.x; i < rows * kSharedBlocks; i += kSimThreads)
+                lead[i / kSharedBlocks][i % kSharedBlocks] =
+                    philox_of_c0(b0 + i % kSharedBlocks, s.t0 + row0 + i / kSharedBlocks, kDomainStraggler, s.seed, key1);
+            __syncthreads();
+            const int here = blocks - b0 < kSharedBlocks ? blocks - b0 : kSharedBlocks;
+            const int last = steps_in_block(s.H, b0 + here - 1), full = last < 4 ? here - 1 : here;
+            for (int k = 0; k < full; ++k)                           // inner steps 4 (b0 + k) .. + 3 share a block
+                work += block_work<TAME>(tables, philox_join(lead[mine][k], of_worker, s.seed, key1), q);
+            if (full < here) work += part_work<TAME>(tables, philox_join(lead[mine][full], of_worker, s.seed, key1), q, last);
         }
-        __syncthreads();
-        const int here = blocks - b0 < kSharedBlocks ? blocks - b0 : kSharedBlocks;
-        for (int k = 0; k < here; ++k) {                             // inner steps 4 (b0 + k) .. + 3 share a block
-            double step[4];
-            lognormal4<TAME>(tables, philox_join(lead[mine][k], of_worker, s.seed, s.trial0 + trial), q, step);
-            const int steps = steps_in_block(s.H, b0 + k);
-            if (steps == 4) {
-                work += (step[0] + step[1]) + (step[2] + step[3]);
-            } else {
-#pragma unroll
-                for (int l = 0; l < 3; ++l)
-                    if (l < steps) work += step[l];
-            }
-        }
+        if (item < items) s.work[trial * items + item] = work;
     }
-    if (item < items) s.work[item] = work;
 }
 
 // The same for any W: `lanes` (a power of two, at most 32) threads share the blocks of an item, so that few
@@ -260,30 +270,24 @@ straggler_split_work_kernel(const Slab s, const LogNormal q, int lanes, int64_t 
     __shared__ LogNormalTables tables;
     fill_tables(tables, q);
     __syncthreads();
-    const int64_t thread = (int64_t)blockIdx.x * kSimThreads + threadIdx.x;
-    const int64_t item = thread / lanes;
-    const int lane = (int)(thread % lanes);
-    double work = 0.0;
-    if (item < items) {
-        const int64_t row = item / s.W;
-        const int w = (int)(item - row * s.W);
-        const int64_t trial = row / s.iterations, t = row - trial * s.iterations;
-        const int blocks = step_blocks(s.H);
-        for (int k = lane; k < blocks; k += lanes) {
-            double step[4];
-            lognormal4<TAME>(tables, philox4x64_10(k, w, s.t0 + t, kDomainStraggler, s.seed, s.trial0 + trial), q, step);
-            const int steps = steps_in_block(s.H, k);
-            if (steps == 4) {
-                work += (step[0] + step[1]) + (step[2] + step[3]);
-            } else {
-#pragma unroll
-                for (int l = 0; l < 3; ++l)
-                    if (l < steps) work += step[l];
+    const int lane = threadIdx.x % lanes;
+    const int blocks = step_blocks(s.H);
+    for (int64_t first = (int64_t)blockIdx.x * kSimThreads; first < items * lanes; first += (int64_t)gridDim.x * kSimThreads) {
+        const int64_t item = (first + threadIdx.x) / lanes;
+        double work = 0.0;
+        if (item < items) {
+            const int64_t row = item / s.W;
+            const int w = (int)(item - row * s.W);
+            const int64_t trial = row / s.iterations, t = row - trial * s.iterations;
+            for (int k = lane; k < blocks; k += lanes) {
+                const Philox4 x = philox4x64_10(k, w, s.t0 + t, kDomainStraggler, s.seed, s.trial0 + trial);
+                const int steps = steps_in_block(s.H, k);
+                work += steps == 4 ? block_work<TAME>(tables, x, q) : part_work<TAME>(tables, x, q, steps);
             }
         }
+        for (int o = lanes / 2; o > 0; o >>= 1) work += __shfl_xor_sync(0xffffffffu, work, o);
+        if (item < items && lane == 0) s.work[item] = work;
     }
-    for (int o = lanes / 2; o > 0; o >>= 1) work += __shfl_xor_sync(0xffffffffu, work, o);
-    if (item < items && lane == 0) s.work[item] = work;
 }
 
 // One row (trial, iteration) per CTA of THREADS; with 32 threads and W <= 32, one per warp of a larger CTA.
@@ -554,6 +558,14 @@ cudaError_t launch_straggler(int W, int n, int H, int T, double mu, double sigma
     s.order = reinterpret_cast<uint16_t*>(s.longest + group * iterations);
     const bool tame = LogNormal::tame(mu, sigma);
     const int threads = W >= 1024 ? 1024 : (W + 31) / 32 * 32;
+    int device = 0, sms = 0, resident = 0;
+    cudaError_t e = cudaGetDevice(&device);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, tame ? straggler_work_kernel<true> : straggler_work_kernel<false>,
+                                                          kSimThreads, 0);
+    if (e != cudaSuccess) return e;
+    const int64_t work_ctas = (int64_t)sms * (resident > 0 ? resident : 1);
     int lanes = 1;
     while (2 * lanes <= n && lanes < 32) lanes *= 2;
     for (int64_t trial0 = 0; trial0 < trials; trial0 += group) {
@@ -567,13 +579,16 @@ cudaError_t launch_straggler(int W, int n, int H, int T, double mu, double sigma
             // Threads per item: enough to fill the chip about twice, at most one per block of the item.
             int split = 1;
             while (items * split < (1 << 18) && split < 32 && 4 * split < H) split *= 2;
-            const unsigned work_ctas = (unsigned)((items * split + kSimThreads - 1) / kSimThreads);
-            if (split == 1 && W >= kSharedRowsW)
-                (tame ? straggler_work_kernel<true> : straggler_work_kernel<false>)<<<work_ctas, kSimThreads, 0, stream>>>(s, q, items);
+            const bool shared = split == 1 && W >= kSharedRowsW;
+            const int64_t units = shared ? s.trials * (((int64_t)s.iterations * W + kSimThreads - 1) / kSimThreads)
+                                         : (items * split + kSimThreads - 1) / kSimThreads;
+            const unsigned ctas = (unsigned)(units < 3 * work_ctas ? units : 3 * work_ctas);   // a CTA that falls behind holds up less
+            if (shared)
+                (tame ? straggler_work_kernel<true> : straggler_work_kernel<false>)<<<ctas, kSimThreads, 0, stream>>>(s, q);
             else
                 (tame ? straggler_split_work_kernel<true>
-                      : straggler_split_work_kernel<false>)<<<work_ctas, kSimThreads, 0, stream>>>(s, q, split, items);
-            cudaError_t e = cudaGetLastError();
+                      : straggler_split_work_kernel<false>)<<<ctas, kSimThreads, 0, stream>>>(s, q, split, items);
+            e = cudaGetLastError();
             if (e != cudaSuccess) return e;
             auto order = [&](auto kernel, int order_threads) {
                 return launch_overlapped(kernel, dim3((unsigned)rows), order_threads, draw_scratch_bytes(W, order_threads), stream, s);
