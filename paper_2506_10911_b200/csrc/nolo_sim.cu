@@ -29,152 +29,135 @@ constexpr uint64_t kDomainStraggler = 4;
 
 // ---- tree all-reduce ---------------------------------------------------------------------------
 //
-// A group of threads per trial: `group` = W/2 of them (one Philox block of each direction each) up to 256;
-// a CTA holds several trials at a time and strides over the trials.  The times of all edges of one
-// direction are made first, by all threads at once, into shared memory, indexed like a binary heap (root 1,
-// children of p are 2p and 2p+1, leaves W .. 2W-1; block q holds those above the nodes 4q .. 4q+3); then the
-// levels are swept, the upper ones (nodes below 128) by one warp, which alone makes and reads those nodes'
-// times: between the last wide level up and the first wide level down no barrier is needed, and the other warps
-// make the times of the way down meanwhile.  (Subtrees per warp need fewer barriers still, but more
-// instructions on part-filled warps, and measured slower.)  What Philox makes of a block's number is the same
-// for all trials, what it makes of a trial's for all blocks: both are kept (LEAD).  Bound by the log-normal times
-// and the barriers (0.505 -> 0.492 ms without those around the root, W = 1024).  Whole call, (W, trials): one CTA
-// per trial that drew the times level by level, two threads for a block -> all times first, a barrier per level ->
-// now, ms: (1024, 20 000) 2.0 -> 0.54 -> 0.49, (256, 100 000) 3.3 -> 0.79 -> 0.73, (16, 400 000) 3.8 -> 0.30 -> 0.21
-// (0.65 of the first was an allocation).
+// The edges of one direction are indexed like a binary heap (root 1, children of p are 2p and 2p + 1, leaves W .. 2W - 1);
+// Philox block q holds the times above the nodes 4q .. 4q + 3.  Either direction is the same recursion from the leaves
+// to the root: a node is ready when the later of its children's messages is there, and the last leaf has the result at
+// the time of the longest way down, which is found from below like the longest way up.  So a trial is two sums of
+// longest ways, and no time is kept for a second sweep.
+//
+// A warp takes one direction of one trial (W / 2 lanes do below 64 workers).  Above 64 workers every lane has a subtree
+// of W / 32 leaves whose blocks it visits children first, with the finished halves of what is above them on a stack
+// of its own; then every lane makes one of the 32 blocks of the nodes below 128, which the warp reduces by shuffles.
+// So all lanes work all the time and nothing waits for another warp, but for the two directions of a trial, which
+// meet every kTreeRounds trials.  What Philox makes of a block's number is the same for all trials and is kept (LEAD).
+// Bound by the log-normal times: 372 thread-instructions per four, of which 323 make them; a sweep up and one down over
+// nodes in shared memory with barriers between the levels took 464.  Whole call, (W, trials): (1024, 20 000) 0.51 -> 0.37 ms,
+// (256, 100 000) 0.77 -> 0.50, (64, 300 000) 0.70 -> 0.48 (0.3 of it the copy of the trials).
+constexpr int kTreeThreads = 512, kTreeWarps = kTreeThreads / 32, kTreeRounds = 32;
+constexpr int kLeadMaxW = 1024;      // 32 KB of shared memory
 
-constexpr int kTreeThreads = 512;
-// Trials of a CTA whose part of Philox is made at a time: a multiple of those that it has at once.
-__host__ __device__ constexpr int trials_ahead(int per_cta) { return per_cta > 32 ? per_cta : 32; }
-constexpr int kLeadMaxW = 1024;      // 32 KB of shared memory; above, one trial per CTA and no LEAD
-
-// Barrier of the threads of one trial.  Trials of more than a warp share the CTA's barrier: all trials of a CTA
-// take the same steps.  (Named barriers, one per trial, cost CTAs per SM: all 16 of a CTA are set aside.)
-__device__ __forceinline__ void sync_group(int group) {
-    if (group <= 32) __syncwarp();
-    else __syncthreads();
-}
+__device__ __forceinline__ double later(double a, double b) { return a > b ? a : b; }      // no NaN here
 
 template <bool TAME, bool LEAD>
-__global__ void __launch_bounds__(LEAD ? kTreeThreads : 256, LEAD ? 2 : 5)
-tree_allreduce_kernel(int W, int group, int64_t trials, LogNormal q, uint64_t seed, double* __restrict__ out) {
+__global__ void __launch_bounds__(kTreeThreads, 2)
+tree_allreduce_kernel(int W, int64_t trials, LogNormal q, uint64_t seed, double* __restrict__ out) {
     extern __shared__ double2 dynamic[];
     __shared__ LogNormalTables tables;
-    __shared__ double part[kTreeThreads / 32];
-    const int blocks = W / 2 > 1 ? W / 2 : 1;         // of four times each, the first two of block 0 above no node
-    const int per_cta = blockDim.x / group, mine = threadIdx.x / group, lane = threadIdx.x % group;
-    const int keep = trials_ahead(per_cta);
-    // [direction][block] a, b and c, d; [trial][direction]; then the nodes of each trial of the CTA
+    __shared__ double ways[kTreeRounds][kTreeWarps];
+    const int blocks = W / 2, lanes = W < 64 ? W / 2 : 32, leaves = W / 128;   // leaf blocks of a lane
+    // [direction][block] a, b and c, d, a level's blocks in the order in which the lanes take them; then [depth][thread]
     ulonglong2* lead_ab = reinterpret_cast<ulonglong2*>(dynamic);
     ulonglong2* lead_cd = lead_ab + (LEAD ? 2 * blocks : 0);
-    PhiloxOfC1* of_trials = reinterpret_cast<PhiloxOfC1*>(lead_cd + (LEAD ? 2 * blocks : 0));
+    double2* stack = reinterpret_cast<double2*>(lead_cd + (LEAD ? 2 * blocks : 0)) + threadIdx.x;
     fill_tables(tables, q);
     if constexpr (LEAD) {
-        for (int i = threadIdx.x; i < 2 * blocks; i += blockDim.x) {
-            const PhiloxOfC0 l = philox_of_c0(i % blocks, i / blocks, kDomainTree, seed, 0);
+        for (int i = threadIdx.x; i < 2 * blocks; i += kTreeThreads) {
+            const int direction = i / blocks, slot = i % blocks;
+            const int first = slot < 32 ? 0 : 1 << (31 - __clz(slot)), each = first / 32;
+            const int block = first == 0 ? slot : first + (slot & 31) * each + (slot - first) / 32;
+            const PhiloxOfC0 l = philox_of_c0(block, direction, kDomainTree, seed, 0);
             lead_ab[i] = make_ulonglong2(l.a, l.b);
             lead_cd[i] = make_ulonglong2(l.c, l.d);
         }
     }
     __syncthreads();
-    double* node = reinterpret_cast<double*>(of_trials + (LEAD ? 2 * keep : 0)) + (size_t)mine * 2 * W;
-    const int wide = group > 32 ? 32 : group;         // threads of the warp, or of the part of one, that a trial has
-    int turn = 0;                                     // of the CTA; its trials' part of Philox is made `keep` at a time
-    for (int64_t first_trial = (int64_t)blockIdx.x * per_cta; first_trial < trials;
-         first_trial += (int64_t)gridDim.x * per_cta, ++turn) {
-        const int64_t trial = first_trial + mine;
-        const int ahead = turn * per_cta & (keep - 1);
-        if constexpr (LEAD) {
-            if (ahead == 0) {
-                __syncthreads();
-                for (int i = threadIdx.x; i < 2 * keep; i += blockDim.x) {
-                    const int later = i / 2 / per_cta, which = i / 2 % per_cta;
-                    of_trials[i] = philox_of_c1(first_trial + (int64_t)later * gridDim.x * per_cta + which, i & 1, seed);
-                }
-                __syncthreads();
-            }
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, mine = lane % lanes;
+    // A warp's tasks of a round: one, or both directions of 16 / lanes trials next to each other in the warp (of 32 trials
+    // for W = 2, one lane each, in two rounds' worth of lanes).
+    const int64_t per_warp = 32 / lanes, workers = (int64_t)gridDim.x * kTreeWarps;
+    const int64_t rounds = (2 * trials + per_warp * workers - 1) / (per_warp * workers);
+    for (int64_t round = 0; round < rounds; ++round) {
+        int direction;
+        int64_t trial;
+        if (lanes == 32) {
+            direction = warp & 1;
+            trial = (round * (kTreeWarps / 2) + (warp >> 1)) * gridDim.x + blockIdx.x;
+        } else {
+            const int64_t task = ((round * kTreeWarps + warp) * gridDim.x + blockIdx.x) * per_warp + lane / lanes;
+            direction = (int)(task & 1);
+            trial = task >> 1;
         }
-        const bool live = trial < trials;             // the threads of other trials only keep the barriers company
-        auto draw = [&](int direction) {
-            if (!live) return;
-            PhiloxOfC1 of_trial;
-            if constexpr (LEAD) of_trial = of_trials[2 * (ahead + mine) + direction];
-            for (int b = lane; b < blocks; b += group) {
-                Philox4 x;
+        double way = 0.0;
+        if (lanes < 32 || trial < trials) {
+            const PhiloxOfC1 of_trial = philox_of_c1(trial, direction, seed);
+            auto words = [&](int block, int slot) {
                 if constexpr (LEAD) {
-                    const ulonglong2 ab = lead_ab[direction * blocks + b], cd = lead_cd[direction * blocks + b];
-                    x = philox_join({ab.x, ab.y, cd.x, cd.y}, of_trial, seed, 0);
+                    const ulonglong2 ab = lead_ab[direction * blocks + slot], cd = lead_cd[direction * blocks + slot];
+                    return philox_join({ab.x, ab.y, cd.x, cd.y}, of_trial, seed, 0);
                 } else {
-                    x = philox4x64_10(b, trial, direction, kDomainTree, seed, 0);
+                    return philox4x64_10(block, trial, direction, kDomainTree, seed, 0);
                 }
-                double t[4];
-                lognormal4<TAME>(tables, x, q, t);
-                double2* to = reinterpret_cast<double2*>(node + 4 * b);
-                to[0] = make_double2(t[0], t[1]);
-                if (4 * b + 2 < 2 * W) to[1] = make_double2(t[2], t[3]);
+            };
+            // when the two parents of the block last made are ready, seen from the leaves
+            double x0 = 0.0, x1 = 0.0;
+            int first = W / 4, turn = 0, done = 0, depth = 0;      // the level's first block, the lane's turn in it
+            double t[4];
+            for (int left = 2 * leaves - 1; left > 0; --left) {
+                const int each = first / 32;
+                lognormal4<TAME>(tables, words(first + mine * each + turn, first + turn * 32 + mine), q, t);
+                if (first == W / 4) {
+                    x0 = later(t[0], t[1]);
+                    x1 = later(t[2], t[3]);
+                } else {
+                    const double2 y = stack[--depth * kTreeThreads];
+                    const double x = later(x0 + t[2], x1 + t[3]);
+                    x0 = later(y.x + t[0], y.y + t[1]);
+                    x1 = x;
+                }
+                if (turn & 1) {                                    // both halves of the block above are there
+                    turn >>= 1;
+                    first >>= 1;
+                } else if (left > 1) {
+                    stack[depth++ * kTreeThreads] = make_double2(x0, x1);
+                    first = W / 4;
+                    turn = ++done;
+                }
             }
-        };
-        // up: node[c] = time at which c's message has reached its parent.  The parents of one level are first ..
-        // 2 * first - 1.
-        auto up = [&](int first, int threads) {
-            for (int i = lane; i < first; i += threads) {
-                const double2 c = reinterpret_cast<const double2*>(node)[first + i];
-                node[first + i] += fmax(c.x, c.y);
-            }
-        };
-        draw(0);
-        sync_group(group);
-        int first = W >> 1;
-        for (; first > 32; first >>= 1) {
-            up(first, group);
-            sync_group(group);
-        }
-        if (lane < wide) {
-            for (; first >= 2; first >>= 1) {
-                up(first, wide);
-                __syncwarp();
-            }
-        }
-        const double root = lane < wide ? fmax(node[2], node[3]) : 0.0;
-        __syncwarp();
-        // down: node[c] = time at which the result has reached c.  Children in sibling pairs, those of the
-        // parents pairs .. 2 * pairs - 1.
-        auto down = [&](int pairs, int threads) {
-            for (int i = lane; i < pairs; i += threads) {
-                double2* c = reinterpret_cast<double2*>(node) + pairs + i;
-                const double parent = node[pairs + i];
-                *c = make_double2(parent + c->x, parent + c->y);
-            }
-        };
-        draw(1);
-        __syncwarp();
-        if (lane < wide) {
-            if (lane == 0) {
-                node[2] += root;
-                node[3] += root;
+            // the nodes below 128, or all of them
+            const Philox4 x = words(mine, mine);
+            if (W > 2) lognormal2<TAME>(tables, x.w0, x.w1, q, t[0], t[1]);
+            lognormal2<TAME>(tables, x.w2, x.w3, q, t[2], t[3]);
+            __syncwarp();
+            double2* own = stack - lane;                           // of the warp, [2][32]: the times above nodes 2i and 2i + 1
+            auto pair = [&](int i) -> double2& { return own[(i & 1) * kTreeThreads + (lane - mine) + (i >> 1)]; };
+            pair(2 * mine) = make_double2(t[0], t[1]);
+            pair(2 * mine + 1) = make_double2(t[2], t[3]);
+            __syncwarp();
+            auto above = [&](int node) { return reinterpret_cast<const double*>(&pair(node >> 1))[node & 1]; };
+            const double2 leaf = pair(lanes + mine);
+            way = later(x0 + leaf.x, x1 + leaf.y);
+            for (int o = 1; o < lanes; o <<= 1) {
+                way += above((lanes + mine) / o);
+                way = later(way, __shfl_xor_sync(0xffffffffu, way, o));
             }
             __syncwarp();
-            for (int pairs = 2; pairs < W && pairs <= 32; pairs <<= 1) {
-                down(pairs, wide);
-                __syncwarp();
+        }
+        if (lanes < 32) {
+            way += __shfl_xor_sync(0xffffffffu, way, lanes);
+            if (lane % (2 * lanes) == 0 && trial < trials) out[trial] = way;
+        } else {
+            if (lane == 0) ways[round % kTreeRounds][warp] = way;
+            if (round % kTreeRounds == kTreeRounds - 1 || round == rounds - 1) {
+                __syncthreads();
+                for (int i = threadIdx.x; i < kTreeRounds * kTreeWarps / 2; i += kTreeThreads) {
+                    const int64_t r = round - round % kTreeRounds + i / (kTreeWarps / 2);
+                    const int p = i % (kTreeWarps / 2);
+                    const int64_t at = (r * (kTreeWarps / 2) + p) * gridDim.x + blockIdx.x;
+                    if (r <= round && at < trials) out[at] = ways[r % kTreeRounds][2 * p] + ways[r % kTreeRounds][2 * p + 1];
+                }
+                __syncthreads();
             }
         }
-        sync_group(group);
-        for (int pairs = 64; pairs < W; pairs <<= 1) {
-            down(pairs, group);
-            sync_group(group);
-        }
-        double m = 0.0;
-        for (int leaf = W + lane; leaf < 2 * W; leaf += group) m = fmax(m, node[leaf]);
-        for (int o = wide / 2; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-        if (group > 32) {
-            if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = m;
-            sync_group(group);
-            if (lane == 0)
-                for (int w = 1; w < group / 32; ++w) m = fmax(m, part[(threadIdx.x >> 5) + w]);
-        }
-        if (live && lane == 0) out[trial] = m;
-        sync_group(group);                      // node[] and part[] are used again
     }
 }
 
@@ -515,13 +498,10 @@ size_t tree_scratch() { return sizeof(double2) * kStatsCtas; }
 
 cudaError_t launch_tree_allreduce(int W, double mu, double sigma, int64_t trials, uint64_t seed,
                                   double* per_trial, double* stats, void* scratch, cudaStream_t stream) {
-    const int blocks = W / 2 > 1 ? W / 2 : 1;
-    const int group = blocks < 256 ? blocks : 256;
     const bool lead = W <= kLeadMaxW, tame = LogNormal::tame(mu, sigma);
-    const int threads = group <= 128 ? 256 : lead ? 512 : 256;
-    const int per_cta = threads / group;
-    const size_t smem = sizeof(double) * 2 * (size_t)W * per_cta + 
-                        (lead ? sizeof(PhiloxOfC0) * 2 * (size_t)blocks + sizeof(PhiloxOfC1) * 2 * trials_ahead(per_cta) : 0);
+    int depth = 2;                       // of a lane's stack, as much as it needs for the last exchange
+    for (int leaves = W / 128; leaves > 4; leaves /= 2) ++depth;
+    const size_t smem = sizeof(double2) * depth * kTreeThreads + (lead ? sizeof(PhiloxOfC0) * W : 0);
     auto kernel = tame ? (lead ? tree_allreduce_kernel<true, true> : tree_allreduce_kernel<true, false>)
                        : (lead ? tree_allreduce_kernel<false, true> : tree_allreduce_kernel<false, false>);
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -529,11 +509,11 @@ cudaError_t launch_tree_allreduce(int W, double mu, double sigma, int64_t trials
     int device = 0, sms = 0, resident = 0;
     e = cudaGetDevice(&device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, kernel, threads, smem);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, kernel, kTreeThreads, smem);
     if (e != cudaSuccess) return e;
-    const int64_t ctas = (trials + per_cta - 1) / per_cta, most = (int64_t)sms * (resident > 0 ? resident : 1);
-    kernel<<<(unsigned)(ctas < most ? ctas : most), threads, smem, stream>>>(W, group, trials, LogNormal::make(mu, sigma), seed,
-                                                                            per_trial);
+    const int64_t per_cta = W < 64 ? 32 / W : 1, ctas = (trials + per_cta - 1) / per_cta;     // a warp's worth each, at least
+    const int64_t most = (int64_t)sms * (resident > 0 ? resident : 1);
+    kernel<<<(unsigned)(ctas < most ? ctas : most), kTreeThreads, smem, stream>>>(W, trials, LogNormal::make(mu, sigma), seed, per_trial);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     return launch_stats<1>(per_trial, trials, stats, scratch, stream);
