@@ -104,14 +104,14 @@ cudaError_t launch_divergence(const float* phi, int W, int64_t stride, int64_t P
                               double* out2, cudaStream_t stream, int* launches);
 
 // Latency simulations (Section 4.3).  per_trial: device [trials] resp. [trials][2];
-// stats: device, the column means followed by their standard errors.
+// stats: device or mapped host memory, the column means followed by their standard errors; copy: of per_trial, in mapped host memory, or NULL.
 // scratch: device, tree_scratch() bytes.
 size_t tree_scratch();
 cudaError_t launch_tree_allreduce(int W, double mu, double sigma, int64_t trials, uint64_t seed,
-                                  double* per_trial, double* stats, void* scratch, cudaStream_t stream);
+                                  double* per_trial, double* stats, double* copy, void* scratch, cudaStream_t stream);
 // scratch: device, straggler_scratch() bytes (at most about 46 MB).
 size_t straggler_scratch(int W, int T, int64_t trials);
-cudaError_t launch_straggler(int W, int n, int H, int T, double mu, double sigma, int64_t trials,
-                             uint64_t seed, double* per_trial, double* stats, void* scratch, cudaStream_t stream);
+cudaError_t launch_straggler(int W, int n, int H, int T, double mu, double sigma, int64_t trials, uint64_t seed,
+                             double* per_trial, double* stats, double* copy, void* scratch, cudaStream_t stream);
 
 }  // namespace nolo

@@ -50,21 +50,22 @@ __device__ __forceinline__ double later(double a, double b) { return a > b ? a :
 
 template <bool TAME, bool LEAD>
 __global__ void __launch_bounds__(kTreeThreads, 2)
-tree_allreduce_kernel(int W, int64_t trials, LogNormal q, uint64_t seed, double* __restrict__ out) {
+tree_allreduce_kernel(int W, int lanes, int64_t trials, LogNormal q, uint64_t seed, double* __restrict__ out, unsigned* arrived) {
     extern __shared__ double2 dynamic[];
     __shared__ LogNormalTables tables;
     __shared__ double ways[kTreeRounds][kTreeWarps];
-    const int blocks = W / 2, lanes = W < 64 ? W / 2 : 32, leaves = W / 128;   // leaf blocks of a lane
+    const int blocks = W / 2, leaves = W / (4 * lanes);       // leaf blocks of a lane
     // [direction][block] a, b and c, d, a level's blocks in the order in which the lanes take them; then [depth][thread]
     ulonglong2* lead_ab = reinterpret_cast<ulonglong2*>(dynamic);
     ulonglong2* lead_cd = lead_ab + (LEAD ? 2 * blocks : 0);
     double2* stack = reinterpret_cast<double2*>(lead_cd + (LEAD ? 2 * blocks : 0)) + threadIdx.x;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *arrived = 0;
     fill_tables(tables, q);
     if constexpr (LEAD) {
         for (int i = threadIdx.x; i < 2 * blocks; i += kTreeThreads) {
             const int direction = i / blocks, slot = i % blocks;
-            const int first = slot < 32 ? 0 : 1 << (31 - __clz(slot)), each = first / 32;
-            const int block = first == 0 ? slot : first + (slot & 31) * each + (slot - first) / 32;
+            const int first = slot < lanes ? 0 : 1 << (31 - __clz(slot)), each = first / lanes;
+            const int block = first == 0 ? slot : first + slot % lanes * each + (slot - first) / lanes;
             const PhiloxOfC0 l = philox_of_c0(block, direction, kDomainTree, seed, 0);
             lead_ab[i] = make_ulonglong2(l.a, l.b);
             lead_cd[i] = make_ulonglong2(l.c, l.d);
@@ -72,8 +73,7 @@ tree_allreduce_kernel(int W, int64_t trials, LogNormal q, uint64_t seed, double*
     }
     __syncthreads();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, mine = lane % lanes;
-    // A warp's tasks of a round: one, or both directions of 16 / lanes trials next to each other in the warp (of 32 trials
-    // for W = 2, one lane each, in two rounds' worth of lanes).
+    // A warp's tasks of a round: one, or both directions of 16 / lanes trials next to each other.
     const int64_t per_warp = 32 / lanes, workers = (int64_t)gridDim.x * kTreeWarps;
     const int64_t rounds = (2 * trials + per_warp * workers - 1) / (per_warp * workers);
     for (int64_t round = 0; round < rounds; ++round) {
@@ -103,8 +103,8 @@ tree_allreduce_kernel(int W, int64_t trials, LogNormal q, uint64_t seed, double*
             int first = W / 4, turn = 0, done = 0, depth = 0;      // the level's first block, the lane's turn in it
             double t[4];
             for (int left = 2 * leaves - 1; left > 0; --left) {
-                const int each = first / 32;
-                lognormal4<TAME>(tables, words(first + mine * each + turn, first + turn * 32 + mine), q, t);
+                const int each = first / lanes;
+                lognormal4<TAME>(tables, words(first + mine * each + turn, first + turn * lanes + mine), q, t);
                 if (first == W / 4) {
                     x0 = later(t[0], t[1]);
                     x1 = later(t[2], t[3]);
@@ -123,7 +123,7 @@ tree_allreduce_kernel(int W, int64_t trials, LogNormal q, uint64_t seed, double*
                     turn = ++done;
                 }
             }
-            // the nodes below 128, or all of them
+            // the nodes below 4 * lanes
             const Philox4 x = words(mine, mine);
             if (W > 2) lognormal2<TAME>(tables, x.w0, x.w1, q, t[0], t[1]);
             lognormal2<TAME>(tables, x.w2, x.w3, q, t[2], t[3]);
@@ -181,6 +181,7 @@ struct Slab {
     double* longest;           // [trials][iterations]
     double* clock;             // [trials][W], from slab to slab
     double* out;               // [trials][2]: barrier and subgroup time so far
+    unsigned* arrived;         // counter of the statistics
 };
 
 // The times of one block.
@@ -216,6 +217,7 @@ template <bool TAME>
 __global__ void __launch_bounds__(kSimThreads, 4)
 straggler_work_kernel(const Slab s, const LogNormal q) {
     __shared__ LogNormalTables tables;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *s.arrived = 0;
     __shared__ PhiloxOfC0 lead[kSharedRows][kSharedBlocks];
     fill_tables(tables, q);
     const int items = s.iterations * s.W;                            // of a trial
@@ -251,6 +253,7 @@ template <bool TAME>
 __global__ void __launch_bounds__(kSimThreads, 4)
 straggler_split_work_kernel(const Slab s, const LogNormal q, int lanes, int64_t items) {
     __shared__ LogNormalTables tables;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *s.arrived = 0;
     fill_tables(tables, q);
     __syncthreads();
     const int lane = threadIdx.x % lanes;
@@ -402,6 +405,38 @@ straggler_clock_kernel(const Slab s, int lanes) {
     }
 }
 
+// One subgroup of all workers waits for the longest work of every iteration, as the barrier does: no partition and
+// no clocks, and the two times are the same.  The longest work of a row per warp, then the sum over the
+// iterations, in their order, per warp.  (512, 512, 50, 500, 83) 5.6 -> 4.2 ms, (100, 100, 100, 500, 50) 1.46 -> 0.97.
+__global__ void __launch_bounds__(kSimThreads)
+straggler_longest_kernel(const Slab s, int64_t rows) {
+    wait_for_predecessors();
+    let_successor_start();
+    const int64_t row = ((int64_t)blockIdx.x * kSimThreads + threadIdx.x) >> 5;
+    if (row >= rows) return;
+    double m = 0.0;
+    for (int w = threadIdx.x & 31; w < s.W; w += 32) m = fmax(m, s.work[row * s.W + w]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((threadIdx.x & 31) == 0) s.longest[row] = m;
+}
+
+__global__ void __launch_bounds__(kSimThreads)
+straggler_barrier_kernel(const Slab s) {
+    wait_for_predecessors();
+    let_successor_start();
+    const int64_t trial = ((int64_t)blockIdx.x * kSimThreads + threadIdx.x) >> 5;
+    if (trial >= s.trials) return;
+    const int lane = threadIdx.x & 31;
+    double barrier = s.t0 ? s.out[2 * trial] : 0.0;
+    for (int i0 = 0; i0 < s.iterations; i0 += 32) {
+        const double longest = i0 + lane < s.iterations ? s.longest[trial * s.iterations + i0 + lane] : 0.0;
+#pragma unroll
+        for (int k = 0; k < 32; ++k) barrier += __shfl_sync(0xffffffffu, longest, k);
+    }
+    if (lane < 2) s.out[2 * trial + lane] = barrier;
+}
+
 // ---- means and standard errors ------------------------------------------------------------------------
 
 constexpr int kStatsThreads = 512, kStatsCtas = 64;
@@ -419,120 +454,151 @@ __device__ __forceinline__ double cta_sum(double v) {          // in a fixed ord
     return v;
 }
 
-// Sum, and sum of squared deviations from the mean, of each column of rows [r0, r1) of x[][COLS], one slice of
-// the rows per CTA; the slices are put together by the next kernel.  stats[cta][column] = {sum, deviations}.
+// Means of the columns of x[rows][COLS] to out[c], the standard error of each, sqrt(sample variance / rows), to
+// out[COLS + c]; x itself to `copy`, unless that is NULL.  out and copy may be page-locked host memory.  One slice of the rows
+// per CTA gives its sum and the squared deviations from its mean, which the last CTA to be done puts together in
+// a fixed order.  `arrived` counts them, from zero.  One kernel whose results are there when it ends, instead of two kernels
+// and two copies through the driver's buffer: tree of (64, 2000) 46 -> 27 us a call, (2, 45 226) 71 -> 43.
 template <int COLS>
 __global__ void __launch_bounds__(kStatsThreads)
-column_moments_kernel(const double* x, int64_t rows, double2* __restrict__ moments) {
+trial_stats_kernel(const double* x, int64_t rows, double2* moments, unsigned* arrived, double* out, double* copy) {
+    static_assert(COLS == 1 || COLS == 2, "a row is one access");
     wait_for_predecessors();
     let_successor_start();
     const int64_t r0 = rows * blockIdx.x / gridDim.x, r1 = rows * (blockIdx.x + 1) / gridDim.x;
     double sum[COLS] = {}, dev[COLS] = {};
-#pragma unroll 4
-    for (int64_t i = r0 + threadIdx.x; i < r1; i += kStatsThreads)
-        for (int c = 0; c < COLS; ++c) sum[c] += x[i * COLS + c];
+#pragma unroll 8
+    for (int64_t i = r0 + threadIdx.x; i < r1; i += kStatsThreads) {
+        if constexpr (COLS == 1) {
+            const double v = x[i];
+            if (copy) copy[i] = v;
+            sum[0] += v;
+        } else {
+            const double2 v = reinterpret_cast<const double2*>(x)[i];
+            if (copy) reinterpret_cast<double2*>(copy)[i] = v;
+            sum[0] += v.x;
+            sum[1] += v.y;
+        }
+    }
 #pragma unroll
     for (int c = 0; c < COLS; ++c) sum[c] = cta_sum(sum[c]);
-#pragma unroll 4
+#pragma unroll 8
     for (int64_t i = r0 + threadIdx.x; i < r1; i += kStatsThreads) {
+#pragma unroll
         for (int c = 0; c < COLS; ++c) {
             const double d = x[i * COLS + c] - sum[c] / (double)(r1 - r0);
             dev[c] += d * d;
         }
     }
+    __shared__ bool last;
 #pragma unroll
     for (int c = 0; c < COLS; ++c) {
         dev[c] = cta_sum(dev[c]);
         if (threadIdx.x == 0) moments[blockIdx.x * COLS + c] = make_double2(sum[c], dev[c]);
     }
-}
-
-// Column means to out[c]; the standard error of each mean, sqrt(sample variance / rows), to out[COLS + c].
-template <int COLS>
-__global__ void __launch_bounds__(32)
-column_stats_kernel(const double2* moments, int slices, int64_t rows, double* __restrict__ out) {
-    wait_for_predecessors();
-    let_successor_start();
-    const int c = threadIdx.x;
-    if (c >= COLS) return;
-    double total = 0.0;
-    for (int k = 0; k < slices; ++k) total += moments[k * COLS + c].x;
-    const double mean = total / (double)rows;
-    double dev = 0.0;
-    for (int k = 0; k < slices; ++k) {
-        const double n = (double)(rows * (k + 1) / slices - rows * k / slices), d = moments[k * COLS + c].x / n - mean;
-        dev += moments[k * COLS + c].y + n * d * d;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(arrived, 1u) == gridDim.x - 1;
     }
-    out[c] = mean;
-    out[COLS + c] = rows > 1 ? sqrt(dev / (double)(rows - 1) / (double)rows) : 0.0;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    const int k = threadIdx.x, slices = gridDim.x;
+    const double n = (double)(rows * (k + 1) / slices - rows * k / slices);
+#pragma unroll
+    for (int c = 0; c < COLS; ++c) {
+        const double2 m = k < slices ? __ldcg(moments + k * COLS + c) : make_double2(0.0, 0.0);
+        const double mean = cta_sum(m.x) / (double)rows;
+        const double d = k < slices ? m.x / n - mean : 0.0;
+        const double total = cta_sum(k < slices ? m.y + n * d * d : 0.0);
+        if (threadIdx.x == 0) {
+            out[c] = mean;
+            out[COLS + c] = rows > 1 ? sqrt(total / (double)(rows - 1) / (double)rows) : 0.0;
+        }
+    }
 }
 
+constexpr size_t kStatsScratch = sizeof(double2) * (2 * kStatsCtas + 1);      // moments, then the counter
+
+unsigned* stats_counter(void* scratch) { return reinterpret_cast<unsigned*>(static_cast<double2*>(scratch) + 2 * kStatsCtas); }
+
 template <int COLS>
-cudaError_t launch_stats(const double* x, int64_t rows, double* out, void* scratch, cudaStream_t stream) {
+cudaError_t launch_stats(const double* x, int64_t rows, double* out, double* copy, void* scratch, cudaStream_t stream) {
     const int64_t wanted = rows / 4096;
     const int slices = (int)(wanted < 1 ? 1 : wanted > kStatsCtas ? kStatsCtas : wanted);
-    double2* moments = static_cast<double2*>(scratch);
-    const cudaError_t e = launch_overlapped(column_moments_kernel<COLS>, dim3((unsigned)slices), kStatsThreads, 0, stream, x,
-                                            rows, moments);
-    if (e != cudaSuccess) return e;
-    return launch_overlapped(column_stats_kernel<COLS>, dim3(1), 32, 0, stream, static_cast<const double2*>(moments), slices, rows,
-                             out);
+    return launch_overlapped(trial_stats_kernel<COLS>, dim3((unsigned)slices), kStatsThreads, 0, stream, x, rows,
+                             static_cast<double2*>(scratch), stats_counter(scratch), out, copy);
 }
 
 // Iterations and trials whose work sums are held at a time.
 constexpr int64_t kSlabItems = 1 << 21;
 
-int64_t slab_trials(int W, int64_t trials) {
-    const int64_t most = kSlabItems / W;
-    return trials < most ? trials : most;
+// As few slabs as that allows, of equal sizes.
+int64_t even_share(int64_t all, int64_t most) {
+    const int64_t parts = (all + most - 1) / most;
+    return (all + parts - 1) / parts;
 }
 
+int64_t slab_trials(int W, int64_t trials) { return even_share(trials, kSlabItems / W); }
+
 int64_t slab_iterations(int W, int T, int64_t trials) {
-    const int64_t most = kSlabItems / (W * slab_trials(W, trials));
-    return T < most ? T : most;
+    return even_share(T, kSlabItems / (W * slab_trials(W, trials)));
 }
 
 }  // namespace
 
-size_t tree_scratch() { return sizeof(double2) * kStatsCtas; }
+size_t tree_scratch() { return kStatsScratch; }
 
 cudaError_t launch_tree_allreduce(int W, double mu, double sigma, int64_t trials, uint64_t seed,
-                                  double* per_trial, double* stats, void* scratch, cudaStream_t stream) {
+                                  double* per_trial, double* stats, double* copy, void* scratch, cudaStream_t stream) {
     const bool lead = W <= kLeadMaxW, tame = LogNormal::tame(mu, sigma);
+    // Lanes per direction of a trial.  What several do together costs about 0.14 of a block for each of their log2(lanes)
+    // exchanges, few lanes per trial leave the last turn of the chip's warps emptier.
+    int device = 0, sms = 0, resident = 0, lanes = 1;
+    cudaError_t e = cudaGetDevice(&device);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+    if (e != cudaSuccess) return e;
+    double least = 0.0;
+    for (int l = 1, log2 = 0; l <= W / 2 && l <= 32; l *= 2, ++log2) {
+        const int64_t threads = (int64_t)sms * 2 * kTreeThreads;
+        const double cost = (double)((2 * trials * l + threads - 1) / threads) * (W / (2 * l) + 0.14 * log2);
+        if (l == 1 || cost <= least) {
+            least = cost;
+            lanes = l;
+        }
+    }
     int depth = 2;                       // of a lane's stack, as much as it needs for the last exchange
-    for (int leaves = W / 128; leaves > 4; leaves /= 2) ++depth;
+    for (int leaves = W / (4 * lanes); leaves > 4; leaves /= 2) ++depth;
     const size_t smem = sizeof(double2) * depth * kTreeThreads + (lead ? sizeof(PhiloxOfC0) * W : 0);
     auto kernel = tame ? (lead ? tree_allreduce_kernel<true, true> : tree_allreduce_kernel<true, false>)
                        : (lead ? tree_allreduce_kernel<false, true> : tree_allreduce_kernel<false, false>);
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    int device = 0, sms = 0, resident = 0;
-    e = cudaGetDevice(&device);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, kernel, kTreeThreads, smem);
     if (e != cudaSuccess) return e;
-    const int64_t per_cta = W < 64 ? 32 / W : 1, ctas = (trials + per_cta - 1) / per_cta;     // a warp's worth each, at least
+    const int64_t per_warp = lanes < 32 ? 16 / lanes : 1, ctas = (trials + per_warp - 1) / per_warp;
     const int64_t most = (int64_t)sms * (resident > 0 ? resident : 1);
-    kernel<<<(unsigned)(ctas < most ? ctas : most), kTreeThreads, smem, stream>>>(W, trials, LogNormal::make(mu, sigma), seed, per_trial);
+    kernel<<<(unsigned)(ctas < most ? ctas : most), kTreeThreads, smem, stream>>>(W, lanes, trials, LogNormal::make(mu, sigma), seed,
+                                                                                 per_trial, stats_counter(scratch));
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    return launch_stats<1>(per_trial, trials, stats, scratch, stream);
+    return launch_stats<1>(per_trial, trials, stats, copy, scratch, stream);
 }
 
 size_t straggler_scratch(int W, int T, int64_t trials) {
     const size_t rows = (size_t)slab_trials(W, trials) * slab_iterations(W, T, trials);
     return rows * W * (sizeof(double) + sizeof(uint16_t)) + rows * sizeof(double) +
-           (size_t)slab_trials(W, trials) * W * sizeof(double) + sizeof(double2) * 2 * kStatsCtas;
+           (size_t)slab_trials(W, trials) * W * sizeof(double) + kStatsScratch;
 }
 
 cudaError_t launch_straggler(int W, int n, int H, int T, double mu, double sigma, int64_t trials, uint64_t seed,
-                             double* per_trial, double* stats, void* scratch, cudaStream_t stream) {
+                             double* per_trial, double* stats, double* copy, void* scratch, cudaStream_t stream) {
     const int64_t group = slab_trials(W, trials), iterations = slab_iterations(W, T, trials);
     Slab s;
     s.W = W; s.n = n; s.H = H;
     const LogNormal q = LogNormal::make(mu, sigma);
     s.seed = seed;
-    s.work = static_cast<double*>(scratch);
+    s.arrived = stats_counter(scratch);
+    s.work = static_cast<double*>(scratch) + kStatsScratch / sizeof(double);
     s.clock = s.work + group * iterations * W;
     s.longest = s.clock + group * W;
     s.order = reinterpret_cast<uint16_t*>(s.longest + group * iterations);
@@ -570,6 +636,16 @@ cudaError_t launch_straggler(int W, int n, int H, int T, double mu, double sigma
                       : straggler_split_work_kernel<false>)<<<ctas, kSimThreads, 0, stream>>>(s, q, split, items);
             e = cudaGetLastError();
             if (e != cudaSuccess) return e;
+            if (n == W) {
+                auto warps = [&](auto kernel, int64_t count, auto... args) {
+                    return launch_overlapped(kernel, dim3((unsigned)((count * 32 + kSimThreads - 1) / kSimThreads)), kSimThreads, 0,
+                                             stream, args...);
+                };
+                e = warps(straggler_longest_kernel, rows, s, rows);
+                if (e == cudaSuccess) e = warps(straggler_barrier_kernel, s.trials, s);
+                if (e != cudaSuccess) return e;
+                continue;
+            }
             auto order = [&](auto kernel, int order_threads) {
                 return launch_overlapped(kernel, dim3((unsigned)rows), order_threads, draw_scratch_bytes(W, order_threads), stream, s);
             };
@@ -589,7 +665,7 @@ cudaError_t launch_straggler(int W, int n, int H, int T, double mu, double sigma
             if (e != cudaSuccess) return e;
         }
     }
-    return launch_stats<2>(per_trial, trials, stats, scratch, stream);      // the slabs are done with it
+    return launch_stats<2>(per_trial, trials, stats, copy, scratch, stream);
 }
 
 }  // namespace nolo
