@@ -177,7 +177,7 @@ struct Slab {
     int64_t t0, trial0, trials;
     uint64_t seed;
     double* work;              // [trials][iterations][W]
-    uint16_t* order;           // [trials][iterations][W]: the worker in each position of the partition
+    uint32_t* rank;            // [trials][iterations][W]: each worker's position in the partition
     double* longest;           // [trials][iterations]
     double* clock;             // [trials][W], from slab to slab
     double* out;               // [trials][2]: barrier and subgroup time so far
@@ -233,11 +233,12 @@ straggler_work_kernel(const Slab s, const LogNormal q) {
         double work = 0.0;
         for (int b0 = 0; b0 < blocks; b0 += kSharedBlocks) {
             __syncthreads();
-            for (int i = threadIdx.x; i < rows * kSharedBlocks; i += kSimThreads)
-                lead[i / kSharedBlocks][i % kSharedBlocks] =
-                    philox_of_c0(b0 + i % kSharedBlocks, s.t0 + row0 + i / kSharedBlocks, kDomainStraggler, s.seed, key1);
-            __syncthreads();
             const int here = blocks - b0 < kSharedBlocks ? blocks - b0 : kSharedBlocks;
+            for (int i = threadIdx.x; i < rows * here; i += kSimThreads) {
+                const int r = i / here, k = i - r * here;
+                lead[r][k] = philox_of_c0(b0 + k, s.t0 + row0 + r, kDomainStraggler, s.seed, key1);
+            }
+            __syncthreads();
             const int last = steps_in_block(s.H, b0 + here - 1), full = last < 4 ? here - 1 : here;
             for (int k = 0; k < full; ++k)                           // inner steps 4 (b0 + k) .. + 3 share a block
                 work += block_work<TAME>(tables, philox_join(lead[mine][k], of_worker, s.seed, key1), q);
@@ -276,7 +277,7 @@ straggler_split_work_kernel(const Slab s, const LogNormal q, int lanes, int64_t 
     }
 }
 
-// One row (trial, iteration) per CTA of THREADS; with 32 threads and W <= 32, one per warp of a larger CTA.
+// One row (trial, iteration) per CTA of THREADS; up to 32 workers, 32 / width rows per warp.
 template <int THREADS>
 __global__ void __launch_bounds__(THREADS)
 straggler_order_kernel(const Slab s) {
@@ -295,7 +296,7 @@ straggler_order_kernel(const Slab s) {
     for (int k = 0; k < kDrawPerThread; ++k) {
         const int w = threadIdx.x + k * THREADS;
         if (w < s.W) {
-            s.order[row * s.W + rank[k]] = (uint16_t)w;
+            s.rank[row * s.W + w] = (uint32_t)rank[k];
             m = fmax(m, s.work[row * s.W + w]);
         }
     }
@@ -310,98 +311,147 @@ straggler_order_kernel(const Slab s) {
 }
 
 __global__ void __launch_bounds__(kSimThreads)
-straggler_order_warp_kernel(const Slab s, int64_t rows) {
-    const int64_t row = ((int64_t)blockIdx.x * kSimThreads + threadIdx.x) >> 5;
+straggler_order_warp_kernel(const Slab s, int64_t rows, int width) {
+    const int lane = threadIdx.x & (width - 1);
+    const int64_t row = ((int64_t)blockIdx.x * kSimThreads + threadIdx.x) / width;
+    const int64_t trial = row / s.iterations, t = row - trial * s.iterations;
+    const uint64_t key = draw_key(lane, s.trial0 + trial, 0, kDomainGroups, s.seed, s.t0 + t);
+    int rank = 0;
+    for (int j = 0; j < s.W; ++j) {
+        const uint64_t other = __shfl_sync(0xffffffffu, key, j, width);
+        rank += other < key || (other == key && j < lane);
+    }
     wait_for_predecessors();
     let_successor_start();
-    if (row >= rows) return;
-    const int lane = threadIdx.x & 31;
-    const int64_t trial = row / s.iterations, t = row - trial * s.iterations;
-    const int rank = rank_by_warp(s.W, s.trial0 + trial, 0, kDomainGroups, s.seed, s.t0 + t);
-    double m = 0.0;
-    if (lane < s.W) {
-        s.order[row * s.W + rank] = (uint16_t)lane;
-        m = s.work[row * s.W + lane];
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if (lane == 0) s.longest[row] = m;
+    const bool mine = row < rows && lane < s.W;
+    double m = mine ? s.work[row * s.W + lane] : 0.0;
+    if (mine) s.rank[row * s.W + lane] = (uint32_t)rank;
+    for (int o = width / 2; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (row < rows && lane == 0) s.longest[row] = m;
 }
 
-// The clocks of one trial per CTA.  `lanes` (a power of two, at most 32 and n) threads share a subgroup.  The
-// work and the partition of an iteration are read AHEAD iterations ahead: an iteration is two short exchanges
-// through shared memory, a read from L2 several times that.
-template <int MOST, int AHEAD>
+// The sum of the longest work of a trial's iterations, in their order, added to `sum`; by one warp.
+__device__ __forceinline__ double barrier_time(const Slab& s, int64_t trial, double sum) {
+    const int lane = threadIdx.x & 31;
+    for (int i0 = 0; i0 < s.iterations; i0 += 32) {
+        const double longest = i0 + lane < s.iterations ? s.longest[trial * s.iterations + i0 + lane] : 0.0;
+#pragma unroll
+        for (int k = 0; k < 32; ++k) sum += __shfl_sync(0xffffffffu, longest, k);
+    }
+    return sum;
+}
+
+// The clocks of one trial per CTA, each in a register of its worker's thread; the members of a subgroup meet in
+// shared memory, in the order of the partition.  Bound by the latency of that exchange, iteration after iteration, so
+// the work and the ranks are copied to shared memory AHEAD iterations ahead, each by the thread that will use it (loads into
+// registers are waited for by six counters, whoever shares one waits for the latest: no more than four iterations ahead).
+// PAIRS: each of the two looks at the other, one barrier per iteration, two buffers.  Else `lanes` (a power of two, at most 32)
+// threads share a subgroup (members who look at all the others hit the same banks: 2.9 us per iteration at n = 8, W = 1024).
+// In a kernel of 500 iterations: 246 -> 60 us with pairs of 16 workers.
+template <int BYTES>
+__device__ __forceinline__ void copy_ahead(void* to, const void* from) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((unsigned)__cvta_generic_to_shared(to)), "l"(from), "n"(BYTES)
+                 : "memory");
+}
+
+__host__ __device__ constexpr size_t clock_bytes(int W, int groups, int ahead, bool pairs) {
+    return (size_t)W * ahead * (sizeof(double) + sizeof(uint32_t)) + (pairs ? 2 * W : W + groups) * sizeof(double);
+}
+
+template <int MOST, int AHEAD, bool PAIRS>
 __global__ void __launch_bounds__(1024)
-straggler_clock_kernel(const Slab s, int lanes) {
-    extern __shared__ uint64_t raw[];
-    double* clock = reinterpret_cast<double*>(raw);           // [W] when each worker is done with its work
-    uint16_t* order = reinterpret_cast<uint16_t*>(clock + s.W);   // [W]
+straggler_clock_kernel(const Slab s, int lanes, unsigned inverse_n) {
+    extern __shared__ double shared[];
     const int64_t trial = blockIdx.x;
-    const int lane = threadIdx.x % lanes, groups = s.W / s.n;
-    let_successor_start();
-    for (int w = threadIdx.x; w < s.W; w += blockDim.x) clock[w] = s.t0 ? s.clock[trial * s.W + w] : 0.0;
-    double barrier = s.t0 ? s.out[2 * trial] : 0.0;
-    double work[AHEAD][MOST], longest[AHEAD];
-    uint16_t position[AHEAD][MOST];
-    auto read = [&](int slot, int i) {
-        if (i >= s.iterations) return;
-        const int64_t row = trial * s.iterations + i;
+    const int lane = threadIdx.x % lanes, turn = threadIdx.x / lanes, per_turn = blockDim.x / lanes, groups = s.W / s.n;
+    double* buffer = shared;                                  // [W], twice for PAIRS
+    double* longest_of = shared + s.W;                        // [groups], unless PAIRS
+    double* works = shared + (PAIRS ? 2 * s.W : s.W + groups);  // [AHEAD][W]
+    uint32_t* ranks = reinterpret_cast<uint32_t*>(works + AHEAD * s.W);      // [AHEAD][W]
+    const double* next_work = s.work + trial * s.iterations * s.W + threadIdx.x;
+    const uint32_t* next_rank = s.rank + trial * s.iterations * s.W + threadIdx.x;
+    double clock[MOST];
+    bool mine[MOST];
 #pragma unroll
-        for (int k = 0; k < MOST; ++k) {
-            const int w = threadIdx.x + k * blockDim.x;
-            if (w < s.W) {
-                work[slot][k] = s.work[row * s.W + w];
-                position[slot][k] = s.order[row * s.W + w];
-            }
-        }
-        longest[slot] = s.longest[row];
-    };
-#pragma unroll
-    for (int u = 0; u < AHEAD; ++u) read(u, u);
-    __syncthreads();
-    for (int i0 = 0; i0 < s.iterations; i0 += AHEAD) {
-#pragma unroll
-        for (int u = 0; u < AHEAD; ++u) {
-            if (i0 + u >= s.iterations) break;
+    for (int k = 0; k < MOST; ++k) {
+        const int w = threadIdx.x + k * blockDim.x;
+        mine[k] = w < s.W;
+        clock[k] = s.t0 && mine[k] ? s.clock[trial * s.W + w] : 0.0;
+    }
+    auto ahead = [&](int slot, int i) {
+        if (i < s.iterations) {
 #pragma unroll
             for (int k = 0; k < MOST; ++k) {
                 const int w = threadIdx.x + k * blockDim.x;
-                if (w < s.W) {
-                    clock[w] += work[u][k];
-                    order[w] = position[u][k];
+                if (mine[k]) {
+                    copy_ahead<8>(works + slot * s.W + w, next_work + k * blockDim.x);
+                    copy_ahead<4>(ranks + slot * s.W + w, next_rank + k * blockDim.x);
                 }
             }
-            barrier += longest[u];
-            read(u, i0 + u + AHEAD);
-            __syncthreads();
-            for (int g0 = 0; g0 < groups; g0 += blockDim.x / lanes) {     // every lane of a subgroup takes the same turns
-                const int g = g0 + threadIdx.x / lanes;
-                const uint16_t* member = order + (g < groups ? g : 0) * s.n;
+            next_work += s.W;
+            next_rank += s.W;
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    for (int u = 0; u < AHEAD; ++u) ahead(u, u);
+    int slot = 0;
+    for (int i = 0; i < s.iterations; ++i) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(AHEAD - 1) : "memory");
+        int at[MOST];
+#pragma unroll
+        for (int k = 0; k < MOST; ++k) {
+            if (mine[k]) {
+                const int w = threadIdx.x + k * blockDim.x;
+                at[k] = (int)ranks[slot * s.W + w];
+                clock[k] += works[slot * s.W + w];
+                buffer[at[k]] = clock[k];
+                if (!PAIRS && inverse_n) at[k] = (int)__umulhi((unsigned)at[k], inverse_n);     // the subgroup
+            }
+        }
+        ahead(slot, i + AHEAD);
+        slot = slot + 1 == AHEAD ? 0 : slot + 1;
+        __syncthreads();
+        if constexpr (PAIRS) {
+#pragma unroll
+            for (int k = 0; k < MOST; ++k)
+                if (mine[k]) clock[k] = later(clock[k], buffer[at[k] ^ 1]);
+            buffer = buffer == shared ? shared + s.W : shared;
+        } else {
+            for (int g0 = 0; g0 < groups; g0 += per_turn) {               // every lane of a subgroup takes the same turns
+                const int g = g0 + turn;
                 double m = 0.0;
                 if (g < groups)
-                    for (int j = lane; j < s.n; j += lanes) m = fmax(m, clock[member[j]]);
-                for (int o = lanes / 2; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-                if (g < groups)
-                    for (int j = lane; j < s.n; j += lanes) clock[member[j]] = m;
+                    for (int j = lane; j < s.n; j += lanes) m = later(m, buffer[g * s.n + j]);
+                for (int o = lanes / 2; o > 0; o >>= 1) m = later(m, __shfl_xor_sync(0xffffffffu, m, o));
+                if (g < groups && lane == 0) longest_of[g] = m;
             }
             __syncthreads();
+#pragma unroll
+            for (int k = 0; k < MOST; ++k)
+                if (mine[k]) clock[k] = longest_of[at[k]];
         }
     }
     double m = 0.0;
-    for (int w = threadIdx.x; w < s.W; w += blockDim.x) {
-        m = fmax(m, clock[w]);
-        s.clock[trial * s.W + w] = clock[w];
+#pragma unroll
+    for (int k = 0; k < MOST; ++k) {
+        const int w = threadIdx.x + k * blockDim.x;
+        if (w < s.W) {
+            m = fmax(m, clock[k]);
+            s.clock[trial * s.W + w] = clock[k];
+        }
     }
     __shared__ double part[32];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
     if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = m;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < (int)blockDim.x / 32; ++w) m = fmax(m, part[w]);
-        s.out[2 * trial] = barrier;
-        s.out[2 * trial + 1] = m;
+    if (threadIdx.x < 32) {
+        const double barrier = barrier_time(s, trial, s.t0 ? s.out[2 * trial] : 0.0);
+        if (threadIdx.x == 0) {
+            for (int w = 1; w < (int)blockDim.x / 32; ++w) m = fmax(m, part[w]);
+            s.out[2 * trial] = barrier;
+            s.out[2 * trial + 1] = m;
+        }
     }
 }
 
@@ -427,14 +477,8 @@ straggler_barrier_kernel(const Slab s) {
     let_successor_start();
     const int64_t trial = ((int64_t)blockIdx.x * kSimThreads + threadIdx.x) >> 5;
     if (trial >= s.trials) return;
-    const int lane = threadIdx.x & 31;
-    double barrier = s.t0 ? s.out[2 * trial] : 0.0;
-    for (int i0 = 0; i0 < s.iterations; i0 += 32) {
-        const double longest = i0 + lane < s.iterations ? s.longest[trial * s.iterations + i0 + lane] : 0.0;
-#pragma unroll
-        for (int k = 0; k < 32; ++k) barrier += __shfl_sync(0xffffffffu, longest, k);
-    }
-    if (lane < 2) s.out[2 * trial + lane] = barrier;
+    const double barrier = barrier_time(s, trial, s.t0 ? s.out[2 * trial] : 0.0);
+    if ((threadIdx.x & 31) < 2) s.out[2 * trial + (threadIdx.x & 31)] = barrier;
 }
 
 // ---- means and standard errors ------------------------------------------------------------------------
@@ -494,8 +538,16 @@ trial_stats_kernel(const double* x, int64_t rows, double2* moments, unsigned* ar
 #pragma unroll
     for (int c = 0; c < COLS; ++c) {
         dev[c] = cta_sum(dev[c]);
+        if (gridDim.x == 1) {
+            if (threadIdx.x == 0) {
+                out[c] = sum[c] / (double)rows;
+                out[COLS + c] = rows > 1 ? sqrt(dev[c] / (double)(rows - 1) / (double)rows) : 0.0;
+            }
+            continue;
+        }
         if (threadIdx.x == 0) moments[blockIdx.x * COLS + c] = make_double2(sum[c], dev[c]);
     }
+    if (gridDim.x == 1) return;
     if (threadIdx.x == 0) {
         __threadfence();
         last = atomicAdd(arrived, 1u) == gridDim.x - 1;
@@ -531,7 +583,7 @@ cudaError_t launch_stats(const double* x, int64_t rows, double* out, double* cop
 }
 
 // Iterations and trials whose work sums are held at a time.
-constexpr int64_t kSlabItems = 1 << 21;
+constexpr int64_t kSlabItems = 31 << 16;
 
 // As few slabs as that allows, of equal sizes.
 int64_t even_share(int64_t all, int64_t most) {
@@ -586,7 +638,7 @@ cudaError_t launch_tree_allreduce(int W, double mu, double sigma, int64_t trials
 
 size_t straggler_scratch(int W, int T, int64_t trials) {
     const size_t rows = (size_t)slab_trials(W, trials) * slab_iterations(W, T, trials);
-    return rows * W * (sizeof(double) + sizeof(uint16_t)) + rows * sizeof(double) +
+    return rows * W * (sizeof(double) + sizeof(uint32_t)) + rows * sizeof(double) +
            (size_t)slab_trials(W, trials) * W * sizeof(double) + kStatsScratch;
 }
 
@@ -601,7 +653,7 @@ cudaError_t launch_straggler(int W, int n, int H, int T, double mu, double sigma
     s.work = static_cast<double*>(scratch) + kStatsScratch / sizeof(double);
     s.clock = s.work + group * iterations * W;
     s.longest = s.clock + group * W;
-    s.order = reinterpret_cast<uint16_t*>(s.longest + group * iterations);
+    s.rank = reinterpret_cast<uint32_t*>(s.longest + group * iterations);
     const bool tame = LogNormal::tame(mu, sigma);
     const int threads = W >= 1024 ? 1024 : (W + 31) / 32 * 32;
     int device = 0, sms = 0, resident = 0;
@@ -649,8 +701,11 @@ cudaError_t launch_straggler(int W, int n, int H, int T, double mu, double sigma
             auto order = [&](auto kernel, int order_threads) {
                 return launch_overlapped(kernel, dim3((unsigned)rows), order_threads, draw_scratch_bytes(W, order_threads), stream, s);
             };
-            e = W <= 32 ? launch_overlapped(straggler_order_warp_kernel, dim3((unsigned)((rows * 32 + kSimThreads - 1) / kSimThreads)),
-                                            kSimThreads, 0, stream, s, rows)
+            int width = 4;
+            while (width < W) width *= 2;
+            e = W <= 32 ? launch_overlapped(straggler_order_warp_kernel,
+                                            dim3((unsigned)((rows * width + kSimThreads - 1) / kSimThreads)), kSimThreads, 0,
+                                            stream, s, rows, width)
               : W <= 512  ? order(straggler_order_kernel<128>, 128)
               : W <= 1024 ? order(straggler_order_kernel<256>, 256)
               : W <= 2048 ? order(straggler_order_kernel<512>, 512)
@@ -658,10 +713,16 @@ cudaError_t launch_straggler(int W, int n, int H, int T, double mu, double sigma
             if (e != cudaSuccess) return e;
             // Not ahead of the order kernel's end: CTAs that come in as it leaves crowd on the first free SMs, and these
             // run for long (1.03 -> 1.16 ms in all for (4, 2, 100, 500, 592)).
-            auto clock = [&](auto kernel) { kernel<<<(unsigned)s.trials, threads, (size_t)W * 10, stream>>>(s, lanes); };
-            if (W <= 1024) clock(straggler_clock_kernel<1, 4>);
-            else clock(straggler_clock_kernel<NOLO_MAX_WORKERS / 1024, 1>);
-            e = cudaGetLastError();
+            auto clock = [&](auto kernel, int ahead, bool pairs) {
+                const size_t bytes = clock_bytes(W, W / n, ahead, pairs);
+                cudaError_t set = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+                if (set != cudaSuccess) return set;
+                kernel<<<(unsigned)s.trials, threads, bytes, stream>>>(s, lanes, n > 1 ? 0xffffffffu / n + 1 : 0u);
+                return cudaGetLastError();
+            };
+            e = W > 1024 ? clock(straggler_clock_kernel<NOLO_MAX_WORKERS / 1024, 2, false>, 2, false)
+              : n == 2   ? clock(straggler_clock_kernel<1, 4, true>, 4, true)
+                         : clock(straggler_clock_kernel<1, 4, false>, 4, false);
             if (e != cudaSuccess) return e;
         }
     }
