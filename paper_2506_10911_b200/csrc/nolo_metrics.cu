@@ -187,19 +187,23 @@ struct Shape {
 };
 
 // Four quads per thread and a second kernel for the sums where that leaves enough CTAs, else one quad and one
-// kernel, in as many parts as give the chip about four CTAs per SM while every part keeps a worker.  Enough are eight per
+// kernel, in parts while there are few CTAs and every part keeps a worker.  Enough are eight per
 // SM, so that the last, part-filled wave of four weighs little ((128, 3e6) 247 us with one quad, 301 with four, which
 // are 1.2 waves); with few workers a CTA is soon done and their number weighs more, the one counter that they all
 // add to included: three per SM ((1, 2^22) 45 us with one quad, 29 with four, (12, 3e6) 57 / 53, (16, 3e6) 58 / 62).
-// Few columns in parts: (1024, 1000) 331 us unparted, 21 now.  Four quads want four CTAs of 64 registers per SM: at 66
-// registers, three CTAs, (16, 2^26) measured 675 us instead of 622.
-constexpr int64_t kManyCtas = 148 * 8, kManyShortCtas = 148 * 3, kFewCtas = 148 * 4;
+// Few are less than one per SM, or two where a part has 64 workers and more to walk; the counter makes more of them
+// dearer again.  us, with four per SM for few / now: (16, 100 000) 26.2 / 17.1, (64, 100 000) 29.7 / 21.0, (32, 50 000) 21.7 / 17.0,
+// (64, 390 625) 38.2 / 31.0, (1024, 390 625) 270 / 250, (1024, 24 414) 43.3 / 36.5; unparted (1024, 1000) 331, now 21.
+// Four quads want four CTAs of 64 registers per SM: at 66
+// registers, three CTAs, (16, 2^26) measured 675 us instead of 622.  (Sums of each thread in float32 pairs instead of float64,
+// to save its conversions, measured slower: (2, 2e8) 330 -> 360.)
+constexpr int64_t kManyCtas = 148 * 8, kManyShortCtas = 148 * 3, kFewCtas = 148 * 2;
 constexpr int kShortMaxW = 12;
 Shape shape_for(int W, int64_t P) {
     Shape s = {4, 1};
     if (s.ctas(P) >= (W <= kShortMaxW ? kManyShortCtas : kManyCtas)) return s;
     s.items = 1;
-    while (s.parts < 32 && s.ctas(P) < kFewCtas && W >= 4 * s.parts) s.parts *= s.parts == 16 ? 2 : 4;
+    while (s.parts < 32 && W >= 4 * s.parts && s.ctas(P) < (W >= 64 * s.parts ? kFewCtas : kFewCtas / 2)) s.parts *= s.parts == 16 ? 2 : 4;
     return s;
 }
 
