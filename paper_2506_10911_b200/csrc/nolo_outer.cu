@@ -582,12 +582,15 @@ __device__ __forceinline__ void store_mean4(double* out, double a, double b, dou
     }
 }
 
-// ITEMS quads per thread, 256 quads apart: small subgroups have few rows to keep in flight per
-// quad, so each thread takes two quads up to n = 4.
-template <int ITEMS, bool WIDE>
+// ITEMS quads per thread: small subgroups have few rows to keep in flight per quad, so each thread takes two quads up
+// to n = 4.  PARTS groups of the CTA's threads share out the members of the same columns and join their sums in
+// shared memory, for states with few columns, whose CTAs would not fill the chip and whose threads would walk the members
+// one after the other.
+template <int ITEMS, int PARTS, bool WIDE>
 __global__ void __launch_bounds__(kThreads)
 group_mean_kernel(const float* phi, const int32_t* perm, int n, int64_t stride,
                   int64_t P, double* __restrict__ mean, int64_t mean_stride, double inv_n) {
+    constexpr int COLS = kThreads / PARTS;             // threads of one part
     wait_for_predecessors();
     let_successor_start();
     const int g = blockIdx.y;
@@ -604,36 +607,49 @@ group_mean_kernel(const float* phi, const int32_t* perm, int n, int64_t stride,
         if ((threadIdx.x & 31) == 0) mean[(int64_t)g * mean_stride + c] = t * inv_n;
         return;
     }
-    const int64_t q0 = (int64_t)(blockIdx.x - tail) * (kThreads * ITEMS) + threadIdx.x;
+    const int part = threadIdx.x / COLS;
+    const int64_t q0 = (int64_t)(blockIdx.x - tail) * (COLS * ITEMS) + threadIdx.x % COLS;
     const int64_t quads = P >> 2;
     PairSum s[ITEMS];
 #pragma unroll
     for (int it = 0; it < ITEMS; ++it) s[it].clear();
-    for (int j = 0; j < n; j += kMeanUnroll) {
+    for (int j = part; j < n; j += PARTS * kMeanUnroll) {
         float4 v[ITEMS][kMeanUnroll];
 #pragma unroll
         for (int i = 0; i < kMeanUnroll; ++i) {
-            if (j + i < n) {
-                const float4* row = reinterpret_cast<const float4*>(phi + (int64_t)load_written(members + j + i) * stride);
+            if (j + i * PARTS < n) {
+                const float4* row = reinterpret_cast<const float4*>(phi + (int64_t)load_written(members + j + i * PARTS) * stride);
 #pragma unroll
                 for (int it = 0; it < ITEMS; ++it) {
-                    const int64_t q = q0 + (int64_t)it * kThreads;
+                    const int64_t q = q0 + (int64_t)it * COLS;
                     if (q < quads) v[it][i] = __ldcs(row + q);
                 }
             }
         }
 #pragma unroll
         for (int i = 0; i < kMeanUnroll; ++i) {
-            if (j + i < n) {
+            if (j + i * PARTS < n) {
 #pragma unroll
                 for (int it = 0; it < ITEMS; ++it)
-                    if (q0 + (int64_t)it * kThreads < quads) s[it].add(v[it][i]);
+                    if (q0 + (int64_t)it * COLS < quads) s[it].add(v[it][i]);
             }
         }
     }
+    if constexpr (PARTS > 1) {
+        __shared__ PairSum shared[PARTS][COLS];
+        shared[part][threadIdx.x % COLS] = s[0];
+        for (int half = PARTS / 2; half >= 1; half /= 2) {         // part p takes over the members of part p + half
+            __syncthreads();
+            if (part < half) {
+                s[0].add(shared[part + half][threadIdx.x % COLS]);
+                shared[part][threadIdx.x % COLS] = s[0];
+            }
+        }
+        if (part > 0) return;
+    }
 #pragma unroll
     for (int it = 0; it < ITEMS; ++it) {
-        const int64_t q = q0 + (int64_t)it * kThreads;
+        const int64_t q = q0 + (int64_t)it * COLS;
         if (q < quads) {
             store_mean4<WIDE>(mean + (int64_t)g * mean_stride + 4 * q,
                               ((double)s[it].hi.x + (double)s[it].lo.x) * inv_n, ((double)s[it].hi.y + (double)s[it].lo.y) * inv_n,
@@ -738,13 +754,22 @@ cudaError_t dispatch(KArgs& k, bool draw, int groups, cudaStream_t stream) {
 
 }  // namespace
 
+// Parts: as many as give the chip two CTAs per SM while every part keeps four rounds of loads, or half a CTA per SM while
+// it keeps a member.  us of prepare and prepared step, unparted /
+// in parts: n = W, float32, (32, 3125) 15.0 / 8.6, (96, 66 666) 46.9 / 32.3, (256, 25 000) 87 / 41, (1024, 1563) 232 / 33.
+constexpr int64_t kMeanFewCtas = 148 * 2;
+
 cudaError_t launch_group_mean(const float* phi, const int32_t* perm, int W, int n, int64_t stride, int64_t P,
                               double* mean, int64_t mean_stride, cudaStream_t stream) {
     if (P <= 0 || W <= 0) return cudaSuccess;
-    const int items = n <= 4 ? 2 : 1;
-    const int64_t per_cta = (int64_t)kThreads * items;
-    const int64_t tiles = ((P >> 2) + per_cta - 1) / per_cta + ((P & 3) != 0);
-    const int groups = W / n;
+    const int items = n <= 4 ? 2 : 1, groups = W / n;
+    const int64_t quads = P >> 2;
+    int parts = 1;
+    while (items == 1 && parts < 32 && n >= 4 * parts &&
+           (quads * parts + kThreads - 1) / kThreads * groups < (n >= 16 * parts ? kMeanFewCtas : kMeanFewCtas / 4))
+        parts *= parts == 16 ? 2 : 4;
+    const int64_t per_cta = (int64_t)(kThreads / parts) * items;
+    const int64_t tiles = (quads + per_cta - 1) / per_cta + ((P & 3) != 0);
     if (tiles > 0x7fffffffll || groups > 65535) return cudaErrorInvalidConfiguration;
     dim3 grid((unsigned)tiles, (unsigned)groups);
     const double inv_n = 1.0 / (double)n;
@@ -753,8 +778,13 @@ cudaError_t launch_group_mean(const float* phi, const int32_t* perm, int W, int 
     auto launch = [&](auto kernel) {
         return launch_overlapped(kernel, grid, kThreads, 0, stream, phi, perm, n, stride, P, mean, mean_stride, inv_n);
     };
-    if (items == 2) return launch(wide ? group_mean_kernel<2, true> : group_mean_kernel<2, false>);
-    return launch(wide ? group_mean_kernel<1, true> : group_mean_kernel<1, false>);
+    if (items == 2) return launch(wide ? group_mean_kernel<2, 1, true> : group_mean_kernel<2, 1, false>);
+    switch (parts) {
+        case 1: return launch(wide ? group_mean_kernel<1, 1, true> : group_mean_kernel<1, 1, false>);
+        case 4: return launch(wide ? group_mean_kernel<1, 4, true> : group_mean_kernel<1, 4, false>);
+        case 16: return launch(wide ? group_mean_kernel<1, 16, true> : group_mean_kernel<1, 16, false>);
+        default: return launch(wide ? group_mean_kernel<1, 32, true> : group_mean_kernel<1, 32, false>);
+    }
 }
 
 // Drawing in the kernel saves the launch of the draw and costs every CTA the draw's 0.3 us.  It is the faster, for a call
