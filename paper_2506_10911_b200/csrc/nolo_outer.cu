@@ -11,9 +11,10 @@
 //   phi_i'   = phi_i + delta_i'                                           (Eq. 3)
 //   theta_i' = phi_i'   (start of the next inner phase)
 //
-// Two kernels cover the subgroup sizes:
+// Three kernels cover the subgroup sizes:
 //   n <= 8        register-resident: one thread holds its oct of every member;
-//   n > 8         two passes over the members, the second read of phi served by L1/L2.
+//   n > 8         two passes over the members, the second read of phi served by L1/L2;
+//                 with few columns the threads of a CTA hold all members, and the sums are taken in shared memory.
 //
 // Arithmetic.  Delta_j is formed per member and summed in float32 in short fixed-order partial
 // sums.  gamma * (phi_i - mean phi) is a small number formed from large ones: a mean rounded to
@@ -34,6 +35,7 @@ namespace nolo {
 
 namespace {
 
+constexpr int kMostSlots = 32;  // of a two-pass CTA
 constexpr int kThreads = 256;   // CTA size of the subgroup-mean kernel
 
 struct KArgs {
@@ -562,6 +564,111 @@ outer_step_twopass_kernel(const KArgs a) {
     }
 }
 
+// ---- n > 8, few columns: every row in flight at once ------------------------------------------
+//
+// One CTA owns one subgroup x ROWQ quads, and its threads hold every member's piece: ROWS members each, phi and delta in
+// registers, phi and Delta in shared memory as well.  There the sums are taken column by column, by a thread for each column,
+// slot and kind of sum; the slots are those of the two-pass shape that these states would have otherwise, and their sums meet in
+// its order, so every bit is the same, whatever the number of columns.
+//
+// Bound by latency: the table's, one read of all rows, three barriers.  (W, n, P) float32, us in a train, two passes / this: (32, 32, 3125)
+// 5.5 / 3.3, (60, 60, 1667) 9.8 / 5.1, (96, 96, 4166) 13.1 / 5.3, (256, 256, 1562) 11.1 / 7.5, (1024, 1024, 1563) 31.2 / 18.0.
+template <typename ThetaT, int THREADS, int ROWQ, int ROWS, bool DRAW>
+__global__ void __launch_bounds__(THREADS, 1)
+outer_step_staged_kernel(const KArgs a, int slots) {
+    constexpr int WALK = THREADS / ROWQ, COLS = 4 * ROWQ;
+    extern __shared__ float4 staged[];                         // [n][ROWQ] phi, [n][ROWQ] Delta
+    __shared__ float part_D[kMostSlots][COLS], part_hi[kMostSlots][COLS], part_lo[kMostSlots][COLS];
+    __shared__ float4 total_D[ROWQ], total_hi[ROWQ], total_lo[ROWQ];
+    const int g = blockIdx.y, n = a.n;
+    __shared__ int drawn[DRAW ? 32 : 1];
+    Members<DRAW> members;
+    members.init(a, g, drawn);
+    if (a.tail && blockIdx.x == 0) {
+        ragged_tail<ThetaT, THREADS, 4>(a, g, members);
+        return;
+    }
+    const int ql = threadIdx.x % ROWQ, walk = threadIdx.x / ROWQ;
+    const int64_t q = (int64_t)(blockIdx.x - a.tail) * ROWQ + ql;
+    const bool ok = q < (a.P >> 2);
+    float4 p[ROWS], d[ROWS];
+    typename ThetaRaw<ThetaT>::type t[ROWS];
+    int row[ROWS];
+#pragma unroll
+    for (int i = 0; i < ROWS; ++i) {
+        const int j = walk + i * WALK;
+        if (ok && j < n) row[i] = members[j];
+    }
+#pragma unroll
+    for (int i = 0; i < ROWS; ++i) {
+        if (ok && walk + i * WALK < n) {
+            const int64_t off = row[i] * a.stride;
+            p[i] = __ldcs(reinterpret_cast<const float4*>(a.phi + off) + q);
+            t[i] = load_theta_raw(static_cast<const ThetaT*>(a.theta) + off, q);
+            d[i] = __ldcs(reinterpret_cast<const float4*>(a.delta + off) + q);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < ROWS; ++i) {
+        const int j = walk + i * WALK;
+        if (ok && j < n) {
+            staged[j * ROWQ + ql] = p[i];
+            staged[(n + j) * ROWQ + ql] = f4_sub(p[i], widen(t[i]));                    // Eq. 1
+        }
+    }
+    __syncthreads();
+    const float* phi = reinterpret_cast<const float*>(staged);
+    const float* Delta = phi + n * COLS;
+    for (int task = threadIdx.x; task < 2 * slots * COLS; task += THREADS) {
+        const int c = task % COLS, slot = task / COLS % slots;
+        if (task < slots * COLS) {
+            float sum = 0.f;
+            for (int j = slot; j < n; j += slots) sum += Delta[j * COLS + c];
+            part_D[slot][c] = sum;
+        } else {
+            float hi = 0.f, lo = 0.f;
+            for (int j = slot; j < n; j += slots) two_sum(hi, lo, phi[j * COLS + c]);
+            part_hi[slot][c] = hi;
+            part_lo[slot][c] = lo;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < COLS) {
+        // as the two-pass kernel does it: the two slots of a warp first, where it has 16 quads per slot
+        const int c = threadIdx.x, pair = slots >= 16 ? 2 : 1;
+        float sD = 0.f, hi = 0.f, lo = 0.f;
+        for (int w = 0; w < slots; w += pair) {
+            float D = part_D[w][c], h = part_hi[w][c], l = part_lo[w][c];
+            if (pair == 2) {
+                D += part_D[w + 1][c];
+                two_sum(h, l, part_hi[w + 1][c]);
+                l += part_lo[w + 1][c];
+            }
+            if (w == 0) {
+                sD = D; hi = h; lo = l;
+            } else {
+                sD += D;
+                two_sum(hi, lo, h);
+                lo += l;
+            }
+        }
+        reinterpret_cast<float*>(total_D)[c] = sD;
+        reinterpret_cast<float*>(total_hi)[c] = hi;
+        reinterpret_cast<float*>(total_lo)[c] = lo;
+    }
+    __syncthreads();
+    if (!ok) return;
+    const float4 sD = total_D[ql];
+    PairSum sP;
+    sP.hi = total_hi[ql];
+    sP.lo = total_lo[ql];
+    if (a.mean_phi) sP = load_prepared_mean(a, g, q);
+    else sP.divide(a);
+#pragma unroll
+    for (int i = 0; i < ROWS; ++i)
+        if (walk + i * WALK < n) update_store<ThetaT>(a, row[i] * a.stride, q, p[i], sP.deviation(p[i]), d[i], sD);
+}
+
 // ---- subgroup means of phi alone (first half of the split-phase step) ------------------------
 //
 // mean[g][p] = (1/n) sum_{j in subgroup g} phi_j[p], stored as float64.  Section 3.2 notes that
@@ -706,8 +813,35 @@ cudaError_t launch_reg(KArgs& k, bool draw, int groups, cudaStream_t stream) {
                 : launch_reg_shape<N, ThetaT, 64, true, false>(k, groups, stream);
 }
 
+// CTAs up to which all rows are taken at once: with 8 quads each (n <= 128) about what runs at a time, with 4 quads (n <= 1024,
+// 512 threads) two turns.  us in a train, two passes / staged, float32: 521 CTAs (96, 96, 16 667) 13.1 / 9.8, 391 (32, 32, 12 501) 5.6 /
+// 3.9, 1042 (24, 12, 16 667) 5.8 / 6.1; of 4 quads 196 (512, 512, 3125) 19.3 / 16.5, 392 (1024, 256, 1563) 13.9 / 19.0.
+constexpr int64_t kStagedCtas = 148 * 4, kStagedCtasWide = 148 * 2;
+
+template <typename ThetaT, int THREADS, int ROWQ, int ROWS, bool DRAW>
+cudaError_t launch_staged(KArgs& k, int slots, int groups, cudaStream_t stream) {
+    dim3 grid;
+    if (!tile_grid(k, 4, (int64_t)ROWQ * 4, groups, &grid)) return cudaErrorInvalidConfiguration;
+    const size_t smem = (size_t)k.n * ROWQ * 2 * sizeof(float4);
+    auto kernel = outer_step_staged_kernel<ThetaT, THREADS, ROWQ, ROWS, DRAW>;
+    if (smem > 32768) {
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    return launch_overlapped(kernel, grid, THREADS, smem, stream, k, slots);
+}
+
 template <typename ThetaT, int THREADS, int ROWQ, int U, int MINB>
 cudaError_t launch_twopass(KArgs& k, bool draw, int groups, cudaStream_t stream) {
+    constexpr int SLOTS = THREADS / ROWQ;
+    static_assert(SLOTS <= kMostSlots && (SLOTS >= 16) == (ROWQ == 16), "the staged kernel adds the slots in the same order");
+    if (k.n <= 128 && (k.P + 31) / 32 * groups <= kStagedCtas) {
+        if (k.n <= 32) return draw ? launch_staged<ThetaT, 256, 8, 1, true>(k, SLOTS, groups, stream)
+                                   : launch_staged<ThetaT, 256, 8, 1, false>(k, SLOTS, groups, stream);
+        if (!draw) return launch_staged<ThetaT, 256, 8, 4, false>(k, SLOTS, groups, stream);
+    }
+    if (k.n > 128 && k.n <= 1024 && !draw && (k.P + 15) / 16 * groups <= kStagedCtasWide)
+        return launch_staged<ThetaT, 512, 4, 8, false>(k, SLOTS, groups, stream);
     dim3 grid;
     if (!tile_grid(k, 4, (int64_t)ROWQ * 4, groups, &grid)) return cudaErrorInvalidConfiguration;
     if constexpr (ROWQ >= 64 && U * THREADS / ROWQ <= 16) {       // the shapes of up to 32 members

@@ -1,0 +1,145 @@
+"""Kernels and rules for states with few columns and for small simulations, at the sizes where they change."""
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import latency_oracle as L
+from oracle import nolo_oracle as O
+from paper_2506_10911_b200 import synth
+from tests.helpers import to_np
+from tests.test_gpu_magnitudes import step_and_compare
+
+pytestmark = pytest.mark.gpu
+HP = (0.5, 0.7, 0.5)
+
+
+@pytest.fixture(scope="module")
+def nolo():
+    from paper_2506_10911_b200 import binding
+    return binding
+
+
+# All members at once up to 592 CTAs of 32 columns (n <= 128) or 296 of 16 columns (n <= 1024), else two passes: both
+# sides of each line, for every shape whose order of the sums the former keeps.
+LINES = [(12, 12, 592 * 32), (24, 12, 296 * 32), (24, 24, 592 * 32), (32, 32, 592 * 32), (64, 64, 592 * 32), (96, 96, 592 * 32),
+         (128, 128, 592 * 32), (129, 129, 296 * 16), (224, 224, 296 * 16), (225, 225, 296 * 16), (641, 641, 296 * 16),
+         (1024, 1024, 296 * 16)]
+
+
+@pytest.mark.parametrize("W,n,P", LINES + [(W, n, P + 3) for W, n, P in LINES] + [
+    (9, 9, 4), (32, 32, 1), (64, 64, 31), (40, 40, 130), (128, 128, 33), (130, 130, 5), (225, 225, 17), (1024, 1024, 1000), (2050, 1025, 150)])
+@pytest.mark.parametrize("bf16", [False, True])
+def test_outer_step_shapes(nolo, W, n, P, bf16):
+    step_and_compare(nolo, W, n, P, torch.bfloat16 if bf16 else torch.float32, HP, seed=n + P)
+
+
+@pytest.mark.parametrize("W,n,P", LINES)
+@pytest.mark.parametrize("bf16", [False, True])
+def test_bits_do_not_depend_on_the_number_of_columns(nolo, W, n, P, bf16):
+    """The same columns in a state on either side of the line: the sums are added in the same order."""
+    got = []
+    state = synth.make_state(W, P + 64, n, torch.bfloat16 if bf16 else torch.float32)
+    for cols in (P, P + 64):
+        dev = [x.cuda() for x in state]
+        h = nolo.nolo_create(W, n, cols, 1, *HP)
+        nolo.nolo_bind_state(h, *dev)
+        nolo.nolo_outer_step(h, 5, 6)
+        torch.cuda.synchronize()
+        nolo.nolo_destroy(h)
+        got.append([x[:, :P] for x in dev])
+    assert all(torch.equal(a, b) for a, b in zip(*got))
+
+
+# 1, 4, 16 or 32 parts of a CTA share out the members of a column.
+@pytest.mark.parametrize("W,n,P", [(5, 5, 3), (7, 7, 1030), (15, 15, 2051), (16, 16, 4096), (63, 63, 517), (64, 64, 514), (65, 65, 4097),
+                                   (130, 130, 6), (24, 12, 80_003), (64, 32, 40_001), (128, 128, 20_003)])
+def test_subgroup_means_in_parts(nolo, W, n, P):
+    phi, theta, delta = synth.make_state(W, P, n, pad_value=float("nan"))
+    dev = [x.cuda() for x in (phi, theta, delta)]
+    mean = torch.full((W // n, synth.padded_stride(P, 8)), float("nan"), dtype=torch.float64, device="cuda")
+    h = nolo.nolo_create(W, n, P, 1, *HP)
+    nolo.nolo_bind_state(h, *dev)
+    nolo.nolo_bind_prepared(h, mean)
+    nolo.nolo_outer_prepare(h, 3, 3)
+    got = mean.cpu().numpy()
+    nolo.nolo_destroy(h)
+    x = to_np(phi)[:, :P]
+    # float32 pairs hold about 46 bits of a sum of n values
+    np.testing.assert_allclose(got[:, :P], O.subgroup_mean_phi(x, O.draw_groups(3, 3, W, n), n), rtol=1e-12,
+                               atol=1e-12 * float(np.abs(x).max()))
+    assert np.isnan(got[:, P:]).all()
+
+
+@pytest.mark.parametrize("W,P", [(63, 1024 * 147), (64, 1024 * 147), (64, 1024 * 295 + 1), (16, 1024 * 148), (15, 1024 * 100 + 3)])
+def test_divergence_in_parts(nolo, W, P):
+    gen = torch.Generator().manual_seed(W)
+    phi = 0.02 * torch.randn(1, synth.padded_stride(P), generator=gen) + 1e-3 * torch.randn(W, synth.padded_stride(P), generator=gen)
+    dev = phi.cuda()
+    h = nolo.nolo_create(W, 1, P, 1, *HP)
+    nolo.nolo_bind_state(h, dev, torch.zeros_like(dev), torch.zeros_like(dev))
+    got = nolo.nolo_divergence(h)
+    nolo.nolo_destroy(h)
+    std = phi[:, :P].double().std(0, correction=0)
+    # a float32 variance per parameter: a few roundings of 2^-24 each
+    assert got == pytest.approx((float(std.mean()), float(std.square().mean().sqrt())), rel=1e-6)
+
+
+# Lanes per trial from 1 to 32 (many trials take few), subtrees of 0 to 32 leaf blocks per lane.
+@pytest.mark.parametrize("W", [2, 4, 8, 32, 64, 128, 512, 1024, 2048, 4096])
+@pytest.mark.parametrize("many", [1, 70_000])
+def test_tree_lanes(nolo, W, many):
+    trials = max(1, many * 2 // W)
+    *_, per = nolo.nolo_sim_tree_allreduce(W, 0.1, 0.9, trials, 17, return_trials=True)
+    count = min(trials, max(1, 512 // W))
+    assert per.shape == (trials,) and (per > 0).all()
+    for first in {0, trials - count}:
+        want = [_tree(W, s, 0.1, 0.9, 17) for s in range(first, first + count)]
+        np.testing.assert_allclose(per[first:first + count], want, rtol=1e-11)
+
+
+def _tree(W, trial, mu, sigma, seed):
+    """Completion of one trial, level by level from the oracle's message times."""
+    up, down = (L.message_times(W, trial, phase, mu, sigma, seed) for phase in (0, 1))
+    ready = np.zeros(2 * W)
+    for node in range(W - 1, 0, -1):
+        ready[node] = max(ready[2 * node] + up[2 * node], ready[2 * node + 1] + up[2 * node + 1])
+    at = np.zeros(2 * W)
+    at[1] = ready[1]
+    for node in range(2, 2 * W):
+        at[node] = at[node // 2] + down[node]
+    return at[W:].max()
+
+
+# Results of up to 2^17 values are written to page-locked memory by the kernel, others copied.
+@pytest.mark.parametrize("trials", [(1 << 17) - 1, 1 << 17, (1 << 17) + 1])
+def test_results_at_the_size_where_they_are_copied(nolo, trials):
+    mean, _, per = nolo.nolo_sim_tree_allreduce(2, 0.1, 0.6, trials, 5, return_trials=True)
+    *_, few = nolo.nolo_sim_tree_allreduce(2, 0.1, 0.6, 50, 5, return_trials=True)
+    assert np.array_equal(per[:50], few) and (per > 0).all() and mean == pytest.approx(per.mean(), rel=1e-13)
+    *_, per = nolo.nolo_sim_straggler(1, 1, 1, 1, 0.1, 0.6, trials // 2, 5, return_trials=True)
+    *_, few = nolo.nolo_sim_straggler(1, 1, 1, 1, 0.1, 0.6, 50, 5, return_trials=True)
+    assert np.array_equal(per[:50], few) and (per > 0).all()
+
+
+# One subgroup of all workers; partitions of 4 to 32 lanes each; pairs and other subgroups; several slabs of each; the last
+# block of an item with one to four inner steps.
+@pytest.mark.parametrize("W,n,H,T,trials", [
+    (3, 3, 5, 40, 3), (64, 64, 6, 33, 2), (4096, 4096, 2, 3, 2), (4, 2, 7, 37, 9), (5, 1, 3, 4, 7), (8, 4, 4, 9, 3), (9, 3, 1, 5, 2),
+    (16, 2, 2, 9, 5), (17, 17, 4, 3, 2), (64, 2, 9, 8, 3), (66, 2, 10, 7, 2), (1024, 8, 3, 5, 1), (1026, 2, 3, 6, 1), (2048, 1, 2, 3, 1),
+])
+def test_straggler_rules(nolo, W, n, H, T, trials):
+    *_, per = nolo.nolo_sim_straggler(W, n, H, T, 0.4, 0.8, trials, 21, return_trials=True)
+    np.testing.assert_allclose(per, L.sim_straggler(W, n, H, T, 0.4, 0.8, trials, 21), rtol=1e-11)
+    if n == W:
+        assert np.array_equal(per[:, 0], per[:, 1])
+
+
+@pytest.mark.parametrize("W,n,H,T,trials", [(1024, 1024, 1, 5, 900), (512, 2, 2, 9, 700), (64, 64, 40, 37, 900)])
+def test_straggler_slabs_and_shared_rows(nolo, W, n, H, T, trials):
+    """Several slabs; the first and last trials are those of the oracle or of a small call."""
+    *_, per = nolo.nolo_sim_straggler(W, n, H, T, 0.4, 0.8, trials, 21, return_trials=True)
+    *_, few = nolo.nolo_sim_straggler(W, n, H, T, 0.4, 0.8, 2, 21, return_trials=True)
+    np.testing.assert_allclose(per[:2], few, rtol=1e-14)
+    np.testing.assert_allclose(few, L.sim_straggler(W, n, H, T, 0.4, 0.8, 2, 21), rtol=1e-11)
+    assert (per[:, 1] <= per[:, 0] * (1 + 1e-15)).all() and (per > 0).all()
