@@ -206,19 +206,22 @@ __device__ __forceinline__ double part_work(const LogNormalTables& tables, const
 
 // A thread per item (iteration, worker) of a trial, for W >= kSharedRowsW.  A CTA's kSimThreads items lie in few rows
 // (iterations), so the part of the Philox rounds that depends on the row and the block only is made once for
-// the CTA, kSharedBlocks blocks at a time; they are of one trial, so the round keys are the same for the CTA.
+// the CTA, up to kSharedBlocks blocks at a time; they are of one trial, so the round keys are the same for the CTA.
 // Bound as nolo_lognormal.cuh says: 323 thread-instructions per four times, 0.60 of the issue slots.  The tables are filled
 // once for several units of 256 items.  (1024, 2, 100, 250, 148) 16.1 -> 14.7 ms; 3 CTAs per SM 14.8, 5 14.8, 2 of 512 threads 14.6.
-constexpr int kSharedRowsW = 64;
-constexpr int kSharedRows = (kSimThreads - 2) / kSharedRowsW + 2;
-constexpr int kSharedBlocks = 32;
+// Few workers (from kSharedRowsW on) lie in many rows, a few blocks of which are made at a time: (4, 2, 100, 500, 592)
+// 611 -> 570 us, (16, 2, 50, 250, 500) 540 -> 493 against whole Philox blocks in the kernel below.
+constexpr int kSharedRowsW = 4;
+constexpr int kSharedBlocks = 32, kSharedLead = 400;
+static_assert(kSharedLead >= 4 * ((kSimThreads - 2) / kSharedRowsW + 2), "at least four blocks of every row");
 
 template <bool TAME>
 __global__ void __launch_bounds__(kSimThreads, 4)
 straggler_work_kernel(const Slab s, const LogNormal q) {
     __shared__ LogNormalTables tables;
     if (blockIdx.x == 0 && threadIdx.x == 0) *s.arrived = 0;
-    __shared__ PhiloxOfC0 lead[kSharedRows][kSharedBlocks];
+    __shared__ PhiloxOfC0 lead[kSharedLead];                         // [row][at_once]
+    const int at_once = min(kSharedBlocks, kSharedLead / ((kSimThreads - 2) / s.W + 2));
     fill_tables(tables, q);
     const int items = s.iterations * s.W;                            // of a trial
     const int chunks = (items + kSimThreads - 1) / kSimThreads;
@@ -231,18 +234,18 @@ straggler_work_kernel(const Slab s, const LogNormal q) {
         const PhiloxOfC1 of_worker = philox_of_c1(item - row * s.W, s.t0 + row, s.seed);
         const uint64_t key1 = s.trial0 + trial;
         double work = 0.0;
-        for (int b0 = 0; b0 < blocks; b0 += kSharedBlocks) {
+        for (int b0 = 0; b0 < blocks; b0 += at_once) {
             __syncthreads();
-            const int here = blocks - b0 < kSharedBlocks ? blocks - b0 : kSharedBlocks;
+            const int here = blocks - b0 < at_once ? blocks - b0 : at_once;
             for (int i = threadIdx.x; i < rows * here; i += kSimThreads) {
                 const int r = i / here, k = i - r * here;
-                lead[r][k] = philox_of_c0(b0 + k, s.t0 + row0 + r, kDomainStraggler, s.seed, key1);
+                lead[r * at_once + k] = philox_of_c0(b0 + k, s.t0 + row0 + r, kDomainStraggler, s.seed, key1);
             }
             __syncthreads();
             const int last = steps_in_block(s.H, b0 + here - 1), full = last < 4 ? here - 1 : here;
             for (int k = 0; k < full; ++k)                           // inner steps 4 (b0 + k) .. + 3 share a block
-                work += block_work<TAME>(tables, philox_join(lead[mine][k], of_worker, s.seed, key1), q);
-            if (full < here) work += part_work<TAME>(tables, philox_join(lead[mine][full], of_worker, s.seed, key1), q, last);
+                work += block_work<TAME>(tables, philox_join(lead[mine * at_once + k], of_worker, s.seed, key1), q);
+            if (full < here) work += part_work<TAME>(tables, philox_join(lead[mine * at_once + full], of_worker, s.seed, key1), q, last);
         }
         if (item < items) s.work[trial * items + item] = work;
     }
@@ -677,9 +680,10 @@ cudaError_t launch_straggler(int W, int n, int H, int T, double mu, double sigma
             // Threads per item: enough to fill the chip about twice, at most one per block of the item.
             int split = 1;
             while (items * split < (1 << 18) && split < 32 && 4 * split < H) split *= 2;
-            const bool shared = split == 1 && W >= kSharedRowsW;
-            const int64_t units = shared ? s.trials * (((int64_t)s.iterations * W + kSimThreads - 1) / kSimThreads)
-                                         : (items * split + kSimThreads - 1) / kSimThreads;
+            // (and items of a trial that fill its units, of which the last may be part-filled)
+            const int64_t of_trial = (int64_t)s.iterations * W, chunks = (of_trial + kSimThreads - 1) / kSimThreads;
+            const bool shared = split == 1 && W >= kSharedRowsW && (W >= 64 || 8 * of_trial >= 7 * chunks * kSimThreads);
+            const int64_t units = shared ? s.trials * chunks : (items * split + kSimThreads - 1) / kSimThreads;
             const unsigned ctas = (unsigned)(units < 3 * work_ctas ? units : 3 * work_ctas);   // a CTA that falls behind holds up less
             if (shared)
                 (tame ? straggler_work_kernel<true> : straggler_work_kernel<false>)<<<ctas, kSimThreads, 0, stream>>>(s, q);

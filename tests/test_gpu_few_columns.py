@@ -135,7 +135,8 @@ def test_straggler_rules(nolo, W, n, H, T, trials):
         assert np.array_equal(per[:, 0], per[:, 1])
 
 
-@pytest.mark.parametrize("W,n,H,T,trials", [(1024, 1024, 1, 5, 900), (512, 2, 2, 9, 700), (64, 64, 40, 37, 900)])
+@pytest.mark.parametrize("W,n,H,T,trials", [(1024, 1024, 1, 5, 900), (512, 2, 2, 9, 700), (64, 64, 40, 37, 900), (4, 2, 30, 250, 300),
+                                            (5, 5, 9, 250, 300), (16, 2, 130, 112, 160), (63, 3, 6, 61, 80), (3, 3, 13, 90, 1200)])
 def test_straggler_slabs_and_shared_rows(nolo, W, n, H, T, trials):
     """Several slabs; the first and last trials are those of the oracle or of a small call."""
     *_, per = nolo.nolo_sim_straggler(W, n, H, T, 0.4, 0.8, trials, 21, return_trials=True)
