@@ -436,7 +436,7 @@ def extra_configs(nolo, dev, peak, copy_gbs, args):
 # its 20 64 x 64 -> 128-bit products, the rest is shared) and half a table-driven logarithm, square root
 # and sine/cosine pair plus one exponential in float64 per sample; the tree kernel also walks the tree.
 # The bound is SMs x 4 schedulers x 32 lanes x SM clock / that count.
-SIM_THREAD_INSTR_PER_SAMPLE = {"straggler_work_kernel": 95.1, "tree_allreduce_kernel": 129.7}
+SIM_THREAD_INSTR_PER_SAMPLE = {"straggler_work_kernel": 79.2, "tree_allreduce_kernel": 90.6}
 
 
 def sim_records(nolo):

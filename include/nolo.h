@@ -318,7 +318,8 @@ int nolo_divergence(nolo_handle* h, double* host_out);
  *   host_stats   host, 2 doubles: mean completion time, its standard error
  *   host_trials  host, [trials] completion times, or NULL
  * float64 arithmetic.  Synchronous; allocates its own scratch, of which the
- * library keeps up to 64 MB for later calls until a handle is destroyed (which
+ * library keeps up to 64 MB on the device and 4 MB of page-locked host memory
+ * for later calls until a handle is destroyed (which
  * a process that resets the device has to do first).
  * Errors: NOLO_EINVAL, NOLO_ENOMEM, NOLO_ECUDA.
  */

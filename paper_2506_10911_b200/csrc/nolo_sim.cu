@@ -165,12 +165,12 @@ tree_allreduce_kernel(int W, int lanes, int64_t trials, LogNormal q, uint64_t se
 //
 // Only the clocks depend on the iteration before: the work of every worker in every iteration and the
 // partitions do not.  So a slab of iterations is done by three kernels: the work sums (all of the random
-// times; bound by issue slots, any number of trials fills the chip), the partitions with the longest
-// work of each iteration (one CTA or warp each), and the clocks (one CTA per trial, a few exchanges
-// through shared memory per iteration).  One CTA per trial for everything used as many SMs as there were
-// trials, ranked the keys by O(W^2) comparisons in each iteration, and waited for itself.  Whole call, before ->
-// now, (W, n, H, T, trials): (1024, 2, 100, 250, 148) 39.0 -> 16.1 ms, (1024, 512, 100, 500, 8) 91.7 -> 3.1,
-// (100, 100, 100, 500, 50) 16.9 -> 1.54, (4, 2, 100, 500, 592) 15.7 -> 0.94, (64, 2, 50, 100, 8) 2.3 -> 0.13.
+// times; any number of trials fills the chip), the partitions with the longest
+// work of each iteration (a CTA, a warp or a part of one each), and the clocks (one CTA per trial, one exchange
+// through shared memory per iteration for pairs, two for other subgroups).  Whole call, one CTA per trial for everything ->
+// three kernels -> now, (W, n, H, T, trials): (1024, 2, 100, 250, 148) 39.0 -> 16.1 -> 14.5 ms, (1024, 512, 100, 500, 8) 91.7 ->
+// 2.9 -> 2.3, (100, 100, 100, 500, 50) 16.9 -> 1.55 -> 0.97, (4, 2, 100, 500, 592) 15.7 -> 0.95 -> 0.57,
+// (64, 2, 50, 100, 8) 2.3 -> 0.11 -> 0.065.
 struct Slab {
     int W, n, H;
     int iterations;            // of this slab, from t0 on
