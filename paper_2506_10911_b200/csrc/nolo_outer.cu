@@ -824,8 +824,10 @@ cudaError_t launch_staged(KArgs& k, int slots, int groups, cudaStream_t stream) 
     if (!tile_grid(k, 4, (int64_t)ROWQ * 4, groups, &grid)) return cudaErrorInvalidConfiguration;
     const size_t smem = (size_t)k.n * ROWQ * 2 * sizeof(float4);
     auto kernel = outer_step_staged_kernel<ThetaT, THREADS, ROWQ, ROWS, DRAW>;
-    if (smem > 32768) {
-        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // the most that any subgroup needs, so that calls of different sizes from several threads do not undo each other's
+    constexpr int kMost = ROWS * THREADS * 2 * (int)sizeof(float4);
+    if constexpr (kMost > 32768) {
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost);
         if (e != cudaSuccess) return e;
     }
     return launch_overlapped(kernel, grid, THREADS, smem, stream, k, slots);

@@ -45,6 +45,8 @@ constexpr uint64_t kDomainStraggler = 4;
 // (256, 100 000) 0.77 -> 0.50, (64, 300 000) 0.70 -> 0.48 (0.3 of it the copy of the trials).
 constexpr int kTreeThreads = 512, kTreeWarps = kTreeThreads / 32, kTreeRounds = 32;
 constexpr int kLeadMaxW = 1024;      // 32 KB of shared memory
+constexpr int kTreeMostDepth = 10;    // log2(NOLO_MAX_WORKERS / 4)
+static_assert(4 << kTreeMostDepth == NOLO_MAX_WORKERS, "a lane's subtree has at most NOLO_MAX_WORKERS / 4 leaf blocks");
 
 __device__ __forceinline__ double later(double a, double b) { return a > b ? a : b; }      // no NaN here
 
@@ -627,7 +629,9 @@ cudaError_t launch_tree_allreduce(int W, double mu, double sigma, int64_t trials
     const size_t smem = sizeof(double2) * depth * kTreeThreads + (lead ? sizeof(PhiloxOfC0) * W : 0);
     auto kernel = tame ? (lead ? tree_allreduce_kernel<true, true> : tree_allreduce_kernel<true, false>)
                        : (lead ? tree_allreduce_kernel<false, true> : tree_allreduce_kernel<false, false>);
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // the most that any call needs (lanes = 1), so that calls of different sizes from several threads do not undo each other's
+    const int most_smem = (int)sizeof(double2) * kTreeMostDepth * kTreeThreads + (lead ? (int)sizeof(PhiloxOfC0) * kLeadMaxW : 0);
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most_smem);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, kernel, kTreeThreads, smem);
     if (e != cudaSuccess) return e;
     const int64_t per_warp = lanes < 32 ? 16 / lanes : 1, ctas = (trials + per_warp - 1) / per_warp;
@@ -719,7 +723,9 @@ cudaError_t launch_straggler(int W, int n, int H, int T, double mu, double sigma
             // run for long (1.03 -> 1.16 ms in all for (4, 2, 100, 500, 592)).
             auto clock = [&](auto kernel, int ahead, bool pairs) {
                 const size_t bytes = clock_bytes(W, W / n, ahead, pairs);
-                cudaError_t set = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+                const int most = W > 1024 ? NOLO_MAX_WORKERS : 1024;         // as above: for any call of this kernel
+                cudaError_t set = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                       (int)clock_bytes(most, most, ahead, pairs));
                 if (set != cudaSuccess) return set;
                 kernel<<<(unsigned)s.trials, threads, bytes, stream>>>(s, lanes, n > 1 ? 0xffffffffu / n + 1 : 0u);
                 return cudaGetLastError();

@@ -144,3 +144,36 @@ def test_straggler_slabs_and_shared_rows(nolo, W, n, H, T, trials):
     np.testing.assert_allclose(per[:2], few, rtol=1e-14)
     np.testing.assert_allclose(few, L.sim_straggler(W, n, H, T, 0.4, 0.8, 2, 21), rtol=1e-11)
     assert (per[:, 1] <= per[:, 0] * (1 + 1e-15)).all() and (per > 0).all()
+
+
+def test_calls_of_different_sizes_from_several_threads(nolo):
+    """The kernels' shared memory depends on the sizes; what one call sets up must do for the others."""
+    import threading
+    trees, stragglers, states = [(1024, 300), (64, 300), (4096, 20), (2048, 20)], [(1024, 512), (100, 10), (64, 2), (1024, 2)], [130, 1024, 256, 700]
+    want = {}
+    bad = []
+
+    def work(k):
+        try:
+            stream = torch.cuda.Stream()
+            dev = [x.cuda() for x in synth.make_state(states[k], 900, k)]
+            h = nolo.nolo_create(states[k], states[k], 900, 1, *HP)
+            torch.cuda.synchronize()
+            nolo.nolo_bind_state(h, *dev, stream=stream)
+            for turn in range(30):
+                got = (nolo.nolo_sim_tree_allreduce(*trees[k][:1], 0.0, 1.0, trees[k][1], 3, stream, return_trials=True)[2],
+                       nolo.nolo_sim_straggler(*stragglers[k], 3, 4, 0.0, 0.5, 5, 3, stream, return_trials=True)[4])
+                nolo.nolo_outer_step(h, 1, turn)
+                if not all(np.array_equal(a, b) for a, b in zip(got, want.setdefault(k, got))):
+                    bad.append(k)
+            stream.synchronize()
+            nolo.nolo_destroy(h)
+        except Exception as e:
+            bad.append(e)
+
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(4)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad
