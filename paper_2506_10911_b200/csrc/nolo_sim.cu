@@ -634,7 +634,8 @@ cudaError_t launch_tree_allreduce(int W, double mu, double sigma, int64_t trials
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most_smem);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, kernel, kTreeThreads, smem);
     if (e != cudaSuccess) return e;
-    const int64_t per_warp = lanes < 32 ? 16 / lanes : 1, ctas = (trials + per_warp - 1) / per_warp;
+    // whole CTAs of busy warps, for each fills its tables: (16, 1855) 26.2 us with as many CTAs as run at a time, 23.4 so
+    const int64_t ctas = (2 * trials * lanes + kTreeThreads - 1) / kTreeThreads;
     const int64_t most = (int64_t)sms * (resident > 0 ? resident : 1);
     kernel<<<(unsigned)(ctas < most ? ctas : most), kTreeThreads, smem, stream>>>(W, lanes, trials, LogNormal::make(mu, sigma), seed,
                                                                                  per_trial, stats_counter(scratch));
@@ -688,7 +689,10 @@ cudaError_t launch_straggler(int W, int n, int H, int T, double mu, double sigma
             const int64_t of_trial = (int64_t)s.iterations * W, chunks = (of_trial + kSimThreads - 1) / kSimThreads;
             const bool shared = split == 1 && W >= kSharedRowsW && (W >= 64 || 8 * of_trial >= 7 * chunks * kSimThreads);
             const int64_t units = shared ? s.trials * chunks : (items * split + kSimThreads - 1) / kSimThreads;
-            const unsigned ctas = (unsigned)(units < 3 * work_ctas ? units : 3 * work_ctas);   // a CTA that falls behind holds up less
+            // Every CTA fills its tables (2 us), but of three per place one that falls behind holds up less: 2744 units, (100, 100, 50,
+            // 250, 28), 176 us with one CTA per place, 170 with three; 1775 units, (4, 2, 100, 100, 71), 58 and 65.
+            const int64_t most = units >= 4 * work_ctas ? 3 * work_ctas : work_ctas;
+            const unsigned ctas = (unsigned)(units < most ? units : most);
             if (shared)
                 (tame ? straggler_work_kernel<true> : straggler_work_kernel<false>)<<<ctas, kSimThreads, 0, stream>>>(s, q);
             else
