@@ -350,28 +350,34 @@ __device__ __forceinline__ double barrier_time(const Slab& s, int64_t trial, dou
 // shared memory, in the order of the partition.  Bound by the latency of that exchange, iteration after iteration, so
 // the work and the ranks are copied to shared memory AHEAD iterations ahead, each by the thread that will use it (loads into
 // registers are waited for by six counters, whoever shares one waits for the latest: no more than four iterations ahead).
-// PAIRS: each of the two looks at the other, one barrier per iteration, two buffers.  Else `lanes` (a power of two, at most 32)
-// threads share a subgroup (members who look at all the others hit the same banks: 2.9 us per iteration at n = 8, W = 1024).
-// In a kernel of 500 iterations: 246 -> 60 us with pairs of 16 workers.
+// LOOK > 0: subgroups of at most that many, each of whose members looks at all the others: one barrier per iteration, two buffers.
+// Else `lanes` (a power of two, at most 32) threads share a subgroup, with shuffles and two barriers: from 512 workers on the
+// faster for more than pairs, since members who look at all take n accesses each.  Whole call, us, shared / looked at: (16, 8, 10, 500,
+// 100) 299 / 233, (100, 5, 10, 250, 50) 241 / 204, (256, 8, 10, 250, 50) 377 / 360, (1024, 4, 10, 100, 20) 275 / 294.  Pairs of 16
+// workers, a kernel of 500 iterations: 246 -> 60 us.
+constexpr int kLookMost = 8, kLookMaxW = 256;
+
 template <int BYTES>
 __device__ __forceinline__ void copy_ahead(void* to, const void* from) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((unsigned)__cvta_generic_to_shared(to)), "l"(from), "n"(BYTES)
                  : "memory");
 }
 
-__host__ __device__ constexpr size_t clock_bytes(int W, int groups, int ahead, bool pairs) {
-    return (size_t)W * ahead * (sizeof(double) + sizeof(uint32_t)) + (pairs ? 2 * W : W + groups) * sizeof(double);
+__host__ __device__ constexpr size_t clock_bytes(int W, int groups, int ahead, bool look) {
+    return (size_t)W * ahead * (sizeof(double) + sizeof(uint32_t)) + (look ? 2 * (W + groups) : W + groups) * sizeof(double);
 }
 
-template <int MOST, int AHEAD, bool PAIRS>
+template <int MOST, int AHEAD, int LOOK>
 __global__ void __launch_bounds__(1024)
 straggler_clock_kernel(const Slab s, int lanes, unsigned inverse_n) {
     extern __shared__ double shared[];
     const int64_t trial = blockIdx.x;
     const int lane = threadIdx.x % lanes, turn = threadIdx.x / lanes, per_turn = blockDim.x / lanes, groups = s.W / s.n;
-    double* buffer = shared;                                  // [W], twice for PAIRS
-    double* longest_of = shared + s.W;                        // [groups], unless PAIRS
-    double* works = shared + (PAIRS ? 2 * s.W : s.W + groups);  // [AHEAD][W]
+    // [W], or twice [groups][pitch]: an odd pitch spreads the subgroups over the banks
+    const int pitch = LOOK > 2 ? s.n | 1 : s.n, half = LOOK > 2 ? s.W + groups : s.W;
+    double* buffer = shared;
+    double* longest_of = shared + s.W;                        // [groups], unless LOOK
+    double* works = shared + (LOOK ? 2 * half : s.W + groups);            // [AHEAD][W]
     uint32_t* ranks = reinterpret_cast<uint32_t*>(works + AHEAD * s.W);      // [AHEAD][W]
     const double* next_work = s.work + trial * s.iterations * s.W + threadIdx.x;
     const uint32_t* next_rank = s.rank + trial * s.iterations * s.W + threadIdx.x;
@@ -409,18 +415,31 @@ straggler_clock_kernel(const Slab s, int lanes, unsigned inverse_n) {
                 const int w = threadIdx.x + k * blockDim.x;
                 at[k] = (int)ranks[slot * s.W + w];
                 clock[k] += works[slot * s.W + w];
-                buffer[at[k]] = clock[k];
-                if (!PAIRS && inverse_n) at[k] = (int)__umulhi((unsigned)at[k], inverse_n);     // the subgroup
+                const int group = LOOK != 2 && inverse_n ? (int)__umulhi((unsigned)at[k], inverse_n) : at[k];
+                buffer[LOOK > 2 ? at[k] + group * (pitch - s.n) : at[k]] = clock[k];
+                if (LOOK != 2) at[k] = group;
             }
         }
         ahead(slot, i + AHEAD);
         slot = slot + 1 == AHEAD ? 0 : slot + 1;
         __syncthreads();
-        if constexpr (PAIRS) {
+        if constexpr (LOOK > 0) {
 #pragma unroll
-            for (int k = 0; k < MOST; ++k)
-                if (mine[k]) clock[k] = later(clock[k], buffer[at[k] ^ 1]);
-            buffer = buffer == shared ? shared + s.W : shared;
+            for (int k = 0; k < MOST; ++k) {
+                if (mine[k]) {
+                    if constexpr (LOOK == 2) {
+                        clock[k] = later(clock[k], buffer[at[k] ^ 1]);
+                    } else {
+                        const double* member = buffer + at[k] * pitch;
+                        double c[LOOK];
+#pragma unroll
+                        for (int j = 0; j < LOOK; ++j) c[j] = j < s.n ? member[j] : 0.0;
+#pragma unroll
+                        for (int j = 0; j < LOOK; ++j) clock[k] = later(clock[k], c[j]);
+                    }
+                }
+            }
+            buffer = buffer == shared ? shared + half : shared;
         } else {
             for (int g0 = 0; g0 < groups; g0 += per_turn) {               // every lane of a subgroup takes the same turns
                 const int g = g0 + turn;
@@ -725,18 +744,19 @@ cudaError_t launch_straggler(int W, int n, int H, int T, double mu, double sigma
             if (e != cudaSuccess) return e;
             // Not ahead of the order kernel's end: CTAs that come in as it leaves crowd on the first free SMs, and these
             // run for long (1.03 -> 1.16 ms in all for (4, 2, 100, 500, 592)).
-            auto clock = [&](auto kernel, int ahead, bool pairs) {
-                const size_t bytes = clock_bytes(W, W / n, ahead, pairs);
+            auto clock = [&](auto kernel, int ahead, bool look) {
+                const size_t bytes = clock_bytes(W, W / n, ahead, look);
                 const int most = W > 1024 ? NOLO_MAX_WORKERS : 1024;         // as above: for any call of this kernel
                 cudaError_t set = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                       (int)clock_bytes(most, most, ahead, pairs));
+                                                       (int)clock_bytes(most, most, ahead, look));
                 if (set != cudaSuccess) return set;
                 kernel<<<(unsigned)s.trials, threads, bytes, stream>>>(s, lanes, n > 1 ? 0xffffffffu / n + 1 : 0u);
                 return cudaGetLastError();
             };
-            e = W > 1024 ? clock(straggler_clock_kernel<NOLO_MAX_WORKERS / 1024, 2, false>, 2, false)
-              : n == 2   ? clock(straggler_clock_kernel<1, 4, true>, 4, true)
-                         : clock(straggler_clock_kernel<1, 4, false>, 4, false);
+            e = W > 1024                         ? clock(straggler_clock_kernel<NOLO_MAX_WORKERS / 1024, 2, 0>, 2, false)
+              : n == 2                           ? clock(straggler_clock_kernel<1, 4, 2>, 4, true)
+              : n <= kLookMost && W <= kLookMaxW ? clock(straggler_clock_kernel<1, 4, kLookMost>, 4, true)
+                                                 : clock(straggler_clock_kernel<1, 4, 0>, 4, false);
             if (e != cudaSuccess) return e;
         }
     }

@@ -126,7 +126,7 @@ def test_results_at_the_size_where_they_are_copied(nolo, trials):
 # block of an item with one to four inner steps.
 @pytest.mark.parametrize("W,n,H,T,trials", [
     (3, 3, 5, 40, 3), (64, 64, 6, 33, 2), (4096, 4096, 2, 3, 2), (4, 2, 7, 37, 9), (5, 1, 3, 4, 7), (8, 4, 4, 9, 3), (9, 3, 1, 5, 2),
-    (16, 2, 2, 9, 5), (17, 17, 4, 3, 2), (64, 2, 9, 8, 3), (66, 2, 10, 7, 2), (1024, 8, 3, 5, 1), (1026, 2, 3, 6, 1), (2048, 1, 2, 3, 1),
+    (16, 2, 2, 9, 5), (17, 17, 4, 3, 2), (15, 5, 3, 9, 3), (32, 8, 2, 5, 2), (256, 8, 2, 6, 2), (252, 7, 2, 6, 2), (258, 6, 2, 3, 1), (64, 2, 9, 8, 3), (66, 2, 10, 7, 2), (1024, 8, 3, 5, 1), (1026, 2, 3, 6, 1), (2048, 1, 2, 3, 1),
 ])
 def test_straggler_rules(nolo, W, n, H, T, trials):
     *_, per = nolo.nolo_sim_straggler(W, n, H, T, 0.4, 0.8, trials, 21, return_trials=True)
