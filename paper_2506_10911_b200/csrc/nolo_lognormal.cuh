@@ -12,7 +12,7 @@
 // Bound by the dispatch of 32- and 64-bit operands, to which the float64 operations (19 to 20 per time) and Philox's
 // products contribute alike: an instruction less of any kind shows.  Intervals of 2^-9 (logarithm), entries of 2 pi / 512 and
 // 2^(1 / 2048) (33 KB in all) need 39 float64 operations per pair of times, those of 128, 256 and 256 entries (9 KB) needed
-// 48: 380 -> 323 thread-instructions per four times in the straggler simulation, and errors no larger (root mean square
+// 48: 380 -> 317 thread-instructions per four times in the straggler simulation, and errors no larger (root mean square
 // 1.28e-16 -> 1.18e-16 at sigma = 1, 4.9e-16 -> 2.6e-16 at mu = -3, sigma = 2.5).
 #pragma once
 

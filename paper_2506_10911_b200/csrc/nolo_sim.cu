@@ -35,13 +35,13 @@ constexpr uint64_t kDomainStraggler = 4;
 // the time of the longest way down, which is found from below like the longest way up.  So a trial is two sums of
 // longest ways, and no time is kept for a second sweep.
 //
-// A warp takes one direction of one trial (W / 2 lanes do below 64 workers).  Above 64 workers every lane has a subtree
-// of W / 32 leaves whose blocks it visits children first, with the finished halves of what is above them on a stack
-// of its own; then every lane makes one of the 32 blocks of the nodes below 128, which the warp reduces by shuffles.
-// So all lanes work all the time and nothing waits for another warp, but for the two directions of a trial, which
-// meet every kTreeRounds trials.  What Philox makes of a block's number is the same for all trials and is kept (LEAD).
-// Bound by the log-normal times: 372 thread-instructions per four, of which 323 make them; a sweep up and one down over
-// nodes in shared memory with barriers between the levels took 464.  Whole call, (W, trials): (1024, 20 000) 0.51 -> 0.37 ms,
+// `lanes` lanes (a power of two, at most 32 and W / 2) take one direction of one trial.  Every lane has a subtree of W / lanes
+// leaves, whose blocks it visits children first, with the finished halves of what is above them on a stack
+// of its own; then every lane makes one of the `lanes` blocks of the nodes below 4 lanes, which they reduce by shuffles.
+// So all lanes work all the time and nothing waits for another warp, but for the two directions of a trial
+// of 32 lanes, which meet every kTreeRounds trials.  What Philox makes of a block's number is the same for all trials and is kept (LEAD).
+// Bound by the log-normal times: 363 thread-instructions per four (those of the stragglers 317); a sweep up and one down
+// over nodes in shared memory with barriers between the levels took 464.  Whole call, (W, trials): (1024, 20 000) 0.51 -> 0.37 ms,
 // (256, 100 000) 0.77 -> 0.50, (64, 300 000) 0.70 -> 0.48 (0.3 of it the copy of the trials).
 constexpr int kTreeThreads = 512, kTreeWarps = kTreeThreads / 32, kTreeRounds = 32;
 constexpr int kLeadMaxW = 1024;      // 32 KB of shared memory
@@ -209,8 +209,9 @@ __device__ __forceinline__ double part_work(const LogNormalTables& tables, const
 // A thread per item (iteration, worker) of a trial, for W >= kSharedRowsW.  A CTA's kSimThreads items lie in few rows
 // (iterations), so the part of the Philox rounds that depends on the row and the block only is made once for
 // the CTA, up to kSharedBlocks blocks at a time; they are of one trial, so the round keys are the same for the CTA.
-// Bound as nolo_lognormal.cuh says: 323 thread-instructions per four times, 0.60 of the issue slots.  The tables are filled
-// once for several units of 256 items.  (1024, 2, 100, 250, 148) 16.1 -> 14.7 ms; 3 CTAs per SM 14.8, 5 14.8, 2 of 512 threads 14.6.
+// Bound as nolo_lognormal.cuh says: 317 thread-instructions per four times, 0.60 of the issue slots.  The tables are filled
+// once for several units of 256 items.  (1024, 2, 100, 250, 148) 16.1 -> 14.5 ms; with 3 CTAs
+// per SM 1 % more, with 5 the same, with 2 of 512 threads 0.3 % less.
 // Few workers (from kSharedRowsW on) lie in many rows, a few blocks of which are made at a time: (4, 2, 100, 500, 592)
 // 611 -> 570 us, (16, 2, 50, 250, 500) 540 -> 493 against whole Philox blocks in the kernel below.
 constexpr int kSharedRowsW = 4;
