@@ -210,14 +210,19 @@ cudaError_t launch_copy_probe(const void* in, void* out, int64_t bytes, cudaStre
 }
 
 // Drawing in the copy saves the launch of the draw, lets the copy ask for its data ahead of its wait, and costs every
-// CTA the draw's 0.3 us.  It is the faster, for a call alone and for calls that follow each other, as long as the grid is
-// few waves.  us alone, drawn in the copy / by a kernel ahead: 6 MB 10.2 / 11.3, 134 MB (multiples of 32 bytes) 47.1 / 48.1,
-// 67 MB of other blocks 28.7 / 29.7; 400 MB 251 / 248 there and back.
-constexpr int64_t kDrawMaxBytes = 64ll << 20, kDrawMaxBytesWide = 128ll << 20;   // the latter for multiples of 32 bytes
+// CTA the draw, 0.3 us and the more the more replicas there are.  It is the faster, for a call alone and for calls that follow
+// each other, as long as the grid is few waves, and for few replicas long after.  us alone, drawn in the copy / by a kernel ahead:
+// 6 MB 10.2 / 11.3, 134 MB (multiples of 32 bytes) 47.1 / 48.1, 67 MB of other blocks 28.7 / 29.7.  There and back, 8 replicas:
+// 140 MB a way 85.8 / 90.5, 420 MB 240 / 245, 944 MB 536 / 543, at odd offsets 73 MB 46.2 / 50.3, 94 MB 59.2 / 62.5, 126 MB 79.1 /
+// 80.4; 32 replicas: 420 MB 255 / 245, at odd offsets 84 MB 58.9 / 56.8.
+constexpr int kFewReplicas = 8;
+constexpr int64_t kDrawMaxBytes = 64ll << 20, kDrawMaxBytesFew = 100ll << 20;
+constexpr int64_t kDrawMaxBytesWide = 128ll << 20, kDrawMaxBytesWideFew = 1024ll << 20;   // for multiples of 32 bytes
 
 bool route_draws(const RouteArgs& a) {
-    const int64_t block = a.E * a.elem_size;
-    return a.R <= 32 && (int64_t)a.B * a.R * a.K * block <= (block % 32 == 0 ? kDrawMaxBytesWide : kDrawMaxBytes);
+    const int64_t block = a.E * a.elem_size, bytes = (int64_t)a.B * a.R * a.K * block;
+    if (block % 32 == 0) return a.R <= 32 && bytes <= (a.R <= kFewReplicas ? kDrawMaxBytesWideFew : kDrawMaxBytesWide);
+    return a.R <= 32 && bytes <= (a.R <= kFewReplicas ? kDrawMaxBytesFew : kDrawMaxBytes);
 }
 
 template <typename V, int THREADS, int N>

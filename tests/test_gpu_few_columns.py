@@ -177,3 +177,25 @@ def test_calls_of_different_sizes_from_several_threads(nolo):
     for t in threads:
         t.join()
     assert not bad
+
+
+# Copies draw for themselves up to 1 GB, of blocks that are no multiple of 32 bytes 100 MB, for up to 8 replicas (128 and 64 MB
+# for more): both sides of each line.
+@pytest.mark.parametrize("W,E", [(8, 1 << 24), ((8), (1 << 24) + 8), (8, 100 * 32768 - 1), (8, 100 * 32768 + 1), (7, 3_000_000), (9, 3_000_001)])
+def test_routing_at_the_sizes_where_copies_stop_drawing(nolo, W, E):
+    stages, K = (3, 2) if E > 1 << 23 else (3, 1)
+    acts = torch.randint(-2**31, 2**31 - 1, (stages - 1, W, K, E), dtype=torch.int32, device="cuda").view(torch.float32)
+    out, back = torch.zeros_like(acts), torch.zeros_like(acts)
+    h = nolo.nolo_create(W, 1, 8, stages, *HP)
+    nolo.nolo_bind_route(h, W * K, E, out, True)
+    nolo.nolo_route(h, 11, 3, acts)
+    table = torch.from_numpy(O.draw_route(11, 3, stages, W, K, per_microbatch=True)).long()
+    assert np.array_equal(nolo.nolo_get_route(h), table.numpy())
+    for b in range(stages - 1):
+        for k in range(K):
+            for r in range(W):
+                assert torch.equal(out[b, r, k].view(torch.int32), acts[b, int(table[b, k, r]), k].view(torch.int32))
+    nolo.nolo_route_backward(h, 11, 3, out, back)
+    torch.cuda.synchronize()
+    assert torch.equal(back.view(torch.int32), acts.view(torch.int32))
+    nolo.nolo_destroy(h)
