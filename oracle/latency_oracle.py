@@ -135,12 +135,12 @@ def sim_tree_allreduce(W, mu, sigma, trials, seed):
     return out
 
 
-def sim_straggler(W, n, H, T, mu, sigma, trials, seed):
+def sim_straggler(W, n, H, T, mu, sigma, trials, seed, first=0):
     """[trials, 2]: time for all workers to finish T outer iterations of H inner
-    steps under (global barrier every outer step, wait only for the subgroup)."""
+    steps under (global barrier every outer step, wait only for the subgroup).  Trials first .. first + trials - 1."""
     out = np.empty((trials, 2), dtype=np.float64)
     w = np.arange(W, dtype=np.uint64)
-    for s in range(trials):
+    for s in range(first, first + trials):
         barrier_clock = 0.0
         clock = np.zeros(W)
         for t in range(T):
@@ -156,5 +156,5 @@ def sim_straggler(W, n, H, T, mu, sigma, trials, seed):
                 members = perm[g * n:(g + 1) * n]
                 new[members] = done[members].max()
             clock = new
-        out[s] = (barrier_clock, clock.max())
+        out[s - first] = (barrier_clock, clock.max())
     return out

@@ -206,9 +206,10 @@ __device__ __forceinline__ double part_work(const LogNormalTables& tables, const
     return work;
 }
 
-// A thread per item (iteration, worker) of a trial, for W >= kSharedRowsW.  A CTA's kSimThreads items lie in few rows
+// A thread per item (iteration, worker), for W >= kSharedRowsW.  A CTA's kSimThreads items lie in few rows
 // (iterations), so the part of the Philox rounds that depends on the row and the block only is made once for
-// the CTA, up to kSharedBlocks blocks at a time; they are of one trial, so the round keys are the same for the CTA.
+// the CTA, up to kSharedBlocks blocks at a time.  They are of one trial, so that the round keys are the same for the CTA, unless
+// that would leave threads idle: many trials leave a slab few iterations, and a trial of it fewer items than threads (ACROSS).
 // Bound as nolo_lognormal.cuh says: 317 thread-instructions per four times, 0.60 of the issue slots.  The tables are filled
 // once for several units of 256 items.  (1024, 2, 100, 250, 148) 16.1 -> 14.5 ms; with 3 CTAs
 // per SM 1 % more, with 5 the same, with 2 of 512 threads 0.3 % less.
@@ -218,31 +219,33 @@ constexpr int kSharedRowsW = 4;
 constexpr int kSharedBlocks = 32, kSharedLead = 400;
 static_assert(kSharedLead >= 4 * ((kSimThreads - 2) / kSharedRowsW + 2), "at least four blocks of every row");
 
-template <bool TAME>
+template <bool TAME, bool ACROSS>
 __global__ void __launch_bounds__(kSimThreads, 4)
-straggler_work_kernel(const Slab s, const LogNormal q) {
+straggler_work_kernel(const Slab s, const LogNormal q, int items, int chunks, int64_t units) {
     __shared__ LogNormalTables tables;
     if (blockIdx.x == 0 && threadIdx.x == 0) *s.arrived = 0;
     __shared__ PhiloxOfC0 lead[kSharedLead];                         // [row][at_once]
     const int at_once = min(kSharedBlocks, kSharedLead / ((kSimThreads - 2) / s.W + 2));
     fill_tables(tables, q);
-    const int items = s.iterations * s.W;                            // of a trial
-    const int chunks = (items + kSimThreads - 1) / kSimThreads;
     const int blocks = step_blocks(s.H);
-    for (int64_t unit = blockIdx.x; unit < s.trials * chunks; unit += gridDim.x) {
-        const int64_t trial = unit / chunks;
-        const int base = (int)(unit - trial * chunks) * kSimThreads, item = base + threadIdx.x;
+    for (int64_t unit = blockIdx.x; unit < units; unit += gridDim.x) {
+        const int64_t unit_trial = ACROSS ? 0 : unit / chunks;
+        const int base = (int)(unit - unit_trial * chunks) * kSimThreads, item = base + threadIdx.x;
         const int row0 = base / s.W, rows = (min(base + kSimThreads, items) - 1) / s.W - row0 + 1;
         const int row = item / s.W, mine = item < items ? row - row0 : 0;
-        const PhiloxOfC1 of_worker = philox_of_c1(item - row * s.W, s.t0 + row, s.seed);
-        const uint64_t key1 = s.trial0 + trial;
+        // of a row, counted from the unit's trial on
+        auto trial_of = [&](int r) { return ACROSS ? r / s.iterations : 0; };
+        auto iteration_of = [&](int r) { return s.t0 + (ACROSS ? r % s.iterations : r); };
+        const PhiloxOfC1 of_worker = philox_of_c1(item - row * s.W, iteration_of(row), s.seed);
+        const uint64_t key1 = s.trial0 + unit_trial + trial_of(row);
         double work = 0.0;
         for (int b0 = 0; b0 < blocks; b0 += at_once) {
             __syncthreads();
             const int here = blocks - b0 < at_once ? blocks - b0 : at_once;
             for (int i = threadIdx.x; i < rows * here; i += kSimThreads) {
                 const int r = i / here, k = i - r * here;
-                lead[r * at_once + k] = philox_of_c0(b0 + k, s.t0 + row0 + r, kDomainStraggler, s.seed, key1);
+                lead[r * at_once + k] = philox_of_c0(b0 + k, iteration_of(row0 + r), kDomainStraggler, s.seed,
+                                                     s.trial0 + unit_trial + trial_of(row0 + r));
             }
             __syncthreads();
             const int last = steps_in_block(s.H, b0 + here - 1), full = last < 4 ? here - 1 : here;
@@ -250,7 +253,7 @@ straggler_work_kernel(const Slab s, const LogNormal q) {
                 work += block_work<TAME>(tables, philox_join(lead[mine * at_once + k], of_worker, s.seed, key1), q);
             if (full < here) work += part_work<TAME>(tables, philox_join(lead[mine * at_once + full], of_worker, s.seed, key1), q, last);
         }
-        if (item < items) s.work[trial * items + item] = work;
+        if (item < items) s.work[unit_trial * items + item] = work;
     }
 }
 
@@ -688,7 +691,7 @@ cudaError_t launch_straggler(int W, int n, int H, int T, double mu, double sigma
     cudaError_t e = cudaGetDevice(&device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, tame ? straggler_work_kernel<true> : straggler_work_kernel<false>,
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, tame ? straggler_work_kernel<true, false> : straggler_work_kernel<false, false>,
                                                           kSimThreads, 0);
     if (e != cudaSuccess) return e;
     const int64_t work_ctas = (int64_t)sms * (resident > 0 ? resident : 1);
@@ -705,16 +708,18 @@ cudaError_t launch_straggler(int W, int n, int H, int T, double mu, double sigma
             // Threads per item: enough to fill the chip about twice, at most one per block of the item.
             int split = 1;
             while (items * split < (1 << 18) && split < 32 && 4 * split < H) split *= 2;
-            // (and items of a trial that fill its units, of which the last may be part-filled)
-            const int64_t of_trial = (int64_t)s.iterations * W, chunks = (of_trial + kSimThreads - 1) / kSimThreads;
-            const bool shared = split == 1 && W >= kSharedRowsW && (W >= 64 || 8 * of_trial >= 7 * chunks * kSimThreads);
-            const int64_t units = shared ? s.trials * chunks : (items * split + kSimThreads - 1) / kSimThreads;
+            const WorkUnits u = WorkUnits::of(W, s.iterations, s.trials, kSimThreads);
+            const bool shared = split == 1 && W >= kSharedRowsW;
+            const int64_t units = shared ? u.count : (items * split + kSimThreads - 1) / kSimThreads;
             // Every CTA fills its tables (2 us), but of three per place one that falls behind holds up less: 2744 units, (100, 100, 50,
             // 250, 28), 176 us with one CTA per place, 170 with three; 1775 units, (4, 2, 100, 100, 71), 58 and 65.
             const int64_t most = units >= 4 * work_ctas ? 3 * work_ctas : work_ctas;
             const unsigned ctas = (unsigned)(units < most ? units : most);
             if (shared)
-                (tame ? straggler_work_kernel<true> : straggler_work_kernel<false>)<<<ctas, kSimThreads, 0, stream>>>(s, q);
+                (tame ? (u.across ? straggler_work_kernel<true, true> : straggler_work_kernel<true, false>)
+                      : (u.across ? straggler_work_kernel<false, true>
+                                  : straggler_work_kernel<false, false>))<<<ctas, kSimThreads, 0, stream>>>(s, q, (int)u.items,
+                                                                                                           (int)u.chunks, units);
             else
                 (tame ? straggler_split_work_kernel<true>
                       : straggler_split_work_kernel<false>)<<<ctas, kSimThreads, 0, stream>>>(s, q, split, items);

@@ -146,6 +146,19 @@ def test_straggler_slabs_and_shared_rows(nolo, W, n, H, T, trials):
     assert (per[:, 1] <= per[:, 0] * (1 + 1e-15)).all() and (per > 0).all()
 
 
+# Many trials leave a slab few iterations: units of 256 items lie across trials where one trial does not fill them.
+@pytest.mark.parametrize("W,n,H,T,trials", [(64, 2, 6, 9, 4000), (100, 4, 5, 3, 9000), (257, 257, 3, 2, 7000), (65, 5, 9, 1, 3000),
+                                            (64, 64, 130, 2, 17_000), (1000, 8, 2, 1, 300), (300, 10, 34, 2, 900), (128, 8, 3, 3, 31),
+                                            (4, 2, 29, 1, 9000), (5, 1, 2, 20, 70_000), (63, 9, 30, 2, 40_000)])
+@pytest.mark.parametrize("sigma", [0.8, 90.0])
+def test_straggler_units_across_trials(nolo, W, n, H, T, trials, sigma):
+    *_, per = nolo.nolo_sim_straggler(W, n, H, T, 0.4, sigma, trials, 21, return_trials=True)
+    for first in (0, trials // 2, trials - 2):
+        want = L.sim_straggler(W, n, H, T, 0.4, sigma, 2, 21, first)
+        # (an exponent of 8.7 sigma has units of 2^-53 times that)
+        np.testing.assert_allclose(per[first:first + 2], want, rtol=1e-11)
+
+
 def test_calls_of_different_sizes_from_several_threads(nolo):
     """The kernels' shared memory depends on the sizes; what one call sets up must do for the others."""
     import threading

@@ -195,3 +195,31 @@ int main() {
     return 0;
 }
 """)
+
+
+def test_units_of_the_straggler_simulation_are_filled(tmp_path):
+    """However many trials leave a slab however few iterations, at most an eighth of the threads is idle, but for the last
+    unit; and the units cover the items."""
+    run_host_code(tmp_path, r"""
+#include "nolo_steps.h"
+#include <cstdio>
+#include <initializer_list>
+int main() {
+    const int threads = 256;
+    for (int W = 4; W <= 4096; W += W < 300 ? 1 : 37)
+        for (int iterations = 1; iterations <= 60; iterations += iterations < 9 ? 1 : 7)
+            for (long long trials : {1ll, 2ll, 3ll, 50ll, 700ll, 20000ll}) {
+                const int64_t work = (int64_t)W * iterations * trials;
+                if (work > 31 << 16) continue;
+                const nolo::WorkUnits u = nolo::WorkUnits::of(W, iterations, trials, threads);
+                const int64_t laid = u.count * threads;
+                bool ok = 7 * laid <= 8 * work + 7 * threads;
+                ok &= u.items == (int64_t)W * iterations * (u.across ? trials : 1);
+                ok &= u.chunks * threads >= u.items && (u.chunks - 1) * threads < u.items;
+                ok &= u.count == u.chunks * (u.across ? 1 : trials);
+                if (!ok) return printf("W %d, %d iterations, %lld trials: %lld threads for %lld items\n", W, iterations, trials,
+                                       (long long)laid, (long long)work), 1;
+            }
+    return 0;
+}
+""")
