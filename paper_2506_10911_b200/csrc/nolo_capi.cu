@@ -257,10 +257,14 @@ struct DeviceMemory {
     }
     static bool exhausted(Status e) { return e == cudaErrorMemoryAllocation; }
     static void release(void* p) { cudaFree(p); }
+    using Stream = cudaStream_t;
+    static Status copy(void* host, const void* device, size_t bytes, Stream s) {
+        return cudaMemcpyAsync(host, device, bytes, cudaMemcpyDeviceToHost, s);
+    }
+    static Status wait(Stream s) { return cudaStreamSynchronize(s); }
 };
-using Scratches = nolo::ScratchBlocks<DeviceMemory>;
 
-Scratches g_scratch;
+nolo::ScratchBlocks<DeviceMemory> g_scratch;
 
 // Page-locked memory, which any device may write, for their results: blocks of one size, so at most 4 MB are kept.
 struct HostMemory : DeviceMemory {
@@ -272,44 +276,10 @@ struct HostMemory : DeviceMemory {
     }
     static void release(void* p) { cudaFreeHost(p); }
 };
-using HostScratches = nolo::ScratchBlocks<HostMemory>;
 
-HostScratches g_host_scratch;
+nolo::ScratchBlocks<HostMemory> g_host_scratch;
 
-// Scratch of one simulation call and page-locked memory for its results, kept for the next one if the call comes to its
-// end.  The results are the statistics and, up to kHostTrials values, the trials: the last kernel writes them there.
-struct SimScratch {
-    static constexpr int64_t kHostTrials = 1 << 17;
-    static constexpr int kStats = 4;
-    Scratches::Block block;
-    HostScratches::Block host;
-    ~SimScratch() {
-        if (block.p) cudaFree(block.p);
-        if (host.p) cudaFreeHost(host.p);
-    }
-    cudaError_t take(size_t want) {
-        const cudaError_t e = g_scratch.take(want < (size_t(1) << 20) ? size_t(1) << 20 : want, &block);   // small calls of all sizes share blocks
-        return e != cudaSuccess ? e : g_host_scratch.take(sizeof(double) * (kStats + kHostTrials), &host);
-    }
-    double* stats() const { return static_cast<double*>(host.p); }
-    double* trials() const { return stats() + kStats; }
-    // Waits for the results and hands them over; e: how the launches went.
-    int finish(cudaError_t e, const double* per_trial, int64_t values, double* host_trials, double* host_stats, int stats_count,
-               cudaStream_t s) {
-        const bool in_place = values <= kHostTrials;
-        if (e == cudaSuccess && host_trials && !in_place)
-            e = cudaMemcpyAsync(host_trials, per_trial, sizeof(double) * (size_t)values, cudaMemcpyDeviceToHost, s);
-        const cudaError_t end = cudaStreamSynchronize(s);
-        if (e == cudaSuccess) e = end;
-        if (e != cudaSuccess) return NOLO_ECUDA;
-        memcpy(host_stats, stats(), sizeof(double) * (size_t)stats_count);
-        if (host_trials && in_place) memcpy(host_trials, trials(), sizeof(double) * (size_t)values);
-        g_scratch.put(block);
-        g_host_scratch.put(host);
-        block.p = host.p = nullptr;
-        return NOLO_OK;
-    }
-};
+using SimScratch = nolo::SimScratch<DeviceMemory, HostMemory>;
 
 int ensure_host_streams(nolo_handle* h) {
     if (h->s_in) return NOLO_OK;
@@ -746,15 +716,12 @@ int nolo_sim_tree_allreduce(int W, double mu, double sigma, int64_t trials, uint
         !std::isfinite(mu) || !std::isfinite(sigma) || sigma < 0 || !host_stats)
         return NOLO_EINVAL;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    SimScratch scratch;
-    const size_t results = sizeof(double) * (((size_t)trials + 1) & ~size_t(1));
-    cudaError_t e = scratch.take(results + nolo::tree_scratch());
+    SimScratch scratch(g_scratch, g_host_scratch);
+    cudaError_t e = scratch.take(trials, nolo::tree_scratch());
     if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? NOLO_ENOMEM : NOLO_ECUDA;
-    double* d = static_cast<double*>(scratch.block.p);
-    e = nolo::launch_tree_allreduce(W, mu, sigma, trials, seed, d, scratch.stats(),
-                                    host_trials && trials <= SimScratch::kHostTrials ? scratch.trials() : nullptr,
-                                    reinterpret_cast<char*>(d) + results, s);
-    return scratch.finish(e, d, trials, host_trials, host_stats, 2, s);
+    e = nolo::launch_tree_allreduce(W, mu, sigma, trials, seed, scratch.values(), scratch.stats(),
+                                    scratch.values_in_place(host_trials), scratch.scratch(), s);
+    return scratch.finish(e, host_trials, host_stats, 2, s) == cudaSuccess ? NOLO_OK : NOLO_ECUDA;
 }
 
 int nolo_sim_straggler(int W, int n, int H, int T, double mu, double sigma, int64_t trials, uint64_t seed,
@@ -765,15 +732,12 @@ int nolo_sim_straggler(int W, int n, int H, int T, double mu, double sigma, int6
     // One launch draws W*H*T samples per trial; a mistyped H or T must not occupy the GPU for hours.
     if ((double)W * (double)H * (double)T * (double)trials > (double)NOLO_SIM_MAX_SAMPLES) return NOLO_EINVAL;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    SimScratch scratch;
-    const size_t results = sizeof(double) * 2 * (size_t)trials;
-    cudaError_t e = scratch.take(results + nolo::straggler_scratch(W, T, trials));
+    SimScratch scratch(g_scratch, g_host_scratch);
+    cudaError_t e = scratch.take(2 * trials, nolo::straggler_scratch(W, T, trials));
     if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? NOLO_ENOMEM : NOLO_ECUDA;
-    double* d = static_cast<double*>(scratch.block.p);
-    e = nolo::launch_straggler(W, n, H, T, mu, sigma, trials, seed, d, scratch.stats(),
-                               host_trials && 2 * trials <= SimScratch::kHostTrials ? scratch.trials() : nullptr,
-                               reinterpret_cast<char*>(d) + results, s);
-    return scratch.finish(e, d, 2 * trials, host_trials, host_stats, 4, s);
+    e = nolo::launch_straggler(W, n, H, T, mu, sigma, trials, seed, scratch.values(), scratch.stats(),
+                               scratch.values_in_place(host_trials), scratch.scratch(), s);
+    return scratch.finish(e, host_trials, host_stats, 4, s) == cudaSuccess ? NOLO_OK : NOLO_ECUDA;
 }
 
 double nolo_expected_pair_exchange(double mu, double sigma) {

@@ -223,3 +223,79 @@ int main() {
     return 0;
 }
 """)
+
+
+def test_simulations_do_without_page_locked_memory(tmp_path):
+    """Results are left in page-locked memory where there is some, else on the device and copied; the caller gets the
+    same, and either kind of block is kept or released once."""
+    run_host_code(tmp_path, SCRATCH + r"""
+#include <cstring>
+struct Device : Fake {
+    using Stream = int;
+    struct Copy { void* to; const void* from; size_t bytes; };
+    static inline std::vector<Copy> pending;
+    static inline int copies = 0, wait_fails = 0;
+    static int allocate(void** p, size_t bytes) {
+        *p = calloc(1, bytes);
+        held[*p] = bytes; total += bytes;
+        return 0;
+    }
+    static int copy(void* to, const void* from, size_t bytes, int) { pending.push_back({to, from, bytes}); ++copies; return 0; }
+    static int wait(int) {
+        for (const Copy& c : pending) memcpy(c.to, c.from, c.bytes);
+        pending.clear();
+        return wait_fails;
+    }
+};
+struct Host : Device {
+    static inline int refuses = 0;
+    static int device(int* d) { *d = 0; return 0; }
+    static int allocate(void** p, size_t bytes) { return refuses ? refuses : Device::allocate(p, bytes); }
+};
+using Sim = nolo::SimScratch<Device, Host>;
+int main() {
+    nolo::ScratchBlocks<Device> pool;
+    nolo::ScratchBlocks<Host> host_pool;
+    const int64_t most = Sim::kHostValues;
+    for (int refuses : {0, 2, 5})                       // 2: exhausted, 5: any other error
+        for (int64_t values : {int64_t(1), int64_t(7), most, most + 1, 3 * most})
+            for (int wanted = 0; wanted < 2; ++wanted)
+                for (int fails : {0, 7, 8}) {           // 7: of the launches, 8: of the wait
+                    pool.give_back();
+                    host_pool.give_back();
+                    CHECK(Fake::total == 0);
+                    Host::refuses = refuses;
+                    Device::copies = 0;
+                    std::vector<double> got(values, -1.0), stats(4, -1.0);
+                    {
+                        Sim s(pool, host_pool);
+                        CHECK(s.take(values, 1000) == 0);
+                        CHECK((uintptr_t)s.values() % 16 == 0 && (uintptr_t)s.scratch() % 16 == 0);
+                        CHECK((char*)s.scratch() >= (char*)(s.values() + values));
+                        double* in_place = s.values_in_place(wanted);
+                        CHECK((in_place != nullptr) == (wanted && !refuses && values <= most));
+                        for (int64_t i = 0; i < values; ++i) s.values()[i] = 0.5 * i;
+                        for (int64_t i = 0; in_place && i < values; ++i) in_place[i] = 0.5 * i;
+                        memset(s.scratch(), 255, 1000);
+                        for (int i = 0; i < 3; ++i) s.stats()[i] = 10.0 + i;
+                        Device::wait_fails = fails == 8 ? 8 : 0;
+                        CHECK(s.finish(fails == 7 ? 7 : 0, wanted ? got.data() : nullptr, stats.data(), 3, 0) == fails);
+                        Device::wait_fails = 0;
+                    }
+                    if (fails) {
+                        CHECK(Fake::total == 0);        // nothing of a call that failed is kept
+                        continue;
+                    }
+                    CHECK(stats == std::vector<double>({10.0, 11.0, 12.0, -1.0}));
+                    for (int64_t i = 0; i < values; ++i) CHECK(got[i] == (wanted ? 0.5 * i : -1.0));
+                    CHECK(Device::copies == (refuses != 0) + (wanted && (refuses || values > most)));
+                    const size_t kept = Fake::total;
+                    Sim again(pool, host_pool);
+                    CHECK(again.take(values, 1000) == 0 && Fake::total == kept);
+                }
+    pool.give_back();
+    host_pool.give_back();
+    CHECK(Fake::total == 0);
+    return 0;
+}
+""")
