@@ -22,11 +22,34 @@ struct Moments {
         mean += d * inv_k;
         m2 += d * (x - mean);
     }
-    // this one of n values, o of the m that follow (Chan, Golub, LeVeque: updating formulae, 1979)
-    __device__ __forceinline__ void join(const Moments& o, float n, float m) {
-        const float d = o.mean - mean, share = m / (n + m);
+    // this one of n values, o of the m that follow; share = m / (n + m), weight = n * share
+    // (Chan, Golub, LeVeque: updating formulae, 1979)
+    __device__ __forceinline__ void join(const Moments& o, float share, float weight) {
+        const float d = o.mean - mean;
         mean += d * share;
-        m2 += o.m2 + d * (n * share * d);      // (d * d may overflow where this does not)
+        m2 += o.m2 + d * (weight * d);         // (d * d may overflow where this does not)
+    }
+    static __device__ __forceinline__ Moments of_pair(float a, float b) {
+        const float d = b - a, half = 0.5f * d;
+        return {a + half, half * d};
+    }
+};
+
+// Moments of `rows` (1 to 4) values at once; those that are missing may be anything.  A part joins its workers by fours: a quarter of
+// the roundings in a row, whose errors do not cancel, and a quarter of the dependent operations of one worker after the other.  Relative
+// error of the returned mean against 64 bits, sixteen parts with single workers / four with fours (with single workers):
+// (64, 100 000) -7e-10 / 9e-10 (-8e-9), (32, 50 000) 0 / 4e-10 (-7e-9); at the same number of parts (1000, 100 000) 2e-8 / 4e-9.
+struct Quad {
+    bool second, third, fourth;
+    float share, weight;
+    __device__ __forceinline__ explicit Quad(int rows)
+        : second(rows > 1), third(rows > 2), fourth(rows > 3), share(fourth ? 0.5f : third ? 1.f / 3.f : 0.f),
+          weight(fourth ? 1.f : third ? 2.f / 3.f : 0.f) {}
+    __device__ __forceinline__ Moments moments(float a, float b, float c, float d) const {
+        Moments m = Moments::of_pair(a, second ? b : a);
+        const float x = third ? c : a;
+        m.join(Moments::of_pair(x, fourth ? d : x), share, weight);
+        return m;
     }
 };
 
@@ -74,7 +97,7 @@ __device__ __forceinline__ void finish(const double2* partial, int64_t count, in
 // CTAs would not fill the chip and whose threads would walk the workers one after the other.  FUSED: the
 // last CTA to leave its sums adds them up; `arrived` counts them and is zero before and after.
 template <int ITEMS, int PARTS, bool FUSED>
-__global__ void __launch_bounds__(kThreads, ITEMS == 4 ? 4 : 1)
+__global__ void __launch_bounds__(kThreads, ITEMS == 4 || PARTS > 1 ? 4 : 1)
 divergence_kernel(const float* phi, int W, int64_t stride, int64_t P, double2* partial, unsigned* arrived,
                   double* out) {
     constexpr int COLS = kThreads / PARTS;             // threads of one part
@@ -106,12 +129,24 @@ divergence_kernel(const float* phi, int W, int64_t stride, int64_t P, double2* p
         }
 #pragma unroll
         for (int i = 0; i < ROWS; ++i) {
-            const float inv_k = __frcp_rn((float)(w + i - w0 + 1));
+            if constexpr (PARTS > 1) {
+                static_assert(PARTS == 1 || ROWS == 4, "four rows at once");
+                if (i > 0 || !ok[0]) break;
+                const int n = w - w0, rows = w1 - w < 4 ? w1 - w : 4;
+                const Quad quad(rows);
+                const float share = (float)rows * __frcp_rn((float)(n + rows)), weight = (float)n * share;
+                acc[0][0].join(quad.moments(x[0][0].x, x[1][0].x, x[2][0].x, x[3][0].x), share, weight);
+                acc[0][1].join(quad.moments(x[0][0].y, x[1][0].y, x[2][0].y, x[3][0].y), share, weight);
+                acc[0][2].join(quad.moments(x[0][0].z, x[1][0].z, x[2][0].z, x[3][0].z), share, weight);
+                acc[0][3].join(quad.moments(x[0][0].w, x[1][0].w, x[2][0].w, x[3][0].w), share, weight);
+            } else {
+                const float inv_k = __frcp_rn((float)(w + i - w0 + 1));
 #pragma unroll
-            for (int it = 0; it < ITEMS; ++it) {
-                if (ok[it] && w + i < w1) {
-                    acc[it][0].push(x[i][it].x, inv_k); acc[it][1].push(x[i][it].y, inv_k);
-                    acc[it][2].push(x[i][it].z, inv_k); acc[it][3].push(x[i][it].w, inv_k);
+                for (int it = 0; it < ITEMS; ++it) {
+                    if (ok[it] && w + i < w1) {
+                        acc[it][0].push(x[i][it].x, inv_k); acc[it][1].push(x[i][it].y, inv_k);
+                        acc[it][2].push(x[i][it].z, inv_k); acc[it][3].push(x[i][it].w, inv_k);
+                    }
                 }
             }
         }
@@ -131,20 +166,22 @@ divergence_kernel(const float* phi, int W, int64_t stride, int64_t P, double2* p
                     n += (int)((int64_t)W * (p + 1) / PARTS) - (int)((int64_t)W * p / PARTS);
                     m += (int)((int64_t)W * (p + half + 1) / PARTS) - (int)((int64_t)W * (p + half) / PARTS);
                 }
+                const float share = (float)m / (float)(n + m), weight = (float)n * share;
 #pragma unroll
-                for (int e = 0; e < 4; ++e) acc[0][e].join(shared[threadIdx.x + half * COLS][e], (float)n, (float)m);
+                for (int e = 0; e < 4; ++e) acc[0][e].join(shared[threadIdx.x + half * COLS][e], share, weight);
             }
         }
     }
     double2 sum = make_double2(0.0, 0.0);              // of the standard deviations, of the variances
     if (part == 0) {
         const float inv_W = 1.0f / (float)W;
+        auto variance = [&](const Moments& m) { return PARTS > 1 ? m.m2 / (float)W : m.m2 * inv_W; };
         const int64_t full = P >> 2;
         const int ragged = (int)(P & 3);
 #pragma unroll
         for (int it = 0; it < ITEMS; ++it) {
             if (!ok[it]) continue;
-            float4 v = make_float4(acc[it][0].m2 * inv_W, acc[it][1].m2 * inv_W, acc[it][2].m2 * inv_W, acc[it][3].m2 * inv_W);
+            float4 v = make_float4(variance(acc[it][0]), variance(acc[it][1]), variance(acc[it][2]), variance(acc[it][3]));
             const int64_t q = q0 + it * COLS;
             if (q == full) {                           // the partial quad
                 if (ragged < 2) v.y = 0.f;
@@ -191,19 +228,20 @@ struct Shape {
 // SM, so that the last, part-filled wave of four weighs little ((128, 3e6) 247 us with one quad, 301 with four, which
 // are 1.2 waves); with few workers a CTA is soon done and their number weighs more, the one counter that they all
 // add to included: three per SM ((1, 2^22) 45 us with one quad, 29 with four, (12, 3e6) 57 / 53, (16, 3e6) 58 / 62).
-// Few are less than one per SM, or two where a part has 64 workers and more to walk; the counter makes more of them
-// dearer again.  us, with four per SM for few / now: (16, 100 000) 26.2 / 17.1, (64, 100 000) 29.7 / 21.0, (32, 50 000) 21.7 / 17.0,
-// (64, 390 625) 38.2 / 31.0, (1024, 390 625) 270 / 250, (1024, 24 414) 43.3 / 36.5; unparted (1024, 1000) 331, now 21.
+// Few are less than four per SM; for further parts than four less than one, unless a part has 64 workers and more to walk, for the
+// counter makes more of them dearer again.  us, with four per SM for few throughout / now: (16, 100 000) 26.2 / 15.3,
+// (64, 100 000) 29.4 / 18.9, (32, 50 000) 20.3 / 15.8, (40, 60 000) 21.7 / 15.7, (1024, 24 414) 41.8 / 39.6; unparted (1024, 1000) 331, now 21.
 // Four quads want four CTAs of 64 registers per SM: at 66
 // registers, three CTAs, (16, 2^26) measured 675 us instead of 622.  (Sums of each thread in float32 pairs instead of float64,
 // to save its conversions, measured slower: (2, 2e8) 330 -> 360.)
-constexpr int64_t kManyCtas = 148 * 8, kManyShortCtas = 148 * 3, kFewCtas = 148 * 2;
+constexpr int64_t kManyCtas = 148 * 8, kManyShortCtas = 148 * 3, kFewCtas = 148 * 4;
 constexpr int kShortMaxW = 12;
 Shape shape_for(int W, int64_t P) {
     Shape s = {4, 1};
     if (s.ctas(P) >= (W <= kShortMaxW ? kManyShortCtas : kManyCtas)) return s;
     s.items = 1;
-    while (s.parts < 32 && W >= 4 * s.parts && s.ctas(P) < (W >= 64 * s.parts ? kFewCtas : kFewCtas / 2)) s.parts *= s.parts == 16 ? 2 : 4;
+    while (s.parts < 32 && W >= 4 * s.parts && s.ctas(P) < (s.parts == 1 || W >= 64 * s.parts ? kFewCtas : kFewCtas / 4))
+        s.parts *= s.parts == 16 ? 2 : 4;
     return s;
 }
 
