@@ -30,7 +30,7 @@ __device__ __forceinline__ double2 load_written(const double2* p) {
 // The next kernel may be a caller's, and what such kernels read ahead of their wait is what the kernel before them is
 // not expected to write: weights.  So the kernels that write the state never call this (their successor starts when all
 // their CTAs are done, as after any kernel that does not), and the others that can end a call do so behind their own
-// wait.  Only a draw, which the same call follows with a kernel that waits, calls it earlier.
+// wait, if at all.  Only a draw, which the same call follows with a kernel that waits, calls it earlier.
 __device__ __forceinline__ void let_successor_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Asks for memory to be brought to L2: the 128-byte line that holds *p, or a range (16-byte aligned, a multiple of

@@ -689,80 +689,137 @@ __device__ __forceinline__ void store_mean4(double* out, double a, double b, dou
     }
 }
 
-// ITEMS quads per thread: small subgroups have few rows to keep in flight per quad, so each thread takes two quads up
-// to n = 4.  PARTS groups of the CTA's threads share out the members of the same columns and join their sums in
-// shared memory, for states with few columns, whose CTAs would not fill the chip and whose threads would walk the members
-// one after the other.
-template <int ITEMS, int PARTS, bool WIDE>
+__device__ __forceinline__ void copy_ahead16(void* to, const void* from) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(to)), "l"(from) : "memory");
+}
+
+// The columns of the partial quad, one warp per column.
+__device__ __forceinline__ void mean_tail(const float* phi, const int32_t* members, int n, int64_t stride, int64_t P, double* mean,
+                                          double inv_n) {
+    const int64_t c = (P & ~int64_t(3)) + (threadIdx.x >> 5);
+    if (c >= P) return;
+    double t = 0.0;
+#pragma unroll 4
+    for (int j = threadIdx.x & 31; j < n; j += 32) t += (double)phi[(int64_t)load_written(members + j) * stride + c];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if ((threadIdx.x & 31) == 0) mean[c] = t * inv_n;
+}
+
+// A thread adds the members of ITEMS quads, 256 quads apart: small subgroups have few rows to keep in flight per
+// quad, so each thread takes two quads up to n = 4.
+template <int ITEMS, bool WIDE>
 __global__ void __launch_bounds__(kThreads)
 group_mean_kernel(const float* phi, const int32_t* perm, int n, int64_t stride,
                   int64_t P, double* __restrict__ mean, int64_t mean_stride, double inv_n) {
-    constexpr int COLS = kThreads / PARTS;             // threads of one part
     wait_for_predecessors();
     let_successor_start();
     const int g = blockIdx.y;
     const int32_t* members = perm + (int64_t)g * n;
+    mean += (int64_t)g * mean_stride;
     const int tail = (P & 3) != 0;
-    if (tail && blockIdx.x == 0) {            // the partial quad, one warp per column
-        const int64_t c = (P & ~int64_t(3)) + (threadIdx.x >> 5);
-        if (c >= P) return;
-        double t = 0.0;
-#pragma unroll 4
-        for (int j = threadIdx.x & 31; j < n; j += 32) t += (double)phi[(int64_t)load_written(members + j) * stride + c];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-        if ((threadIdx.x & 31) == 0) mean[(int64_t)g * mean_stride + c] = t * inv_n;
-        return;
-    }
-    const int part = threadIdx.x / COLS;
-    const int64_t q0 = (int64_t)(blockIdx.x - tail) * (COLS * ITEMS) + threadIdx.x % COLS;
+    if (tail && blockIdx.x == 0) return mean_tail(phi, members, n, stride, P, mean, inv_n);
+    const int64_t q0 = (int64_t)(blockIdx.x - tail) * (kThreads * ITEMS) + threadIdx.x;
     const int64_t quads = P >> 2;
     PairSum s[ITEMS];
 #pragma unroll
     for (int it = 0; it < ITEMS; ++it) s[it].clear();
-    for (int j = part; j < n; j += PARTS * kMeanUnroll) {
+    for (int j = 0; j < n; j += kMeanUnroll) {
         float4 v[ITEMS][kMeanUnroll];
 #pragma unroll
         for (int i = 0; i < kMeanUnroll; ++i) {
-            if (j + i * PARTS < n) {
-                const float4* row = reinterpret_cast<const float4*>(phi + (int64_t)load_written(members + j + i * PARTS) * stride);
+            if (j + i < n) {
+                const float4* row = reinterpret_cast<const float4*>(phi + (int64_t)load_written(members + j + i) * stride);
 #pragma unroll
                 for (int it = 0; it < ITEMS; ++it) {
-                    const int64_t q = q0 + (int64_t)it * COLS;
+                    const int64_t q = q0 + (int64_t)it * kThreads;
                     if (q < quads) v[it][i] = __ldcs(row + q);
                 }
             }
         }
 #pragma unroll
         for (int i = 0; i < kMeanUnroll; ++i) {
-            if (j + i * PARTS < n) {
+            if (j + i < n) {
 #pragma unroll
                 for (int it = 0; it < ITEMS; ++it)
-                    if (q0 + (int64_t)it * COLS < quads) s[it].add(v[it][i]);
+                    if (q0 + (int64_t)it * kThreads < quads) s[it].add(v[it][i]);
             }
         }
-    }
-    if constexpr (PARTS > 1) {
-        __shared__ PairSum shared[PARTS][COLS];
-        shared[part][threadIdx.x % COLS] = s[0];
-        for (int half = PARTS / 2; half >= 1; half /= 2) {         // part p takes over the members of part p + half
-            __syncthreads();
-            if (part < half) {
-                s[0].add(shared[part + half][threadIdx.x % COLS]);
-                shared[part][threadIdx.x % COLS] = s[0];
-            }
-        }
-        if (part > 0) return;
     }
 #pragma unroll
     for (int it = 0; it < ITEMS; ++it) {
-        const int64_t q = q0 + (int64_t)it * COLS;
+        const int64_t q = q0 + (int64_t)it * kThreads;
         if (q < quads) {
-            store_mean4<WIDE>(mean + (int64_t)g * mean_stride + 4 * q,
+            store_mean4<WIDE>(mean + 4 * q,
                               ((double)s[it].hi.x + (double)s[it].lo.x) * inv_n, ((double)s[it].hi.y + (double)s[it].lo.y) * inv_n,
                               ((double)s[it].hi.z + (double)s[it].lo.z) * inv_n, ((double)s[it].hi.w + (double)s[it].lo.w) * inv_n);
         }
     }
+}
+
+// The same for few columns, whose CTAs would not fill the chip and whose threads would walk the members in many latencies:
+// the CTA's threads bring the members of 4 QUADS columns to shared memory, three stages of 8 KB ahead, and a thread per column adds
+// them in the order of the kernel above, so that no bit depends on the number of columns.  Bound by latency up to about a
+// hundred members, then by the additions, whose chain is 4 cycles and whose 7 instructions a member has in each column's thread
+// alone.  (Groups of threads that share out the members and join their sums in a tree took 126 us at (1024, 37 888) and gave other
+// bits than a thread per quad; rows brought through registers, one stage of 16 KB ahead, 189.)
+//
+// It does not let its successor start early: the step that follows would find the SMs set up for this kernel's shared memory and
+// keep them so, with little L1 left for its loads in flight (prepare and prepared step (1024, 24 415) 192 us, now 154,
+// (64, 300 000) 118, now 95).
+constexpr int kMeanStages = 4, kMeanStageQuads = 2 * kThreads;
+
+template <int QUADS>
+__global__ void __launch_bounds__(kThreads)
+staged_mean_kernel(const float* phi, const int32_t* perm, int n, int64_t stride, int64_t P, double* __restrict__ mean,
+                   int64_t mean_stride, double inv_n) {
+    constexpr int COLS = 4 * QUADS, ROWS = kMeanStageQuads / QUADS, HALF = ROWS / 2;
+    __shared__ float4 staged[kMeanStages][ROWS][QUADS];
+    wait_for_predecessors();
+    const int g = blockIdx.y;
+    const int32_t* members = perm + (int64_t)g * n;
+    mean += (int64_t)g * mean_stride;
+    const int tail = (P & 3) != 0;
+    if (tail && blockIdx.x == 0) return mean_tail(phi, members, n, stride, P, mean, inv_n);
+    const int ql = threadIdx.x % QUADS, row = threadIdx.x / QUADS;
+    const int64_t first = (int64_t)(blockIdx.x - tail) * QUADS, quads = P >> 2;
+    const bool ok = first + ql < quads;
+    phi += 4 * (first + ql);
+    int m0[kMeanStages - 1], m1[kMeanStages - 1];              // this thread's members of the stages ahead
+#pragma unroll
+    for (int u = 0; u < kMeanStages - 1; ++u) {
+        const int j = u * ROWS + row;
+        if (j < n) m0[u] = load_written(members + j);
+        if (j + HALF < n) m1[u] = load_written(members + j + HALF);
+    }
+    auto ahead = [&](int j0, int slot, int a, int b) {
+        if (ok && j0 + row < n) copy_ahead16(&staged[slot][row][ql], phi + (int64_t)a * stride);
+        if (ok && j0 + row + HALF < n) copy_ahead16(&staged[slot][row + HALF][ql], phi + (int64_t)b * stride);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+#pragma unroll
+    for (int u = 0; u < kMeanStages - 1; ++u) ahead(u * ROWS, u, m0[u], m1[u]);
+    float hi = 0.f, lo = 0.f;
+    int slot = 0;
+    for (int j0 = 0; j0 < n; j0 += ROWS) {
+        const int next = j0 + (kMeanStages - 1) * ROWS;
+        int a = 0, b = 0;
+        if (next + row < n) a = load_written(members + next + row);
+        if (next + row + HALF < n) b = load_written(members + next + row + HALF);
+        asm volatile("cp.async.wait_group %0;" ::"n"(kMeanStages - 2) : "memory");
+        __syncthreads();
+        ahead(next, (slot + kMeanStages - 1) % kMeanStages, a, b);      // where the stage before this one was
+        if (threadIdx.x < COLS) {
+            const float* x = reinterpret_cast<const float*>(staged[slot]) + threadIdx.x;
+            const int count = n - j0 < ROWS ? n - j0 : ROWS;
+#pragma unroll 8
+            for (int j = 0; j < count; ++j) two_sum(hi, lo, x[j * COLS]);
+        }
+        slot = (slot + 1) % kMeanStages;
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    const int64_t c = 4 * first + threadIdx.x;
+    if (threadIdx.x < COLS && c < 4 * quads) mean[c] = ((double)hi + (double)lo) * inv_n;
 }
 
 // ---- launches ---------------------------------------------------------------------------
@@ -890,37 +947,35 @@ cudaError_t dispatch(KArgs& k, bool draw, int groups, cudaStream_t stream) {
 
 }  // namespace
 
-// Parts: as many as give the chip two CTAs per SM while every part keeps four rounds of loads, or half a CTA per SM while
-// it keeps a member.  us of prepare and prepared step, unparted /
-// in parts: n = W, float32, (32, 3125) 15.0 / 8.6, (96, 66 666) 46.9 / 32.3, (256, 25 000) 87 / 41, (1024, 1563) 232 / 33.
-constexpr int64_t kMeanFewCtas = 148 * 2;
+// Few columns: at most two CTAs of 256 quads per SM (one for fewer than 32 members, which a thread walks in few latencies).  us of a draw
+// and the means (the draw alone 5.7), a thread per quad / staged, one subgroup of n, quads: (32, 18 944) 7.8 / 5.8, (20, 75 776) 7.6 / 9.7, (32, 75 776) 11.4 /
+// 10.6, (32, 303 104) 30 / 36, (64, 9472) 13.2 / 6.0, (128, 37 888) 34 / 15, (256, 18 944) 65 / 19, (1024, 37 888) 271 / 111.
+// Row pieces of 128 bytes where CTAs of 512-byte ones would leave SMs idle: (1024, 1024) 25.9 / 14.0, (256, 1024) 7.6 / 5.9,
+// (256, 4096) 7.7 / 8.6.
+constexpr int64_t kMeanFewQuads = 148 * 256, kMeanNarrowCtas = 148 * 2;
+constexpr int kMeanDirectMaxN = 16, kMeanManyN = 32;
 
 cudaError_t launch_group_mean(const float* phi, const int32_t* perm, int W, int n, int64_t stride, int64_t P,
                               double* mean, int64_t mean_stride, cudaStream_t stream) {
     if (P <= 0 || W <= 0) return cudaSuccess;
-    const int items = n <= 4 ? 2 : 1, groups = W / n;
+    const int groups = W / n;
     const int64_t quads = P >> 2;
-    int parts = 1;
-    while (items == 1 && parts < 32 && n >= 4 * parts &&
-           (quads * parts + kThreads - 1) / kThreads * groups < (n >= 16 * parts ? kMeanFewCtas : kMeanFewCtas / 4))
-        parts *= parts == 16 ? 2 : 4;
-    const int64_t per_cta = (int64_t)(kThreads / parts) * items;
-    const int64_t tiles = (quads + per_cta - 1) / per_cta + ((P & 3) != 0);
-    if (tiles > 0x7fffffffll || groups > 65535) return cudaErrorInvalidConfiguration;
-    dim3 grid((unsigned)tiles, (unsigned)groups);
+    if (groups > 65535) return cudaErrorInvalidConfiguration;
     const double inv_n = 1.0 / (double)n;
     // rows of the means are 32-byte aligned when the base is (the stride is a multiple of 64 bytes)
     const bool wide = (reinterpret_cast<uintptr_t>(mean) & 31u) == 0;
-    auto launch = [&](auto kernel) {
-        return launch_overlapped(kernel, grid, kThreads, 0, stream, phi, perm, n, stride, P, mean, mean_stride, inv_n);
+    auto launch = [&](auto kernel, int64_t quads_per_cta) {
+        const int64_t tiles = (quads + quads_per_cta - 1) / quads_per_cta + ((P & 3) != 0);
+        if (tiles > 0x7fffffffll) return cudaErrorInvalidConfiguration;
+        return launch_overlapped(kernel, dim3((unsigned)tiles, (unsigned)groups), kThreads, 0, stream, phi, perm, n, stride, P, mean,
+                                 mean_stride, inv_n);
     };
-    if (items == 2) return launch(wide ? group_mean_kernel<2, 1, true> : group_mean_kernel<2, 1, false>);
-    switch (parts) {
-        case 1: return launch(wide ? group_mean_kernel<1, 1, true> : group_mean_kernel<1, 1, false>);
-        case 4: return launch(wide ? group_mean_kernel<1, 4, true> : group_mean_kernel<1, 4, false>);
-        case 16: return launch(wide ? group_mean_kernel<1, 16, true> : group_mean_kernel<1, 16, false>);
-        default: return launch(wide ? group_mean_kernel<1, 32, true> : group_mean_kernel<1, 32, false>);
+    if (n <= 4) return launch(wide ? group_mean_kernel<2, true> : group_mean_kernel<2, false>, 2 * kThreads);
+    if (n > kMeanDirectMaxN && quads * groups <= (n < kMeanManyN ? 1 : 2) * kMeanFewQuads) {
+        if ((quads + 7) / 8 * groups <= kMeanNarrowCtas) return launch(staged_mean_kernel<8>, 8);
+        return launch(staged_mean_kernel<32>, 32);
     }
+    return launch(wide ? group_mean_kernel<1, true> : group_mean_kernel<1, false>, kThreads);
 }
 
 // Drawing in the kernel saves the launch of the draw and costs every CTA the draw's 0.3 us.  It is the faster, for a call

@@ -51,10 +51,11 @@ def test_bits_do_not_depend_on_the_number_of_columns(nolo, W, n, P, bf16):
     assert all(torch.equal(a, b) for a, b in zip(*got))
 
 
-# 1, 4, 16 or 32 parts of a CTA share out the members of a column.
+# A thread per quad or the members staged in pieces of 8 or 32 quads, in one to many stages of 64 or 16 rows.
 @pytest.mark.parametrize("W,n,P", [(5, 5, 3), (7, 7, 1030), (15, 15, 2051), (16, 16, 4096), (63, 63, 517), (64, 64, 514), (65, 65, 4097),
-                                   (130, 130, 6), (24, 12, 80_003), (64, 32, 40_001), (128, 128, 20_003)])
-def test_subgroup_means_in_parts(nolo, W, n, P):
+                                   (130, 130, 6), (24, 12, 80_003), (64, 32, 40_001), (128, 128, 20_003),
+                                   (17, 17, 4 * 2368 + 1), (34, 17, 4 * 1185), (1024, 1024, 9475), (2049, 2049, 260), (193, 193, 30_002)])
+def test_subgroup_means_of_few_columns(nolo, W, n, P):
     phi, theta, delta = synth.make_state(W, P, n, pad_value=float("nan"))
     dev = [x.cuda() for x in (phi, theta, delta)]
     mean = torch.full((W // n, synth.padded_stride(P, 8)), float("nan"), dtype=torch.float64, device="cuda")
@@ -69,6 +70,30 @@ def test_subgroup_means_in_parts(nolo, W, n, P):
     np.testing.assert_allclose(got[:, :P], O.subgroup_mean_phi(x, O.draw_groups(3, 3, W, n), n), rtol=1e-12,
                                atol=1e-12 * float(np.abs(x).max()))
     assert np.isnan(got[:, P:]).all()
+
+
+@pytest.mark.parametrize("W,n", [(5, 5), (16, 16), (17, 17), (34, 17), (32, 32), (64, 64), (96, 48), (255, 255), (256, 256), (1024, 1024), (2500, 1250)])
+def test_subgroup_means_do_not_depend_on_the_number_of_columns(nolo, W, n):
+    """A state cut by columns has the means of the whole, bit for bit: 8 quads, and both sides of each line."""
+    groups = W // n
+    few = 148 * 256 * (1 if n < 32 else 2) // groups
+    sizes = [32, 4 * (148 * 2 * 8 // groups), 4 * (148 * 2 * 8 // groups + 1), 4 * few, 4 * few + 4]
+    cols = max(sizes)
+    phi = 0.02 * torch.randn(W, synth.padded_stride(cols), device="cuda", generator=torch.Generator("cuda").manual_seed(n))
+    z, d = torch.zeros_like(phi), torch.zeros_like(phi)
+    got = []
+    for P in sizes:
+        mean = torch.full((groups, synth.padded_stride(P, 8)), float("nan"), dtype=torch.float64, device="cuda")
+        h = nolo.nolo_create(W, n, P, 1, *HP)
+        nolo.nolo_bind_state(h, phi, z, d)
+        nolo.nolo_bind_prepared(h, mean)
+        nolo.nolo_outer_prepare(h, 3, 3)
+        torch.cuda.synchronize()
+        nolo.nolo_destroy(h)
+        got.append(mean)
+    whole = got[sizes.index(cols)]
+    for P, mean in zip(sizes, got):
+        assert torch.equal(mean[:, :P], whole[:, :P])
 
 
 @pytest.mark.parametrize("W,P", [(63, 1024 * 147), (64, 1024 * 147), (64, 1024 * 295 + 1), (16, 1024 * 148), (15, 1024 * 100 + 3)])
