@@ -35,22 +35,25 @@ constexpr uint64_t kDomainStraggler = 4;
 // the time of the longest way down, which is found from below like the longest way up.  So a trial is two sums of
 // longest ways, and no time is kept for a second sweep.
 //
-// `lanes` lanes (a power of two, at most 32 and W / 2) take one direction of one trial.  Every lane has a subtree of W / lanes
+// `lanes` lanes (a power of two, at most kTreeMostLanes and W / 2) take one direction of one trial.  Every lane has a subtree of W / lanes
 // leaves, whose blocks it visits children first, with the finished halves of what is above them on a stack
 // of its own; then every lane makes one of the `lanes` blocks of the nodes below 4 lanes, which they reduce by shuffles.
 // So all lanes work all the time and nothing waits for another warp, but for the two directions of a trial
-// of 32 lanes, which meet every kTreeRounds trials.  What Philox makes of a block's number is the same for all trials and is kept (LEAD).
+// of 32 lanes, which meet every kTreeRounds trials.  Where few trials leave most of the chip idle, several warps share a direction and
+// meet in shared memory for the nodes below 2 lanes / 32 (WIDE): (2048, 148) 66 -> 28 us, (4096, 148) 108 -> 34 (46 and
+// 50 with 256 threads that swept the nodes).  What Philox makes of a block's number is the same for all trials and is kept (LEAD).
 // Bound by the log-normal times: 363 thread-instructions per four (those of the stragglers 317); a sweep up and one down
 // over nodes in shared memory with barriers between the levels took 464.  Whole call, (W, trials): (1024, 20 000) 0.51 -> 0.37 ms,
 // (256, 100 000) 0.77 -> 0.50, (64, 300 000) 0.70 -> 0.48 (0.3 of it the copy of the trials).
 constexpr int kTreeThreads = 512, kTreeWarps = kTreeThreads / 32, kTreeRounds = 32;
+constexpr int kTreeMostLanes = kTreeThreads / 2;      // both directions of a trial in a CTA
 constexpr int kLeadMaxW = 1024;      // 32 KB of shared memory
 constexpr int kTreeMostDepth = 10;    // log2(NOLO_MAX_WORKERS / 4)
 static_assert(4 << kTreeMostDepth == NOLO_MAX_WORKERS, "a lane's subtree has at most NOLO_MAX_WORKERS / 4 leaf blocks");
 
 __device__ __forceinline__ double later(double a, double b) { return a > b ? a : b; }      // no NaN here
 
-template <bool TAME, bool LEAD>
+template <bool TAME, bool LEAD, bool WIDE>
 __global__ void __launch_bounds__(kTreeThreads, 2)
 tree_allreduce_kernel(int W, int lanes, int64_t trials, LogNormal q, uint64_t seed, double* __restrict__ out, unsigned* arrived) {
     extern __shared__ double2 dynamic[];
@@ -74,14 +77,19 @@ tree_allreduce_kernel(int W, int lanes, int64_t trials, LogNormal q, uint64_t se
         }
     }
     __syncthreads();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, mine = lane % lanes;
-    // A warp's tasks of a round: one, or both directions of 16 / lanes trials next to each other.
-    const int64_t per_warp = 32 / lanes, workers = (int64_t)gridDim.x * kTreeWarps;
-    const int64_t rounds = (2 * trials + per_warp * workers - 1) / (per_warp * workers);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, mine = threadIdx.x % lanes;
+    // A warp's tasks of a round: one, or both directions of 16 / lanes trials next to each other.  WIDE: the CTA's, both directions of
+    // its trials next to each other.
+    const int64_t per_warp = WIDE ? 1 : 32 / lanes, per_cta = kTreeThreads / lanes;
+    const int64_t rounds = (2 * trials + per_cta * gridDim.x - 1) / (per_cta * gridDim.x);
     for (int64_t round = 0; round < rounds; ++round) {
         int direction;
         int64_t trial;
-        if (lanes == 32) {
+        if (WIDE) {
+            const int64_t task = (round * gridDim.x + blockIdx.x) * per_cta + threadIdx.x / lanes;
+            direction = (int)(task & 1);
+            trial = task >> 1;
+        } else if (lanes == 32) {
             direction = warp & 1;
             trial = (round * (kTreeWarps / 2) + (warp >> 1)) * gridDim.x + blockIdx.x;
         } else {
@@ -90,7 +98,7 @@ tree_allreduce_kernel(int W, int lanes, int64_t trials, LogNormal q, uint64_t se
             trial = task >> 1;
         }
         double way = 0.0;
-        if (lanes < 32 || trial < trials) {
+        if (WIDE || lanes < 32 || trial < trials) {
             const PhiloxOfC1 of_trial = philox_of_c1(trial, direction, seed);
             auto words = [&](int block, int slot) {
                 if constexpr (LEAD) {
@@ -130,21 +138,39 @@ tree_allreduce_kernel(int W, int lanes, int64_t trials, LogNormal q, uint64_t se
             if (W > 2) lognormal2<TAME>(tables, x.w0, x.w1, q, t[0], t[1]);
             lognormal2<TAME>(tables, x.w2, x.w3, q, t[2], t[3]);
             __syncwarp();
-            double2* own = stack - lane;                           // of the warp, [2][32]: the times above nodes 2i and 2i + 1
-            auto pair = [&](int i) -> double2& { return own[(i & 1) * kTreeThreads + (lane - mine) + (i >> 1)]; };
+            double2* own = stack - mine;                           // of the lanes, [2][lanes]: the times above nodes 2i and 2i + 1
+            auto pair = [&](int i) -> double2& { return own[(i & 1) * kTreeThreads + (i >> 1)]; };
             pair(2 * mine) = make_double2(t[0], t[1]);
             pair(2 * mine + 1) = make_double2(t[2], t[3]);
-            __syncwarp();
+            if constexpr (WIDE) __syncthreads();
+            else __syncwarp();
             auto above = [&](int node) { return reinterpret_cast<const double*>(&pair(node >> 1))[node & 1]; };
             const double2 leaf = pair(lanes + mine);
             way = later(x0 + leaf.x, x1 + leaf.y);
-            for (int o = 1; o < lanes; o <<= 1) {
+            for (int o = 1; o < (WIDE ? 32 : lanes); o <<= 1) {
                 way += above((lanes + mine) / o);
                 way = later(way, __shfl_xor_sync(0xffffffffu, way, o));
             }
             __syncwarp();
+            if constexpr (WIDE) {                                  // the nodes that a warp each has come to
+                const int warps = lanes / 32;
+                if (lane == 0) ways[0][warp] = way;
+                __syncthreads();
+                if (mine < 32) {
+                    const int i = lane % warps;
+                    way = ways[0][warp + i];
+                    for (int o = 1; o < warps; o <<= 1) {
+                        way += above((warps + i) / o);
+                        way = later(way, __shfl_xor_sync(0xffffffffu, way, o));
+                    }
+                    if (lane == 0) ways[1][threadIdx.x / lanes] = way;
+                }
+                __syncthreads();
+            }
         }
-        if (lanes < 32) {
+        if (WIDE) {
+            if (mine == 0 && direction == 0 && trial < trials) out[trial] = ways[1][threadIdx.x / lanes] + ways[1][threadIdx.x / lanes + 1];
+        } else if (lanes < 32) {
             way += __shfl_xor_sync(0xffffffffu, way, lanes);
             if (lane % (2 * lanes) == 0 && trial < trials) out[trial] = way;
         } else {
@@ -639,7 +665,7 @@ cudaError_t launch_tree_allreduce(int W, double mu, double sigma, int64_t trials
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
     if (e != cudaSuccess) return e;
     double least = 0.0;
-    for (int l = 1, log2 = 0; l <= W / 2 && l <= 32; l *= 2, ++log2) {
+    for (int l = 1, log2 = 0; l <= W / 2 && l <= kTreeMostLanes; l *= 2, ++log2) {
         const int64_t threads = (int64_t)sms * 2 * kTreeThreads;
         const double cost = (double)((2 * trials * l + threads - 1) / threads) * (W / (2 * l) + 0.14 * log2);
         if (l == 1 || cost <= least) {
@@ -650,8 +676,10 @@ cudaError_t launch_tree_allreduce(int W, double mu, double sigma, int64_t trials
     int depth = 2;                       // of a lane's stack, as much as it needs for the last exchange
     for (int leaves = W / (4 * lanes); leaves > 4; leaves /= 2) ++depth;
     const size_t smem = sizeof(double2) * depth * kTreeThreads + (lead ? sizeof(PhiloxOfC0) * W : 0);
-    auto kernel = tame ? (lead ? tree_allreduce_kernel<true, true> : tree_allreduce_kernel<true, false>)
-                       : (lead ? tree_allreduce_kernel<false, true> : tree_allreduce_kernel<false, false>);
+    auto kernel = lanes > 32 ? (tame ? (lead ? tree_allreduce_kernel<true, true, true> : tree_allreduce_kernel<true, false, true>)
+                                     : (lead ? tree_allreduce_kernel<false, true, true> : tree_allreduce_kernel<false, false, true>))
+                             : (tame ? (lead ? tree_allreduce_kernel<true, true, false> : tree_allreduce_kernel<true, false, false>)
+                                     : (lead ? tree_allreduce_kernel<false, true, false> : tree_allreduce_kernel<false, false, false>));
     // the most that any call needs (lanes = 1), so that calls of different sizes from several threads do not undo each other's
     const int most_smem = (int)sizeof(double2) * kTreeMostDepth * kTreeThreads + (lead ? (int)sizeof(PhiloxOfC0) * kLeadMaxW : 0);
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most_smem);

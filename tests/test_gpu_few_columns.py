@@ -141,6 +141,19 @@ def test_tree_lanes(nolo, W, many):
         np.testing.assert_allclose(per[first:first + count], want, rtol=1e-11)
 
 
+# 64 to 256 lanes, of several warps, in one round and several; the last trials of a CTA missing.
+@pytest.mark.parametrize("W,trials", [(128, 148), (256, 300), (512, 1), (1024, 5), (1024, 601), (2048, 149), (2048, 1593), (4096, 3), (4096, 90),
+                                      (4096, 1501)])
+@pytest.mark.parametrize("sigma", [0.9, 90.0])
+def test_tree_lanes_of_several_warps(nolo, W, trials, sigma):
+    mean, _, per = nolo.nolo_sim_tree_allreduce(W, 0.1, sigma, trials, 17, return_trials=True)
+    assert per.shape == (trials,) and (per > 0).all() and mean == pytest.approx(per.mean(), rel=1e-13)
+    for first in {0, trials // 2, max(0, trials - 3)}:
+        count = min(3, trials - first)
+        want = [_tree(W, s, 0.1, sigma, 17) for s in range(first, first + count)]
+        np.testing.assert_allclose(per[first:first + count], want, rtol=1e-11)
+
+
 def _tree(W, trial, mu, sigma, seed):
     """Completion of one trial, level by level from the oracle's message times."""
     up, down = (L.message_times(W, trial, phase, mu, sigma, seed) for phase in (0, 1))
