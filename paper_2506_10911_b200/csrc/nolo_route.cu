@@ -211,18 +211,25 @@ cudaError_t launch_copy_probe(const void* in, void* out, int64_t bytes, cudaStre
 
 // Drawing in the copy saves the launch of the draw, lets the copy ask for its data ahead of its wait, and costs every
 // CTA the draw, 0.3 us and the more the more replicas there are.  It is the faster, for a call alone and for calls that follow
-// each other, as long as the grid is few waves, and for few replicas long after.  us alone, drawn in the copy / by a kernel ahead:
+// each other, as long as the grid is few waves, and for few replicas long after if the CTAs' tiles are filled to four fifths.  us alone,
+// drawn in the copy / by a kernel ahead:
 // 6 MB 10.2 / 11.3, 134 MB (multiples of 32 bytes) 47.1 / 48.1, 67 MB of other blocks 28.7 / 29.7.  There and back, 8 replicas:
 // 140 MB a way 85.8 / 90.5, 420 MB 240 / 245, 944 MB 536 / 543, at odd offsets 73 MB 46.2 / 50.3, 94 MB 59.2 / 62.5, 126 MB 79.1 /
-// 80.4; 32 replicas: 420 MB 255 / 245, at odd offsets 84 MB 58.9 / 56.8.
+// 80.4; 32 replicas: 420 MB 255 / 245, at odd offsets 84 MB 58.9 / 56.8.  300 MB in blocks of 2 KB 611 / 246, 8 KB (half a tile) 220 /
+// 189, 16 KB 175 / 184, 18 KB (two tiles) 199 / 184, 24 KB 180 / 183, 32 KB 175 / 182; 97 MB at odd offsets, 8 KB 87.9 / 80.6, 12 KB 71.4 / 70.4,
+// 16 KB 64.4 / 67.1, 33 KB (three tiles) 69.9 / 67.6, 66 KB (five) 64.4 / 65.3.  The lines of 1 GB and 100 MB are where it was measured
+// to; the gain beyond is a percent.
 constexpr int kFewReplicas = 8;
 constexpr int64_t kDrawMaxBytes = 64ll << 20, kDrawMaxBytesFew = 100ll << 20;
 constexpr int64_t kDrawMaxBytesWide = 128ll << 20, kDrawMaxBytesWideFew = 1024ll << 20;   // for multiples of 32 bytes
+constexpr int64_t kDrawTile = 16 << 10;           // bytes per CTA of every copy that draws
 
 bool route_draws(const RouteArgs& a) {
     const int64_t block = a.E * a.elem_size, bytes = (int64_t)a.B * a.R * a.K * block;
-    if (block % 32 == 0) return a.R <= 32 && bytes <= (a.R <= kFewReplicas ? kDrawMaxBytesWideFew : kDrawMaxBytesWide);
-    return a.R <= 32 && bytes <= (a.R <= kFewReplicas ? kDrawMaxBytesFew : kDrawMaxBytes);
+    const int64_t tiles = (block + kDrawTile - 1) / kDrawTile;
+    const bool wide = block % 32 == 0, few = a.R <= kFewReplicas && 5 * block >= 4 * tiles * kDrawTile;
+    const int64_t most = wide ? (few ? kDrawMaxBytesWideFew : kDrawMaxBytesWide) : (few ? kDrawMaxBytesFew : kDrawMaxBytes);
+    return a.R <= 32 && bytes <= most;
 }
 
 template <typename V, int THREADS, int N>
@@ -230,6 +237,7 @@ cudaError_t launch_shape(const CopyArgs& c, bool draw, cudaStream_t stream) {
     constexpr int64_t tile = (int64_t)THREADS * N * (sizeof(V) < 16 ? 16 : sizeof(V));
     const int64_t tiles = (c.bytes + tile - 1) / tile, rk = (int64_t)c.R * c.K;
     if (tiles > 0x7fffffffll) return cudaErrorInvalidConfiguration;
+    if (draw && tile != kDrawTile) return cudaErrorInvalidValue;
     const dim3 grid((unsigned)tiles, (unsigned)(rk < 65535 ? rk : 65535), (unsigned)(c.B < 65535 ? c.B : 65535));
     return launch_overlapped(draw ? route_copy_kernel<V, THREADS, N, true> : route_copy_kernel<V, THREADS, N, false>, grid,
                              THREADS, 0, stream, c);

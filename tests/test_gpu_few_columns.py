@@ -248,23 +248,30 @@ def test_calls_of_different_sizes_from_several_threads(nolo):
     assert not bad
 
 
-# Copies draw for themselves up to 1 GB, of blocks that are no multiple of 32 bytes 100 MB, for up to 8 replicas (128 and 64 MB
-# for more): both sides of each line.
-@pytest.mark.parametrize("W,E", [(8, 1 << 24), ((8), (1 << 24) + 8), (8, 100 * 32768 - 1), (8, 100 * 32768 + 1), (7, 3_000_000), (9, 3_000_001)])
-def test_routing_at_the_sizes_where_copies_stop_drawing(nolo, W, E):
-    stages, K = (3, 2) if E > 1 << 23 else (3, 1)
-    acts = torch.randint(-2**31, 2**31 - 1, (stages - 1, W, K, E), dtype=torch.int32, device="cuda").view(torch.float32)
+# Copies draw for themselves up to 1 GB, of blocks that are no multiple of 32 bytes 100 MB, for up to 8 replicas and tiles of 16 KB that
+# are filled to four fifths (128 and 64 MB otherwise): both sides of each line, E float32 elements in each of 2 boundaries x K x W.
+@pytest.mark.parametrize("W,K,E,draws", [
+    (8, 1, 1 << 24, True), (8, 1, (1 << 24) + 8, False), (8, 1, 50 * 32768 - 1, True), (8, 1, 50 * 32768 + 1, False),
+    (9, 1, 932_067, True), (9, 1, 932_069, False), (9, 1, 1_864_128, True), (9, 1, 1_864_136, False), (7, 1, 3_000_000, True), (3, 1, 4_000_001, True),
+    (8, 3000, 1000, False), (4, 8000, 512, True), (4, 8200, 512, False), (8, 700, 3280, True), (8, 700, 3272, False), (2, 1000, 4104, True),
+    (6, 700, 4104, False), (8, 300, 3277, True), (8, 400, 3277, True), (8, 400, 3275, False), (3, 900, 4099, False), (5, 2, 1_200_001, True)])
+def test_routing_at_the_sizes_where_copies_stop_drawing(nolo, W, K, E, draws):
+    stages = 3
+    acts = torch.randint(-2**31, 2**31 - 1, (stages - 1, W, K, E), dtype=torch.int32, device="cuda")
     out, back = torch.zeros_like(acts), torch.zeros_like(acts)
     h = nolo.nolo_create(W, 1, 8, stages, *HP)
-    nolo.nolo_bind_route(h, W * K, E, out, True)
-    nolo.nolo_route(h, 11, 3, acts)
+    nolo.nolo_bind_route(h, W * K, E, out.view(torch.float32), True)
+    before = nolo.nolo_launch_count(h)
+    nolo.nolo_route(h, 11, 3, acts.view(torch.float32))
+    assert nolo.nolo_launch_count(h) - before == (1 if draws else 2)
     table = torch.from_numpy(O.draw_route(11, 3, stages, W, K, per_microbatch=True)).long()
     assert np.array_equal(nolo.nolo_get_route(h), table.numpy())
+    k = torch.arange(K)[:, None].cuda()
     for b in range(stages - 1):
-        for k in range(K):
-            for r in range(W):
-                assert torch.equal(out[b, r, k].view(torch.int32), acts[b, int(table[b, k, r]), k].view(torch.int32))
-    nolo.nolo_route_backward(h, 11, 3, out, back)
+        from_replica = table[b].cuda()                          # [K][W]
+        for r in range(W):
+            assert torch.equal(out[b, r], acts[b][from_replica[:, r], k[:, 0]])
+    nolo.nolo_route_backward(h, 11, 3, out.view(torch.float32), back.view(torch.float32))
     torch.cuda.synchronize()
-    assert torch.equal(back.view(torch.int32), acts.view(torch.int32))
+    assert torch.equal(back, acts)
     nolo.nolo_destroy(h)
