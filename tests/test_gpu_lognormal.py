@@ -46,34 +46,40 @@ def probe(tmp_path_factory):
     return fn
 
 
-def words():
-    """Both ends of every interval of the tables, the ends of the whole range, and random words."""
+def words(sigma):
+    """Both ends of every interval of the tables (of the power table next to them), the ends of the whole range, and random words."""
     rng = np.random.default_rng(3)
     radius, angle = [0, 1, 2, 3, 2**53 - 1, 2**53 - 2, 2**53 - 3], [0, 1, 2**53 - 1]
-    for e in range(0, 54, 3):                                   # u = m 2^(e - 54), m at the ends of the 128 intervals
-        for j in range(129):
-            m = 0.6875 + j / 128 * (0.5 if j < 80 else 1.0) if e == 0 else 0.5 + j / 256
-            radius += [int(m * 2.0**e) + d for d in (-1, 0, 1)]
+    # u = m 2^(e - 53), m at the ends of the logarithm's 512 intervals of [0.6875, 1.375), which are 2^-10 wide below 1
+    ends = [0.6875 + j / 1024 for j in range(320)] + [1.0 + j / 512 for j in range(193)]
+    for e in range(54):
+        radius += [int(m * 2.0**e) + d for m in ends for d in (-1, 0, 1)]
     for j in range(1, 129):                                     # u next to 1, where nothing may cancel
         radius += [2**53 - j, 2**53 - (j << 40), 2**53 - (j << 45)]
-    for j in range(257):
-        angle += [(j << 45) + d for d in (-1, 0, 1)]
-        angle += [(j << 45) + (1 << 44) + d for d in (-1, 0, 1)]      # the middle of the entry
-    radius = np.array([x for x in radius if 0 <= x < 2**53], dtype=np.uint64)
+    for j in range(513):                                        # the 512 entries of sine and cosine
+        angle += [(j << 44) + d for d in (-1, 0, 1)]
+        angle += [(j << 44) + (1 << 43) + d for d in (-1, 0, 1)]      # the middle of the entry
+    radius = np.unique(np.array([x for x in radius if 0 <= x < 2**53], dtype=np.uint64))
     angle = np.array([x for x in angle if 0 <= x < 2**53], dtype=np.uint64)
+    # sigma r half-way between two entries of the power table, 2^(1 / 2048) apart, at angles 0 and pi: of each sign
+    half = (np.arange(0, 8.5 * sigma * 2048 / np.log(2), max(1.0, sigma)) + 0.5) * np.log(2) / 2048 / sigma
+    half = (np.exp(-0.5 * half * half) * 2.0**53).astype(np.uint64)
     n = 1 << 19
+    assert max(len(radius), 2 * len(half)) <= n // 4
     wa = rng.integers(0, 2**53, n, dtype=np.uint64)
     wb = rng.integers(0, 2**53, n, dtype=np.uint64)
     wa[:len(radius)] = radius
-    wb[n // 2:n // 2 + len(angle)] = angle
     wa[n // 4:n // 4 + len(radius)], wb[n // 4:n // 4 + len(radius)] = radius, rng.choice(angle, len(radius))
+    wb[n // 2:n // 2 + len(angle)] = angle
+    for at, turn in ((3 * n // 4, 0), (7 * n // 8, 2**52)):
+        wa[at:at + len(half)], wb[at:at + len(half)] = half, turn
     low = rng.integers(0, 2**11, n, dtype=np.uint64)            # the bits that are not used
     return (wa << np.uint64(11)) | low, (wb << np.uint64(11)) | low
 
 
 @pytest.mark.parametrize("mu,sigma", [(0.0, 1.0), (1.0, 0.5**0.5), (0.0, 0.1), (-3.0, 2.5), (0.5, 1e-9), (300.0, 40.0), (0.0, 80.0)])
 def test_times_are_good_to_a_few_units_in_the_last_place(probe, mu, sigma):
-    wa, wb = words()
+    wa, wb = words(sigma)
     a, b = (torch.from_numpy(x.view(np.int64)).cuda() for x in (wa, wb))
     out = torch.empty((len(wa), 2), dtype=torch.float64, device="cuda")
     torch.cuda.synchronize()
@@ -94,11 +100,11 @@ def test_times_are_good_to_a_few_units_in_the_last_place(probe, mu, sigma):
     c = cos8[q] * np.cos(rest) - sin8[q] * np.sin(rest)
     s = sin8[q] * np.cos(rest) + cos8[q] * np.sin(rest)
     # Units of 2^-53: the radius is good to 3 (logarithm and square root), sine and cosine to 2 of 1; the exponent is
-    # formed from mu and sigma scaled to units of ln 2 / 256 (2 each for the scaled values, 1 for the sum), and each unit
-    # of it is a unit of the time relative to 1; the power itself is good to 3.
+    # formed from sigma scaled to units of ln 2 / 2048 (2 for the scaled value, 1 for the sum), and each unit
+    # of it is a unit of the time relative to 1; the power itself, e^mu 2^(j / 2048) from a table, is good to 3.
     for k, trig in ((0, c), (1, s)):
         want = np.exp(L(mu) + L(sigma) * (r * trig))
-        unit = 2.0 ** -53 * (3 + 3 * abs(mu) + 8 * sigma * np.maximum(r, 1e-30).astype(np.float64))
+        unit = 2.0 ** -53 * (3 + 8 * sigma * np.maximum(r, 1e-30).astype(np.float64))
         err = np.abs((got[:, k].astype(L) - want) / want).astype(np.float64)
         worst = int(np.argmax(err / unit))
         assert (err <= unit).all(), (hex(wa[worst]), hex(wb[worst]), err[worst] / unit[worst])
