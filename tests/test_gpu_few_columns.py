@@ -178,7 +178,7 @@ def test_results_at_the_size_where_they_are_copied(nolo, trials):
     assert np.array_equal(per[:50], few) and (per > 0).all()
 
 
-# One subgroup of all workers; partitions of 4 to 32 lanes each; pairs and other subgroups; several slabs of each; the last
+# One subgroup of all workers; partitions of 4 to 32 lanes each; pairs and other subgroups; the last
 # block of an item with one to four inner steps.
 @pytest.mark.parametrize("W,n,H,T,trials", [
     (3, 3, 5, 40, 3), (64, 64, 6, 33, 2), (4096, 4096, 2, 3, 2), (4, 2, 7, 37, 9), (5, 1, 3, 4, 7), (8, 4, 4, 9, 3), (9, 3, 1, 5, 2),
@@ -191,14 +191,16 @@ def test_straggler_rules(nolo, W, n, H, T, trials):
         assert np.array_equal(per[:, 0], per[:, 1])
 
 
-@pytest.mark.parametrize("W,n,H,T,trials", [(1024, 1024, 1, 5, 900), (512, 2, 2, 9, 700), (64, 64, 40, 37, 900), (4, 2, 30, 250, 300),
-                                            (5, 5, 9, 250, 300), (16, 2, 130, 112, 160), (63, 3, 6, 61, 80), (3, 3, 13, 90, 1200)])
+# One slab (the first five) and several, of 31 * 2^16 work sums, from which pairs, the members of small subgroups, shared subgroups, more than
+# 1024 workers and one subgroup of all go on.
+@pytest.mark.parametrize("W,n,H,T,trials", [
+    (4, 2, 30, 250, 300), (5, 5, 9, 250, 300), (16, 2, 130, 112, 160), (63, 3, 6, 61, 80), (3, 3, 13, 90, 1200),
+    (64, 64, 40, 37, 900), (1024, 1024, 1, 5, 900), (512, 2, 2, 9, 700), (256, 8, 2, 40, 300), (252, 7, 2, 40, 300),
+    (15, 3, 2, 100, 1500), (1024, 8, 2, 5, 900), (1024, 32, 2, 3, 2000), (288, 9, 1, 30, 300), (2048, 2, 2, 4, 600)])
 def test_straggler_slabs_and_shared_rows(nolo, W, n, H, T, trials):
-    """Several slabs; the first and last trials are those of the oracle or of a small call."""
     *_, per = nolo.nolo_sim_straggler(W, n, H, T, 0.4, 0.8, trials, 21, return_trials=True)
-    *_, few = nolo.nolo_sim_straggler(W, n, H, T, 0.4, 0.8, 2, 21, return_trials=True)
-    np.testing.assert_allclose(per[:2], few, rtol=1e-14)
-    np.testing.assert_allclose(few, L.sim_straggler(W, n, H, T, 0.4, 0.8, 2, 21), rtol=1e-11)
+    for first in (0, trials // 2, trials - 2):
+        np.testing.assert_allclose(per[first:first + 2], L.sim_straggler(W, n, H, T, 0.4, 0.8, 2, 21, first), rtol=1e-11)
     assert (per[:, 1] <= per[:, 0] * (1 + 1e-15)).all() and (per > 0).all()
 
 
@@ -216,27 +218,37 @@ def test_straggler_units_across_trials(nolo, W, n, H, T, trials, sigma):
 
 
 def test_calls_of_different_sizes_from_several_threads(nolo):
-    """The kernels' shared memory depends on the sizes; what one call sets up must do for the others."""
+    """The kernels' shared memory depends on the sizes; what one call sets up must do for the others.  Every call gives what
+    it gives when nothing else runs."""
     import threading
     trees, stragglers, states = [(1024, 300), (64, 300), (4096, 20), (2048, 20)], [(1024, 512), (100, 10), (64, 2), (1024, 2)], [130, 1024, 256, 700]
-    want = {}
+
+    def calls(k):
+        """The simulations of every turn and, at the end, the state."""
+        stream = torch.cuda.Stream()
+        dev = [x.cuda() for x in synth.make_state(states[k], 900, k)]
+        h = nolo.nolo_create(states[k], states[k], 900, 1, *HP)
+        torch.cuda.synchronize()
+        nolo.nolo_bind_state(h, *dev, stream=stream)
+        sims = []
+        for turn in range(30):
+            sims += [nolo.nolo_sim_tree_allreduce(trees[k][0], 0.0, 1.0, trees[k][1], 3, stream, return_trials=True)[2],
+                     nolo.nolo_sim_straggler(*stragglers[k], 3, 4, 0.0, 0.5, 5, 3, stream, return_trials=True)[4]]
+            nolo.nolo_outer_step(h, 1, turn)
+        stream.synchronize()
+        nolo.nolo_destroy(h)
+        return sims, [x.cpu() for x in dev]
+
+    want = [calls(k) for k in range(4)]
     bad = []
 
     def work(k):
         try:
-            stream = torch.cuda.Stream()
-            dev = [x.cuda() for x in synth.make_state(states[k], 900, k)]
-            h = nolo.nolo_create(states[k], states[k], 900, 1, *HP)
-            torch.cuda.synchronize()
-            nolo.nolo_bind_state(h, *dev, stream=stream)
-            for turn in range(30):
-                got = (nolo.nolo_sim_tree_allreduce(*trees[k][:1], 0.0, 1.0, trees[k][1], 3, stream, return_trials=True)[2],
-                       nolo.nolo_sim_straggler(*stragglers[k], 3, 4, 0.0, 0.5, 5, 3, stream, return_trials=True)[4])
-                nolo.nolo_outer_step(h, 1, turn)
-                if not all(np.array_equal(a, b) for a, b in zip(got, want.setdefault(k, got))):
-                    bad.append(k)
-            stream.synchronize()
-            nolo.nolo_destroy(h)
+            sims, state = calls(k)
+            if not all(np.array_equal(a, b) for a, b in zip(sims, want[k][0])):
+                bad.append(f"simulations {k}")
+            if not all(torch.equal(a, b) for a, b in zip(state, want[k][1])):
+                bad.append(f"state {k}")
         except Exception as e:
             bad.append(e)
 
