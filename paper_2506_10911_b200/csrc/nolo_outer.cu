@@ -761,21 +761,22 @@ group_mean_kernel(const float* phi, const int32_t* perm, int n, int64_t stride,
 // the CTA's threads bring the members of 4 QUADS columns to shared memory, three stages of 8 KB ahead, and a thread per column adds
 // them in the order of the kernel above, so that no bit depends on the number of columns.  Bound by latency up to about a
 // hundred members, then by the additions, whose chain is 4 cycles and whose 7 instructions a member has in each column's thread
-// alone.  (Groups of threads that share out the members and join their sums in a tree took 126 us at (1024, 37 888) and gave other
+// alone.  (Groups of threads that share out the members and join their sums in a tree took 124 us at (1024, 37 888) and gave other
 // bits than a thread per quad; rows brought through registers, one stage of 16 KB ahead, 189.)
 //
-// It does not let its successor start early: the step that follows would find the SMs set up for this kernel's shared memory and
-// keep them so, with little L1 left for its loads in flight (prepare and prepared step (1024, 24 415) 192 us, now 154,
-// (64, 300 000) 118, now 95).
+// It lets its successor start early for small states only: else the step that follows would find the SMs set up for this kernel's
+// shared memory and keep them so, with little L1 left for its loads in flight.  us of prepare and prepared step, early / not, n = W:
+// (1024, 24 415) 192 / 154, (64, 300 000) 118 / 95, (96, 66 666) 36.9 / 31.1, (256, 6251) 18.8 / 19.1, (1024, 1563) 31.0 / 32.9.
 constexpr int kMeanStages = 4, kMeanStageQuads = 2 * kThreads;
 
 template <int QUADS>
 __global__ void __launch_bounds__(kThreads)
 staged_mean_kernel(const float* phi, const int32_t* perm, int n, int64_t stride, int64_t P, double* __restrict__ mean,
-                   int64_t mean_stride, double inv_n) {
+                   int64_t mean_stride, double inv_n, bool early) {
     constexpr int COLS = 4 * QUADS, ROWS = kMeanStageQuads / QUADS, HALF = ROWS / 2;
     __shared__ float4 staged[kMeanStages][ROWS][QUADS];
     wait_for_predecessors();
+    if (early) let_successor_start();
     const int g = blockIdx.y;
     const int32_t* members = perm + (int64_t)g * n;
     mean += (int64_t)g * mean_stride;
@@ -947,13 +948,14 @@ cudaError_t dispatch(KArgs& k, bool draw, int groups, cudaStream_t stream) {
 
 }  // namespace
 
-// Few columns: at most two CTAs of 256 quads per SM (one for fewer than 32 members, which a thread walks in few latencies).  us of a draw
-// and the means (the draw alone 5.7), a thread per quad / staged, one subgroup of n, quads: (32, 18 944) 7.8 / 5.8, (20, 75 776) 7.6 / 9.7, (32, 75 776) 11.4 /
-// 10.6, (32, 303 104) 30 / 36, (64, 9472) 13.2 / 6.0, (128, 37 888) 34 / 15, (256, 18 944) 65 / 19, (1024, 37 888) 271 / 111.
-// Row pieces of 128 bytes where CTAs of 512-byte ones would leave SMs idle: (1024, 1024) 25.9 / 14.0, (256, 1024) 7.6 / 5.9,
-// (256, 4096) 7.7 / 8.6.
-constexpr int64_t kMeanFewQuads = 148 * 256, kMeanNarrowCtas = 148 * 2;
-constexpr int kMeanDirectMaxN = 16, kMeanManyN = 32;
+// Few columns: up to two CTAs of 256 quads per SM, three quarters of one for fewer than 32 members, which a thread walks in few latencies.
+// us of a draw (alone 5.7) and the means, a thread per quad / staged, one subgroup of n, quads: (24, 28 416) 6.8 / 5.7, (20, 37 888) 6.2 / 6.9,
+// (32, 37 888) 8.3 / 7.3, (32, 75 776) 12.8 / 11.0, (64, 9472) 13.2 / 5.8, (128, 37 888) 35 / 17, (256, 18 944) 66 / 18, (1024, 37 888) 273 /
+// 115.  Row pieces of 128 bytes for the smallest of them, where 512-byte ones leave SMs idle: (128, 4096) 5.9, of 512 bytes 6.5, (256, 4096) 8.2 / 9.5,
+// (1024, 4096) 19.8 / 29.4, (64, 9472) 6.3 / 5.8, (256, 9472) 13.0 / 12.2, (1024, 9472) 37 / 41.
+constexpr int64_t kMeanFewQuads = 148 * 512, kMeanFewQuadsSmall = 148 * 192, kMeanNarrowQuads = 148 * 32;
+constexpr int64_t kMeanEarlyQuads = 1 << 19;       // of all members
+constexpr int kMeanDirectMaxN = 16, kMeanSmallMaxN = 31;
 
 cudaError_t launch_group_mean(const float* phi, const int32_t* perm, int W, int n, int64_t stride, int64_t P,
                               double* mean, int64_t mean_stride, cudaStream_t stream) {
@@ -964,16 +966,16 @@ cudaError_t launch_group_mean(const float* phi, const int32_t* perm, int W, int 
     const double inv_n = 1.0 / (double)n;
     // rows of the means are 32-byte aligned when the base is (the stride is a multiple of 64 bytes)
     const bool wide = (reinterpret_cast<uintptr_t>(mean) & 31u) == 0;
-    auto launch = [&](auto kernel, int64_t quads_per_cta) {
+    auto launch = [&](auto kernel, int64_t quads_per_cta, auto... more) {
         const int64_t tiles = (quads + quads_per_cta - 1) / quads_per_cta + ((P & 3) != 0);
         if (tiles > 0x7fffffffll) return cudaErrorInvalidConfiguration;
         return launch_overlapped(kernel, dim3((unsigned)tiles, (unsigned)groups), kThreads, 0, stream, phi, perm, n, stride, P, mean,
-                                 mean_stride, inv_n);
+                                 mean_stride, inv_n, more...);
     };
     if (n <= 4) return launch(wide ? group_mean_kernel<2, true> : group_mean_kernel<2, false>, 2 * kThreads);
-    if (n > kMeanDirectMaxN && quads * groups <= (n < kMeanManyN ? 1 : 2) * kMeanFewQuads) {
-        if ((quads + 7) / 8 * groups <= kMeanNarrowCtas) return launch(staged_mean_kernel<8>, 8);
-        return launch(staged_mean_kernel<32>, 32);
+    if (n > kMeanDirectMaxN && quads > 0 && quads * groups <= (n <= kMeanSmallMaxN ? kMeanFewQuadsSmall : kMeanFewQuads)) {
+        const bool early = quads * W <= kMeanEarlyQuads;
+        return quads * groups <= kMeanNarrowQuads ? launch(staged_mean_kernel<8>, 8, early) : launch(staged_mean_kernel<32>, 32, early);
     }
     return launch(wide ? group_mean_kernel<1, true> : group_mean_kernel<1, false>, kThreads);
 }

@@ -54,7 +54,7 @@ def test_bits_do_not_depend_on_the_number_of_columns(nolo, W, n, P, bf16):
 # A thread per quad or the members staged in pieces of 8 or 32 quads, in one to many stages of 64 or 16 rows.
 @pytest.mark.parametrize("W,n,P", [(5, 5, 3), (7, 7, 1030), (15, 15, 2051), (16, 16, 4096), (63, 63, 517), (64, 64, 514), (65, 65, 4097),
                                    (130, 130, 6), (24, 12, 80_003), (64, 32, 40_001), (128, 128, 20_003),
-                                   (17, 17, 4 * 2368 + 1), (34, 17, 4 * 1185), (1024, 1024, 9475), (2049, 2049, 260), (193, 193, 30_002)])
+                                   (17, 17, 4 * 4736 + 1), (34, 17, 4 * 2369), (1024, 1024, 9475), (2049, 2049, 260), (193, 193, 30_002), (569, 569, 2)])
 def test_subgroup_means_of_few_columns(nolo, W, n, P):
     phi, theta, delta = synth.make_state(W, P, n, pad_value=float("nan"))
     dev = [x.cuda() for x in (phi, theta, delta)]
@@ -76,8 +76,8 @@ def test_subgroup_means_of_few_columns(nolo, W, n, P):
 def test_subgroup_means_do_not_depend_on_the_number_of_columns(nolo, W, n):
     """A state cut by columns has the means of the whole, bit for bit: 8 quads, and both sides of each line."""
     groups = W // n
-    few = 148 * 256 * (1 if n < 32 else 2) // groups
-    sizes = [32, 4 * (148 * 2 * 8 // groups), 4 * (148 * 2 * 8 // groups + 1), 4 * few, 4 * few + 4]
+    few, narrow = 148 * (192 if n < 32 else 512) // groups, 148 * 32 // groups
+    sizes = [32, 4 * narrow, 4 * narrow + 4, 4 * few, 4 * few + 4]
     cols = max(sizes)
     phi = 0.02 * torch.randn(W, synth.padded_stride(cols), device="cuda", generator=torch.Generator("cuda").manual_seed(n))
     z, d = torch.zeros_like(phi), torch.zeros_like(phi)
