@@ -572,7 +572,8 @@ outer_step_twopass_kernel(const KArgs a) {
 // its order, so every bit is the same, whatever the number of columns.
 //
 // Bound by latency: the table's, one read of all rows, three barriers.  (W, n, P) float32, us in a train, two passes / this: (32, 32, 3125)
-// 5.5 / 3.3, (60, 60, 1667) 9.8 / 5.1, (96, 96, 4166) 13.1 / 5.3, (256, 256, 1562) 11.1 / 7.5, (1024, 1024, 1563) 31.2 / 18.0.
+// 5.6 / 3.4, (60, 60, 1667) 10.3 / 5.5, (96, 96, 4166) 13.2 / 5.8, (256, 256, 1562) 11.1 / 7.2, (512, 512, 3125) 18.9 / 15.6,
+// (1024, 1024, 1563) 30.6 / 16.1.
 template <typename ThetaT, int THREADS, int ROWQ, int ROWS, bool DRAW>
 __global__ void __launch_bounds__(THREADS, 1)
 outer_step_staged_kernel(const KArgs a, int slots) {
