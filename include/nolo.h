@@ -348,7 +348,7 @@ double nolo_expected_pair_exchange(double mu, double sigma);
  *   host_stats   host, 4 doubles: mean time with the global barrier, mean time
  *           with subgroup waits, then the standard errors of the two means
  *   host_trials  host, [trials][2] (barrier, subgroup) per trial, or NULL
- * Synchronous; scratch as above (at most about 65 MB).  trials 1..2^20, and the
+ * Synchronous; scratch as above (at most about 67 MB).  trials 1..2^20, and the
  * total number of samples W*H*T*trials at most NOLO_SIM_MAX_SAMPLES (2^40, about
  * 20 s of GPU time): a larger request is refused with NOLO_EINVAL rather than
  * left to occupy the device.

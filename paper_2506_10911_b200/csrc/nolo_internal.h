@@ -109,7 +109,7 @@ cudaError_t launch_divergence(const float* phi, int W, int64_t stride, int64_t P
 size_t tree_scratch();
 cudaError_t launch_tree_allreduce(int W, double mu, double sigma, int64_t trials, uint64_t seed,
                                   double* per_trial, double* stats, double* copy, void* scratch, cudaStream_t stream);
-// scratch: device, straggler_scratch() bytes (at most about 49 MB).
+// scratch: device, straggler_scratch() bytes (at most about 50 MB).
 size_t straggler_scratch(int W, int T, int64_t trials);
 cudaError_t launch_straggler(int W, int n, int H, int T, double mu, double sigma, int64_t trials, uint64_t seed,
                              double* per_trial, double* stats, double* copy, void* scratch, cudaStream_t stream);

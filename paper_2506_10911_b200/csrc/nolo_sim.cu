@@ -636,8 +636,9 @@ cudaError_t launch_stats(const double* x, int64_t rows, double* out, double* cop
                              static_cast<double2*>(scratch), stats_counter(scratch), out, copy);
 }
 
-// Iterations and trials whose work sums are held at a time.
-constexpr int64_t kSlabItems = 31 << 16;
+// Iterations and trials whose work sums are held at a time: as many as keep a call's scratch with its results below the 64 MB that are kept
+// between calls (67.0e6 bytes at one worker, 2 iterations, 1 046 528 trials).
+constexpr int64_t kSlabItems = (1 << 21) - (1 << 12);
 
 // As few slabs as that allows, of equal sizes.
 int64_t even_share(int64_t all, int64_t most) {

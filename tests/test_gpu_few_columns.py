@@ -191,7 +191,7 @@ def test_straggler_rules(nolo, W, n, H, T, trials):
         assert np.array_equal(per[:, 0], per[:, 1])
 
 
-# One slab (the first five) and several, of 31 * 2^16 work sums, from which pairs, the members of small subgroups, shared subgroups, more than
+# One slab (the first five) and several, of 2^21 - 2^12 work sums, from which pairs, the members of small subgroups, shared subgroups, more than
 # 1024 workers and one subgroup of all go on.
 @pytest.mark.parametrize("W,n,H,T,trials", [
     (4, 2, 30, 250, 300), (5, 5, 9, 250, 300), (16, 2, 130, 112, 160), (63, 3, 6, 61, 80), (3, 3, 13, 90, 1200),
@@ -202,6 +202,22 @@ def test_straggler_slabs_and_shared_rows(nolo, W, n, H, T, trials):
     for first in (0, trials // 2, trials - 2):
         np.testing.assert_allclose(per[first:first + 2], L.sim_straggler(W, n, H, T, 0.4, 0.8, 2, 21, first), rtol=1e-11)
     assert (per[:, 1] <= per[:, 0] * (1 + 1e-15)).all() and (per > 0).all()
+
+
+def test_the_largest_scratch_of_stragglers_is_kept(nolo):
+    """One worker, two iterations and 1 046 528 trials need the most: 67.0e6 bytes, below the 2^26 that are kept (the driver hands memory
+    out in pieces of 2 MB)."""
+    def give_back():
+        nolo.nolo_destroy(nolo.nolo_create(2, 1, 8, 1, *HP))
+        torch.cuda.synchronize()
+
+    nolo.nolo_sim_straggler(1, 1, 1, 1, 0.0, 0.5, 10, 1)
+    give_back()
+    free = torch.cuda.mem_get_info()[0]
+    nolo.nolo_sim_straggler(1, 1, 1, 2, 0.0, 0.5, 1_046_528, 1)
+    assert 64 << 20 >= free - torch.cuda.mem_get_info()[0] >= 62 << 20
+    give_back()
+    assert free - torch.cuda.mem_get_info()[0] <= 4 << 20
 
 
 # Many trials leave a slab few iterations: units of 256 items lie across trials where one trial does not fill them.

@@ -210,7 +210,7 @@ int main() {
         for (int iterations = 1; iterations <= 60; iterations += iterations < 9 ? 1 : 7)
             for (long long trials : {1ll, 2ll, 3ll, 50ll, 700ll, 20000ll}) {
                 const int64_t work = (int64_t)W * iterations * trials;
-                if (work > 31 << 16) continue;
+                if (work > 1 << 21) continue;
                 const nolo::WorkUnits u = nolo::WorkUnits::of(W, iterations, trials, threads);
                 const int64_t laid = u.count * threads;
                 bool ok = 7 * laid <= 8 * work + 7 * threads;
