@@ -8,8 +8,7 @@
 // logarithm): a table in shared memory takes the leading bits, a short polynomial the rest.  Two arrangements are those of
 // the log and exp of Arm's optimized-routines: the logarithm's intervals of equal high word from 0.6875 on, found and reduced by
 // subtraction of integers, with a reciprocal of 1 next to 1; and powers stored with their index taken off the high word, so that one
-// addition of the shifted exponent puts either right.  The tables' values are computed from their definitions (the parts of
-// kLogGroup, kExpCoarse, kExpFine and kSinTable rounded from 60 digits).  The arguments are confined
+// addition of the shifted exponent puts either right.  The tables' values are computed from their definitions.  The arguments are confined
 // (u in (0, 1], angles as integers, exponents checked once on the host), so no special case is left in the loop, the
 // angle is reduced in integers and the factors 2, pi, sigma, e^mu and 2048 / ln 2 are folded into tables and constants.
 //

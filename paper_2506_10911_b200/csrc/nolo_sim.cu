@@ -195,8 +195,8 @@ tree_allreduce_kernel(int W, int lanes, int64_t trials, LogNormal q, uint64_t se
 // partitions do not.  So a slab of iterations is done by three kernels: the work sums (all of the random
 // times; any number of trials fills the chip), the partitions with the longest
 // work of each iteration (a CTA, a warp or a part of one each), and the clocks (one CTA per trial, one exchange
-// through shared memory per iteration for pairs and for the members of small subgroups, two for other subgroups).  Whole call, one CTA per trial for everything ->
-// three kernels -> now, (W, n, H, T, trials): (1024, 2, 100, 250, 148) 39.0 -> 16.1 -> 14.5 ms, (1024, 512, 100, 500, 8) 91.7 ->
+// through shared memory per iteration for pairs and for the members of small subgroups, two for other subgroups).
+// Whole call, one CTA per trial for everything -> three kernels -> now, (W, n, H, T, trials): (1024, 2, 100, 250, 148) 39.0 -> 16.1 -> 14.5 ms, (1024, 512, 100, 500, 8) 91.7 ->
 // 2.9 -> 2.3, (100, 100, 100, 500, 50) 16.9 -> 1.55 -> 0.97, (4, 2, 100, 500, 592) 15.7 -> 0.95 -> 0.57,
 // (64, 2, 50, 100, 8) 2.3 -> 0.11 -> 0.065.
 struct Slab {
